@@ -1194,6 +1194,13 @@ rr_status autotune(Graph &g, uint32_t k, uint32_t *best_ppl, uint32_t *best_chun
     RR_CUDA(cudaEventCreate(&e1));
     rr_query q{0, k, 0x7E57ull, nullptr};
     const uint32_t save_ppl = g.tune_ppl[k], save_chunk = g.tune_chunk[k];
+    // the candidates are shapes of the sieve-point engine: keep the query on it
+    // while they are timed
+    struct Forced {
+        bool &f, saved;
+        explicit Forced(bool &x) : f(x), saved(x) { f = true; }
+        ~Forced() { f = saved; }
+    } forced(g.tune_forced[k]);
     auto set_shape = [&](const Cand &c) {
         g.tune_ppl[k] = c.ppl;
         g.tune_chunk[k] = c.chunk;

@@ -176,7 +176,7 @@ rr_status rr_reach_sync(const rr_graph *g, const rr_query *q, uint8_t *bitmap, u
     if (bitmap)
         RR_CUDA(cudaMemcpyAsync(bitmap, g->ws.bitmap.p, nb, cudaMemcpyDeviceToHost, g->stream));
     RR_CUDA(cudaStreamSynchronize(g->stream));
-    return RR_OK;
+    return frontier_error(g->ws);
 }
 
 rr_status rr_reach_device(const rr_graph *g, const rr_query *q, uint8_t *d_bitmap,
@@ -387,6 +387,7 @@ rr_status rr_set_tuning(rr_graph *g, uint32_t k, uint32_t ppl, uint32_t chunk)
     std::lock_guard<std::mutex> lk(g->mu);
     g->tune_ppl[k] = ppl;
     g->tune_chunk[k] = chunk;
+    g->tune_forced[k] = ppl != 0 || chunk != 0;
     g->tune_gen++;
     return RR_OK;
 }

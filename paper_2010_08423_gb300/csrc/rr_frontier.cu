@@ -1,0 +1,1652 @@
+// rr_frontier.cu -- the frontier engine: a query's sums over the rows that
+// matter to it, without sieve points.
+//
+// Rows that matter. P_l[e] can be non-zero only when a walk of l edges from the
+// source ends with e, and it reaches an output only when a walk goes on from e
+// to the query's last layer. Both sets are found first, per layer, as bitmaps
+// over the row lists: forward, a row is active at layer l when its window holds
+// a row active at l - 1 (k_plan); backward, an active row is needed when a
+// needed row of the next layer has it in its window. The layers then run over
+// the needed rows alone, stored densely in list order (k_wedge).
+//
+// Wedge form. Summed over all sieve points L, a walk contributes the permanent
+// of its vertices' z rows, which in characteristic 2 is their determinant.
+//  * Columns are eliminated with the source's row: with pivot label p
+//    (z_{s,p} != 0) and rho_j = z_{s,j} / z_{s,p}, z'_{u,j} = z_{u,j} + z_{u,p}
+//    rho_j leaves the determinant unchanged and makes z'_s zero outside p, so it
+//    is z_{s,p} times the determinant of the other vertices' z' over the
+//    K = k - 1 other labels.
+//  * That determinant is the wedge product of the z' rows, so layer l keeps per
+//    row the values on the (l-1)-subsets of the K labels instead of one per
+//    sieve point: R_l[e]_T = y_{e,l} sum_{j in T} z'_{u,j} W_{T\j}, u the tail
+//    of e, W = the sum of R_{l-1} over e's window (layer 1: y_{e,1} z_{s,p});
+//    the last layer ends with witness[w] += sum_j z'_{w,j} (sum of R_{k-1})_{[K]\j}.
+// Each value is the same element of GF(2^64) as the sum over the sieve points.
+//
+// Why. On a Chung-Lu graph with n = 1e6, m = 1e7 the sieve-point engine
+// multiplies 1,024 points for each of 330,000 rows at each layer of a k = 10
+// query; walks from the source that reach the last layer pass 1,400 to 62,000
+// of them per layer, with at most 126 values each. Measured there 21 to 25 ms ->
+// 0.9 to 1.0 ms a query; n = 2e5, m = 2e6, k = 12: 23 -> 0.9 ms; a dense contact
+// graph (n = 2,000, m = 30,011, k = 12): 4.6 -> 0.26 ms; uniform n = 1e5, m = 1e6,
+// k = 8 (a handful of rows): 0.053 -> 0.033 ms; n = 1,000, k = 5: 26 -> 25 us.
+#include <algorithm>
+#include <cstring>
+#include <type_traits>
+
+#include "rr_frontier.cuh"
+
+namespace rr {
+
+namespace {
+
+constexpr int kThreads = 512;
+constexpr int kWarps = kThreads / 32;
+constexpr uint32_t kTeamLog = 4;      // log2 of the warps of a wedge block
+constexpr uint32_t kMaxRows = 16;     // rows of one wedge item
+constexpr uint32_t kSplit = 36;       // words of a split multiplier: 9 pieces of 3 classes, each padded to 16 bytes
+constexpr uint32_t kSup1 = 16, kSup2 = 256;  // blocks per partial sum
+// Bitmap words per scan tile: one tile up to 8,192 words (a block scans them in
+// 8 steps), else at most 256 tiles of whole 1,024s.
+__host__ __device__ constexpr uint32_t x_tile_words(uint32_t words)
+{
+    return words <= 8192u ? 8192u : ((words + 255u) / 256u + 1023u) / 1024u * 1024u;
+}
+
+__host__ __device__ constexpr uint32_t x_binom(uint32_t n, uint32_t d)
+{
+    uint64_t r = 1;
+    if (d > n) return 0;
+    for (uint32_t i = 1; i <= d; ++i) r = r * (n - d + i) / i;
+    return (uint32_t)r;
+}
+
+// the same at run time (n, d <= kXMaxLabels + 1)
+__constant__ uint16_t c_binom[kXMaxLabels + 2][kXMaxLabels + 2];
+__constant__ uint32_t c_tab_off[kXMaxLabels + 2];
+__device__ __forceinline__ uint32_t x_binom_dev(uint32_t n, uint32_t d) { return c_binom[n][d]; }
+
+// Subset tables: for every subset size d and d-subset T of [kXMaxLabels] in
+// colexicographic order, element i of T and the rank of T without it, packed
+// j | rank << 8, stored [i][T]. Colex order lists the subsets of the first K
+// labels first, so one table serves every K.
+__host__ __device__ constexpr uint32_t x_tab_off(uint32_t d)
+{
+    uint32_t o = 0;
+    for (uint32_t i = 1; i < d; ++i) o += i * x_binom(kXMaxLabels, i);
+    return o;
+}
+
+__device__ __forceinline__ uint32_t x_tab_off_dev(uint32_t d) { return c_tab_off[d]; }
+
+__global__ void __launch_bounds__(128) k_subset_table(uint32_t *__restrict__ tab)
+{
+    constexpr uint32_t W = kXMaxLabels + 1;
+    __shared__ uint32_t bin[W][W];
+    for (uint32_t i = threadIdx.x; i < W * W; i += blockDim.x) bin[i / W][i % W] = x_binom(i / W, i % W);
+    __syncthreads();
+    const uint32_t d = blockIdx.y + 1, cm = bin[kXMaxLabels][d];
+    const uint32_t T = blockIdx.x * blockDim.x + threadIdx.x;
+    if (T >= cm) return;
+    uint32_t set = 0, t = T, c = kXMaxLabels;
+    for (uint32_t i = d; i >= 1; --i) {  // the largest c with C(c, i) <= t
+        do --c;
+        while (bin[c][i] > t);
+        set |= 1u << c;
+        t -= bin[c][i];
+    }
+    // rank without element i: the elements above it move down one place
+    uint32_t below = 0, above = 0, pos = 0;
+    for (uint32_t m = set; m; m &= m - 1) {
+        const uint32_t e = (uint32_t)__ffs((int)m) - 1u;
+        if (pos) above += bin[e][pos];  // places 1.. with the lowest element gone
+        ++pos;
+    }
+    pos = 0;
+    uint32_t *o = tab + x_tab_off(d) + T;
+    for (uint32_t m = set; m; m &= m - 1) {
+        const uint32_t e = (uint32_t)__ffs((int)m) - 1u;
+        o[pos * cm] = e | ((below + above) << 8);
+        const uint32_t rest = m & (m - 1);
+        below += bin[e][pos + 1];
+        if (rest) above -= bin[__ffs((int)rest) - 1][pos + 1];
+        ++pos;
+    }
+}
+
+__device__ __forceinline__ uint64_t now_ns()
+{
+    uint64_t t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
+
+// The blocks that work together: the whole grid (cooperative launch, a barrier
+// on a counter in device memory), or one block with a query of its own. The
+// counter wait is bounded by time and by iterations; when it gives up it sets
+// the error flag, and the blocks return.
+struct View {
+    uint32_t b, n;  // this block among n
+    uint32_t *ctr, *err;
+    uint32_t target;
+    // worker w of n, the items before `base` dealt out: its first item from there on
+    __device__ static uint32_t first_item(uint32_t base, uint32_t w, uint32_t n)
+    {
+        if (!base) return w;
+        const uint32_t r = base % n;
+        return w >= r ? w - r : w + n - r;
+    }
+    __device__ bool sync()
+    {
+        if (n == 1) {
+            __syncthreads();
+            return true;
+        }
+        __shared__ int ok;
+        target += n;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            __threadfence();
+            atomicAdd(ctr, 1u);
+            int good = 0;
+            const uint64_t t0 = now_ns();
+            for (uint32_t it = 0; it < 200000000u; ++it) {
+                uint32_t v;
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(ctr) : "memory");
+                if ((int32_t)(v - target) >= 0) {
+                    good = 1;
+                    break;
+                }
+                if ((it & 1023u) == 1023u && (*(volatile uint32_t *)err || now_ns() - t0 > 10000000000ull)) break;
+            }
+            if (!good) *(volatile uint32_t *)err = 1u;
+            __threadfence();
+            ok = good;
+        }
+        __syncthreads();
+        return ok != 0;
+    }
+};
+
+// Some active row at positions [lo, hi) of a bitmap.
+__device__ __forceinline__ bool any_in(const uint32_t *A, uint32_t lo, uint32_t hi)
+{
+    if (hi <= lo) return false;
+    const uint32_t w0 = lo >> 5, w1 = (hi - 1) >> 5;
+    const uint32_t m0 = 0xffffffffu << (lo & 31u), m1 = 0xffffffffu >> (31u - ((hi - 1) & 31u));
+    if (w0 == w1) return (A[w0] & m0 & m1) != 0;
+    if ((A[w1] & m1) || (A[w0] & m0)) return true;
+    for (uint32_t w = w0 + 1; w < w1; ++w)
+        if (A[w]) return true;
+    return false;
+}
+
+// Needed rows of a level at positions below x.
+__device__ __forceinline__ uint32_t rank_below(const XLL &L, uint32_t x)
+{
+    const uint32_t w = x >> 5;
+    return L.pc[w] + __popc(L.N[w] & ((1u << (x & 31u)) - 1u));
+}
+
+// One wedge item: 1 << rows consecutive needed rows of a level, taken by a team
+// of 1 << team warps. Few rows get large teams (all warps of a block on one
+// row: the layer's latency counts), many rows one warp each (no block-wide
+// waits; the warps cover each other's loads): of the team sizes whose share of
+// shared memory holds a row, the one whose busiest team has the fewest product
+// steps, a row's fixed cost (loads, draws, multipliers) counted as kRowSteps.
+// Rows per item grow until every team has one item, at most kMaxRows and what
+// shared memory holds. The next level derives the same rows to read the prefix
+// sums. Chosen once per level list, by the thread that counts its rows.
+struct XShape {
+    uint32_t team, rows;  // log2
+};
+__device__ __forceinline__ XShape x_shape_of(uint32_t s) { return XShape{s & 0xffu, s >> 8}; }
+constexpr uint32_t kRowSteps = 6;
+__device__ __forceinline__ uint32_t x_item_bytes(uint32_t rows, uint32_t K, const XLL &X)
+{
+    return rows * (K * (4u * kSplit) + (X.cin + X.cout + X.uout) * 8u + 32u);
+}
+__device__ __noinline__ XShape x_choose_shape(uint32_t smem, uint32_t blocks, uint32_t cnt, uint32_t K, const XLL &X)
+{
+    XShape s{kTeamLog, 0u};
+    uint32_t best = 0xffffffffu;
+    for (uint32_t t = 0; t <= kTeamLog; ++t) {
+        if (t < kTeamLog && x_item_bytes(1u, K, X) > (smem >> (kTeamLog - t))) continue;
+        const uint32_t teams = blocks << (kTeamLog - t);
+        const uint32_t steps = X.out ? 1u : ((X.cout + (32u << t) - 1u) >> (5 + t)) * X.d;
+        const uint32_t cost = (cnt + teams - 1u) / teams * (steps + kRowSteps);
+        if (cost < best) {
+            best = cost;
+            s.team = t;
+        }
+    }
+    const uint32_t teams = blocks << (kTeamLog - s.team), share = smem >> (kTeamLog - s.team);
+    while ((1u << s.rows) < kMaxRows && cnt > (teams << s.rows) && x_item_bytes(2u << s.rows, K, X) <= share) ++s.rows;
+    return s;
+}
+
+// Carry-less inner products. gf64_mul splits both operands into 9 16-bit pieces
+// (two Karatsuba levels) of 3 bit classes; everything after the 81 integer
+// products of classes is linear, so a sum of products XORs them class by class
+// and is put together and reduced once. The multipliers of a row serve all its
+// subsets: their 27 words are formed once and read from shared memory, a piece
+// (three classes) at a time, so that a product holds few registers.
+// Per product this leaves 81 IMAD, about 41 three-input XORs and the 31
+// instructions that split the other operand, against 240 of gf64_mul.
+__device__ __forceinline__ uint64_t finish27(const uint32_t (&z)[27])
+{
+    uint64_t r[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        uint32_t c[3];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const uint32_t *q = z + 9 * i + 3 * j;
+            c[j] = (q[0] & 0x49249249u) | (q[1] & 0x92492492u) | (q[2] & 0x24924924u);
+        }
+        const uint32_t m = c[2] ^ c[0] ^ c[1];
+        r[i] = ((uint64_t)(c[1] ^ (m >> 16)) << 32) | (uint32_t)(c[0] ^ (m << 16));
+    }
+    const uint64_t m = r[2] ^ r[0] ^ r[1];
+    return gf64_reduce(r[1] ^ (m >> 32), r[0] ^ (m << 32));
+}
+
+// z'_{u,j}: the source's column eliminated (see the top of the file); a set of
+// sources keeps all k labels as they are.
+__device__ __forceinline__ uint64_t zprime(const XQuery &Q, const uint64_t *omega, const uint8_t *color, uint32_t u, uint32_t j)
+{
+    if (!Q.colored) {
+        const uint64_t zj = sm_draw(Q.key_z, (uint64_t)u * 32u + (j < Q.pivot ? j : j + 1u));
+        return Q.multi ? zj : zj ^ gf64_mul(sm_draw(Q.key_z, (uint64_t)u * 32u + Q.pivot), Q.rho[j]);
+    }
+    const uint32_t c = color[u], d0 = Q.first[c], mu = Q.mu[c];
+    uint64_t r = 0;
+    for (uint32_t d = d0; d < d0 + mu; ++d) r ^= gf64_mul(sm_draw(Q.key_g, (uint64_t)u * 32u + d), omega[d * Q.K + j]);
+    return r;
+}
+// omega'_{d,j} at i = d K + j: the shade factor with the source's column eliminated
+__device__ __forceinline__ uint64_t shade_factor(const XQuery &Q, uint32_t i)
+{
+    const uint32_t d = i / Q.K, j = i - d * Q.K;
+    const uint64_t oj = sm_draw(Q.key_o, (uint64_t)d * 32u + (j < Q.pivot ? j : j + 1u));
+    return Q.multi ? oj : oj ^ gf64_mul(sm_draw(Q.key_o, (uint64_t)d * 32u + Q.pivot), Q.rho[j]);
+}
+// A vertex walks may pass: it has a colour of M and is not deleted.
+__device__ __forceinline__ bool allowed(const XQuery &Q, const uint8_t *color, uint32_t v)
+{
+    if (Q.colored && !Q.mu[color[v]]) return false;
+    return !(Q.vmask && Q.vmask[v]);
+}
+
+// Forward and backward passes, ranks and row records of one query.
+__device__ __noinline__ bool x_plan(const XArgs &a, const XOne &o, View &v)
+{
+    const XQuery &Q = o.q;
+    const XTmpl &t = o.t;
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    const uint32_t gw = v.b * kWarps + warp, nw = v.n * kWarps;
+    const uint32_t gt = v.b * kThreads + threadIdx.x, nt = v.n * kThreads;
+    constexpr uint32_t U = 4;  // bitmap words per warp and step
+
+    // cleared first: needed-row bitmaps, flags
+    for (uint32_t i = gt; i < t.clear4; i += nt) t.clear[i] = make_uint4(0, 0, 0, 0);
+    if (v.b == 0)
+        for (uint32_t i = threadIdx.x; i < t.nll; i += kThreads) {
+            t.live[i] = t.ll[i].level == 1 ? 1u : 0u;
+            t.cnt[i] = 0;
+        }
+    if (Q.colored && v.b == v.n - 1)
+        // shade factors with the source's column eliminated
+        for (uint32_t i = threadIdx.x; i < Q.k * Q.K; i += kThreads) t.omega[i] = shade_factor(Q, i);
+    const bool check = Q.colored || Q.vmask;
+    uint32_t lmax = t.maxlev;
+    for (uint32_t l = 1; l <= t.maxlev; ++l) {
+        for (uint32_t li = t.runs[l].first; li < t.runs[l].first + t.runs[l].count; ++li) {
+            const XLL &X = t.ll[li];
+            const XList &L = a.lists[X.list];
+            const uint32_t steps = (L.words + U - 1) / U;
+            const uint32_t *const Ap = t.ll[X.prev].A;
+            if (l > 1 && !t.live[X.prev]) continue;
+            const bool none = Q.dead || (X.out && Q.pivot > l && !Q.multi);  // z_s is zero over the labels of k' = l + 1
+            bool warp_live = false;
+            for (uint32_t i = gw; i < steps; i += nw) {
+                const uint32_t w0 = i * U;
+                bool act[U];
+                if (l == 1) {
+                    uint32_t u[U];
+#pragma unroll
+                    for (uint32_t x = 0; x < U; ++x) {
+                        const uint32_t r = (w0 + x) * 32u + lane;
+                        u[x] = r < L.count ? L.src[r] : 0xffffffffu;
+                    }
+#pragma unroll
+                    for (uint32_t x = 0; x < U; ++x) {
+                        act[x] = Q.multi ? u[x] != 0xffffffffu && Q.smask[u[x]] : u[x] == Q.source && u[x] != 0xffffffffu;
+                        if (act[x] && Q.vmask && Q.vmask[u[x]]) act[x] = false;
+                    }
+                } else {
+                    uint32_t lo[U], hi[U];
+#pragma unroll
+                    for (uint32_t x = 0; x < U; ++x) {
+                        const uint32_t r = (w0 + x) * 32u + lane;
+                        lo[x] = r < L.count ? L.lo[r] : 0u;
+                        hi[x] = r < L.count ? L.hi[r] : 0u;
+                    }
+#pragma unroll
+                    for (uint32_t x = 0; x < U; ++x) act[x] = any_in(Ap, lo[x], hi[x]);
+                }
+                if (check) {
+#pragma unroll
+                    for (uint32_t x = 0; x < U; ++x)
+                        // walks through vertices without a colour of M, or deleted ones, are zero
+                        if (act[x] && !allowed(Q, a.color, L.head[(w0 + x) * 32u + lane])) act[x] = false;
+                }
+#pragma unroll
+                for (uint32_t x = 0; x < U; ++x) {
+                    const uint32_t word = __ballot_sync(0xffffffffu, act[x] && !none);
+                    if (lane == x && w0 + x < L.words) X.A[w0 + x] = word;
+                    warp_live |= word != 0;
+                }
+            }
+            // one write per block: one line written by every warp would queue in L2
+            const bool some = __syncthreads_or(warp_live);
+            if (some && threadIdx.x == 0 && l > 1) t.live[li] = 1u;
+        }
+        if (!v.sync()) return false;
+        if (l == 1) continue;
+        bool some = false;
+        for (uint32_t li = t.runs[l].first; li < t.runs[l].first + t.runs[l].count; ++li) some |= t.live[li] != 0;
+        if (!some) {
+            lmax = l - 1;
+            break;
+        }
+    }
+
+    // backward: the rows of layer l - 1 in the window of a needed row of layer l
+    // (at-most-k: every layer has outputs, every active row is needed)
+    if (!t.every)
+        for (uint32_t l = lmax; l >= 2; --l) {
+            for (uint32_t li = t.runs[l].first; li < t.runs[l].first + t.runs[l].count; ++li) {
+                const XLL &X = t.ll[li];
+                const XList &L = a.lists[X.list];
+                const uint32_t steps = (L.words + U - 1) / U;
+                if (!t.live[li]) continue;
+                const uint32_t *const Ap = t.ll[X.prev].A;
+                uint32_t *const Np = t.ll[X.prev].N;
+                for (uint32_t i = gw; i < steps; i += nw) {
+                    const uint32_t w0 = i * U;
+                    const uint32_t mine = lane < U && w0 + lane < L.words ? X.N[w0 + lane] : 0u;
+                    if (!__any_sync(0xffffffffu, mine != 0)) continue;
+                    uint32_t lo[U], hi[U];
+#pragma unroll
+                    for (uint32_t x = 0; x < U; ++x) {
+                        const bool on = (__shfl_sync(0xffffffffu, mine, (int)x) >> lane) & 1u;
+                        const uint32_t r = (w0 + x) * 32u + lane;
+                        lo[x] = on ? L.lo[r] : 0u;
+                        hi[x] = on ? L.hi[r] : 0u;
+                    }
+                    uint32_t m[U], have[U];  // the window's first words
+#pragma unroll
+                    for (uint32_t x = 0; x < U; ++x) {
+                        m[x] = have[x] = 0;
+                        if (hi[x] > lo[x]) {
+                            m[x] = Ap[lo[x] >> 5] & (0xffffffffu << (lo[x] & 31u));
+                            have[x] = Np[lo[x] >> 5];
+                        }
+                    }
+#pragma unroll
+                    for (uint32_t x = 0; x < U; ++x) {
+                        if (hi[x] <= lo[x]) continue;
+                        const uint32_t b0 = lo[x] >> 5, b1 = (hi[x] - 1) >> 5;
+                        const uint32_t last = 0xffffffffu >> (31u - ((hi[x] - 1) & 31u));
+                        if (b1 == b0) m[x] &= last;
+                        if (m[x] & ~have[x]) atomicOr(Np + b0, m[x]);
+                        for (uint32_t w = b0 + 1; w <= b1; ++w) {
+                            const uint32_t mw = Ap[w] & (w == b1 ? last : 0xffffffffu);
+                            if (mw & ~Np[w]) atomicOr(Np + w, mw);
+                        }
+                    }
+                }
+            }
+            if (!v.sync()) return false;
+        }
+
+    // ranks: exclusive popcounts per bitmap word, and the levels' row counts.
+    // Long bitmaps are cut into tiles, whose sums come first.
+    __shared__ uint32_t part[32];
+    if (threadIdx.x < 32) part[threadIdx.x] = 0;
+    __syncthreads();
+    bool tiled = false;
+    for (uint32_t l = 1; l <= lmax; ++l)
+        for (uint32_t li = t.runs[l].first; li < t.runs[l].first + t.runs[l].count; ++li)
+            tiled |= t.ll[li].words > x_tile_words(t.ll[li].words);
+    const uint32_t nll = t.runs[lmax].first + t.runs[lmax].count;  // level lists up to lmax
+    for (uint32_t pass = tiled ? 0u : 1u; pass < 2; ++pass) {
+        uint32_t base_item = 0;
+        for (uint32_t li = 0; li < nll; ++li) {
+            const XLL &X = t.ll[li];
+            const uint32_t words = X.words;
+            const uint32_t tw = x_tile_words(words), tiles = (words + tw - 1) / tw;
+            if ((pass == 0 && tiles == 1) || !t.live[li]) continue;  // block-uniform
+            for (uint32_t i = View::first_item(base_item, v.b, v.n); i < tiles; i += v.n) {
+                const uint32_t end = min(words, (i + 1) * tw);
+                uint32_t sum = 0;
+                if (pass == 0) {
+                    for (uint32_t w = i * tw + threadIdx.x; w < end; w += kThreads) sum += __popc(X.N[w]);
+                } else if (tiles > 1) {
+                    if (threadIdx.x < i) sum = X.tsum[threadIdx.x];  // rows before the tile
+                }
+                uint32_t run_base = 0;
+                if (tiles > 1) {
+                    sum = __reduce_add_sync(0xffffffffu, sum);
+                    __syncthreads();
+                    if (lane == 0) part[warp] = sum;
+                    __syncthreads();
+                    run_base = __reduce_add_sync(0xffffffffu, part[lane]);
+                }
+                if (pass == 0) {
+                    if (threadIdx.x == 0) X.tsum[i] = run_base;
+                    continue;
+                }
+                for (uint32_t w0 = i * tw; w0 < end; w0 += 4u * kThreads) {
+                    // four words per thread
+                    const uint32_t w = w0 + 4u * threadIdx.x;
+                    uint32_t c[4], mysum = 0;
+#pragma unroll
+                    for (uint32_t x = 0; x < 4; ++x) {
+                        c[x] = w + x < end ? __popc(X.N[w + x]) : 0u;
+                        mysum += c[x];
+                    }
+                    uint32_t inc = mysum;
+#pragma unroll
+                    for (int d = 1; d < 32; d <<= 1) {
+                        const uint32_t y = __shfl_up_sync(0xffffffffu, inc, d);
+                        if (lane >= (uint32_t)d) inc += y;
+                    }
+                    __syncthreads();
+                    if (lane == 31) part[warp] = inc;
+                    __syncthreads();
+                    const uint32_t other = part[lane];
+                    const uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? other : 0u);
+                    uint32_t at = run_base + before + inc - mysum;
+#pragma unroll
+                    for (uint32_t x = 0; x < 4; ++x) {
+                        if (w + x < end) X.pc[w + x] = at;
+                        at += c[x];
+                    }
+                    run_base += __reduce_add_sync(0xffffffffu, other);
+                }
+                if (end == words && threadIdx.x == 0) {
+                    t.cnt[li] = run_base;
+                    const XShape sh = x_choose_shape(a.smem, v.n, run_base, Q.K, X);
+                    t.shape[li] = sh.team | sh.rows << 8;
+                }
+            }
+            base_item += tiles;
+        }
+        if (!v.sync()) return false;
+    }
+
+    // the needed rows' windows, edges and tails, in list order
+    for (uint32_t li = 0; li < nll; ++li) {
+        const XLL &X = t.ll[li];
+        const XList &L = a.lists[X.list];
+        const uint32_t steps = (L.words + U - 1) / U;
+        if (!t.live[li]) continue;
+        const bool window = X.level > 1;
+        const XLL &P = t.ll[X.prev];
+        for (uint32_t i = gw; i < steps; i += nw) {
+            const uint32_t w0 = i * U;
+            const uint32_t mine = lane < U && w0 + lane < L.words ? X.N[w0 + lane] : 0u;
+            if (!__any_sync(0xffffffffu, mine != 0)) continue;
+            const uint32_t mypc = lane < U && w0 + lane < L.words ? X.pc[w0 + lane] : 0u;
+            uint32_t lo[U], hi[U], at[U];
+#pragma unroll
+            for (uint32_t x = 0; x < U; ++x) {
+                const uint32_t word = __shfl_sync(0xffffffffu, mine, (int)x);
+                at[x] = __shfl_sync(0xffffffffu, mypc, (int)x) + __popc(word & ((1u << lane) - 1u));
+                const bool on = (word >> lane) & 1u;
+                const uint32_t r = (w0 + x) * 32u + lane;
+                lo[x] = hi[x] = 0;
+                if (!on) {
+                    at[x] = 0xffffffffu;
+                } else if (window) {
+                    lo[x] = L.lo[r];
+                    hi[x] = L.hi[r];
+                }
+            }
+#pragma unroll
+            for (uint32_t x = 0; x < U; ++x)
+                if (at[x] != 0xffffffffu) {
+                    const uint32_t r = (w0 + x) * 32u + lane;
+                    X.meta[at[x]] = make_uint4(window ? rank_below(P, lo[x]) : 0u, window ? rank_below(P, hi[x]) : 0u,
+                                               L.eid[r], L.src[r]);
+                    if (X.mhead) X.mhead[at[x]] = L.head[r];
+                    if (X.mtime) X.mtime[at[x]] = L.time[r];
+                }
+        }
+    }
+    // the partial sums of layer 1's blocks
+    for (uint32_t li = t.runs[1].first; li < t.runs[1].first + t.runs[1].count; ++li) {
+        const XLL &X = t.ll[li];
+        const uint32_t c = t.cnt[li];
+        if (X.out || !c) continue;
+        const uint32_t words = (c / kSup1 + 1 + c / kSup2 + 1) * (X.cout + X.uout);
+        for (uint32_t w = gt; w < words; w += nt) X.sup[w] = 0;
+    }
+    return v.sync();
+}
+
+__device__ __forceinline__ void store_split(uint32_t *o, uint64_t v)
+{
+    const uint32_t w[3] = {(uint32_t)v, (uint32_t)(v >> 32), (uint32_t)v ^ (uint32_t)(v >> 32)};
+    uint4 *q = reinterpret_cast<uint4 *>(o);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const uint32_t x[3] = {w[i], w[i] >> 16, w[i] ^ (w[i] >> 16)};
+#pragma unroll
+        for (int j = 0; j < 3; ++j) q[3 * i + j] = make_uint4(x[j] & 0x9249u, x[j] & 0x2492u, x[j] & 0x4924u, 0u);
+    }
+}
+
+// sum over the d elements j of subset T of m_j w_{T \ j} (m: split multipliers)
+__device__ __forceinline__ uint64_t wedge_at(const uint32_t *__restrict__ tb, uint32_t cm, uint32_t T, uint32_t d,
+                                             const uint32_t *m, const uint64_t *w)
+{
+    uint32_t z[27];
+#pragma unroll
+    for (int i = 0; i < 27; ++i) z[i] = 0;
+    uint32_t e = __ldg(tb + T);
+#pragma unroll 1
+    for (uint32_t i = 1; i <= d; ++i) {
+        const uint32_t next = i < d ? __ldg(tb + i * cm + T) : 0u;
+        const uint64_t v = w[e >> 8];
+        const uint4 *const mv = reinterpret_cast<const uint4 *>(m + (e & 255u) * kSplit);
+#pragma unroll
+        for (int h = 0; h < 3; ++h) {
+            const uint32_t x = h == 0 ? (uint32_t)v : h == 1 ? (uint32_t)(v >> 32) : (uint32_t)v ^ (uint32_t)(v >> 32);
+            const uint32_t xh = x >> 16;
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                const uint32_t piece = j == 0 ? x : j == 1 ? xh : x ^ xh;
+                const uint32_t x0 = piece & 0x9249u, x1 = piece & 0x2492u, x2 = piece & 0x4924u;
+                const uint4 y = mv[3 * h + j];
+                uint32_t *const q = z + 9 * h + 3 * j;
+                q[0] ^= (x0 * y.x) ^ (x1 * y.z) ^ (x2 * y.y);
+                q[1] ^= (x0 * y.y) ^ (x1 * y.x) ^ (x2 * y.z);
+                q[2] ^= (x0 * y.z) ^ (x1 * y.y) ^ (x2 * y.x);
+            }
+        }
+        e = next;
+    }
+    return finish27(z);
+}
+
+// XOR of rows [ra, rb) of a level's values from their prefix sums (blocks of
+// 1 << ps rows, sums of 16 and 256 blocks), `count` values per row, into dst;
+// one warp. The two ends' rows come first, several loads in flight, then the
+// whole blocks between them.
+__device__ __forceinline__ void window_sum(const uint64_t *R, const uint64_t *sup1, const uint64_t *sup2, uint32_t stride,
+                                           uint32_t ps, uint32_t ra, uint32_t rb, uint32_t count, uint32_t lane, uint64_t *dst)
+{
+    const uint32_t pm = (1u << ps) - 1u;
+    const bool ha = ra & pm, hb = rb & pm;
+    const uint64_t *pa = R + (size_t)(ha ? ra - 1 : 0) * stride, *pb = R + (size_t)(hb ? rb - 1 : 0) * stride;
+#pragma unroll 4
+    for (uint32_t s = lane; s < count; s += 32u) dst[s] = (ha ? pa[s] : 0ull) ^ (hb ? pb[s] : 0ull);
+    uint32_t i = ra >> ps;
+    const uint32_t e = rb >> ps;
+    while (i < e) {  // warp-uniform
+        const uint64_t *p;
+        if (!(i % kSup2) && i + kSup2 <= e) {
+            p = sup2 + (size_t)(i / kSup2) * stride;
+            i += kSup2;
+        } else if (!(i % kSup1) && i + kSup1 <= e) {
+            p = sup1 + (size_t)(i / kSup1) * stride;
+            i += kSup1;
+        } else {
+            p = R + ((size_t)(i << ps) + pm) * stride;
+            ++i;
+        }
+#pragma unroll 4
+        for (uint32_t s = lane; s < count; s += 32u) dst[s] ^= p[s];
+    }
+}
+
+// Layers lbeg..lend of a query over its needed rows. One item = a
+// block of consecutive needed rows of one level, taken by one team of warps:
+// their window sums of the level below, the multipliers y z'_j (split), one
+// thread per (row, subset) for the wedge, the running XOR over the block's rows.
+// The store level below an out level keeps U = z'_v ^ (its value), v the row's
+// head, on the label sets the output needs: the window of an out row lies in one
+// vertex's rows, so the wedge with that vertex is taken once per stored row, not
+// per out row, and an out row needs y U only.
+__device__ __noinline__ bool x_wedge(const XArgs &a, const XOne &o, View &v, uint32_t lbeg, uint32_t lend, bool last_sync)
+{
+    extern __shared__ __align__(16) uint64_t sm_all[];
+    const XQuery &Q = o.q;
+    const XTmpl &t_ = o.t;
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint32_t gt = v.b * kThreads + threadIdx.x, nt = v.n * kThreads;
+    for (uint32_t l = lbeg; l <= lend; ++l) {
+        bool any = false;
+        uint32_t base_item = 0;
+            for (uint32_t li = t_.runs[l].first; li < t_.runs[l].first + t_.runs[l].count; ++li) {
+                const uint32_t cnt = t_.cnt[li];
+                if (!cnt) continue;
+                any = true;
+                const XLL &X = t_.ll[li];
+                const uint32_t cin = X.cin, cout = X.cout, uout = X.uout, d = X.d;
+                const uint32_t K = X.out ? cout : Q.K;  // labels in use
+                const XShape sh = x_shape_of(t_.shape[li]);
+                const uint32_t qs = sh.rows, rows = 1u << qs;
+                const uint32_t nb = (cnt + rows - 1) >> qs;
+                // the thread's team, its number in the grid and its shared memory
+                const uint32_t tsize = 32u << sh.team, team = threadIdx.x / tsize, tid = threadIdx.x % tsize;
+                const uint32_t per_block = (1u << kTeamLog) >> sh.team;
+                const uint32_t nteam = v.n * per_block, gteam = team * v.n + v.b;
+                const uint32_t tsmem = a.smem >> (kTeamLog - sh.team);
+                uint64_t *const sm = sm_all + (size_t)team * (tsmem / 8);
+                uint32_t *const msp = reinterpret_cast<uint32_t *>(sm);  // rows x K split multipliers
+                uint64_t *const dr = sm + (size_t)rows * K * (kSplit / 2), *const G = dr + rows * cin, *const Us = G + rows * cout;
+                uint4 *const smeta = reinterpret_cast<uint4 *>(sm + (tsmem / 8 - rows * 4u));
+                uint32_t *const shead = reinterpret_cast<uint32_t *>(smeta + rows);
+                auto sync = [&] {
+                    if (sh.team == 0) __syncwarp();
+                    else if (sh.team == kTeamLog) __syncthreads();
+                    else asm volatile("bar.sync %0, %1;" ::"r"(team + 1u), "r"(tsize) : "memory");
+                };
+                // the level below: its prefix sums come in blocks of 1 << ps rows
+                const XLL &P = t_.ll[X.prev];
+                const uint32_t pcnt = l > 1 ? t_.cnt[X.prev] : 0u;
+                const uint32_t ps = l > 1 ? x_shape_of(t_.shape[X.prev]).rows : 0u;
+                const uint32_t pn1 = (((pcnt + (1u << ps) - 1) >> ps) / kSup1) + 1, pn2 = (((pcnt + (1u << ps) - 1) >> ps) / kSup2) + 1;
+                const uint32_t pst = X.out ? P.uout : P.cout;  // values per row read from below
+                const uint64_t *const pR = X.out ? P.U : P.R;
+                const uint64_t *const psup1 = P.sup + (X.out ? (size_t)(pn1 + pn2) * P.cout : 0), *const psup2 = psup1 + (size_t)pn1 * pst;
+                const uint32_t n1 = nb / kSup1 + 1, n2 = nb / kSup2 + 1;
+                uint64_t *const E = X.out ? Q.E : nullptr, *const S = Q.S + (size_t)X.row * a.n;
+                const bool per_row = E || X.Ec;  // out levels: every row's own sum is wanted
+                for (uint32_t it = View::first_item(base_item, gteam, nteam); it < nb; it += nteam) {
+                    const uint32_t row0 = it << qs, nr = min(rows, cnt - row0);
+                    sync();
+                    for (uint32_t t = tid; t < nr; t += tsize) {
+                        smeta[t] = X.meta[row0 + t];
+                        if (X.mhead) shead[t] = X.mhead[row0 + t];
+                    }
+                    sync();
+                    if (l > 1)
+                        for (uint32_t q = tid >> 5; q < nr; q += 1u << sh.team)
+                            window_sum(pR, psup1, psup2, pst, ps, smeta[q].x, smeta[q].y, X.out ? cout : cin, lane,
+                                       (X.out ? G + q * cout : dr + q * cin));
+                    if (!X.out) {
+                        if (l == 1) {
+                            // y_{e,1} z_{s,p}; a set of sources: y_{e,1} z_{s,j}
+                            for (uint32_t t = tid; t < nr * cout; t += tsize) {
+                                const uint32_t q = t / cout;
+                                G[t] = gf64_mul(sm_draw(Q.key_y, (uint64_t)smeta[q].z * 32u),
+                                                Q.multi ? zprime(Q, t_.omega, a.color, smeta[q].w, t - q * cout) : Q.d0);
+                            }
+                        } else {
+                            for (uint32_t t = tid; t < nr * K; t += tsize) {
+                                const uint32_t q = t / K, j = t - q * K;
+                                const uint64_t y = sm_draw(Q.key_y, (uint64_t)smeta[q].z * 32u + (l - 1u));
+                                store_split(msp + (size_t)t * kSplit, gf64_mul(y, zprime(Q, t_.omega, a.color, smeta[q].w, j)));
+                            }
+                            sync();
+                            const uint32_t *const tb = a.tab + x_tab_off_dev(d);
+                            const uint32_t cm = x_binom_dev(kXMaxLabels, d);
+                            for (uint32_t t = tid; t < nr * cout; t += tsize) {
+                                const uint32_t q = t / cout, T = t - q * cout;
+                                G[t] = wedge_at(tb, cm, T, d, msp + (size_t)q * K * kSplit, dr + q * cin);
+                            }
+                        }
+                        sync();
+                        if (uout) {  // U on the d+1-subsets of the first d + 2 labels
+                            for (uint32_t t = tid; t < nr * uout; t += tsize) {
+                                const uint32_t q = t / uout, j = t - q * uout;
+                                store_split(msp + (size_t)t * kSplit, zprime(Q, t_.omega, a.color, shead[q], j));
+                            }
+                            sync();
+                            const uint32_t *const tb = a.tab + x_tab_off_dev(d + 1u);
+                            const uint32_t cm = x_binom_dev(kXMaxLabels, d + 1u);
+                            for (uint32_t t = tid; t < nr * uout; t += tsize) {
+                                const uint32_t q = t / uout, T = t - q * uout;
+                                Us[t] = wedge_at(tb, cm, T, d + 1u, msp + (size_t)q * uout * kSplit, G + q * cout);
+                            }
+                            sync();
+                        }
+                        const bool whole = nb >= kSup1 && nr == rows;
+                        for (uint32_t s = tid; s < cout + uout; s += tsize) {
+                            const bool isU = s >= cout;
+                            const uint32_t st = isU ? uout : cout, c = isU ? s - cout : s;
+                            const uint64_t *const g = (isU ? Us : G) + c;
+                            uint64_t *const o = (isU ? X.U : X.R) + c;
+                            uint64_t acc = 0;
+                            if (isU || X.R) {
+                                for (uint32_t q = 0; q < nr; ++q) {
+                                    acc ^= g[q * st];
+                                    o[(size_t)(row0 + q) * st] = acc;
+                                }
+                                if (whole) {
+                                    uint64_t *const s1 = X.sup + (isU ? (size_t)(n1 + n2) * cout : 0) + c;
+                                    atomicXor(reinterpret_cast<unsigned long long *>(s1 + (size_t)(it / kSup1) * st), (unsigned long long)acc);
+                                    if (nb >= kSup2)
+                                        atomicXor(reinterpret_cast<unsigned long long *>(s1 + (size_t)(n1 + it / kSup2) * st), (unsigned long long)acc);
+                                }
+                            }
+                        }
+                    } else {
+                        // y U per row (layer 1: the source's z row itself), then z'_w over runs of
+                        // equal heads -- or row by row when every row's own sum is wanted
+                        sync();
+                        for (uint32_t t = tid; t < nr * K; t += tsize) {
+                            const uint32_t q = t / K;
+                            const uint64_t y = sm_draw(Q.key_y, (uint64_t)smeta[q].z * 32u + (l - 1u));
+                            G[t] = gf64_mul(y, l > 1 ? G[t] : Q.multi ? zprime(Q, t_.omega, a.color, smeta[q].w, t - q * K) : Q.d0);
+                        }
+                        sync();
+                        for (uint32_t t = tid; t < nr * K; t += tsize) {
+                            const uint32_t q = t / K, T = t - q * K;
+                            if (!per_row && q && shead[q] == shead[q - 1]) continue;
+                            uint64_t x = G[t];
+                            if (!per_row)
+                                for (uint32_t o = q + 1; o < nr && shead[o] == shead[q]; ++o) x ^= G[o * K + T];
+                            sm[t] = gf64_mul(x, zprime(Q, t_.omega, a.color, shead[q], K - 1u - T));  // the label T misses
+                        }
+                        sync();
+                        for (uint32_t q = tid; q < nr; q += tsize) {
+                            if (!per_row && q && shead[q] == shead[q - 1]) continue;
+                            uint64_t x = 0;
+                            for (uint32_t s = 0; s < K; ++s) x ^= sm[q * K + s];
+                            if (E) E[smeta[q].z] = x;
+                            if (X.Ec) X.Ec[row0 + q] = x;
+                            if (x) atomicXor(reinterpret_cast<unsigned long long *>(S + shead[q]), (unsigned long long)x);
+                        }
+                    }
+                }
+                base_item += nb;
+                __syncthreads();  // the next level list may form other teams
+            }
+        if (l < t_.maxlev)  // clear the next level's partial sums
+            for (uint32_t li = t_.runs[l + 1].first; li < t_.runs[l + 1].first + t_.runs[l + 1].count; ++li) {
+                const uint32_t cnt = t_.cnt[li];
+                const XLL &X = t_.ll[li];
+                if (X.out || !cnt) continue;
+                const uint32_t qs = x_shape_of(t_.shape[li]).rows;
+                const uint32_t nb = (cnt + (1u << qs) - 1) >> qs;
+                if (nb < kSup1) continue;
+                const uint32_t w = (nb / kSup1 + 1 + nb / kSup2 + 1) * (X.cout + X.uout);
+                for (uint32_t i = gt; i < w; i += nt) X.sup[i] = 0;
+            }
+        if (any && (l < lend || last_sync))
+            if (!v.sync()) return false;
+    }
+    return true;
+}
+
+// Minimum arrival times and bitmaps, after the last layer.
+__device__ __noinline__ void x_outputs(const XArgs &a, const XOne &o, const View &v)
+{
+    const XQuery &Q = o.q;
+    const uint32_t gt = v.b * kThreads + threadIdx.x, nt = v.n * kThreads;
+    for (uint32_t li = 0; li < o.t.nll; ++li) {
+        const XLL &X = o.t.ll[li];
+        if (!X.Ec) continue;
+        uint32_t *const R = Q.R + (size_t)X.row * a.n;
+        // runs of equal head and time among the out rows (consecutive: the
+        // rows keep the list's order)
+        const uint32_t cnt = o.t.cnt[li];
+        for (uint32_t i = gt; i < cnt; i += nt) {
+            const uint32_t h = X.mhead[i], t = X.mtime[i];
+            if (i && X.mhead[i - 1] == h && X.mtime[i - 1] == t) continue;
+            uint64_t e = X.Ec[i];
+            for (uint32_t x = i + 1; x < cnt && X.mhead[x] == h && X.mtime[x] == t; ++x) e ^= X.Ec[x];
+            if (e) atomicMin(R + h, t);
+        }
+    }
+    if (!Q.bitmap) return;
+    const uint32_t nbytes = (a.n + 7) / 8, rows = o.t.every ? Q.k - 1 : 1u;
+    for (uint32_t b = gt; b < nbytes; b += nt) {
+        uint32_t bits = 0;
+        for (uint32_t w = 0; w < rows; ++w)
+#pragma unroll
+            for (uint32_t i = 0; i < 8; ++i) {
+                const uint32_t x = b * 8 + i;
+                if (x < a.n && Q.S[(size_t)w * a.n + x] != 0) bits |= 1u << i;
+            }
+        Q.bitmap[b] = (uint8_t)bits;
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Queries whose walks are few: one block, everything in shared memory, no
+// bitmaps. The frontier is pushed along the edges sorted by (tail, time); a
+// level holds at most kTinyRows rows, each with the set of the level below's
+// rows in its window (a bit mask), so the backward pass and the window sums
+// need no memory traffic. The multipliers y z'_j of all levels are formed at
+// once, before the layers, and a layer's products (row, subset, element) are
+// spread over the threads while they fit: what is left is a chain of about two
+// dependent loads a layer forward and one product a layer after that.
+// Returns false, with nothing written, when the query does not fit.
+// ---------------------------------------------------------------------------
+constexpr uint32_t kTinyRows = 128, kTinyWords = kTinyRows / 32, kTinyTotal = 768, kTinyPairs = 1024, kTinyHash = 512;
+
+struct TinyMem {
+    uint4 row[kTinyTotal];                  // tail, head, time, edge
+    uint32_t mask[kTinyTotal][kTinyWords];  // rows of the level below in the window
+    uint32_t need[kXMaxLevels + 1][kTinyWords];
+    uint32_t base[kXMaxLevels + 2];         // first row of each level
+    uint32_t cn[kXMaxLevels + 2];           // needed rows before each level
+    uint32_t hkey[kTinyHash], hval[kTinyHash];
+    uint32_t pair[kTinyPairs];
+    uint32_t npair, count, over;
+    uint16_t list[kTinyTotal];              // needed rows: level << 12 is kept in lev
+    uint8_t lev[kTinyTotal];
+    uint64_t acc[kTinyRows];
+};
+
+__device__ __forceinline__ void xor_shared(uint64_t *p, uint64_t v)
+{
+    uint32_t *w = reinterpret_cast<uint32_t *>(p);
+    if ((uint32_t)v) atomicXor(w, (uint32_t)v);
+    if ((uint32_t)(v >> 32)) atomicXor(w + 1, (uint32_t)(v >> 32));
+}
+
+__device__ __noinline__ bool x_tiny(const XArgs &a, const XQuery &Q, bool every)
+{
+    extern __shared__ __align__(16) uint64_t sm_all[];
+    TinyMem &M = *reinterpret_cast<TinyMem *>(sm_all);
+    uint64_t *const pool = sm_all + (sizeof(TinyMem) + 15) / 16 * 2;
+    const uint32_t pool_n = a.smem / 8 - (uint32_t)((sizeof(TinyMem) + 15) / 16 * 2);
+    const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+    const uint32_t k = Q.k, K = Q.K, sh = Q.multi ? 1u : 0u, last = k - 1;
+
+    // layer 1: the edges leaving the source(s)
+    if (tid == 0) {
+        M.count = M.over = 0;
+        M.base[1] = 0;
+    }
+    __syncthreads();
+    if (!Q.dead) {
+        const uint32_t ns = Q.multi ? Q.nslist : 1u;
+        for (uint32_t i = warp; i < ns; i += kWarps) {
+            const uint32_t s = Q.multi ? Q.slist[i] : Q.source;
+            if (Q.vmask && Q.vmask[s]) continue;
+            const uint32_t o0 = a.ooff[s], o1 = a.ooff[s + 1];
+            if (o1 - o0 > kTinyRows) {
+                if (lane == 0) M.over = 1;
+                continue;
+            }
+            for (uint32_t o = o0 + lane; o < o1; o += 32u) {
+                const uint4 r = make_uint4(s, a.odst[o], a.otime[o], a.oeid[o]);
+                if (!allowed(Q, a.color, r.y) || (!Q.multi && r.y == s)) continue;
+                const uint32_t at = atomicAdd(&M.count, 1u);
+                if (at < kTinyRows) M.row[at] = r;
+            }
+        }
+    }
+    __syncthreads();
+    if (M.over || M.count > kTinyRows) return false;
+    uint32_t n = M.count, lmax = 1;
+    __syncthreads();
+    if (tid == 0) M.base[2] = n;
+    // forward
+    for (uint32_t l = 2; l <= last && n; ++l) {
+        for (uint32_t i = tid; i < kTinyHash; i += kThreads) M.hkey[i] = 0;
+        if (tid == 0) M.count = M.npair = 0;
+        __syncthreads();
+        const uint32_t b0 = M.base[l - 1], b1 = M.base[l];
+        for (uint32_t f = warp; f < n; f += kWarps) {
+            const uint4 r = M.row[b0 + f];
+            const uint32_t v = r.y;
+            uint32_t o = a.ooff[v];
+            const uint32_t o1 = a.ooff[v + 1], t0 = r.z;
+            const uint64_t t1 = (uint64_t)t0 + a.delta[v];
+            if (o1 - o > 64u) {  // the first edge at or after t0
+                uint32_t hi = o1;
+                while (o < hi) {
+                    const uint32_t mid = o + (hi - o) / 2;
+                    if (a.otime[mid] < t0) o = mid + 1;
+                    else hi = mid;
+                }
+            }
+            for (; o < o1; o += 32u) {  // warp-uniform
+                const uint32_t p = o + lane;
+                const bool in = p < o1;
+                const uint32_t t = in ? a.otime[p] : 0xffffffffu, w = in ? a.odst[p] : 0u, e = in ? a.oeid[p] : 0u;
+                const bool past = !in || (uint64_t)t > t1;
+                if (!past && t >= t0 && allowed(Q, a.color, w) && (Q.multi || w != Q.source)) {
+                    // the row's place in the level (one per edge)
+                    uint32_t h = (p * 2654435761u) >> 23;  // 9 bits: kTinyHash
+                    bool placed = false;
+                    for (uint32_t tries = 0; tries < kTinyHash && !placed; ++tries) {
+                        const uint32_t key = atomicCAS(&M.hkey[h], 0u, p + 1u);
+                        if (key == 0u) {
+                            const uint32_t at = atomicAdd(&M.count, 1u);
+                            M.hval[h] = at;
+                            if (at < kTinyRows && b1 + at < kTinyTotal) {
+                                M.row[b1 + at] = make_uint4(v, w, t, e);
+#pragma unroll
+                                for (uint32_t x = 0; x < kTinyWords; ++x) M.mask[b1 + at][x] = 0;
+                            }
+                        }
+                        placed = key == 0u || key == p + 1u;
+                        if (!placed) h = (h + 1u) % kTinyHash;
+                    }
+                    const uint32_t pp = atomicAdd(&M.npair, 1u);
+                    if (!placed || pp >= kTinyPairs) M.over = 1;
+                    else M.pair[pp] = f << 16 | h;
+                }
+                if (__all_sync(0xffffffffu, past)) break;
+                if (M.count > kTinyRows) break;
+            }
+        }
+        __syncthreads();
+        n = M.count;
+        if (M.over || n > kTinyRows || b1 + n > kTinyTotal) return false;
+        for (uint32_t i = tid; i < M.npair; i += kThreads) {
+            const uint32_t f = M.pair[i] >> 16, e = M.hval[M.pair[i] & 0xffffu];
+            atomicOr(&M.mask[b1 + e][f >> 5], 1u << (f & 31u));
+        }
+        if (tid == 0) M.base[l + 1] = b1 + n;
+        if (n) lmax = l;
+        __syncthreads();
+    }
+    if (n == 0 && !every) return true;  // no walk of k vertices: every sum is zero
+    if (lmax == 1 && M.base[2] == 0) return true;
+    const uint32_t top = every ? lmax : last;
+
+    // backward: the needed rows
+    for (uint32_t i = tid; i < (kXMaxLevels + 1) * kTinyWords; i += kThreads) {
+        const uint32_t l = i / kTinyWords;
+        uint32_t all = 0;
+        if (l >= 1 && l <= top && (every || l == top)) {
+            const uint32_t c = M.base[l + 1] - M.base[l], b = (i % kTinyWords) * 32u;
+            all = c >= b + 32u ? 0xffffffffu : c > b ? (1u << (c - b)) - 1u : 0u;
+        }
+        M.need[l][i % kTinyWords] = all;
+    }
+    __syncthreads();
+    if (!every)
+        for (uint32_t l = top; l >= 2; --l) {
+            const uint32_t c = M.base[l + 1] - M.base[l];
+            for (uint32_t i = tid; i < c * kTinyWords; i += kThreads) {
+                const uint32_t e = i / kTinyWords, x = i % kTinyWords;
+                if ((M.need[l][e >> 5] >> (e & 31u)) & 1u) {
+                    const uint32_t m = M.mask[M.base[l] + e][x];
+                    if (m) atomicOr(&M.need[l - 1][x], m);
+                }
+            }
+            __syncthreads();
+        }
+    if (tid == 0) {
+        uint32_t c = 0;
+        for (uint32_t l = 1; l <= top; ++l) {
+            M.cn[l] = c;
+            for (uint32_t x = 0; x < kTinyWords; ++x) c += __popc(M.need[l][x]);
+        }
+        M.cn[top + 1] = c;
+    }
+    __syncthreads();
+    const uint32_t total = M.cn[top + 1];
+    // shared memory: multipliers, the shade factors, then window sums and two levels' values
+    uint32_t need_g = 0, need_d = 0;
+    for (uint32_t l = 1; l <= top; ++l) {
+        const uint32_t c = M.cn[l + 1] - M.cn[l], d = l - 1 + sh;
+        need_g = max(need_g, c * x_binom_dev(K, d));
+        if (l > 1) need_d = max(need_d, c * x_binom_dev(K, d - 1));
+    }
+    const uint32_t om_n = Q.colored ? Q.k * K : 0u;
+    if (2u * total * K + om_n + need_d + 2u * need_g > pool_n) return false;
+    uint64_t *const mul = pool, *const zw = mul + total * K, *const omega = zw + total * K, *const dr = omega + om_n,
+                    *const G0 = dr + need_d, *const G1 = G0 + need_g;
+    for (uint32_t i = tid; i < om_n; i += kThreads) omega[i] = shade_factor(Q, i);
+    // the needed rows by level
+    for (uint32_t i = tid; i < M.base[top + 1]; i += kThreads) {
+        uint32_t l = 1;
+        while (i >= M.base[l + 1]) ++l;
+        const uint32_t e = i - M.base[l];
+        if (!((M.need[l][e >> 5] >> (e & 31u)) & 1u)) continue;
+        uint32_t at = M.cn[l] + __popc(M.need[l][e >> 5] & ((1u << (e & 31u)) - 1u));
+        for (uint32_t x = 0; x < (e >> 5); ++x) at += __popc(M.need[l][x]);
+        M.list[at] = (uint16_t)i;
+        M.lev[at] = (uint8_t)l;
+    }
+    __syncthreads();
+    for (uint32_t i = tid; i < 2u * total * K; i += kThreads) {
+        const bool second = i >= total * K;
+        const uint32_t x = second ? i - total * K : i, at = x / K, j = x - at * K, l = M.lev[at];
+        const uint4 r = M.row[M.list[at]];
+        if (second) {
+            if (every || l == top) zw[x] = zprime(Q, omega, a.color, r.y, j);
+        } else {
+            const uint64_t y = sm_draw(Q.key_y, (uint64_t)r.w * 32u + (l - 1u));
+            mul[x] = gf64_mul(y, l > 1 || Q.multi ? zprime(Q, omega, a.color, r.x, j) : Q.d0);
+        }
+    }
+    __syncthreads();
+    // the layers
+    uint64_t *G = G0, *Gp = G1;
+    for (uint32_t l = 1; l <= top; ++l) {
+        const uint32_t c = M.cn[l + 1] - M.cn[l], d = l - 1 + sh, cout = x_binom_dev(K, d);
+        uint64_t *const t_ = G;
+        G = Gp;
+        Gp = t_;
+        const uint64_t *const ml = mul + M.cn[l] * K;
+        if (l == 1) {
+            for (uint32_t i = tid; i < c * cout; i += kThreads) G[i] = ml[i / cout * K + i % cout];
+        } else {
+            const uint32_t cin = x_binom_dev(K, d - 1);
+            const bool spread = c * cout * d <= 4u * kThreads;
+            for (uint32_t i = tid; i < c * cin; i += kThreads) {
+                const uint32_t q = i / cin, s = i - q * cin;
+                const uint32_t *const mk = M.mask[M.list[M.cn[l] + q]];
+                uint64_t v = 0;
+                uint32_t before = 0;
+#pragma unroll
+                for (uint32_t x = 0; x < kTinyWords; ++x) {
+                    const uint32_t nd = M.need[l - 1][x];
+                    for (uint32_t m = mk[x] & nd; m; m &= m - 1)
+                        v ^= Gp[(before + __popc(nd & ((m & (0u - m)) - 1u))) * cin + s];
+                    before += __popc(nd);
+                }
+                dr[i] = v;
+            }
+            if (spread)
+                for (uint32_t i = tid; i < c * cout; i += kThreads) G[i] = 0;
+            __syncthreads();
+            const uint32_t *const tb = a.tab + x_tab_off_dev(d);
+            const uint32_t cm = x_binom_dev(kXMaxLabels, d);
+            if (spread) {
+                for (uint32_t i = tid; i < c * cout * d; i += kThreads) {
+                    const uint32_t q = i / (cout * d), r = i - q * cout * d, x = r / cout, T = r - x * cout;
+                    const uint32_t e = __ldg(tb + x * cm + T);
+                    xor_shared(&G[q * cout + T], gf64_mul(ml[q * K + (e & 255u)], dr[q * cin + (e >> 8)]));
+                }
+            } else {
+                for (uint32_t i = tid; i < c * cout; i += kThreads) {
+                    const uint32_t q = i / cout, T = i - q * cout;
+                    uint64_t v = 0;
+                    for (uint32_t x = 0; x < d; ++x) {
+                        const uint32_t e = __ldg(tb + x * cm + T);
+                        v ^= gf64_mul(ml[q * K + (e & 255u)], dr[q * cin + (e >> 8)]);
+                    }
+                    G[i] = v;
+                }
+            }
+        }
+        const bool out = every ? !(Q.pivot > l && !Q.multi) : l == top;
+        if (!out) {
+            __syncthreads();
+            continue;
+        }
+        // witness: z'_w over the first K2 labels
+        for (uint32_t i = tid; i < c; i += kThreads) M.acc[i] = 0;
+        __syncthreads();
+        const uint32_t K2 = l + sh;
+        for (uint32_t i = tid; i < c * K2; i += kThreads) {
+            const uint32_t q = i / K2, T = i - q * K2;
+            xor_shared(&M.acc[q], gf64_mul(G[q * cout + T], zw[(M.cn[l] + q) * K + (K2 - 1u - T)]));
+        }
+        __syncthreads();
+        const uint32_t row = every ? l - 1u : 0u;
+        for (uint32_t q = tid; q < c; q += kThreads) {
+            const uint4 r = M.row[M.list[M.cn[l] + q]];
+            const uint64_t v = M.acc[q];
+            if (v) atomicXor(reinterpret_cast<unsigned long long *>(Q.S + (size_t)row * a.n + r.y), (unsigned long long)v);
+            if (Q.E) Q.E[r.w] = v;
+            if (Q.R) {  // the XOR over the head's rows of the same time
+                uint64_t sum = 0;
+                for (uint32_t x = 0; x < c; ++x) {
+                    const uint4 o = M.row[M.list[M.cn[l] + x]];
+                    if (o.y == r.y && o.z == r.z) sum ^= M.acc[x];
+                }
+                if (sum) atomicMin(Q.R + (size_t)row * a.n + r.y, r.z);
+            }
+        }
+        __syncthreads();
+    }
+    if (Q.bitmap) {  // the bytes of the out rows' heads (the rest is clear)
+        __threadfence();
+        __syncthreads();
+        const uint32_t rows = every ? k - 1 : 1u;
+        for (uint32_t at = tid; at < total; at += kThreads) {
+            if (!every && M.lev[at] != top) continue;
+            const uint32_t b = M.row[M.list[at]].y >> 3;
+            uint32_t bits = 0;
+            for (uint32_t w = 0; w < rows; ++w)
+                for (uint32_t i = 0; i < 8; ++i) {
+                    const uint32_t x = b * 8 + i;
+                    if (x < a.n && __ldcg(Q.S + (size_t)w * a.n + x) != 0) bits |= 1u << i;
+                }
+            Q.bitmap[b] = (uint8_t)bits;
+        }
+    }
+    return true;
+}
+
+// The scratch pointers of a template, from offsets + 1 to addresses.
+__device__ __forceinline__ void relocate(XTmpl &t, uint8_t *base)
+{
+    const uint64_t b = reinterpret_cast<uint64_t>(base) - 1u;
+    auto fix = [b](auto &p) {
+        if (p) p = reinterpret_cast<std::remove_reference_t<decltype(p)>>(reinterpret_cast<uint64_t>(p) + b);
+    };
+    for (uint32_t i = threadIdx.x; i < t.nll; i += blockDim.x) {
+        XLL &x = t.ll[i];
+        fix(x.A);
+        fix(x.N);
+        fix(x.pc);
+        fix(x.tsum);
+        fix(x.meta);
+        fix(x.mhead);
+        fix(x.mtime);
+        fix(x.R);
+        fix(x.U);
+        fix(x.sup);
+        fix(x.Ec);
+    }
+    if (threadIdx.x == 0) {
+        fix(t.clear);
+        fix(t.live);
+        fix(t.cnt);
+        fix(t.shape);
+        fix(t.omega);
+    }
+}
+
+__device__ __forceinline__ void copy_words(void *dst, const void *src, uint32_t bytes)
+{
+    for (uint32_t i = threadIdx.x; i < bytes / 4; i += blockDim.x)
+        static_cast<uint32_t *>(dst)[i] = static_cast<const uint32_t *>(src)[i];
+}
+
+// The description of one query, in shared memory (it is read all the time at
+// run-time indexes; indexed reads of the parameter bank took a microsecond a
+// phase).
+template <bool BATCH>
+__device__ __forceinline__ void load_query(XOne &o, const XArgs &a, const XOne &one, uint32_t q, uint32_t lane)
+{
+    __syncthreads();
+    copy_words(&o.q, BATCH ? a.xq + q : &one.q, sizeof(XQuery));
+    __syncthreads();
+    copy_words(&o.t, BATCH ? a.xt + o.q.k : &one.t, sizeof(XTmpl));
+    __syncthreads();
+    relocate(o.t, a.scratch + lane * a.stride);
+    __syncthreads();
+}
+
+// First: every query in one block's shared memory (x_tiny). Those that do not
+// fit are left to the bitmap passes: one query at a time by the whole grid, or,
+// when there are many, one per block.
+template <bool BATCH>
+__global__ void __launch_bounds__(kThreads, 1)
+k_frontier(const __grid_constant__ XArgs a_, const __grid_constant__ XOne one_, uint32_t plan, uint32_t lbeg, uint32_t lend,
+           uint32_t fin)
+{
+    __shared__ __align__(16) XArgs a;
+    __shared__ __align__(16) XOne o;
+    __shared__ uint32_t next;
+    copy_words(&a, &a_, sizeof(XArgs));
+    __syncthreads();
+    const uint32_t gt = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
+    View grid{blockIdx.x, gridDim.x, a.ctl, a.err, 0u};
+    bool ok = true;
+    if (plan) {
+        // cleared first: witnesses and bitmaps
+        if ((reinterpret_cast<uint64_t>(a.szero) & 15u) == 0) {
+            ulonglong2 *z = reinterpret_cast<ulonglong2 *>(a.szero);
+            for (uint64_t i = gt; i < a.szero_n / 2; i += nt) z[i] = make_ulonglong2(0, 0);
+            if (gt == 0 && (a.szero_n & 1)) a.szero[a.szero_n - 1] = 0;
+        } else {
+            for (uint64_t i = gt; i < a.szero_n; i += nt) a.szero[i] = 0;
+        }
+        for (uint64_t i = gt; i < a.bzero_n; i += nt) a.bzero[i] = 0;
+    }
+    uint32_t left = BATCH ? 0u : 1u;
+    if (!BATCH) load_query<BATCH>(o, a, one_, 0, 0);
+    if (plan && a.tiny) {
+        ok = grid.sync();
+        if (ok) {
+            for (;;) {
+                uint32_t q = blockIdx.x;  // one query: block 0's
+                if (BATCH) {
+                    __syncthreads();
+                    if (threadIdx.x == 0) next = atomicAdd(a.ctl + 2, 1u);
+                    __syncthreads();
+                    q = next;
+                    if (q < a.nq) load_query<BATCH>(o, a, one_, q, 0);
+                }
+                if (q >= a.nq) break;
+                if (!x_tiny(a, o.q, o.t.every != 0) && threadIdx.x == 0) {
+                    const uint32_t at = atomicAdd(a.ctl + 3, 1u);
+                    if (BATCH) a.left[at] = q;
+                }
+                if (!BATCH) break;
+            }
+            ok = grid.sync();
+        }
+        if (ok) left = *(volatile uint32_t *)(a.ctl + 3);
+    }
+    if (ok && left) {
+        if (BATCH && a.lanes > 1 && left >= gridDim.x / 4) {
+            View solo{0u, 1u, a.ctl, a.err, 0u};
+            while (blockIdx.x < a.lanes) {
+                __syncthreads();
+                if (threadIdx.x == 0) next = atomicAdd(a.ctl + 4, 1u);
+                __syncthreads();
+                if (next >= left) break;
+                load_query<BATCH>(o, a, one_, a.left[next], blockIdx.x);
+                x_plan(a, o, solo);
+                x_wedge(a, o, solo, 1u, o.t.maxlev, true);
+                x_outputs(a, o, solo);
+            }
+        } else {
+            for (uint32_t i = 0; i < left && ok; ++i) {
+                if (BATCH) load_query<BATCH>(o, a, one_, a.left[i], 0);
+                if (plan) ok = x_plan(a, o, grid);
+                const uint32_t l1 = BATCH ? o.t.maxlev : lend;
+                if (ok && l1) ok = x_wedge(a, o, grid, BATCH ? 1u : lbeg, l1, fin != 0);
+                if (ok && fin) x_outputs(a, o, grid);
+                if (BATCH && ok) ok = grid.sync();  // the scratch is the next query's
+            }
+        }
+    }
+    // the last block to leave clears the counters for the next launch
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(a.ctl + 1, 1u) == gridDim.x - 1)
+            for (int i = 0; i < 5; ++i) a.ctl[i] = 0;
+    }
+}
+
+// start[i] = first position of entry i's window in the list `prev` (0-based):
+// its index b when set, else the first row of the tail's segment there (the
+// rows with smaller heads come before it).
+__global__ void k_window_start(uint32_t count, const uint32_t *__restrict__ a, const uint32_t *__restrict__ b,
+                               const uint32_t *__restrict__ src, const uint32_t *__restrict__ prev_head,
+                               uint32_t prev_count, uint32_t *__restrict__ start)
+{
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) {
+        uint32_t s = b[i];
+        if (!s && a[i]) {
+            const uint32_t u = src[i];
+            uint32_t lo = 0, hi = prev_count;
+            while (lo < hi) {
+                const uint32_t mid = lo + (hi - lo) / 2;
+                if (prev_head[mid] < u) lo = mid + 1;
+                else hi = mid;
+            }
+            s = lo;
+        }
+        start[i] = s;
+    }
+}
+
+}  // namespace
+
+// ---- host side ------------------------------------------------------------------
+
+rr_status frontier_load(Graph &g, cudaStream_t st)
+{
+    RR_CUDA(cudaDeviceGetAttribute(&g.x_sms, cudaDevAttrMultiProcessorCount, g.dev));
+    int smem = 0;
+    RR_CUDA(cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, g.dev));
+    g.x_smem_max = (uint32_t)smem;
+    for (const void *f : {(const void *)k_frontier<false>, (const void *)k_frontier<true>}) {
+        cudaFuncAttributes at{};
+        RR_CUDA(cudaFuncGetAttributes(&at, f));
+        g.x_smem_max = std::min<uint32_t>(g.x_smem_max, (uint32_t)(smem - (int)at.sharedSizeBytes));
+    }
+    g.x_smem_max = g.x_smem_max / 64 * 64;
+    RR_CUDA(cudaFuncSetAttribute(k_frontier<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.x_smem_max));
+    RR_CUDA(cudaFuncSetAttribute(k_frontier<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.x_smem_max));
+    RR_CUDA(g.x_tab.reserve((size_t)x_tab_off(kXMaxLabels + 1) * 4));
+    k_subset_table<<<dim3((x_binom(kXMaxLabels, kXMaxLabels / 2) + 127) / 128, kXMaxLabels), 128, 0, st>>>(g.x_tab.as<uint32_t>());
+    RR_LAUNCHED();
+    {
+        uint16_t bin[kXMaxLabels + 2][kXMaxLabels + 2];
+        uint32_t off[kXMaxLabels + 2];
+        for (uint32_t i = 0; i < kXMaxLabels + 2; ++i) {
+            for (uint32_t d = 0; d < kXMaxLabels + 2; ++d) bin[i][d] = (uint16_t)x_binom(i, d);
+            off[i] = i ? x_tab_off(i) : 0u;
+        }
+        RR_CUDA(cudaMemcpyToSymbolAsync(c_binom, bin, sizeof bin, 0, cudaMemcpyHostToDevice, st));
+        RR_CUDA(cudaMemcpyToSymbolAsync(c_tab_off, off, sizeof off, 0, cudaMemcpyHostToDevice, st));
+        RR_CUDA(cudaStreamSynchronize(st));
+    }
+    struct {
+        RowList *L, *prev;
+        DevBuf *a, *b, *start;
+    } w[] = {{&g.state_list, &g.prod_list, &g.state_list.a0, &g.state_list.b0, &g.state_list.w0},
+             {&g.win_list, &g.prod_list, &g.win_list.a0, &g.win_list.b0, &g.win_list.w0},
+             {&g.deep_list, &g.state_list, &g.deep_list.a1, &g.deep_list.b1, &g.deep_list.w1},
+             {&g.tail_list, &g.state_list, &g.tail_list.a1, &g.tail_list.b1, &g.tail_list.w1},
+             {&g.deep_list, &g.deep_list, &g.deep_list.a3, &g.deep_list.b3, &g.deep_list.w3},
+             {&g.tail3_list, &g.deep_list, &g.tail3_list.a3, &g.tail3_list.b3, &g.tail3_list.w3}};
+    for (auto &x : w) {
+        if (!x.L->count) continue;
+        RR_CUDA(x.start->reserve(x.L->count * 4));
+        const unsigned grid = (unsigned)std::min<uint64_t>(152ull * 32, (x.L->count + 255) / 256);
+        k_window_start<<<grid, 256, 0, st>>>((uint32_t)x.L->count, x.a->as<uint32_t>(), x.b->as<uint32_t>(),
+                                             x.L->src.as<uint32_t>(), x.prev->head.as<uint32_t>(),
+                                             (uint32_t)x.prev->count, x.start->as<uint32_t>());
+        RR_LAUNCHED();
+    }
+    return RR_OK;
+}
+
+static void x_lists(const Graph &g, XList *out)
+{
+    auto set = [&](uint32_t id, const RowList &L, const DevBuf &lo, const DevBuf &hi) {
+        out[id] = XList{L.head.as<uint32_t>(), L.eid.as<uint32_t>(), L.src.as<uint32_t>(), lo.as<uint32_t>(),
+                        hi.as<uint32_t>(), L.time.as<uint32_t>(), (uint32_t)L.count, (uint32_t)(L.count / 32 + 1)};
+    };
+    set(kXProd, g.prod_list, g.prod_list.w0, g.prod_list.a0);
+    set(kXState, g.state_list, g.state_list.w0, g.state_list.a0);
+    set(kXDeep1, g.deep_list, g.deep_list.w1, g.deep_list.a1);
+    set(kXDeep3, g.deep_list, g.deep_list.w3, g.deep_list.a3);
+    set(kXWin, g.win_list, g.win_list.w0, g.win_list.a0);
+    set(kXTail, g.tail_list, g.tail_list.w1, g.tail_list.a1);
+    set(kXTail3, g.tail3_list, g.tail3_list.w3, g.tail3_list.a3);
+    out[kXAll] = XList{g.row_head.as<uint32_t>(), g.row_eid.as<uint32_t>(), g.row_src.as<uint32_t>(), nullptr, nullptr,
+                       g.row_t.as<uint32_t>(), (uint32_t)g.m, (uint32_t)(g.m / 32 + 1)};
+}
+
+// Bump allocation of the scratch: offsets + 1 in place of addresses.
+struct XBump {
+    uint64_t used = 0;
+    template <class T>
+    T *take(uint64_t count)
+    {
+        T *p = reinterpret_cast<T *>(used + 1);
+        used += (count * sizeof(T) + 255) / 256 * 256;
+        return p;
+    }
+};
+
+static uint32_t x_store_list(uint32_t l)
+{
+    return l == 1 ? kXProd : l == 2 ? kXState : l == 3 ? kXDeep1 : kXDeep3;
+}
+static uint32_t x_out_list(uint32_t l)
+{
+    return l == 1 ? kXAll : l == 2 ? kXWin : l == 3 ? kXTail : kXTail3;
+}
+
+// The levels of a k-vertex query, the store level first: store levels 1..k-2, an
+// out level k-1 (every = false) or out levels 1..k-1 (every = true: at-most-k),
+// and their scratch. multi: a set of sources, all k labels, subsets larger by
+// one. Returns the scratch's bytes.
+static uint64_t x_template(const XList *lists, uint32_t k, bool every, bool multi, bool arrivals, XTmpl &t)
+{
+    std::memset(&t, 0, sizeof t);
+    const uint32_t sh = multi ? 1u : 0u, K = k - 1 + sh;
+    t.maxlev = k - 1;
+    t.every = every ? 1u : 0u;
+    uint32_t store[kXMaxLevels + 1] = {0};
+    for (uint32_t l = 1; l <= k - 1; ++l) {
+        t.runs[l].first = t.nll;
+        for (int out = 0; out < 2; ++out) {
+            if (out ? !(every || l == k - 1) : l > k - 2) continue;
+            XLL &x = t.ll[t.nll];
+            x.level = l;
+            x.out = (uint32_t)out;
+            x.list = out ? x_out_list(l) : x_store_list(l);
+            x.words = lists[x.list].words;
+            x.d = l - 1 + sh;
+            x.prev = l > 1 ? store[l - 1] : t.nll;
+            if (out) {
+                x.cout = l + sh;  // labels of k' = l + 1
+                x.row = every ? l - 1 : 0u;
+            } else {
+                x.cin = l >= 2 ? x_binom(K, x.d - 1) : 0u;
+                x.cout = x_binom(K, x.d);
+                x.uout = every || l == k - 2 ? x.d + 2 : 0u;  // the out level above uses d + 2 labels
+                store[l] = t.nll;
+            }
+            ++t.nll;
+        }
+        t.runs[l].count = t.nll - t.runs[l].first;
+    }
+    XBump b;
+    t.clear = b.take<uint4>(0);
+    if (!every)
+        for (uint32_t i = 0; i < t.nll; ++i)
+            if (!t.ll[i].out) t.ll[i].N = b.take<uint32_t>(t.ll[i].words);
+    t.clear4 = (uint32_t)(b.used / 16);
+    uint64_t ping[2] = {0, 0}, supw = 0;
+    for (uint32_t i = 0; i < t.nll; ++i) {
+        const XLL &x = t.ll[i];
+        if (x.out) continue;
+        const uint64_t c = lists[x.list].count, w = x.cout + x.uout;
+        if (x.level >= 3) ping[x.level & 1u] = std::max<uint64_t>(ping[x.level & 1u], c * w);
+        supw = std::max<uint64_t>(supw, (c / kSup1 + c / kSup2 + 2) * w);
+    }
+    uint64_t *pp[2] = {b.take<uint64_t>(ping[0]), b.take<uint64_t>(ping[1])};
+    uint64_t *sup[3] = {b.take<uint64_t>(supw), b.take<uint64_t>(supw), b.take<uint64_t>(supw)};
+    for (uint32_t i = 0; i < t.nll; ++i) {
+        XLL &x = t.ll[i];
+        const uint64_t c = lists[x.list].count;
+        x.A = b.take<uint32_t>(x.words);
+        if (x.out || every) x.N = x.A;
+        x.pc = b.take<uint32_t>(x.words);
+        x.tsum = b.take<uint32_t>(256);
+        x.meta = b.take<uint4>(c);
+        if (x.out || x.uout) x.mhead = b.take<uint32_t>(c);
+        if (x.out && arrivals) {
+            x.mtime = b.take<uint32_t>(c);
+            x.Ec = b.take<uint64_t>(c);
+        }
+        if (!x.out) {
+            x.R = x.level >= 3 ? pp[x.level & 1u] : b.take<uint64_t>(c * (x.cout + x.uout));
+            if (x.uout) x.U = x.R + c * x.cout;
+            x.sup = sup[x.level % 3];
+        }
+    }
+    t.omega = b.take<uint64_t>((uint64_t)k * k);
+    t.live = b.take<uint32_t>(t.nll);
+    t.cnt = b.take<uint32_t>(t.nll);
+    t.shape = b.take<uint32_t>(t.nll);
+    return b.used;
+}
+
+static void x_args(const Graph &g, XArgs &a)
+{
+    x_lists(g, a.lists);
+    a.n = g.n;
+    a.color = g.color.as<uint8_t>();
+    a.tab = g.x_tab.as<uint32_t>();
+    a.ooff = g.o_off.as<uint32_t>();
+    a.otime = g.o_time.as<uint32_t>();
+    a.odst = g.o_dst.as<uint32_t>();
+    a.oeid = g.o_eid.as<uint32_t>();
+    a.delta = g.delta.as<uint32_t>();
+    a.smem = g.x_smem_max / (16u << kTeamLog) * (16u << kTeamLog);  // 16-byte shares per warp
+}
+
+// gf64 inverse by the extended Euclidean algorithm on binary polynomials.
+static uint64_t gf64_inverse(uint64_t x)
+{
+    unsigned __int128 u = x, v = ((unsigned __int128)1 << 64) | 0x1B, g1 = 1, g2 = 0;
+    auto deg = [](unsigned __int128 w) {
+        const uint64_t hi = (uint64_t)(w >> 64), lo = (uint64_t)w;
+        return hi ? 127 - __builtin_clzll(hi) : (lo ? 63 - __builtin_clzll(lo) : -1);
+    };
+    while (u != 1) {
+        int j = deg(u) - deg(v);
+        if (j < 0) {
+            std::swap(u, v);
+            std::swap(g1, g2);
+            j = -j;
+        }
+        u ^= v << j;
+        g1 ^= g2 << j;
+    }
+    return (uint64_t)g1;
+}
+
+static void x_query(const Graph &g, const rr_query &q, bool multi, XQuery &X)
+{
+    std::memset(&X, 0, sizeof X);
+    const QueryKeys keys = make_keys(q.seed);
+    const uint32_t k = q.k, s = q.source;
+    X.source = s;
+    X.k = k;
+    X.K = k - 1;
+    X.colored = q.motif ? 1u : 0u;
+    X.key_y = keys.key_y;
+    X.key_z = keys.key_z;
+    X.key_g = keys.key_gamma;
+    X.key_o = keys.key_omega;
+    uint64_t zs[kXMaxLabels + 1];
+    if (multi) {
+        X.multi = 1;
+        X.K = X.pivot = k;
+    }
+    if (q.motif) {
+        ShadeTable sh;
+        make_shades(q.motif, k, &sh);
+        for (int c = 0; c < 256; ++c) {
+            X.first[c] = (uint8_t)sh.first[c];
+            X.mu[c] = (uint8_t)sh.mu[c];
+        }
+        if (multi) return;
+        const uint32_t c = g.h_color[s];
+        for (uint32_t j = 0; j < k; ++j) {
+            zs[j] = 0;
+            for (uint32_t d = sh.first[c]; d < sh.first[c] + sh.mu[c]; ++d)
+                zs[j] ^= gf64_mul(sm_draw(X.key_g, (uint64_t)s * 32u + d), sm_draw(X.key_o, (uint64_t)d * 32u + j));
+        }
+    } else {
+        if (multi) return;
+        for (uint32_t j = 0; j < k; ++j) zs[j] = sm_draw(X.key_z, (uint64_t)s * 32u + j);
+    }
+    uint32_t p = 0;
+    while (p < k && !zs[p]) ++p;
+    if (p == k) {  // x_s is zero at every point
+        X.dead = 1;
+        return;
+    }
+    X.pivot = p;
+    X.d0 = zs[p];
+    const uint64_t inv = gf64_inverse(zs[p]);
+    for (uint32_t j = 0, t = 0; j < k; ++j)
+        if (j != p) X.rho[t++] = gf64_mul(zs[j], inv);
+}
+
+bool uses_frontier(const Graph &g, uint32_t k)
+{
+    return g.compact && !g.point_flags && k >= 2 && k - 1 <= kXMaxLabels && !g.tune_forced[k];
+}
+
+uint64_t frontier_bytes(const Graph &g, uint32_t k, bool every, bool multi, bool arrivals)
+{
+    XList lists[kXLists];
+    x_lists(g, lists);
+    XTmpl t;
+    return x_template(lists, k, every, multi, arrivals, t);
+}
+
+template <bool BATCH>
+static rr_status x_launch(const Graph &g, const XArgs &a, const XOne &one, cudaStream_t st)
+{
+    cudaLaunchAttribute at[1];
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)g.x_sms);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = a.smem;
+    cfg.stream = st;
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    if (BATCH || a.tiny) {
+        const int ts = timing_begin(st);
+        RR_CUDA(cudaLaunchKernelEx(&cfg, k_frontier<BATCH>, a, one, 1u, 1u, one.t.maxlev, 1u));
+        timing_end(ts, kTimeBatch, st);
+        RR_LAUNCHED();
+        return RR_OK;
+    }
+    // kernel timing: one launch for the passes over the bitmaps and one per
+    // layer, each timed
+    for (uint32_t l = 0; l <= one.t.maxlev; ++l) {
+        const int ts = timing_begin(st);
+        RR_CUDA(cudaLaunchKernelEx(&cfg, k_frontier<BATCH>, a, one, l ? 0u : 1u, l, l, l == one.t.maxlev ? 1u : 0u));
+        timing_end(ts, l == one.t.maxlev ? kTimeLast : l <= 1 ? kTimeFirst : l == 2 ? kTimeSecond : l == 3 ? kTimeThird : kTimeMid, st);
+        RR_LAUNCHED();
+    }
+    return RR_OK;
+}
+
+rr_status frontier_reserve(Workspace &ws, cudaStream_t st)
+{
+    if (!ws.x_bar.p) {
+        RR_CUDA(ws.x_bar.reserve(256));
+        RR_CUDA(cudaMemsetAsync(ws.x_bar.p, 0, 256, st));
+    }
+    if (!ws.x_err) {
+        RR_CUDA(cudaHostAlloc(&ws.x_err, 64, cudaHostAllocMapped));
+        *ws.x_err = 0;
+    }
+    return RR_OK;
+}
+
+rr_status frontier_error(Workspace &ws)
+{
+    if (!ws.x_err || !*(volatile uint32_t *)ws.x_err) return RR_OK;
+    *ws.x_err = 0;
+    return fail(RR_ETIMEDOUT, "a bounded wait of the query's kernel expired");
+}
+
+static rr_status x_control(Workspace &ws, cudaStream_t st, XArgs &a)
+{
+    rr_status s = frontier_reserve(ws, st);
+    if (s == RR_OK) s = frontier_error(ws);
+    if (s != RR_OK) return s;
+    a.ctl = ws.x_bar.as<uint32_t>();
+    uint32_t *d = nullptr;
+    RR_CUDA(cudaHostGetDevicePointer(&d, ws.x_err, 0));
+    a.err = d;
+    return RR_OK;
+}
+
+// One query on st. every: witness rows of k' = 2..k (plain queries); d_R: the
+// minimum arrival times (n per witness row, set to UINT32_MAX by the caller).
+// src: a set of sources.
+rr_status frontier_query(const Graph &g, Workspace &ws, const rr_query *q, bool every, uint8_t *d_bitmap,
+                         uint64_t *d_witness, cudaStream_t st, uint64_t *d_E, const uint8_t *d_vmask, uint32_t *d_R,
+                         const SourceSet *src)
+{
+    XArgs a{};
+    x_args(g, a);
+    rr_status s = x_control(ws, st, a);
+    if (s != RR_OK) return s;
+    XOne one;
+    x_template(a.lists, q->k, every, src != nullptr, d_R != nullptr, one.t);
+    x_query(g, *q, src != nullptr, one.q);
+    XQuery &Q = one.q;
+    Q.S = d_witness;
+    Q.E = d_E;
+    Q.R = d_R;
+    Q.bitmap = d_bitmap;
+    Q.vmask = d_vmask;
+    if (src) {
+        Q.smask = src->mask;
+        Q.slist = src->list;
+        Q.nslist = src->count;
+    }
+    a.nq = 1;
+    a.scratch = ws.state.as<uint8_t>();
+    a.lanes = 1;
+    a.szero = d_witness;
+    a.szero_n = (uint64_t)g.n * (every ? q->k - 1 : 1);
+    a.bzero = d_bitmap;
+    a.bzero_n = d_bitmap ? (g.n + 7) / 8 : 0;
+    a.tiny = g_timing.load(std::memory_order_relaxed) ? 0u : 1u;
+    return x_launch<false>(g, a, one, st);
+}
+
+}  // namespace rr

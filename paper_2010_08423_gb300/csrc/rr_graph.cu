@@ -192,7 +192,7 @@ __global__ void k_v2_index(const uint32_t *__restrict__ lo_in, const uint32_t *_
 }
 
 struct ListOut {
-    uint32_t *head, *eid, *src, *a0, *b0, *a1, *b1, *a3, *b3;
+    uint32_t *head, *eid, *src, *a0, *b0, *a1, *b1, *a3, *b3, *time;
 };
 
 // deep rows: state rows (c1) whose window holds a state row (a1 != b1)
@@ -231,7 +231,8 @@ __global__ void k_v2_scatter3(const uint32_t *__restrict__ row_dst, const uint32
                               const uint32_t *__restrict__ b1, const uint32_t *__restrict__ a3,
                               const uint32_t *__restrict__ b3, const uint32_t *__restrict__ d,
                               const uint32_t *__restrict__ rank_d, const uint32_t *__restrict__ c4,
-                              const uint32_t *__restrict__ rank4, uint64_t m, ListOut D, ListOut T)
+                              const uint32_t *__restrict__ rank4, const uint32_t *__restrict__ row_t,
+                              uint64_t m, ListOut D, ListOut T)
 {
     for (uint64_t r = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; r < m;
          r += (uint64_t)gridDim.x * blockDim.x) {
@@ -243,7 +244,7 @@ __global__ void k_v2_scatter3(const uint32_t *__restrict__ row_dst, const uint32
         if (c4[r]) {
             const uint32_t i = rank4[r] - 1;
             T.head[i] = row_dst[r]; T.eid[i] = row_eid[r]; T.src[i] = row_src[r];
-            T.a3[i] = a3[r]; T.b3[i] = b3[r];
+            T.a3[i] = a3[r]; T.b3[i] = b3[r]; T.time[i] = row_t[r];
         }
     }
 }
@@ -255,8 +256,8 @@ __global__ void k_v2_scatter(const uint32_t *__restrict__ row_dst, const uint32_
                              const uint32_t *__restrict__ rank_p, const uint32_t *__restrict__ c1,
                              const uint32_t *__restrict__ rank1, const uint32_t *__restrict__ c0,
                              const uint32_t *__restrict__ rank0, const uint32_t *__restrict__ c2,
-                             const uint32_t *__restrict__ rank2, uint64_t m, ListOut P, ListOut S,
-                             ListOut W, ListOut T)
+                             const uint32_t *__restrict__ rank2, const uint32_t *__restrict__ row_t,
+                             uint64_t m, ListOut P, ListOut S, ListOut W, ListOut T)
 {
     for (uint64_t r = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; r < m;
          r += (uint64_t)gridDim.x * blockDim.x) {
@@ -273,10 +274,12 @@ __global__ void k_v2_scatter(const uint32_t *__restrict__ row_dst, const uint32_
         if (c0[r]) {
             const uint32_t i = rank0[r] - 1;
             W.head[i] = h; W.eid[i] = e; W.src[i] = u; W.a0[i] = a0[r]; W.b0[i] = b0[r];
+            W.time[i] = row_t[r];
         }
         if (c2[r]) {
             const uint32_t i = rank2[r] - 1;
             T.head[i] = h; T.eid[i] = e; T.src[i] = u; T.a1[i] = a1[r]; T.b1[i] = b1[r];
+            T.time[i] = row_t[r];
         }
     }
 }
@@ -413,15 +416,16 @@ rr_status build_lists_v2(Graph &g, const uint32_t *row_dst, const uint32_t *tpro
             RR_CUDA(R.a1.reserve(bytes));
             RR_CUDA(R.b1.reserve(bytes));
         }
+        if (i >= 2) RR_CUDA(R.time.reserve(bytes));
         out[i] = ListOut{R.head.as<uint32_t>(), R.eid.as<uint32_t>(), R.src.as<uint32_t>(),
                          R.a0.as<uint32_t>(), R.b0.as<uint32_t>(), R.a1.as<uint32_t>(),
-                         R.b1.as<uint32_t>(), nullptr, nullptr};
+                         R.b1.as<uint32_t>(), nullptr, nullptr, R.time.as<uint32_t>()};
     }
     k_v2_scatter<<<grid_for(m, 256), 256, 0, st>>>(
         row_dst, g.row_eid.as<uint32_t>(), g.row_src.as<uint32_t>(), a0.as<uint32_t>(),
         b0.as<uint32_t>(), a1.as<uint32_t>(), b1.as<uint32_t>(), tprod, rank_p.as<uint32_t>(),
         c1.as<uint32_t>(), rank1.as<uint32_t>(), c0.as<uint32_t>(), rank0.as<uint32_t>(),
-        c2.as<uint32_t>(), rank2.as<uint32_t>(), m, out[0], out[1], out[2], out[3]);
+        c2.as<uint32_t>(), rank2.as<uint32_t>(), g.row_t.as<uint32_t>(), m, out[0], out[1], out[2], out[3]);
     RR_LAUNCHED();
 
     // deep rows (layers >= 3) and the last-layer rows that read them
@@ -448,15 +452,15 @@ rr_status build_lists_v2(Graph &g, const uint32_t *row_dst, const uint32_t *tpro
         const size_t db = (size_t)std::max<uint32_t>(1, c3[0]) * 4;
         const size_t tb = (size_t)std::max<uint32_t>(1, c3[1]) * 4;
         for (DevBuf *b : {&D.head, &D.eid, &D.src, &D.a1, &D.b1, &D.a3, &D.b3}) RR_CUDA(b->reserve(db));
-        for (DevBuf *b : {&T.head, &T.eid, &T.src, &T.a3, &T.b3}) RR_CUDA(b->reserve(tb));
+        for (DevBuf *b : {&T.head, &T.eid, &T.src, &T.a3, &T.b3, &T.time}) RR_CUDA(b->reserve(tb));
         ListOut od{D.head.as<uint32_t>(), D.eid.as<uint32_t>(), D.src.as<uint32_t>(), nullptr, nullptr,
-                   D.a1.as<uint32_t>(), D.b1.as<uint32_t>(), D.a3.as<uint32_t>(), D.b3.as<uint32_t>()};
+                   D.a1.as<uint32_t>(), D.b1.as<uint32_t>(), D.a3.as<uint32_t>(), D.b3.as<uint32_t>(), nullptr};
         ListOut ot{T.head.as<uint32_t>(), T.eid.as<uint32_t>(), T.src.as<uint32_t>(), nullptr, nullptr,
-                   nullptr, nullptr, T.a3.as<uint32_t>(), T.b3.as<uint32_t>()};
+                   nullptr, nullptr, T.a3.as<uint32_t>(), T.b3.as<uint32_t>(), T.time.as<uint32_t>()};
         k_v2_scatter3<<<grid_for(m, 256), 256, 0, st>>>(
             row_dst, g.row_eid.as<uint32_t>(), g.row_src.as<uint32_t>(), a1.as<uint32_t>(),
             b1.as<uint32_t>(), a3.as<uint32_t>(), b3.as<uint32_t>(), d.as<uint32_t>(),
-            rank_d.as<uint32_t>(), c4.as<uint32_t>(), rank4.as<uint32_t>(), m, od, ot);
+            rank_d.as<uint32_t>(), c4.as<uint32_t>(), rank4.as<uint32_t>(), g.row_t.as<uint32_t>(), m, od, ot);
         RR_LAUNCHED();
         RR_CUDA(cudaStreamSynchronize(st));
     }
@@ -616,7 +620,9 @@ rr_status graph_load(uint32_t n, uint64_t m, const uint32_t *src, const uint32_t
     cudaStream_t st = g->stream;
 
     RR_CUDA(g->off.reserve((size_t)(n + 1) * 4));
+    g->point_flags = (flags & ~1u) != 0;
     if (color) {
+        g->h_color.assign(color, color + n);
         RR_CUDA(g->color.reserve(n));
         RR_CUDA(cudaMemcpyAsync(g->color.p, color, n, cudaMemcpyHostToDevice, st));
         // counting sort of the vertices by colour
@@ -632,12 +638,14 @@ rr_status graph_load(uint32_t n, uint64_t m, const uint32_t *src, const uint32_t
                       &g->row_hi})
         RR_CUDA(b->reserve(mb * 4));
 
-    DevBuf d_delta;
-    RR_CUDA(d_delta.reserve((size_t)n * 4));
-    RR_CUDA(cudaMemcpyAsync(d_delta.p, delta, (size_t)n * 4, cudaMemcpyHostToDevice, st));
+    RR_CUDA(g->delta.reserve((size_t)n * 4));
+    RR_CUDA(cudaMemcpyAsync(g->delta.p, delta, (size_t)n * 4, cudaMemcpyHostToDevice, st));
+    RR_CUDA(g->o_off.reserve((size_t)(n + 1) * 4));
+    for (DevBuf *b : {&g->o_time, &g->o_dst, &g->o_eid}) RR_CUDA(b->reserve((size_t)(m ? m : 1) * 4));
 
     if (m == 0) {
         RR_CUDA(cudaMemsetAsync(g->off.p, 0, (size_t)(n + 1) * 4, st));
+        RR_CUDA(cudaMemsetAsync(g->o_off.p, 0, (size_t)(n + 1) * 4, st));
     } else {
         DevBuf d_src, d_dst, d_t, key_in, key_out, val_in, tmp;
         RR_CUDA(d_src.reserve(mb * 4));
@@ -664,21 +672,36 @@ rr_status graph_load(uint32_t n, uint64_t m, const uint32_t *src, const uint32_t
                                                 key_out.as<uint64_t>(), val_in.as<uint32_t>(),
                                                 g->row_eid.as<uint32_t>(), (int64_t)m, 0,
                                                 32 + head_bits, st));
-        key_in.release();
-        val_in.release();
-        d_dst.release();
-        d_t.release();
+        // (the key buffers are used once more below)
         RR_CUDA(g->row_t.reserve(mb * 4));
         RR_CUDA(g->row_head.reserve(mb * 4));
         k_unpack_rows<<<grid_for(m, 256), 256, 0, st>>>(
             key_out.as<uint64_t>(), g->row_eid.as<uint32_t>(), d_src.as<uint32_t>(), m,
             g->row_t.as<uint32_t>(), g->row_head.as<uint32_t>(), g->row_src.as<uint32_t>());
         RR_LAUNCHED();
-        key_out.release();
-        d_src.release();
         k_offsets<<<grid_for(m + 1, 256), 256, 0, st>>>(g->row_head.as<uint32_t>(), m, n,
                                                         g->off.as<uint32_t>());
         RR_LAUNCHED();
+        // the edges by (tail, time): what leaves a vertex in a window
+        k_make_keys<<<grid_for(m, 256), 256, 0, st>>>(d_src.as<uint32_t>(), d_t.as<uint32_t>(), m,
+                                                      key_in.as<uint64_t>(), val_in.as<uint32_t>());
+        RR_LAUNCHED();
+        RR_CUDA(cub::DeviceRadixSort::SortPairs(tmp.p, tmp_bytes, key_in.as<uint64_t>(),
+                                                key_out.as<uint64_t>(), val_in.as<uint32_t>(),
+                                                g->o_eid.as<uint32_t>(), (int64_t)m, 0, 32 + head_bits, st));
+        // (the tails go through the value buffer, free again)
+        k_unpack_rows<<<grid_for(m, 256), 256, 0, st>>>(
+            key_out.as<uint64_t>(), g->o_eid.as<uint32_t>(), d_dst.as<uint32_t>(), m,
+            g->o_time.as<uint32_t>(), val_in.as<uint32_t>(), g->o_dst.as<uint32_t>());
+        RR_LAUNCHED();
+        k_offsets<<<grid_for(m + 1, 256), 256, 0, st>>>(val_in.as<uint32_t>(), m, n, g->o_off.as<uint32_t>());
+        RR_LAUNCHED();
+        key_in.release();
+        key_out.release();
+        val_in.release();
+        d_src.release();
+        d_dst.release();
+        d_t.release();
 
         DevBuf diff, cover, prod, tprod, rank, counter;
         RR_CUDA(counter.reserve(16));
@@ -687,7 +710,7 @@ rr_status graph_load(uint32_t n, uint64_t m, const uint32_t *src, const uint32_t
         RR_CUDA(cudaMemsetAsync(diff.p, 0, (mb + 1) * 4, st));
         k_windows<<<grid_for(m, 256), 256, 0, st>>>(
             g->row_t.as<uint32_t>(), g->row_src.as<uint32_t>(), g->off.as<uint32_t>(),
-            d_delta.as<uint32_t>(), m, g->row_lo.as<uint32_t>(), g->row_hi.as<uint32_t>(),
+            g->delta.as<uint32_t>(), m, g->row_lo.as<uint32_t>(), g->row_hi.as<uint32_t>(),
             diff.as<int32_t>(), counter.as<unsigned long long>());
         RR_LAUNCHED();
         RR_CUDA(prod.reserve(mb * 4));
@@ -757,6 +780,8 @@ rr_status graph_load(uint32_t n, uint64_t m, const uint32_t *src, const uint32_t
     if (!items.empty())
         RR_CUDA(cudaMemcpyAsync(g->items.p, items.data(), items.size() * sizeof(uint2),
                                 cudaMemcpyHostToDevice, st));
+    rr_status xs = frontier_load(*g, st);
+    if (xs != RR_OK) return xs;
     RR_CUDA(cudaStreamSynchronize(st));
     *out = guard.release();
     return RR_OK;

@@ -117,6 +117,9 @@ struct Workspace {
     cudaEvent_t ring_ev[kRing] = {};
     bool ring_used[kRing] = {};
     uint32_t ring_pos = 0;
+    // frontier engine: barrier counters, and a host flag its bounded waits set
+    DevBuf x_bar;
+    uint32_t *x_err = nullptr;
     // launch the query's kernels with programmatic dependent launch (off for
     // workspaces whose queries run concurrently with others)
     bool pdl = true;
@@ -143,6 +146,7 @@ struct Workspace {
         if (h_ring) cudaFreeHost(h_ring);
         if (h_bring) cudaFreeHost(h_bring);
         if (side) cudaStreamDestroy(side);
+        if (x_err) cudaFreeHost(x_err);
         for (cudaEvent_t e : bev)
             if (e) cudaEventDestroy(e);
     }
@@ -184,9 +188,13 @@ struct RowList {
     // covers; UINT32_MAX when u heads none)
     DevBuf heads, trank;
     uint32_t nheads = 0;
+    // frontier engine: the windows' first positions in the list of the layer
+    // before (w0 producers, w1 state rows, w3 deep rows; the ends are a0/a1/a3),
+    // and of the lists a last layer reads the edges' times
+    DevBuf w0, w1, w3, time;
     size_t bytes() const
     {
-        return head.bytes + eid.bytes + src.bytes + a0.bytes + b0.bytes + a1.bytes + b1.bytes +
+        return w0.bytes + w1.bytes + w3.bytes + time.bytes + head.bytes + eid.bytes + src.bytes + a0.bytes + b0.bytes + a1.bytes + b1.bytes +
                a3.bytes + b3.bytes + items.bytes + items_coarse.bytes + chains.bytes + fix2.bytes +
                heads.bytes + trank.bytes + row_carry.bytes + chain_slot0.bytes;
     }
@@ -315,6 +323,18 @@ struct Graph {
     //   tail3_list rows whose window holds a deep row (last layer, k >= 5)
     RowList prod_list, state_list, win_list, tail_list, deep_list, tail3_list;
 
+    // frontier engine (rr_frontier.cu): the edges sorted by (tail, time) --
+    // offsets (n + 1), times, heads, input indexes --, the waiting times,
+    // subset tables, launch limits, and the colours on the host (the source's
+    // z row is formed there)
+    DevBuf o_off, o_time, o_dst, o_eid, delta;
+    DevBuf x_tab;
+    int x_sms = 0;
+    uint32_t x_smem_max = 0;
+    std::vector<uint8_t> h_color;
+    // load flags that choose a form of the sieve-point engine keep every query on it
+    bool point_flags = false;
+
     // per-graph scratch for rr_reach_device / rr_reach_sync (serialised by mu)
     mutable std::mutex mu;
     mutable Workspace ws;
@@ -331,6 +351,9 @@ struct Graph {
     uint32_t tune_ppl[32] = {0};
     uint32_t tune_chunk[32] = {0};
     uint64_t tune_gen = 1;
+    // rr_set_tuning chose a point shape for this k: its queries stay on the
+    // sieve-point engine
+    bool tune_forced[32] = {false};
     // shape of the persistent batch (rr_autotune_batch / rr_set_batch_tuning;
     // 0 = the automatic rule): kernel variant by blocks per SM (2, 4 or 6),
     // scheduling ranges (1 fine, 2 coarse) and the largest point chunk
@@ -338,7 +361,7 @@ struct Graph {
 
     size_t device_bytes() const
     {
-        return off.bytes + row_a.bytes + row_b.bytes + row_s.bytes + row_eid.bytes +
+        return x_tab.bytes + o_off.bytes + o_time.bytes + o_dst.bytes + o_eid.bytes + delta.bytes + off.bytes + row_a.bytes + row_b.bytes + row_s.bytes + row_eid.bytes +
                row_src.bytes + row_lo.bytes + row_hi.bytes + row_t.bytes + row_head.bytes +
                color.bytes + color_order.bytes + items.bytes +
                prod_list.bytes() + state_list.bytes() + win_list.bytes() + tail_list.bytes() +
@@ -468,6 +491,26 @@ uint32_t atmost_first_branch(const Graph &g, uint32_t k);
 // lane): the load flags' choice, else atmost_first_branch where the k query's
 // per-point layers are long.
 uint32_t atmost_branches(const Graph &g, uint32_t k);
+
+// Frontier engine (rr_frontier.cu): whole queries of k <= 16 on compact graphs
+// whose load flags and tuning leave the choice to the library.
+bool uses_frontier(const Graph &g, uint32_t k);
+// Scratch bytes (ws.state) of a query; every: at-most-k, arrivals: with d_R.
+struct SourceSet {
+    const uint8_t *mask;   // n flags (device)
+    const uint32_t *list;  // the flagged vertices, each once (device)
+    uint32_t count;
+};
+uint64_t frontier_bytes(const Graph &g, uint32_t k, bool every = false, bool multi = false, bool arrivals = false);
+// Allocates the workspace's barrier counters (otherwise done by its first query).
+rr_status frontier_reserve(Workspace &ws, cudaStream_t st);
+// RR_ETIMEDOUT, once, when a bounded wait of a finished query on ws gave up.
+rr_status frontier_error(Workspace &ws);
+rr_status frontier_load(Graph &g, cudaStream_t st);
+rr_status frontier_query(const Graph &g, Workspace &ws, const rr_query *q, bool every, uint8_t *d_bitmap,
+                         uint64_t *d_witness, cudaStream_t st, uint64_t *d_E = nullptr,
+                         const uint8_t *d_vmask = nullptr, uint32_t *d_R = nullptr,
+                         const SourceSet *src = nullptr);
 
 // Held (under the graph's lock) by every call that uses the graph's scratch:
 // the call's stream first waits for the previous such call's work, and the

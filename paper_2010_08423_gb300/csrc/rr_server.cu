@@ -474,6 +474,8 @@ rr_status rr_server_create(const rr_graph *g, uint64_t device_mem_budget, uint32
         RR_CUDA(sl.ws.z.reserve((size_t)g->n * 20 * 8));
         RR_CUDA(sl.ws.S.reserve((size_t)g->n * 8));
         RR_CUDA(sl.ws.shade.reserve(sizeof(ShadeTable)));
+        rr_status fs = frontier_reserve(sl.ws, sl.stream);
+        if (fs != RR_OK) return fs;
     }
     // one spare result buffer per slot: completed queries keep theirs until
     // polled, and serving allocates only when more than that are waiting

@@ -485,6 +485,10 @@ uint64_t query_scratch_bytes(const Graph &g, uint32_t k, uint64_t budget)
 {
     uint32_t ppl = 0, chunk = 0;
     const uint64_t z = (uint64_t)g.n * k * 8ull + 2048;
+    if (uses_frontier(g, k)) {
+        const uint64_t need = frontier_bytes(g, k);
+        if (need <= budget) return need + z;
+    }
     if (uses_v2(g, k)) {
         if (!choose_shape_v2(g, k, budget, &ppl, &chunk)) return UINT64_MAX;
         return v2_scratch_bytes(g, ppl, chunk, k) + z;
@@ -509,6 +513,19 @@ rr_status reach_on_stream(const Graph &g, Workspace &ws, const rr_query *q, uint
     if (bfirst && (!v2 || q->motif || d_vmask || !range.full(k) || bfirst < atmost_first_branch(g, k) ||
                    k - bfirst > Workspace::kMaxBranches))
         return fail(RR_EINVAL, "internal: at-most-k branches need a plain whole query on the reduced-state engine");
+    if (!bfirst && !d_srcmask && range.full(k) && uses_frontier(g, k)) {
+        const uint64_t need = frontier_bytes(g, k);
+        uint64_t room = budget;
+        if (need > ws.state.bytes && budget == 0) {
+            size_t free_b = 0, total_b = 0;
+            RR_CUDA(cudaMemGetInfo(&free_b, &total_b));
+            room = (uint64_t)(0.6 * (double)(free_b + ws.state.bytes));
+        }
+        if (need <= ws.state.bytes || need <= room) {
+            RR_CUDA(ws.state.reserve(need));
+            return frontier_query(g, ws, q, false, d_bitmap, d_witness, st, d_E, d_vmask);
+        }
+    }
     if (d_srcmask && budget == 0) {
         size_t free_b = 0, total_b = 0;
         RR_CUDA(cudaMemGetInfo(&free_b, &total_b));
