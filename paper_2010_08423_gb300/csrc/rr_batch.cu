@@ -1063,6 +1063,14 @@ rr_status debug_wait_probe(uint64_t timeout_ns, int abort_preset, int32_t *statu
 rr_status atmost_device(const Graph &g, uint32_t source, uint32_t k, uint64_t seed,
                         uint8_t *d_bitmap, uint64_t *d_witness, cudaStream_t st)
 {
+    {
+        // frontier engine: the k query's rows, values on the first k' - 1 labels
+        // and one out level per k' (headline graph, k = 10: 25.9 -> 5.1 ms)
+        const rr_query q{source, k, seed, nullptr};
+        rr_status fs = RR_OK;
+        if (frontier_fits(g, g.ws, k, 0, true, false, false, &fs))
+            return fs != RR_OK ? fs : frontier_query(g, g.ws, &q, true, d_bitmap, d_witness, st);
+    }
     const uint32_t lanes = k - 1;
     size_t free_b = 0, total_b = 0;
     RR_CUDA(cudaMemGetInfo(&free_b, &total_b));

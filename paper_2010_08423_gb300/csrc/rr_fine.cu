@@ -105,6 +105,23 @@ __global__ void k_merge_arrival(uint32_t n, const uint32_t *__restrict__ Rk, uin
     }
 }
 
+// All rows of k' = 2..k at once: R[v] = the smallest of the rows' values, L[v]
+// the first row (as k') with one.
+__global__ void k_merge_rows(uint32_t n, uint32_t k, const uint32_t *__restrict__ rows, uint32_t *__restrict__ R,
+                             uint8_t *__restrict__ L)
+{
+    for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
+        uint32_t best = 0xFFFFFFFFu, len = 0;
+        for (uint32_t kk = 2; kk <= k; ++kk) {
+            const uint32_t r = rows[(size_t)(kk - 2) * n + v];
+            if (r != 0xFFFFFFFFu && !len) len = kk;
+            best = min(best, r);
+        }
+        R[v] = best;
+        if (L) L[v] = (uint8_t)len;
+    }
+}
+
 rr_status arrival_device(const Graph &g, const rr_query *q, uint64_t *d_witness, uint64_t *d_E,
                          uint32_t *d_R, uint8_t *d_bitmap, cudaStream_t st, const uint8_t *d_vmask)
 {
@@ -273,6 +290,28 @@ rr_status sources_device(const Graph &g, const uint32_t *sources, uint32_t nsour
 rr_status atmost_arrival_device(const Graph &g, uint32_t source, uint32_t k, uint64_t seed,
                                 uint32_t *d_R, uint8_t *d_L, uint8_t *d_bitmap, cudaStream_t st)
 {
+    {
+        // frontier engine: every k' from the k query's rows, the arrivals from
+        // its out rows alone (no per-edge sums of all m edges)
+        const rr_query q{source, k, seed, nullptr};
+        rr_status fs = RR_OK;
+        Workspace &ws = g.ws;
+        if (frontier_fits(g, ws, k, 0, true, false, true, &fs)) {
+            if (fs != RR_OK) return fs;
+            RR_CUDA(ws.bS.reserve((size_t)(k - 1) * g.n * 8));
+            RR_CUDA(ws.bR.reserve((size_t)(k - 1) * g.n * 4));
+            RR_CUDA(cudaMemsetAsync(ws.bR.p, 0xFF, (size_t)(k - 1) * g.n * 4, st));
+            fs = frontier_query(g, ws, &q, true, nullptr, ws.bS.as<uint64_t>(), st, nullptr, nullptr, ws.bR.as<uint32_t>());
+            if (fs != RR_OK) return fs;
+            k_merge_rows<<<grid_for(g.n, 256), 256, 0, st>>>(g.n, k, ws.bR.as<uint32_t>(), d_R, d_L);
+            RR_LAUNCHED();
+            if (d_bitmap) {
+                k_arrival_bitmap<<<grid_for((g.n + 7) / 8, 256), 256, 0, st>>>(g.n, d_R, d_bitmap);
+                RR_LAUNCHED();
+            }
+            return RR_OK;
+        }
+    }
     const uint32_t lanes = k - 1;
     const size_t mb = (size_t)std::max<uint64_t>(1, g.m) * 8;
     size_t free_b = 0, total_b = 0;

@@ -1550,6 +1550,26 @@ uint64_t frontier_bytes(const Graph &g, uint32_t k, bool every, bool multi, bool
     return x_template(lists, k, every, multi, arrivals, t);
 }
 
+bool frontier_fits(const Graph &g, Workspace &ws, uint32_t k, uint64_t budget, bool every, bool multi, bool arrivals,
+                   rr_status *st)
+{
+    *st = RR_OK;
+    // a set of sources keeps all k labels, at-most-k answers every smaller k too
+    if (!uses_frontier(g, k) || (multi && k > kXMaxLabels)) return false;
+    for (uint32_t kk = 2; every && kk < k; ++kk)
+        if (!uses_frontier(g, kk)) return false;
+    const uint64_t need = frontier_bytes(g, k, every, multi, arrivals);
+    if (need > ws.state.bytes && budget == 0) {
+        size_t free_b = 0, total_b = 0;
+        if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return false;
+        budget = (uint64_t)(0.6 * (double)(free_b + ws.state.bytes));
+    }
+    if (need > ws.state.bytes && need > budget) return false;
+    const cudaError_t e = ws.state.reserve(need);
+    if (e != cudaSuccess) *st = cuda_fail(e, "cudaMalloc (query scratch)", __FILE__, __LINE__);
+    return true;
+}
+
 template <bool BATCH>
 static rr_status x_launch(const Graph &g, const XArgs &a, const XOne &one, cudaStream_t st)
 {

@@ -502,6 +502,10 @@ struct SourceSet {
     uint32_t count;
 };
 uint64_t frontier_bytes(const Graph &g, uint32_t k, bool every = false, bool multi = false, bool arrivals = false);
+// Reserves ws.state for such a query when it fits `budget` (0: 60% of free device
+// memory, the workspace's own counted in); false: it does not.
+bool frontier_fits(const Graph &g, Workspace &ws, uint32_t k, uint64_t budget, bool every, bool multi, bool arrivals,
+                   rr_status *st);
 // Allocates the workspace's barrier counters (otherwise done by its first query).
 rr_status frontier_reserve(Workspace &ws, cudaStream_t st);
 // RR_ETIMEDOUT, once, when a bounded wait of a finished query on ws gave up.

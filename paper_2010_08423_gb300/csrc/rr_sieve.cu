@@ -513,19 +513,9 @@ rr_status reach_on_stream(const Graph &g, Workspace &ws, const rr_query *q, uint
     if (bfirst && (!v2 || q->motif || d_vmask || !range.full(k) || bfirst < atmost_first_branch(g, k) ||
                    k - bfirst > Workspace::kMaxBranches))
         return fail(RR_EINVAL, "internal: at-most-k branches need a plain whole query on the reduced-state engine");
-    if (!bfirst && !d_srcmask && range.full(k) && uses_frontier(g, k)) {
-        const uint64_t need = frontier_bytes(g, k);
-        uint64_t room = budget;
-        if (need > ws.state.bytes && budget == 0) {
-            size_t free_b = 0, total_b = 0;
-            RR_CUDA(cudaMemGetInfo(&free_b, &total_b));
-            room = (uint64_t)(0.6 * (double)(free_b + ws.state.bytes));
-        }
-        if (need <= ws.state.bytes || need <= room) {
-            RR_CUDA(ws.state.reserve(need));
-            return frontier_query(g, ws, q, false, d_bitmap, d_witness, st, d_E, d_vmask);
-        }
-    }
+    rr_status fs = RR_OK;
+    if (!bfirst && !d_srcmask && range.full(k) && frontier_fits(g, ws, k, budget, false, false, false, &fs))
+        return fs != RR_OK ? fs : frontier_query(g, ws, q, false, d_bitmap, d_witness, st, d_E, d_vmask);
     if (d_srcmask && budget == 0) {
         size_t free_b = 0, total_b = 0;
         RR_CUDA(cudaMemGetInfo(&free_b, &total_b));
