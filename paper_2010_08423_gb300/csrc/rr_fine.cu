@@ -10,6 +10,7 @@
 // values are XOR-ed, and R_u is the smallest time of a run with a non-zero
 // sum (UINT32_MAX when there is none). D = {u : R_u < UINT32_MAX}.
 #include <algorithm>
+#include <cstring>
 
 #include "rr_internal.h"
 
@@ -132,6 +133,21 @@ rr_status arrival_on(const Graph &g, Workspace &ws, const rr_query *q, uint64_t 
                      uint64_t *d_E, uint32_t *d_R, uint8_t *d_bitmap, cudaStream_t st,
                      const uint8_t *d_vmask, uint64_t budget, uint32_t bfirst)
 {
+    rr_status xs = RR_OK;
+    if (!bfirst && frontier_fits(g, ws, q->k, budget, false, false, true, &xs)) {
+        // frontier engine: the arrival times from the out rows alone; the
+        // per-edge sums only when the caller wants them
+        if (xs != RR_OK) return xs;
+        if (d_E && g.m) RR_CUDA(cudaMemsetAsync(d_E, 0, (size_t)g.m * 8, st));
+        RR_CUDA(cudaMemsetAsync(d_R, 0xFF, (size_t)g.n * 4, st));
+        xs = frontier_query(g, ws, q, false, nullptr, d_witness, st, d_E, d_vmask, d_R);
+        if (xs != RR_OK) return xs;
+        if (d_bitmap) {
+            k_arrival_bitmap<<<grid_for((g.n + 7) / 8, 256), 256, 0, st>>>(g.n, d_R, d_bitmap);
+            RR_LAUNCHED();
+        }
+        return RR_OK;
+    }
     if (!d_E) {
         RR_CUDA(ws.edges.reserve((size_t)std::max<uint64_t>(1, g.m) * 8));
         d_E = ws.edges.as<uint64_t>();
@@ -262,8 +278,9 @@ rr_status extract_path(const Graph &g, const rr_query *q, uint32_t target, uint3
 // k-RestlessReach from a set of sources, optionally avoiding separators (Sec.
 // "Discussion": the multi-source variant; the case study's separators). Walks
 // start at every edge leaving a source; the sums are the XOR of the
-// single-source sums. One source runs the reduced-state engine, a larger set
-// the per-point engine with a source mask.
+// single-source sums. One source is a query with deleted vertices; a larger set
+// goes to the frontier engine over all k labels (k <= 15: no source's row can be
+// eliminated) or to the per-point engine with a source mask.
 rr_status sources_device(const Graph &g, const uint32_t *sources, uint32_t nsources, uint32_t k,
                          uint64_t seed, const uint8_t *motif, const uint8_t *d_separators,
                          uint8_t *d_bitmap, uint64_t *d_witness, cudaStream_t st)
@@ -271,12 +288,25 @@ rr_status sources_device(const Graph &g, const uint32_t *sources, uint32_t nsour
     const rr_query q{sources[0], k, seed, motif};
     if (nsources == 1)
         return reach_on_stream(g, g.ws, &q, d_bitmap, d_witness, 0, st, nullptr, d_separators);
-    std::vector<uint8_t> flags(g.n, 0);
-    for (uint32_t i = 0; i < nsources; ++i) flags[sources[i]] = 1;
+    // the flags of all vertices, then the flagged ones, each once
+    const size_t at = ((size_t)g.n + 15) / 16 * 16;
+    std::vector<uint8_t> flags(at + (size_t)nsources * 4, 0);
+    uint32_t count = 0;
+    for (uint32_t i = 0; i < nsources; ++i) {
+        if (flags[sources[i]]) continue;
+        flags[sources[i]] = 1;
+        std::memcpy(flags.data() + at + (size_t)count++ * 4, &sources[i], 4);
+    }
     Workspace &ws = g.ws;
-    RR_CUDA(ws.srcmask.reserve(g.n));
+    RR_CUDA(ws.srcmask.reserve(flags.size()));
     // pageable source: the copy is staged before the call returns
-    RR_CUDA(cudaMemcpyAsync(ws.srcmask.p, flags.data(), g.n, cudaMemcpyHostToDevice, st));
+    RR_CUDA(cudaMemcpyAsync(ws.srcmask.p, flags.data(), flags.size(), cudaMemcpyHostToDevice, st));
+    rr_status xs = RR_OK;
+    if (frontier_fits(g, ws, k, 0, false, true, false, &xs)) {
+        if (xs != RR_OK) return xs;
+        const SourceSet set{ws.srcmask.as<uint8_t>(), reinterpret_cast<const uint32_t *>(ws.srcmask.as<uint8_t>() + at), count};
+        return frontier_query(g, ws, &q, false, d_bitmap, d_witness, st, nullptr, d_separators, nullptr, &set);
+    }
     return reach_on_stream(g, ws, &q, d_bitmap, d_witness, 0, st, nullptr, d_separators,
                            ws.srcmask.as<uint8_t>());
 }
