@@ -360,6 +360,7 @@ rr_status rr_set_batch_tuning(rr_graph *g, const rr_batch_tuning *t)
     g->batch_minb = t->blocks_per_sm;
     g->batch_ranges = t->ranges;
     g->batch_max_chunk = t->max_chunk;
+    g->batch_forced = t->blocks_per_sm || t->ranges || t->max_chunk;
     return RR_OK;
 }
 

@@ -1253,6 +1253,8 @@ k_frontier(const __grid_constant__ XArgs a_, const __grid_constant__ XOne one_, 
             }
         }
     }
+    if (BATCH && !ok && a.status)
+        for (uint32_t i = threadIdx.x; i < a.nq; i += blockDim.x) a.status[i] = (int32_t)RR_ETIMEDOUT;
     // the last block to leave clears the counters for the next launch
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -1488,6 +1490,28 @@ static uint64_t gf64_inverse(uint64_t x)
     return (uint64_t)g1;
 }
 
+// Products with one factor: its 16 multiples by polynomials of degree < 4, and
+// the other factor four bits at a time.
+struct GfTimes {
+    uint64_t t[16];
+    explicit GfTimes(uint64_t a)
+    {
+        t[0] = 0;
+        t[1] = a;
+        for (int i = 2; i < 16; ++i) t[i] = i & 1 ? t[i - 1] ^ a : shl(t[i / 2], 1);
+    }
+    static uint64_t shl(uint64_t v, int n)  // v x^n, n <= 4
+    {
+        return gf64_reduce(v >> (64 - n), v << n);
+    }
+    uint64_t operator()(uint64_t b) const
+    {
+        uint64_t r = t[b >> 60];
+        for (int s = 56; s >= 0; s -= 4) r = shl(r, 4) ^ t[(b >> s) & 15u];
+        return r;
+    }
+};
+
 static void x_query(const Graph &g, const rr_query &q, bool multi, XQuery &X)
 {
     std::memset(&X, 0, sizeof X);
@@ -1532,9 +1556,9 @@ static void x_query(const Graph &g, const rr_query &q, bool multi, XQuery &X)
     }
     X.pivot = p;
     X.d0 = zs[p];
-    const uint64_t inv = gf64_inverse(zs[p]);
+    const GfTimes by_inverse(gf64_inverse(zs[p]));
     for (uint32_t j = 0, t = 0; j < k; ++j)
-        if (j != p) X.rho[t++] = gf64_mul(zs[j], inv);
+        if (j != p) X.rho[t++] = by_inverse(zs[j]);
 }
 
 bool uses_frontier(const Graph &g, uint32_t k)
@@ -1667,6 +1691,75 @@ rr_status frontier_query(const Graph &g, Workspace &ws, const rr_query *q, bool 
     a.bzero_n = d_bitmap ? (g.n + 7) / 8 : 0;
     a.tiny = g_timing.load(std::memory_order_relaxed) ? 0u : 1u;
     return x_launch<false>(g, a, one, st);
+}
+
+// A batch in one launch: the queries' descriptions go to the device with one
+// copy, blocks take queries from a counter (x_tiny), and the queries that do not
+// fit follow, one per block when there are many (each block with its own region
+// of scratch) or one at a time by the whole grid. idx: the queries of qs to run
+// (the witnesses of all nq are cleared); false when one query's scratch does not
+// fit `budget`.
+bool frontier_batch(const Graph &g, const rr_query *qs, uint32_t nq, const std::vector<uint32_t> &idx, uint64_t budget,
+                    uint8_t *d_bitmaps, uint64_t *d_witness, int32_t *d_status, cudaStream_t st, rr_status *ret)
+{
+    *ret = RR_OK;
+    Workspace &ws = g.ws;
+    BatchBuffers &B = g.batch;
+    XArgs a{};
+    x_args(g, a);
+    const uint32_t count = (uint32_t)idx.size();
+    bool used[kXMaxLabels + 2] = {false};
+    for (uint32_t i : idx) used[qs[i].k] = true;
+    const size_t tbytes = sizeof(XTmpl) * (kXMaxLabels + 2), qbytes = sizeof(XQuery) * (size_t)count;
+    auto run = [&]() -> rr_status {
+        uint64_t stride = 0;
+        std::vector<XTmpl> tm(kXMaxLabels + 2);
+        for (uint32_t k = 2; k <= kXMaxLabels + 1; ++k)
+            if (used[k]) stride = std::max(stride, x_template(a.lists, k, false, false, false, tm[k]));
+        stride = (stride + 255) / 256 * 256;
+        if (stride > budget) return RR_EAGAIN;
+        // a region per block while they stay within kBatchScratch
+        constexpr uint64_t kBatchScratch = 24ull << 30;
+        const uint64_t room = std::max<uint64_t>(stride, std::min<uint64_t>(budget, kBatchScratch));
+        a.lanes = (uint32_t)std::min<uint64_t>({(uint64_t)g.x_sms, (uint64_t)count, room / stride});
+        RR_CUDA(ws.state.reserve(a.lanes * stride));
+        rr_status s = x_control(ws, st, a);
+        if (s != RR_OK) return s;
+        RR_CUDA(B.xq.reserve(tbytes + qbytes));
+        RR_CUDA(B.left.reserve((size_t)count * 4));
+        s = B.stage_wait(tbytes + qbytes);
+        if (s != RR_OK) return s;
+        std::memcpy(B.h_stage, tm.data(), tbytes);
+        XQuery *hq = reinterpret_cast<XQuery *>(B.h_stage + tbytes);
+        const size_t nb = (g.n + 7) / 8;
+        for (uint32_t j = 0; j < count; ++j) {
+            const uint32_t i = idx[j];
+            x_query(g, qs[i], false, hq[j]);
+            hq[j].S = d_witness + (size_t)i * g.n;
+            hq[j].bitmap = d_bitmaps ? d_bitmaps + (size_t)i * nb : nullptr;
+        }
+        RR_CUDA(cudaMemcpyAsync(B.xq.p, B.h_stage, tbytes + qbytes, cudaMemcpyHostToDevice, st));
+        s = B.stage_done(st);
+        if (s != RR_OK) return s;
+        a.xt = B.xq.as<XTmpl>();
+        a.xq = reinterpret_cast<const XQuery *>(B.xq.as<uint8_t>() + tbytes);
+        a.left = B.left.as<uint32_t>();
+        a.nq = count;
+        a.scratch = ws.state.as<uint8_t>();
+        a.stride = stride;
+        a.szero = d_witness;
+        a.szero_n = (uint64_t)g.n * nq;
+        a.bzero = d_bitmaps;
+        a.bzero_n = d_bitmaps ? (uint64_t)nb * nq : 0;
+        a.status = d_status && count == nq ? d_status : nullptr;
+        a.tiny = 1;
+        static const XOne none{};
+        return x_launch<true>(g, a, none, st);
+    };
+    *ret = run();
+    if (*ret != RR_EAGAIN) return true;
+    *ret = RR_OK;
+    return false;
 }
 
 }  // namespace rr

@@ -213,6 +213,31 @@ struct BatchBuffers {
     // its register budget is set for; 0 = not queried yet)
     int occupancy[8] = {0};
     int sms = 0;
+    DevBuf xq, left;  // frontier engine: templates and queries, the queries left to the bitmap passes
+    // Waits until the staging area is free and makes it hold `bytes`.
+    rr_status stage_wait(size_t bytes)
+    {
+        if (stage_pending) {
+            RR_CUDA(cudaEventSynchronize(stage_ev));
+            stage_pending = false;
+        }
+        if (bytes > h_cap) {
+            if (h_stage) cudaFreeHost(h_stage);
+            h_stage = nullptr;
+            h_cap = 0;
+            RR_CUDA(cudaMallocHost(&h_stage, bytes));
+            h_cap = bytes;
+        }
+        return RR_OK;
+    }
+    // Marks the staging area busy until the work enqueued on st so far is done.
+    rr_status stage_done(cudaStream_t st)
+    {
+        if (!stage_ev) RR_CUDA(cudaEventCreateWithFlags(&stage_ev, cudaEventDisableTiming));
+        RR_CUDA(cudaEventRecord(stage_ev, st));
+        stage_pending = true;
+        return RR_OK;
+    }
     ~BatchBuffers()
     {
         if (stage_ev) cudaEventDestroy(stage_ev);
@@ -358,6 +383,8 @@ struct Graph {
     // 0 = the automatic rule): kernel variant by blocks per SM (2, 4 or 6),
     // scheduling ranges (1 fine, 2 coarse) and the largest point chunk
     uint32_t batch_minb = 0, batch_ranges = 0, batch_max_chunk = 0;
+    // rr_set_batch_tuning chose a shape: batches stay on the persistent sieve-point kernel
+    bool batch_forced = false;
 
     size_t device_bytes() const
     {
@@ -502,6 +529,8 @@ struct SourceSet {
     uint32_t count;
 };
 uint64_t frontier_bytes(const Graph &g, uint32_t k, bool every = false, bool multi = false, bool arrivals = false);
+bool frontier_batch(const Graph &g, const rr_query *qs, uint32_t nq, const std::vector<uint32_t> &idx, uint64_t budget,
+                    uint8_t *d_bitmaps, uint64_t *d_witness, int32_t *d_status, cudaStream_t st, rr_status *ret);
 // Reserves ws.state for such a query when it fits `budget` (0: 60% of free device
 // memory, the workspace's own counted in); false: it does not.
 bool frontier_fits(const Graph &g, Workspace &ws, uint32_t k, uint64_t budget, bool every, bool multi, bool arrivals,

@@ -98,3 +98,30 @@ def test_windows_over_many_blocks(rows):
             _, w = G.reach(0, k, 31 + k)
             assert np.array_equal(w, oracle.sieve(g, 0, k, 31 + k)), k
             assert w.any()
+
+
+@pytest.mark.parametrize("nq", [1, 5, 60])
+def test_batches_whose_queries_fill_the_rows(nq):
+    # no query fits one block's memory: few go one after another over the whole
+    # grid, many one per block; one with k = 17 goes to the per-point engine
+    import torch
+    g = W.uniform(300, 5_001, 40, 0, 8, 17, ncolors=2)
+    n = g["n"]
+    qs = W.query_set(g, nq, 4, 9, 99, ncolors=2)
+    if nq == 5:
+        qs[2] = {"source": 3, "k": 17, "seed": 8, "motif": None}
+    with capi.Graph(g) as G:
+        d_w = torch.full((nq, n), -1, dtype=torch.int64, device="cuda")
+        d_b = torch.full((nq, (n + 7) // 8), 255, dtype=torch.uint8, device="cuda")
+        d_s = torch.full((nq,), -1, dtype=torch.int32, device="cuda")
+        for _ in range(2):
+            capi.rr_reach_batch_device(G.handle, qs, d_w, d_b, d_s)
+        torch.cuda.synchronize()
+        assert not d_s.cpu().numpy().any()
+        w = d_w.cpu().numpy().view(np.uint64)
+        bm = d_b.cpu().numpy()
+        for i, q in enumerate(qs):
+            b1, w1 = G.reach(q["source"], q["k"], q["seed"], motif=q["motif"])
+            assert np.array_equal(w[i], w1) and np.array_equal(bm[i], b1), i
+            if q["k"] <= 6:
+                assert np.array_equal(w1, oracle.sieve(g, q["source"], q["k"], q["seed"], motif=q["motif"])), i
