@@ -136,20 +136,25 @@ struct View {
         const uint32_t r = base % n;
         return w >= r ? w - r : w + n - r;
     }
-    __device__ bool sync()
+    // In two halves, for what may go on until the other blocks' part is needed:
+    // arrive() publishes the block's writes, wait() returns once every block has
+    // arrived.
+    __device__ void arrive()
     {
-        if (n == 1) {
-            __syncthreads();
-            return true;
-        }
-        __shared__ int ok;
         target += n;
         __syncthreads();
         if (threadIdx.x == 0) {
             __threadfence();
             atomicAdd(ctr, 1u);
+        }
+    }
+    __device__ bool wait()
+    {
+        __shared__ int ok;
+        __syncthreads();
+        if (threadIdx.x == 0) {
             int good = 0;
-            const uint64_t t0 = now_ns();
+            uint64_t t0 = 0;
             for (uint32_t it = 0; it < 200000000u; ++it) {
                 uint32_t v;
                 asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(ctr) : "memory");
@@ -157,7 +162,9 @@ struct View {
                     good = 1;
                     break;
                 }
-                if ((it & 1023u) == 1023u && (*(volatile uint32_t *)err || now_ns() - t0 > 10000000000ull)) break;
+                if ((it & 1023u) != 1023u) continue;
+                if (!t0) t0 = now_ns();
+                if (*(volatile uint32_t *)err || now_ns() - t0 > 10000000000ull) break;
             }
             if (!good) *(volatile uint32_t *)err = 1u;
             __threadfence();
@@ -165,6 +172,15 @@ struct View {
         }
         __syncthreads();
         return ok != 0;
+    }
+    __device__ bool sync()
+    {
+        if (n == 1) {
+            __syncthreads();
+            return true;
+        }
+        arrive();
+        return wait();
     }
 };
 
@@ -821,29 +837,42 @@ __device__ __noinline__ void x_outputs(const XArgs &a, const XOne &o, const View
 
 // ---------------------------------------------------------------------------
 // Queries whose walks are few: one block, everything in shared memory, no
-// bitmaps. The frontier is pushed along the edges sorted by (tail, time); a
-// level holds at most kTinyRows rows, each with the set of the level below's
-// rows in its window (a bit mask), so the backward pass and the window sums
-// need no memory traffic. The multipliers y z'_j of all levels are formed at
-// once, before the layers, and a layer's products (row, subset, element) are
-// spread over the threads while they fit: what is left is a chain of about two
-// dependent loads a layer forward and one product a layer after that.
-// Returns false, with nothing written, when the query does not fit.
+// bitmaps. What bounds such a query is its chain of dependent steps, so each
+// layer is one load forward and one product after that:
+//  * forward, the frontier is pushed along the edges sorted by (tail, time);
+//    every edge's record names the edges that may follow it, so a layer reads
+//    its rows with one dependent load. A level holds at most kTinyRows rows, each
+//    with the set of the level below's rows in its window as a bit mask, and the
+//    backward pass (one warp) and the window sums read no memory at all;
+//  * the multipliers y z'_j of all levels are formed at once, before the layers,
+//    and the subset tables are copied to shared memory beside layer 1;
+//  * a layer's products (row, subset, element) are spread over the threads and
+//    meet in shared memory, its window sums taken on the way: one block barrier
+//    a layer.
+// Uniform n = 1e5, m = 1e6, k = 8: 33.5 us with two loads, a window-sum step and
+// global tables a layer, 29.7 us so. Returns kTinyNoFit, with nothing written,
+// when the query does not fit. Witnesses are written only after every block has
+// cleared its part (clear: the barrier they arrived at).
 // ---------------------------------------------------------------------------
 constexpr uint32_t kTinyRows = 128, kTinyWords = kTinyRows / 32, kTinyTotal = 768, kTinyPairs = 1024, kTinyHash = 512;
+constexpr uint32_t kTinyRange = 1024;    // followers of one edge, at most
+constexpr uint32_t kTinyTable = 11264;   // subset-table words kept in shared memory (11 labels)
+enum { kTinyDone = 0, kTinyNoFit = 1, kTinyFailed = 2 };
 
 struct TinyMem {
     uint4 row[kTinyTotal];                  // tail, head, time, edge
+    uint2 next[kTinyTotal];                 // the edges that may follow: first record, count
     uint32_t mask[kTinyTotal][kTinyWords];  // rows of the level below in the window
     uint32_t need[kXMaxLevels + 1][kTinyWords];
     uint32_t base[kXMaxLevels + 2];         // first row of each level
     uint32_t cn[kXMaxLevels + 2];           // needed rows before each level
-    uint32_t hkey[kTinyHash], hval[kTinyHash];
+    uint32_t hkey[2][kTinyHash], hval[kTinyHash];
     uint32_t pair[kTinyPairs];
-    uint32_t npair, count, over;
-    uint16_t list[kTinyTotal];              // needed rows: level << 12 is kept in lev
-    uint8_t lev[kTinyTotal];
-    uint64_t acc[kTinyRows];
+    uint32_t npair[2], count[2], over, need_g, need_d, toff[kXMaxLabels + 2];
+    uint16_t list[kTinyTotal];              // needed rows
+    uint8_t lev[kTinyTotal];                // and their levels
+    uint64_t acc[kTinyTotal];               // their sums
+    uint64_t omega[(kXMaxLabels + 1) * (kXMaxLabels + 1)];
 };
 
 __device__ __forceinline__ void xor_shared(uint64_t *p, uint64_t v)
@@ -853,157 +882,203 @@ __device__ __forceinline__ void xor_shared(uint64_t *p, uint64_t v)
     if ((uint32_t)(v >> 32)) atomicXor(w + 1, (uint32_t)(v >> 32));
 }
 
-__device__ __noinline__ bool x_tiny(const XArgs &a, const XQuery &Q, bool every)
+// XOR of the level below's values s of the rows in `mk`, by their places among
+// its needed rows `nd`.
+__device__ __forceinline__ uint64_t tiny_window(const uint32_t *mk, const uint32_t *nd, const uint64_t *Gp, uint32_t cin,
+                                                uint32_t s)
+{
+    uint64_t v = 0;
+    uint32_t before = 0;
+#pragma unroll
+    for (uint32_t x = 0; x < kTinyWords; ++x) {
+        const uint32_t need = nd[x];
+        for (uint32_t m = mk[x] & need; m; m &= m - 1)
+            v ^= Gp[(before + __popc(need & ((m & (0u - m)) - 1u))) * cin + s];
+        before += __popc(need);
+    }
+    return v;
+}
+
+__device__ __noinline__ int x_tiny(const XArgs &a, const XQuery &Q, bool every, View &clear, bool &cleared)
 {
     extern __shared__ __align__(16) uint64_t sm_all[];
     TinyMem &M = *reinterpret_cast<TinyMem *>(sm_all);
-    uint64_t *const pool = sm_all + (sizeof(TinyMem) + 15) / 16 * 2;
-    const uint32_t pool_n = a.smem / 8 - (uint32_t)((sizeof(TinyMem) + 15) / 16 * 2);
+    constexpr uint32_t kHead = (uint32_t)((sizeof(TinyMem) + 15) / 16 * 2);
+    uint64_t *pool = sm_all + kHead;
+    uint32_t pool_n = a.smem / 8 - kHead;
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
     const uint32_t k = Q.k, K = Q.K, sh = Q.multi ? 1u : 0u, last = k - 1;
+    // subset tables of the first K labels, where they are small
+    const bool tables = K * (1u << (K - 1u)) <= kTinyTable;
+    uint32_t *const tab = reinterpret_cast<uint32_t *>(pool);
+    if (tables) {
+        const uint32_t w = K * (1u << (K - 1u));
+        pool += (w + 1u) / 2u;
+        pool_n -= (w + 1u) / 2u;
+    }
 
-    // layer 1: the edges leaving the source(s)
     if (tid == 0) {
-        M.count = M.over = 0;
+        M.count[0] = M.count[1] = M.npair[0] = M.npair[1] = M.over = 0;
         M.base[1] = 0;
     }
+    for (uint32_t i = tid; i < 2u * kTinyHash; i += kThreads) M.hkey[0][i] = 0;
     __syncthreads();
-    if (!Q.dead) {
+    // layer 1: the edges leaving the source(s); beside it (the upper warps) the
+    // subset tables and the shade factors
+    if (warp >= kWarps / 2) {
+        const uint32_t t = tid - kThreads / 2;
+        if (tables) {
+            uint32_t off = 0;
+            for (uint32_t d = 1; d <= K; ++d) {
+                const uint32_t c = x_binom_dev(K, d), cm = x_binom_dev(kXMaxLabels, d), w = d * c;
+                const uint32_t *const src = a.tab + x_tab_off_dev(d);
+                if (t == 0) M.toff[d] = off;
+                for (uint32_t i = t; i < w; i += kThreads / 2) tab[off + i] = __ldg(src + i / c * cm + i % c);
+                off += w;
+            }
+        }
+        if (Q.colored)
+            for (uint32_t i = t; i < Q.k * K; i += kThreads / 2) M.omega[i] = shade_factor(Q, i);
+    } else if (!Q.dead) {
         const uint32_t ns = Q.multi ? Q.nslist : 1u;
-        for (uint32_t i = warp; i < ns; i += kWarps) {
+        for (uint32_t i = warp; i < ns; i += kWarps / 2) {
             const uint32_t s = Q.multi ? Q.slist[i] : Q.source;
             if (Q.vmask && Q.vmask[s]) continue;
             const uint32_t o0 = a.ooff[s], o1 = a.ooff[s + 1];
-            if (o1 - o0 > kTinyRows) {
+            if (o1 - o0 > kTinyRange) {
                 if (lane == 0) M.over = 1;
                 continue;
             }
             for (uint32_t o = o0 + lane; o < o1; o += 32u) {
-                const uint4 r = make_uint4(s, a.odst[o], a.otime[o], a.oeid[o]);
-                if (!allowed(Q, a.color, r.y) || (!Q.multi && r.y == s)) continue;
-                const uint32_t at = atomicAdd(&M.count, 1u);
-                if (at < kTinyRows) M.row[at] = r;
+                const uint4 r = a.orec[o];  // head, time, edge, first follower
+                const uint32_t fl = a.olen[o];
+                if (!allowed(Q, a.color, r.x) || (!Q.multi && r.x == s)) continue;
+                const uint32_t at = atomicAdd(&M.count[1], 1u);
+                if (at < kTinyRows) {
+                    M.row[at] = make_uint4(s, r.x, r.y, r.z);
+                    M.next[at] = make_uint2(r.w, fl);
+                }
             }
         }
     }
     __syncthreads();
-    if (M.over || M.count > kTinyRows) return false;
-    uint32_t n = M.count, lmax = 1;
-    __syncthreads();
+    uint32_t n = M.count[1], lmax = 1;
+    const uint32_t n1 = n;
+    if (M.over || n > kTinyRows) return kTinyNoFit;
     if (tid == 0) M.base[2] = n;
-    // forward
+    // forward; the hash table, counters and pairs of a level are cleared while
+    // the one before it uses the other
     for (uint32_t l = 2; l <= last && n; ++l) {
-        for (uint32_t i = tid; i < kTinyHash; i += kThreads) M.hkey[i] = 0;
-        if (tid == 0) M.count = M.npair = 0;
-        __syncthreads();
-        const uint32_t b0 = M.base[l - 1], b1 = M.base[l];
+        const uint32_t b1 = M.base[l - 1] + n, b0 = b1 - n, par = l & 1u;  // (base[l] is written by now or below)
         for (uint32_t f = warp; f < n; f += kWarps) {
-            const uint4 r = M.row[b0 + f];
-            const uint32_t v = r.y;
-            uint32_t o = a.ooff[v];
-            const uint32_t o1 = a.ooff[v + 1], t0 = r.z;
-            const uint64_t t1 = (uint64_t)t0 + a.delta[v];
-            if (o1 - o > 64u) {  // the first edge at or after t0
-                uint32_t hi = o1;
-                while (o < hi) {
-                    const uint32_t mid = o + (hi - o) / 2;
-                    if (a.otime[mid] < t0) o = mid + 1;
-                    else hi = mid;
-                }
+            const uint32_t v = M.row[b0 + f].y;
+            const uint2 nx = M.next[b0 + f];
+            if (nx.y > kTinyRange) {
+                if (lane == 0) M.over = 1;
+                continue;
             }
-            for (; o < o1; o += 32u) {  // warp-uniform
-                const uint32_t p = o + lane;
-                const bool in = p < o1;
-                const uint32_t t = in ? a.otime[p] : 0xffffffffu, w = in ? a.odst[p] : 0u, e = in ? a.oeid[p] : 0u;
-                const bool past = !in || (uint64_t)t > t1;
-                if (!past && t >= t0 && allowed(Q, a.color, w) && (Q.multi || w != Q.source)) {
-                    // the row's place in the level (one per edge)
-                    uint32_t h = (p * 2654435761u) >> 23;  // 9 bits: kTinyHash
-                    bool placed = false;
-                    for (uint32_t tries = 0; tries < kTinyHash && !placed; ++tries) {
-                        const uint32_t key = atomicCAS(&M.hkey[h], 0u, p + 1u);
-                        if (key == 0u) {
-                            const uint32_t at = atomicAdd(&M.count, 1u);
-                            M.hval[h] = at;
-                            if (at < kTinyRows && b1 + at < kTinyTotal) {
-                                M.row[b1 + at] = make_uint4(v, w, t, e);
+            for (uint32_t i = lane; i < nx.y; i += 32u) {
+                const uint32_t p = nx.x + i;
+                const uint4 r = a.orec[p];
+                const uint32_t fl = l < last ? a.olen[p] : 0u;
+                if (!allowed(Q, a.color, r.x) || (!Q.multi && r.x == Q.source)) continue;
+                // the row's place in the level (one per edge)
+                uint32_t h = (p * 2654435761u) >> 23;  // 9 bits: kTinyHash
+                bool placed = false;
+                for (uint32_t tries = 0; tries < kTinyHash && !placed; ++tries) {
+                    const uint32_t key = atomicCAS(&M.hkey[par][h], 0u, p + 1u);
+                    if (key == 0u) {
+                        const uint32_t at = atomicAdd(&M.count[par], 1u);
+                        M.hval[h] = at;
+                        if (at < kTinyRows && b1 + at < kTinyTotal) {
+                            M.row[b1 + at] = make_uint4(v, r.x, r.y, r.z);
+                            M.next[b1 + at] = make_uint2(r.w, fl);
 #pragma unroll
-                                for (uint32_t x = 0; x < kTinyWords; ++x) M.mask[b1 + at][x] = 0;
-                            }
+                            for (uint32_t x = 0; x < kTinyWords; ++x) M.mask[b1 + at][x] = 0;
                         }
-                        placed = key == 0u || key == p + 1u;
-                        if (!placed) h = (h + 1u) % kTinyHash;
                     }
-                    const uint32_t pp = atomicAdd(&M.npair, 1u);
-                    if (!placed || pp >= kTinyPairs) M.over = 1;
-                    else M.pair[pp] = f << 16 | h;
+                    placed = key == 0u || key == p + 1u;
+                    if (!placed) h = (h + 1u) % kTinyHash;
                 }
-                if (__all_sync(0xffffffffu, past)) break;
-                if (M.count > kTinyRows) break;
+                const uint32_t pp = atomicAdd(&M.npair[par], 1u);
+                if (!placed || pp >= kTinyPairs) M.over = 1;
+                else M.pair[pp] = f << 16 | h;
+                if (M.over) break;
             }
         }
         __syncthreads();
-        n = M.count;
-        if (M.over || n > kTinyRows || b1 + n > kTinyTotal) return false;
-        for (uint32_t i = tid; i < M.npair; i += kThreads) {
+        n = M.count[par];
+        if (M.over || n > kTinyRows || b1 + n > kTinyTotal) return kTinyNoFit;
+        for (uint32_t i = tid; i < M.npair[par]; i += kThreads) {
             const uint32_t f = M.pair[i] >> 16, e = M.hval[M.pair[i] & 0xffffu];
             atomicOr(&M.mask[b1 + e][f >> 5], 1u << (f & 31u));
         }
-        if (tid == 0) M.base[l + 1] = b1 + n;
+        for (uint32_t i = tid; i < kTinyHash; i += kThreads) M.hkey[par ^ 1u][i] = 0;
+        if (tid == 0) {
+            M.base[l] = b1;
+            M.base[l + 1] = b1 + n;
+            M.count[par ^ 1u] = M.npair[par ^ 1u] = 0;
+        }
         if (n) lmax = l;
         __syncthreads();
     }
-    if (n == 0 && !every) return true;  // no walk of k vertices: every sum is zero
-    if (lmax == 1 && M.base[2] == 0) return true;
+    if (n == 0 && !every) return kTinyDone;  // no walk of k vertices: every sum is zero
+    if (n1 == 0) return kTinyDone;
     const uint32_t top = every ? lmax : last;
 
-    // backward: the needed rows
-    for (uint32_t i = tid; i < (kXMaxLevels + 1) * kTinyWords; i += kThreads) {
-        const uint32_t l = i / kTinyWords;
-        uint32_t all = 0;
-        if (l >= 1 && l <= top && (every || l == top)) {
-            const uint32_t c = M.base[l + 1] - M.base[l], b = (i % kTinyWords) * 32u;
-            all = c >= b + 32u ? 0xffffffffu : c > b ? (1u << (c - b)) - 1u : 0u;
-        }
-        M.need[l][i % kTinyWords] = all;
-    }
-    __syncthreads();
-    if (!every)
-        for (uint32_t l = top; l >= 2; --l) {
-            const uint32_t c = M.base[l + 1] - M.base[l];
-            for (uint32_t i = tid; i < c * kTinyWords; i += kThreads) {
-                const uint32_t e = i / kTinyWords, x = i % kTinyWords;
-                if ((M.need[l][e >> 5] >> (e & 31u)) & 1u) {
-                    const uint32_t m = M.mask[M.base[l] + e][x];
-                    if (m) atomicOr(&M.need[l - 1][x], m);
-                }
+    // backward, the row counts and the space the layers take: one warp
+    if (warp == 0) {
+        for (uint32_t i = lane; i < (top + 1u) * kTinyWords; i += 32u) {
+            const uint32_t l = i / kTinyWords;
+            uint32_t all = 0;
+            if (l >= 1 && (every || l == top)) {
+                const uint32_t c = M.base[l + 1] - M.base[l], b = (i % kTinyWords) * 32u;
+                all = c >= b + 32u ? 0xffffffffu : c > b ? (1u << (c - b)) - 1u : 0u;
             }
-            __syncthreads();
+            M.need[l][i % kTinyWords] = all;
         }
-    if (tid == 0) {
-        uint32_t c = 0;
-        for (uint32_t l = 1; l <= top; ++l) {
-            M.cn[l] = c;
-            for (uint32_t x = 0; x < kTinyWords; ++x) c += __popc(M.need[l][x]);
+        __syncwarp();
+        for (uint32_t l = top; l >= 2 && !every; --l) {
+            const uint32_t b = M.base[l], c = M.base[l + 1] - b;
+            uint32_t m[kTinyWords] = {};
+            for (uint32_t e = lane; e < c; e += 32u)
+                if ((M.need[l][e >> 5] >> (e & 31u)) & 1u)
+#pragma unroll
+                    for (uint32_t x = 0; x < kTinyWords; ++x) m[x] |= M.mask[b + e][x];
+#pragma unroll
+            for (uint32_t x = 0; x < kTinyWords; ++x) {
+                const uint32_t o = __reduce_or_sync(0xffffffffu, m[x]);
+                if (lane == 0) M.need[l - 1][x] = o;
+            }
+            __syncwarp();
         }
-        M.cn[top + 1] = c;
+        uint32_t c = 0;  // lane l: the needed rows of level l
+        if (lane >= 1 && lane <= top)
+#pragma unroll
+            for (uint32_t x = 0; x < kTinyWords; ++x) c += __popc(M.need[lane][x]);
+        uint32_t inc = c;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t o = __shfl_up_sync(0xffffffffu, inc, d);
+            if (lane >= (uint32_t)d) inc += o;
+        }
+        if (lane >= 1 && lane <= top + 1u) M.cn[lane] = inc - c;
+        const uint32_t d = lane - 1u + sh;
+        const bool on = lane >= 1 && lane <= top;
+        const uint32_t g = __reduce_max_sync(0xffffffffu, on ? c * x_binom_dev(K, d) : 0u);
+        const uint32_t w = __reduce_max_sync(0xffffffffu, on && lane > 1 ? c * x_binom_dev(K, d - 1u) : 0u);
+        if (lane == 0) {
+            M.need_g = g;
+            M.need_d = w;
+        }
     }
     __syncthreads();
-    const uint32_t total = M.cn[top + 1];
-    // shared memory: multipliers, the shade factors, then window sums and two levels' values
-    uint32_t need_g = 0, need_d = 0;
-    for (uint32_t l = 1; l <= top; ++l) {
-        const uint32_t c = M.cn[l + 1] - M.cn[l], d = l - 1 + sh;
-        need_g = max(need_g, c * x_binom_dev(K, d));
-        if (l > 1) need_d = max(need_d, c * x_binom_dev(K, d - 1));
-    }
-    const uint32_t om_n = Q.colored ? Q.k * K : 0u;
-    if (2u * total * K + om_n + need_d + 2u * need_g > pool_n) return false;
-    uint64_t *const mul = pool, *const zw = mul + total * K, *const omega = zw + total * K, *const dr = omega + om_n,
-                    *const G0 = dr + need_d, *const G1 = G0 + need_g;
-    for (uint32_t i = tid; i < om_n; i += kThreads) omega[i] = shade_factor(Q, i);
+    const uint32_t total = M.cn[top + 1], need_g = M.need_g, need_d = M.need_d;
+    if (2u * total * K + need_d + 3u * need_g > pool_n) return kTinyNoFit;
+    uint64_t *const mul = pool, *const zw = mul + total * K, *const dr = zw + total * K;
+    uint64_t *G[3] = {dr + need_d, dr + need_d + need_g, dr + need_d + 2u * need_g};  // level l's values in G[l % 3]
     // the needed rows by level
-    for (uint32_t i = tid; i < M.base[top + 1]; i += kThreads) {
+    for (uint32_t i = tid, rows = M.base[top + 1]; i < rows; i += kThreads) {
         uint32_t l = 1;
         while (i >= M.base[l + 1]) ++l;
         const uint32_t e = i - M.base[l];
@@ -1012,110 +1087,117 @@ __device__ __noinline__ bool x_tiny(const XArgs &a, const XQuery &Q, bool every)
         for (uint32_t x = 0; x < (e >> 5); ++x) at += __popc(M.need[l][x]);
         M.list[at] = (uint16_t)i;
         M.lev[at] = (uint8_t)l;
+        M.acc[at] = 0;
     }
+    for (uint32_t i = tid; i < need_g; i += kThreads) G[2][i] = 0;
     __syncthreads();
     for (uint32_t i = tid; i < 2u * total * K; i += kThreads) {
         const bool second = i >= total * K;
         const uint32_t x = second ? i - total * K : i, at = x / K, j = x - at * K, l = M.lev[at];
         const uint4 r = M.row[M.list[at]];
         if (second) {
-            if (every || l == top) zw[x] = zprime(Q, omega, a.color, r.y, j);
-        } else {
+            if (every || l == top) zw[x] = zprime(Q, M.omega, a.color, r.y, j);
+        } else if (l > 1 || Q.multi) {
             const uint64_t y = sm_draw(Q.key_y, (uint64_t)r.w * 32u + (l - 1u));
-            mul[x] = gf64_mul(y, l > 1 || Q.multi ? zprime(Q, omega, a.color, r.x, j) : Q.d0);
+            mul[x] = gf64_mul(y, zprime(Q, M.omega, a.color, r.x, j));
+            if (l == 1) G[1][at * K + j] = mul[x];
+        } else if (j == 0) {
+            G[1][at] = gf64_mul(sm_draw(Q.key_y, (uint64_t)r.w * 32u), Q.d0);
         }
     }
     __syncthreads();
-    // the layers
-    uint64_t *G = G0, *Gp = G1;
-    for (uint32_t l = 1; l <= top; ++l) {
-        const uint32_t c = M.cn[l + 1] - M.cn[l], d = l - 1 + sh, cout = x_binom_dev(K, d);
-        uint64_t *const t_ = G;
-        G = Gp;
-        Gp = t_;
-        const uint64_t *const ml = mul + M.cn[l] * K;
-        if (l == 1) {
-            for (uint32_t i = tid; i < c * cout; i += kThreads) G[i] = ml[i / cout * K + i % cout];
-        } else {
-            const uint32_t cin = x_binom_dev(K, d - 1);
-            const bool spread = c * cout * d <= 4u * kThreads;
-            for (uint32_t i = tid; i < c * cin; i += kThreads) {
-                const uint32_t q = i / cin, s = i - q * cin;
-                const uint32_t *const mk = M.mask[M.list[M.cn[l] + q]];
-                uint64_t v = 0;
-                uint32_t before = 0;
-#pragma unroll
-                for (uint32_t x = 0; x < kTinyWords; ++x) {
-                    const uint32_t nd = M.need[l - 1][x];
-                    for (uint32_t m = mk[x] & nd; m; m &= m - 1)
-                        v ^= Gp[(before + __popc(nd & ((m & (0u - m)) - 1u))) * cin + s];
-                    before += __popc(nd);
-                }
-                dr[i] = v;
-            }
-            if (spread)
-                for (uint32_t i = tid; i < c * cout; i += kThreads) G[i] = 0;
-            __syncthreads();
-            const uint32_t *const tb = a.tab + x_tab_off_dev(d);
-            const uint32_t cm = x_binom_dev(kXMaxLabels, d);
-            if (spread) {
+    // the layers: step l forms level l's values and the witness terms of level l - 1
+    for (uint32_t l = 2; l <= top + 1u; ++l) {
+        uint64_t *const Gc = G[l % 3u], *const Gp = G[(l + 2u) % 3u], *const Gn = G[(l + 1u) % 3u];
+        if (l <= top) {
+            const uint32_t c0 = M.cn[l], c = M.cn[l + 1] - c0, d = l - 1 + sh, cout = x_binom_dev(K, d), cin = x_binom_dev(K, d - 1);
+            const uint64_t *const ml = mul + c0 * K;
+            const uint32_t *const tb = tables ? tab + M.toff[d] : a.tab + x_tab_off_dev(d);
+            const uint32_t cm = tables ? cout : x_binom_dev(kXMaxLabels, d);
+            const uint32_t *const nd = M.need[l - 1];
+            if (c * cout * d <= 4u * kThreads) {
                 for (uint32_t i = tid; i < c * cout * d; i += kThreads) {
                     const uint32_t q = i / (cout * d), r = i - q * cout * d, x = r / cout, T = r - x * cout;
-                    const uint32_t e = __ldg(tb + x * cm + T);
-                    xor_shared(&G[q * cout + T], gf64_mul(ml[q * K + (e & 255u)], dr[q * cin + (e >> 8)]));
+                    const uint32_t e = tb[x * cm + T];
+                    const uint64_t w = tiny_window(M.mask[M.list[c0 + q]], nd, Gp, cin, e >> 8);
+                    xor_shared(&Gc[q * cout + T], gf64_mul(ml[q * K + (e & 255u)], w));
                 }
             } else {
+                for (uint32_t i = tid; i < c * cin; i += kThreads) {
+                    const uint32_t q = i / cin;
+                    dr[i] = tiny_window(M.mask[M.list[c0 + q]], nd, Gp, cin, i - q * cin);
+                }
+                __syncthreads();
                 for (uint32_t i = tid; i < c * cout; i += kThreads) {
                     const uint32_t q = i / cout, T = i - q * cout;
                     uint64_t v = 0;
                     for (uint32_t x = 0; x < d; ++x) {
-                        const uint32_t e = __ldg(tb + x * cm + T);
+                        const uint32_t e = tb[x * cm + T];
                         v ^= gf64_mul(ml[q * K + (e & 255u)], dr[q * cin + (e >> 8)]);
                     }
-                    G[i] = v;
+                    Gc[i] = v;
                 }
             }
+            if (l < top) {  // the next level's products add up from zero (it was read two steps ago)
+                const uint32_t w = (M.cn[l + 2] - M.cn[l + 1]) * x_binom_dev(K, d + 1u);
+                for (uint32_t i = tid; i < w; i += kThreads) Gn[i] = 0;
+            }
         }
-        const bool out = every ? !(Q.pivot > l && !Q.multi) : l == top;
-        if (!out) {
-            __syncthreads();
-            continue;
-        }
-        // witness: z'_w over the first K2 labels
-        for (uint32_t i = tid; i < c; i += kThreads) M.acc[i] = 0;
-        __syncthreads();
-        const uint32_t K2 = l + sh;
-        for (uint32_t i = tid; i < c * K2; i += kThreads) {
-            const uint32_t q = i / K2, T = i - q * K2;
-            xor_shared(&M.acc[q], gf64_mul(G[q * cout + T], zw[(M.cn[l] + q) * K + (K2 - 1u - T)]));
-        }
-        __syncthreads();
-        const uint32_t row = every ? l - 1u : 0u;
-        for (uint32_t q = tid; q < c; q += kThreads) {
-            const uint4 r = M.row[M.list[M.cn[l] + q]];
-            const uint64_t v = M.acc[q];
-            if (v) atomicXor(reinterpret_cast<unsigned long long *>(Q.S + (size_t)row * a.n + r.y), (unsigned long long)v);
-            if (Q.E) Q.E[r.w] = v;
-            if (Q.R) {  // the XOR over the head's rows of the same time
-                uint64_t sum = 0;
-                for (uint32_t x = 0; x < c; ++x) {
-                    const uint4 o = M.row[M.list[M.cn[l] + x]];
-                    if (o.y == r.y && o.z == r.z) sum ^= M.acc[x];
-                }
-                if (sum) atomicMin(Q.R + (size_t)row * a.n + r.y, r.z);
+        if (every ? !(Q.pivot > l - 1u && !Q.multi) : l == top + 1u) {
+            // times z'_w over the first labels of k' = l
+            const uint32_t c0 = M.cn[l - 1], c = M.cn[l] - c0, K2 = l - 1u + sh, st = x_binom_dev(K, l - 2u + sh);
+            for (uint32_t i = tid; i < c * K2; i += kThreads) {
+                const uint32_t q = i / K2, T = i - q * K2;
+                xor_shared(&M.acc[c0 + q], gf64_mul(Gp[q * st + T], zw[(c0 + q) * K + (K2 - 1u - T)]));
             }
         }
         __syncthreads();
     }
-    if (Q.bitmap) {  // the bytes of the out rows' heads (the rest is clear)
+    // the witnesses: rows of one level and head together
+    if (!cleared) {
+        if (!clear.wait()) return kTinyFailed;
+        cleared = true;
+    }
+    const uint32_t first = every ? 0u : M.cn[top];
+    for (uint32_t at = first + tid; at < total; at += kThreads) {
+        const uint32_t l = M.lev[at], c0 = M.cn[l], c1 = M.cn[l + 1];
+        const uint4 r = M.row[M.list[at]];
+        const size_t off = (size_t)(every ? l - 1u : 0u) * a.n + r.y;
+        uint64_t sum = 0, same = 0;
+        bool lead = true;
+        for (uint32_t x = c0; x < c1; ++x) {
+            const uint4 o = M.row[M.list[x]];
+            if (o.y != r.y) continue;
+            if (x < at) lead = false;
+            sum ^= M.acc[x];
+            if (o.z == r.z) same ^= M.acc[x];
+        }
+        if (lead && sum) {
+            Q.S[off] = sum;
+            if (Q.bitmap && !every) {
+                // the head's byte: every vertex of it with a non-zero sum
+                uint32_t bits = 0;
+                for (uint32_t x = c0; x < c1; ++x) {
+                    const uint32_t h = M.row[M.list[x]].y;
+                    if (h >> 3 != r.y >> 3 || (bits >> (h & 7u)) & 1u) continue;
+                    uint64_t hs = 0;
+                    for (uint32_t z = x; z < c1; ++z)
+                        if (M.row[M.list[z]].y == h) hs ^= M.acc[z];
+                    if (hs) bits |= 1u << (h & 7u);
+                }
+                Q.bitmap[r.y >> 3] = (uint8_t)bits;
+            }
+        }
+        if (Q.E) Q.E[r.w] = M.acc[at];
+        if (Q.R && same) atomicMin(Q.R + off, r.z);  // the XOR over the head's rows of the same time
+    }
+    if (Q.bitmap && every) {  // the bytes of the rows' heads over all witness rows
         __threadfence();
         __syncthreads();
-        const uint32_t rows = every ? k - 1 : 1u;
         for (uint32_t at = tid; at < total; at += kThreads) {
-            if (!every && M.lev[at] != top) continue;
             const uint32_t b = M.row[M.list[at]].y >> 3;
             uint32_t bits = 0;
-            for (uint32_t w = 0; w < rows; ++w)
+            for (uint32_t w = 0; w < k - 1; ++w)
                 for (uint32_t i = 0; i < 8; ++i) {
                     const uint32_t x = b * 8 + i;
                     if (x < a.n && __ldcg(Q.S + (size_t)w * a.n + x) != 0) bits |= 1u << i;
@@ -1123,7 +1205,7 @@ __device__ __noinline__ bool x_tiny(const XArgs &a, const XQuery &Q, bool every)
             Q.bitmap[b] = (uint8_t)bits;
         }
     }
-    return true;
+    return kTinyDone;
 }
 
 // The scratch pointers of a template, from offsets + 1 to addresses.
@@ -1205,30 +1287,32 @@ k_frontier(const __grid_constant__ XArgs a_, const __grid_constant__ XOne one_, 
         for (uint64_t i = gt; i < a.bzero_n; i += nt) a.bzero[i] = 0;
     }
     uint32_t left = BATCH ? 0u : 1u;
-    if (!BATCH) load_query<BATCH>(o, a, one_, 0, 0);
     if (plan && a.tiny) {
-        ok = grid.sync();
-        if (ok) {
-            for (;;) {
-                uint32_t q = blockIdx.x;  // one query: block 0's
-                if (BATCH) {
-                    __syncthreads();
-                    if (threadIdx.x == 0) next = atomicAdd(a.ctl + 2, 1u);
-                    __syncthreads();
-                    q = next;
-                    if (q < a.nq) load_query<BATCH>(o, a, one_, q, 0);
-                }
-                if (q >= a.nq) break;
-                if (!x_tiny(a, o.q, o.t.every != 0) && threadIdx.x == 0) {
-                    const uint32_t at = atomicAdd(a.ctl + 3, 1u);
-                    if (BATCH) a.left[at] = q;
-                }
-                if (!BATCH) break;
+        grid.arrive();
+        bool cleared = false;
+        for (;;) {
+            uint32_t q = blockIdx.x;  // one query: block 0's
+            if (BATCH) {
+                __syncthreads();
+                if (threadIdx.x == 0) next = atomicAdd(a.ctl + 2, 1u);
+                __syncthreads();
+                q = next;
             }
-            ok = grid.sync();
+            if (q >= a.nq || !ok) break;
+            copy_words(&o.q, BATCH ? a.xq + q : &one_.q, sizeof(XQuery));
+            __syncthreads();
+            const int r = x_tiny(a, o.q, !BATCH && one_.t.every, grid, cleared);
+            if (r == kTinyFailed) ok = false;
+            if (r == kTinyNoFit && threadIdx.x == 0) {
+                const uint32_t at = atomicAdd(a.ctl + 3, 1u);
+                if (BATCH) a.left[at] = q;
+            }
+            if (!BATCH) break;
         }
+        ok = ok && grid.sync();
         if (ok) left = *(volatile uint32_t *)(a.ctl + 3);
     }
+    if (!BATCH && ok && left) load_query<BATCH>(o, a, one_, 0, 0);
     if (ok && left) {
         if (BATCH && a.lanes > 1 && left >= gridDim.x / 4) {
             View solo{0u, 1u, a.ctl, a.err, 0u};
@@ -1264,6 +1348,34 @@ k_frontier(const __grid_constant__ XArgs a_, const __grid_constant__ XOne one_, 
     }
 }
 
+// The record of every edge in (tail, time) order: head, time, input index, and
+// the range of edges that may follow it (they leave the head no earlier and at
+// most its waiting time later).
+__global__ void k_out_records(uint32_t m, const uint32_t *__restrict__ off, const uint32_t *__restrict__ time,
+                              const uint32_t *__restrict__ dst, const uint32_t *__restrict__ eid,
+                              const uint32_t *__restrict__ delta, uint4 *__restrict__ rec, uint32_t *__restrict__ len)
+{
+    for (uint32_t o = blockIdx.x * blockDim.x + threadIdx.x; o < m; o += gridDim.x * blockDim.x) {
+        const uint32_t v = dst[o], t = time[o];
+        const uint64_t until = (uint64_t)t + delta[v];
+        uint32_t lo = off[v];
+        const uint32_t end = off[v + 1];
+        for (uint32_t hi = end; lo < hi;) {
+            const uint32_t mid = lo + (hi - lo) / 2;
+            if (time[mid] < t) lo = mid + 1;
+            else hi = mid;
+        }
+        uint32_t e = lo;
+        for (uint32_t hi = end; e < hi;) {
+            const uint32_t mid = e + (hi - e) / 2;
+            if (time[mid] <= until) e = mid + 1;
+            else hi = mid;
+        }
+        rec[o] = make_uint4(v, t, eid[o], lo);
+        len[o] = e - lo;
+    }
+}
+
 // start[i] = first position of entry i's window in the list `prev` (0-based):
 // its index b when set, else the first row of the tail's segment there (the
 // rows with smaller heads come before it).
@@ -1288,6 +1400,19 @@ __global__ void k_window_start(uint32_t count, const uint32_t *__restrict__ a, c
 }
 
 }  // namespace
+
+rr_status frontier_out_records(Graph &g, const uint32_t *d_time, const uint32_t *d_dst, const uint32_t *d_eid,
+                               const uint32_t *d_delta, cudaStream_t st)
+{
+    RR_CUDA(g.o_rec.reserve(std::max<uint64_t>(1, g.m) * sizeof(uint4)));
+    RR_CUDA(g.o_len.reserve(std::max<uint64_t>(1, g.m) * 4));
+    if (!g.m) return RR_OK;
+    const unsigned grid = (unsigned)std::min<uint64_t>(152ull * 64, (g.m + 255) / 256);
+    k_out_records<<<grid, 256, 0, st>>>((uint32_t)g.m, g.o_off.as<uint32_t>(), d_time, d_dst, d_eid, d_delta,
+                                        g.o_rec.as<uint4>(), g.o_len.as<uint32_t>());
+    RR_LAUNCHED();
+    return RR_OK;
+}
 
 // ---- host side ------------------------------------------------------------------
 
@@ -1462,10 +1587,8 @@ static void x_args(const Graph &g, XArgs &a)
     a.color = g.color.as<uint8_t>();
     a.tab = g.x_tab.as<uint32_t>();
     a.ooff = g.o_off.as<uint32_t>();
-    a.otime = g.o_time.as<uint32_t>();
-    a.odst = g.o_dst.as<uint32_t>();
-    a.oeid = g.o_eid.as<uint32_t>();
-    a.delta = g.delta.as<uint32_t>();
+    a.orec = g.o_rec.as<uint4>();
+    a.olen = g.o_len.as<uint32_t>();
     a.smem = g.x_smem_max / (16u << kTeamLog) * (16u << kTeamLog);  // 16-byte shares per warp
 }
 

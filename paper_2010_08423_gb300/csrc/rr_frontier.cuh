@@ -94,7 +94,9 @@ struct XArgs {
     uint32_t *err;         // set when a bounded wait gave up
     const uint8_t *color;
     const uint32_t *tab;   // subset tables
-    const uint32_t *ooff, *otime, *odst, *oeid, *delta;  // edges by (tail, time), waiting times
+    const uint32_t *ooff;  // edges by (tail, time): offsets (n + 1),
+    const uint4 *orec;     // head, time, input index, first edge that may follow
+    const uint32_t *olen;  // and how many
     uint32_t smem;         // dynamic shared memory of a block
     uint32_t tiny;         // try every query in one block's shared memory first
 };

@@ -638,14 +638,16 @@ rr_status graph_load(uint32_t n, uint64_t m, const uint32_t *src, const uint32_t
                       &g->row_hi})
         RR_CUDA(b->reserve(mb * 4));
 
-    RR_CUDA(g->delta.reserve((size_t)n * 4));
-    RR_CUDA(cudaMemcpyAsync(g->delta.p, delta, (size_t)n * 4, cudaMemcpyHostToDevice, st));
+    DevBuf d_delta;
+    RR_CUDA(d_delta.reserve((size_t)n * 4));
+    RR_CUDA(cudaMemcpyAsync(d_delta.p, delta, (size_t)n * 4, cudaMemcpyHostToDevice, st));
     RR_CUDA(g->o_off.reserve((size_t)(n + 1) * 4));
-    for (DevBuf *b : {&g->o_time, &g->o_dst, &g->o_eid}) RR_CUDA(b->reserve((size_t)(m ? m : 1) * 4));
 
     if (m == 0) {
         RR_CUDA(cudaMemsetAsync(g->off.p, 0, (size_t)(n + 1) * 4, st));
         RR_CUDA(cudaMemsetAsync(g->o_off.p, 0, (size_t)(n + 1) * 4, st));
+        rr_status os = frontier_out_records(*g, nullptr, nullptr, nullptr, nullptr, st);
+        if (os != RR_OK) return os;
     } else {
         DevBuf d_src, d_dst, d_t, key_in, key_out, val_in, tmp;
         RR_CUDA(d_src.reserve(mb * 4));
@@ -682,20 +684,27 @@ rr_status graph_load(uint32_t n, uint64_t m, const uint32_t *src, const uint32_t
         k_offsets<<<grid_for(m + 1, 256), 256, 0, st>>>(g->row_head.as<uint32_t>(), m, n,
                                                         g->off.as<uint32_t>());
         RR_LAUNCHED();
-        // the edges by (tail, time): what leaves a vertex in a window
-        k_make_keys<<<grid_for(m, 256), 256, 0, st>>>(d_src.as<uint32_t>(), d_t.as<uint32_t>(), m,
-                                                      key_in.as<uint64_t>(), val_in.as<uint32_t>());
-        RR_LAUNCHED();
-        RR_CUDA(cub::DeviceRadixSort::SortPairs(tmp.p, tmp_bytes, key_in.as<uint64_t>(),
-                                                key_out.as<uint64_t>(), val_in.as<uint32_t>(),
-                                                g->o_eid.as<uint32_t>(), (int64_t)m, 0, 32 + head_bits, st));
-        // (the tails go through the value buffer, free again)
-        k_unpack_rows<<<grid_for(m, 256), 256, 0, st>>>(
-            key_out.as<uint64_t>(), g->o_eid.as<uint32_t>(), d_dst.as<uint32_t>(), m,
-            g->o_time.as<uint32_t>(), val_in.as<uint32_t>(), g->o_dst.as<uint32_t>());
-        RR_LAUNCHED();
-        k_offsets<<<grid_for(m + 1, 256), 256, 0, st>>>(val_in.as<uint32_t>(), m, n, g->o_off.as<uint32_t>());
-        RR_LAUNCHED();
+        // the edges by (tail, time)
+        {
+            DevBuf o_eid, o_time, o_dst;
+            for (DevBuf *b : {&o_eid, &o_time, &o_dst}) RR_CUDA(b->reserve(mb * 4));
+            k_make_keys<<<grid_for(m, 256), 256, 0, st>>>(d_src.as<uint32_t>(), d_t.as<uint32_t>(), m,
+                                                          key_in.as<uint64_t>(), val_in.as<uint32_t>());
+            RR_LAUNCHED();
+            RR_CUDA(cub::DeviceRadixSort::SortPairs(tmp.p, tmp_bytes, key_in.as<uint64_t>(),
+                                                    key_out.as<uint64_t>(), val_in.as<uint32_t>(),
+                                                    o_eid.as<uint32_t>(), (int64_t)m, 0, 32 + head_bits, st));
+            // (the tails go through the value buffer, free again)
+            k_unpack_rows<<<grid_for(m, 256), 256, 0, st>>>(
+                key_out.as<uint64_t>(), o_eid.as<uint32_t>(), d_dst.as<uint32_t>(), m,
+                o_time.as<uint32_t>(), val_in.as<uint32_t>(), o_dst.as<uint32_t>());
+            RR_LAUNCHED();
+            k_offsets<<<grid_for(m + 1, 256), 256, 0, st>>>(val_in.as<uint32_t>(), m, n, g->o_off.as<uint32_t>());
+            RR_LAUNCHED();
+            rr_status os = frontier_out_records(*g, o_time.as<uint32_t>(), o_dst.as<uint32_t>(), o_eid.as<uint32_t>(),
+                                                d_delta.as<uint32_t>(), st);
+            if (os != RR_OK) return os;
+        }
         key_in.release();
         key_out.release();
         val_in.release();
@@ -710,7 +719,7 @@ rr_status graph_load(uint32_t n, uint64_t m, const uint32_t *src, const uint32_t
         RR_CUDA(cudaMemsetAsync(diff.p, 0, (mb + 1) * 4, st));
         k_windows<<<grid_for(m, 256), 256, 0, st>>>(
             g->row_t.as<uint32_t>(), g->row_src.as<uint32_t>(), g->off.as<uint32_t>(),
-            g->delta.as<uint32_t>(), m, g->row_lo.as<uint32_t>(), g->row_hi.as<uint32_t>(),
+            d_delta.as<uint32_t>(), m, g->row_lo.as<uint32_t>(), g->row_hi.as<uint32_t>(),
             diff.as<int32_t>(), counter.as<unsigned long long>());
         RR_LAUNCHED();
         RR_CUDA(prod.reserve(mb * 4));

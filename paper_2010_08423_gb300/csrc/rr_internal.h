@@ -349,10 +349,10 @@ struct Graph {
     RowList prod_list, state_list, win_list, tail_list, deep_list, tail3_list;
 
     // frontier engine (rr_frontier.cu): the edges sorted by (tail, time) --
-    // offsets (n + 1), times, heads, input indexes --, the waiting times,
-    // subset tables, launch limits, and the colours on the host (the source's
-    // z row is formed there)
-    DevBuf o_off, o_time, o_dst, o_eid, delta;
+    // offsets (n + 1), records (head, time, input index, first edge that may
+    // follow), numbers of followers --, subset tables, launch limits, and the
+    // colours on the host (the source's z row is formed there)
+    DevBuf o_off, o_rec, o_len;
     DevBuf x_tab;
     int x_sms = 0;
     uint32_t x_smem_max = 0;
@@ -388,7 +388,7 @@ struct Graph {
 
     size_t device_bytes() const
     {
-        return x_tab.bytes + o_off.bytes + o_time.bytes + o_dst.bytes + o_eid.bytes + delta.bytes + off.bytes + row_a.bytes + row_b.bytes + row_s.bytes + row_eid.bytes +
+        return x_tab.bytes + o_off.bytes + o_rec.bytes + o_len.bytes + off.bytes + row_a.bytes + row_b.bytes + row_s.bytes + row_eid.bytes +
                row_src.bytes + row_lo.bytes + row_hi.bytes + row_t.bytes + row_head.bytes +
                color.bytes + color_order.bytes + items.bytes +
                prod_list.bytes() + state_list.bytes() + win_list.bytes() + tail_list.bytes() +
@@ -540,6 +540,8 @@ rr_status frontier_reserve(Workspace &ws, cudaStream_t st);
 // RR_ETIMEDOUT, once, when a bounded wait of a finished query on ws gave up.
 rr_status frontier_error(Workspace &ws);
 rr_status frontier_load(Graph &g, cudaStream_t st);
+rr_status frontier_out_records(Graph &g, const uint32_t *d_time, const uint32_t *d_dst, const uint32_t *d_eid,
+                               const uint32_t *d_delta, cudaStream_t st);
 rr_status frontier_query(const Graph &g, Workspace &ws, const rr_query *q, bool every, uint8_t *d_bitmap,
                          uint64_t *d_witness, cudaStream_t st, uint64_t *d_E = nullptr,
                          const uint8_t *d_vmask = nullptr, uint32_t *d_R = nullptr,
