@@ -42,10 +42,15 @@ namespace {
 
 constexpr int kThreads = 512;
 constexpr int kWarps = kThreads / 32;
-constexpr uint32_t kTeamLog = 4;      // log2 of the warps of a wedge block
+constexpr uint32_t kTeams = 5;        // team sizes of a wedge block: 1, 2, 4, 8 warps, all of them
+__host__ __device__ constexpr uint32_t team_threads(uint32_t t) { return t + 1 < kTeams ? 32u << t : (uint32_t)kThreads; }
+__host__ __device__ constexpr uint32_t team_count(uint32_t t) { return (uint32_t)kThreads / team_threads(t); }
+// A team's share of the block's shared memory.
+__host__ __device__ constexpr uint32_t team_smem(uint32_t smem, uint32_t t) { return smem / team_count(t) / 16u * 16u; }
 constexpr uint32_t kMaxRows = 16;     // rows of one wedge item
 constexpr uint32_t kSplit = 36;       // words of a split multiplier: 9 pieces of 3 classes, each padded to 16 bytes
-constexpr uint32_t kSup1 = 16, kSup2 = 256;  // blocks per partial sum
+constexpr uint32_t kSup1 = 16, kSup2 = 256, kSup3 = 4096;  // blocks per partial sum
+constexpr uint32_t kScanBlocks = 48, kScanSpan = 6, kScanLong = 1024;  // when a level's prefix sums are completed (x_scans)
 // Bitmap words per scan tile: one tile up to 8,192 words (a block scans them in
 // 8 steps), else at most 256 tiles of whole 1,024s.
 __host__ __device__ constexpr uint32_t x_tile_words(uint32_t words)
@@ -192,53 +197,86 @@ __device__ __forceinline__ bool any_in(const uint32_t *A, uint32_t lo, uint32_t 
     const uint32_t m0 = 0xffffffffu << (lo & 31u), m1 = 0xffffffffu >> (31u - ((hi - 1) & 31u));
     if (w0 == w1) return (A[w0] & m0 & m1) != 0;
     if ((A[w1] & m1) || (A[w0] & m0)) return true;
-    for (uint32_t w = w0 + 1; w < w1; ++w)
+    // the whole words between, four at a time (bitmaps start on 256-byte boundaries)
+    uint32_t w = w0 + 1;
+    for (; w < w1 && (w & 3u); ++w)
+        if (A[w]) return true;
+    for (; w + 4u <= w1; w += 4u) {
+        const uint4 x = *reinterpret_cast<const uint4 *>(A + w);
+        if (x.x | x.y | x.z | x.w) return true;
+    }
+    for (; w < w1; ++w)
         if (A[w]) return true;
     return false;
 }
 
-// Needed rows of a level at positions below x.
-__device__ __forceinline__ uint32_t rank_below(const XLL &L, uint32_t x)
+// Rows of partial sums over nb blocks: of 16, 256 and 4,096 blocks.
+__host__ __device__ __forceinline__ uint32_t x_sup_rows(uint64_t nb)
 {
-    const uint32_t w = x >> 5;
-    return L.pc[w] + __popc(L.N[w] & ((1u << (x & 31u)) - 1u));
+    return (uint32_t)(nb / kSup1 + nb / kSup2 + nb / kSup3 + 3u);
 }
 
-// One wedge item: 1 << rows consecutive needed rows of a level, taken by a team
-// of 1 << team warps. Few rows get large teams (all warps of a block on one
-// row: the layer's latency counts), many rows one warp each (no block-wide
-// waits; the warps cover each other's loads): of the team sizes whose share of
-// shared memory holds a row, the one whose busiest team has the fewest product
-// steps, a row's fixed cost (loads, draws, multipliers) counted as kRowSteps.
-// Rows per item grow until every team has one item, at most kMaxRows and what
-// shared memory holds. The next level derives the same rows to read the prefix
-// sums. Chosen once per level list, by the thread that counts its rows.
-struct XShape {
-    uint32_t team, rows;  // log2
-};
-__device__ __forceinline__ XShape x_shape_of(uint32_t s) { return XShape{s & 0xffu, s >> 8}; }
-constexpr uint32_t kRowSteps = 6;
-__device__ __forceinline__ uint32_t x_item_bytes(uint32_t rows, uint32_t K, const XLL &X)
+// Needed rows of a level at positions below x (rank: the bitmap's word and the
+// rows before it).
+__device__ __forceinline__ uint32_t rank_below(const uint2 *rank, uint32_t x)
 {
-    return rows * (K * (4u * kSplit) + (X.cin + X.cout + X.uout) * 8u + 32u);
+    const uint2 r = rank[x >> 5];
+    return r.y + __popc(r.x & ((1u << (x & 31u)) - 1u));
 }
-__device__ __noinline__ XShape x_choose_shape(uint32_t smem, uint32_t blocks, uint32_t cnt, uint32_t K, const XLL &X)
+
+// One wedge item: `rows` consecutive needed rows of a level, taken by a team of
+// 1 << team warps. Few rows get large teams (all warps of a block on one row:
+// the layer's latency counts), many rows one warp each (no block-wide waits; the
+// warps cover each other's loads). Of the team sizes and rows per item (at most
+// kMaxRows) that a team's share of shared memory holds, the pair is taken whose
+// busiest team has the least to do, counted in product steps of a warp (about
+// 1,000 cycles with four warps on a scheduler) with the measured cost of an
+// item's other parts. Chosen once per level list, by the warp that counts its
+// rows; the next level reads the rows' prefix sums by it. With powers of two and
+// rows added until every team had an item, layers of 2,500 to 4,000 rows left
+// the warps idle for a third of the time.
+struct XShape {
+    uint32_t team, rows, scan;  // team: log2
+};
+__device__ __forceinline__ XShape x_shape_of(uint32_t s) { return XShape{s & 0xffu, (s >> 8) & 0xffu, s >> 16}; }
+__host__ __device__ __forceinline__ uint32_t x_item_bytes(uint32_t rows, uint32_t K, const XLL &X)
 {
-    XShape s{kTeamLog, 0u};
-    uint32_t best = 0xffffffffu;
-    for (uint32_t t = 0; t <= kTeamLog; ++t) {
-        if (t < kTeamLog && x_item_bytes(1u, K, X) > (smem >> (kTeamLog - t))) continue;
-        const uint32_t teams = blocks << (kTeamLog - t);
-        const uint32_t steps = X.out ? 1u : ((X.cout + (32u << t) - 1u) >> (5 + t)) * X.d;
-        const uint32_t cost = (cnt + teams - 1u) / teams * (steps + kRowSteps);
+    return X.out ? rows * (K * 16u + 64u) : rows * (K * (4u * kSplit) + (X.cin + X.cout + X.uout) * 8u + 64u);
+}
+// Quarter steps of one item.
+__device__ __forceinline__ uint32_t x_item_cost(uint32_t rows, uint32_t t, uint32_t K, const XLL &X)
+{
+    const uint32_t T = team_threads(t), W = T / 32u;
+    auto rounds = [&](uint32_t n) { return (n + T - 1u) / T; };
+    if (X.out) return 16u + 24u * rounds(rows * X.cout);
+    const uint32_t per_warp = (rows + W - 1u) / W;
+    uint32_t c = 16u + per_warp * (4u + X.cin / 64u) + rounds(rows * K) * 20u + rounds(rows * X.cout) * X.d * 4u +
+                 rows * rounds(X.cout + X.uout);
+    if (X.uout) c += rounds(rows * X.uout) * (X.d + 5u) * 4u;
+    return c;
+}
+// By one warp; every lane returns the choice.
+__device__ __noinline__ uint32_t x_choose_shape(uint32_t smem, uint32_t blocks, uint32_t cnt, uint32_t K, const XLL &X)
+{
+    const uint32_t lane = threadIdx.x & 31u;
+    uint32_t best = 0xffffffffu, pick = 0;
+    for (uint32_t i = lane; i < kTeams * kMaxRows; i += 32u) {
+        const uint32_t t = i / kMaxRows, rows = i % kMaxRows + 1u;
+        if ((rows > 1u || t + 1u < kTeams) && x_item_bytes(rows, K, X) > team_smem(smem, t)) continue;
+        const uint32_t items = (cnt + rows - 1u) / rows, teams = blocks * team_count(t);
+        const uint32_t cost = (items + teams - 1u) / teams * x_item_cost(rows, t, K, X);
         if (cost < best) {
             best = cost;
-            s.team = t;
+            pick = t | rows << 8;
         }
     }
-    const uint32_t teams = blocks << (kTeamLog - s.team), share = smem >> (kTeamLog - s.team);
-    while ((1u << s.rows) < kMaxRows && cnt > (teams << s.rows) && x_item_bytes(2u << s.rows, K, X) <= share) ++s.rows;
-    return s;
+    const uint32_t least = __reduce_min_sync(0xffffffffu, best);
+    const uint32_t who = __ffs((int)__ballot_sync(0xffffffffu, best == least)) - 1u;
+    pick = __shfl_sync(0xffffffffu, pick, (int)who);
+    // room for the sums of all blocks (taken where the windows span many of them)
+    const uint32_t rows = pick >> 8, nb = (cnt + rows - 1u) / rows;
+    if (!X.out && nb >= kScanBlocks && (rows == 1u || nb <= X.ipcap)) pick |= 1u << 16;
+    return pick;
 }
 
 // Carry-less inner products. gf64_mul splits both operands into 9 16-bit pieces
@@ -302,7 +340,7 @@ __device__ __noinline__ bool x_plan(const XArgs &a, const XOne &o, View &v)
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     const uint32_t gw = v.b * kWarps + warp, nw = v.n * kWarps;
     const uint32_t gt = v.b * kThreads + threadIdx.x, nt = v.n * kThreads;
-    constexpr uint32_t U = 4;  // bitmap words per warp and step
+    constexpr uint32_t U = 2;  // bitmap words per warp and step
 
     // cleared first: needed-row bitmaps, flags
     for (uint32_t i = gt; i < t.clear4; i += nt) t.clear[i] = make_uint4(0, 0, 0, 0);
@@ -310,6 +348,7 @@ __device__ __noinline__ bool x_plan(const XArgs &a, const XOne &o, View &v)
         for (uint32_t i = threadIdx.x; i < t.nll; i += kThreads) {
             t.live[i] = t.ll[i].level == 1 ? 1u : 0u;
             t.cnt[i] = 0;
+            t.span[i] = 0;
         }
     if (Q.colored && v.b == v.n - 1)
         // shade factors with the source's column eliminated
@@ -470,8 +509,8 @@ __device__ __noinline__ bool x_plan(const XArgs &a, const XOne &o, View &v)
                     uint32_t c[4], mysum = 0;
 #pragma unroll
                     for (uint32_t x = 0; x < 4; ++x) {
-                        c[x] = w + x < end ? __popc(X.N[w + x]) : 0u;
-                        mysum += c[x];
+                        c[x] = w + x < end ? X.N[w + x] : 0u;
+                        mysum += __popc(c[x]);
                     }
                     uint32_t inc = mysum;
 #pragma unroll
@@ -487,15 +526,17 @@ __device__ __noinline__ bool x_plan(const XArgs &a, const XOne &o, View &v)
                     uint32_t at = run_base + before + inc - mysum;
 #pragma unroll
                     for (uint32_t x = 0; x < 4; ++x) {
-                        if (w + x < end) X.pc[w + x] = at;
-                        at += c[x];
+                        if (w + x < end) X.rank[w + x] = make_uint2(c[x], at);
+                        at += __popc(c[x]);
                     }
                     run_base += __reduce_add_sync(0xffffffffu, other);
                 }
-                if (end == words && threadIdx.x == 0) {
-                    t.cnt[li] = run_base;
-                    const XShape sh = x_choose_shape(a.smem, v.n, run_base, Q.K, X);
-                    t.shape[li] = sh.team | sh.rows << 8;
+                if (end == words && warp == 0) {
+                    const uint32_t shape = x_choose_shape(a.smem, v.n, run_base, Q.K, X);
+                    if (lane == 0) {
+                        t.cnt[li] = run_base;
+                        t.shape[li] = shape;
+                    }
                 }
             }
             base_item += tiles;
@@ -503,43 +544,61 @@ __device__ __noinline__ bool x_plan(const XArgs &a, const XOne &o, View &v)
         if (!v.sync()) return false;
     }
 
-    // the needed rows' windows, edges and tails, in list order
+    // the needed rows' windows, edges and tails, in list order, and how many rows
+    // of the level below the windows hold together
     for (uint32_t li = 0; li < nll; ++li) {
         const XLL &X = t.ll[li];
         const XList &L = a.lists[X.list];
         const uint32_t steps = (L.words + U - 1) / U;
         if (!t.live[li]) continue;
         const bool window = X.level > 1;
-        const XLL &P = t.ll[X.prev];
+        const uint2 *const rank = X.rank, *const below = t.ll[X.prev].rank;
+        uint64_t span = 0;
         for (uint32_t i = gw; i < steps; i += nw) {
             const uint32_t w0 = i * U;
-            const uint32_t mine = lane < U && w0 + lane < L.words ? X.N[w0 + lane] : 0u;
-            if (!__any_sync(0xffffffffu, mine != 0)) continue;
-            const uint32_t mypc = lane < U && w0 + lane < L.words ? X.pc[w0 + lane] : 0u;
+            const uint2 mine = lane < U && w0 + lane < L.words ? rank[w0 + lane] : make_uint2(0, 0);
+            if (!__any_sync(0xffffffffu, mine.x != 0)) continue;
             uint32_t lo[U], hi[U], at[U];
+            uint4 m[U];
 #pragma unroll
             for (uint32_t x = 0; x < U; ++x) {
-                const uint32_t word = __shfl_sync(0xffffffffu, mine, (int)x);
-                at[x] = __shfl_sync(0xffffffffu, mypc, (int)x) + __popc(word & ((1u << lane) - 1u));
-                const bool on = (word >> lane) & 1u;
+                const uint32_t word = __shfl_sync(0xffffffffu, mine.x, (int)x);
+                at[x] = __shfl_sync(0xffffffffu, mine.y, (int)x) + __popc(word & ((1u << lane) - 1u));
                 const uint32_t r = (w0 + x) * 32u + lane;
                 lo[x] = hi[x] = 0;
-                if (!on) {
+                if (!((word >> lane) & 1u)) {
                     at[x] = 0xffffffffu;
-                } else if (window) {
-                    lo[x] = L.lo[r];
-                    hi[x] = L.hi[r];
+                } else {
+                    if (window) {
+                        lo[x] = L.lo[r];
+                        hi[x] = L.hi[r];
+                    }
+                    m[x].z = L.eid[r];
+                    m[x].w = L.src[r];
+                }
+            }
+#pragma unroll
+            for (uint32_t x = 0; x < U; ++x) {
+                m[x].x = m[x].y = 0;
+                if (window && at[x] != 0xffffffffu) {
+                    m[x].x = rank_below(below, lo[x]);
+                    m[x].y = rank_below(below, hi[x]);
+                    span += m[x].y - m[x].x;
                 }
             }
 #pragma unroll
             for (uint32_t x = 0; x < U; ++x)
                 if (at[x] != 0xffffffffu) {
                     const uint32_t r = (w0 + x) * 32u + lane;
-                    X.meta[at[x]] = make_uint4(window ? rank_below(P, lo[x]) : 0u, window ? rank_below(P, hi[x]) : 0u,
-                                               L.eid[r], L.src[r]);
+                    X.meta[at[x]] = m[x];
                     if (X.mhead) X.mhead[at[x]] = L.head[r];
                     if (X.mtime) X.mtime[at[x]] = L.time[r];
                 }
+        }
+        if (window && __any_sync(0xffffffffu, span != 0)) {
+#pragma unroll
+            for (int f = 16; f > 0; f >>= 1) span += __shfl_xor_sync(0xffffffffu, (unsigned long long)span, f);
+            if (lane == 0) atomicAdd(t.span + X.prev, (unsigned long long)span);
         }
     }
     // the partial sums of layer 1's blocks
@@ -547,7 +606,7 @@ __device__ __noinline__ bool x_plan(const XArgs &a, const XOne &o, View &v)
         const XLL &X = t.ll[li];
         const uint32_t c = t.cnt[li];
         if (X.out || !c) continue;
-        const uint32_t words = (c / kSup1 + 1 + c / kSup2 + 1) * (X.cout + X.uout);
+        const uint32_t words = x_sup_rows(c) * (X.cout + X.uout);
         for (uint32_t w = gt; w < words; w += nt) X.sup[w] = 0;
     }
     return v.sync();
@@ -598,34 +657,153 @@ __device__ __forceinline__ uint64_t wedge_at(const uint32_t *__restrict__ tb, ui
     return finish27(z);
 }
 
-// XOR of rows [ra, rb) of a level's values from their prefix sums (blocks of
-// 1 << ps rows, sums of 16 and 256 blocks), `count` values per row, into dst;
-// one warp. The two ends' rows come first, several loads in flight, then the
-// whole blocks between them.
-__device__ __forceinline__ void window_sum(const uint64_t *R, const uint64_t *sup1, const uint64_t *sup2, uint32_t stride,
-                                           uint32_t ps, uint32_t ra, uint32_t rb, uint32_t count, uint32_t lane, uint64_t *dst)
+__device__ __forceinline__ void xor_shared(uint64_t *p, uint64_t v)
 {
-    const uint32_t pm = (1u << ps) - 1u;
-    const bool ha = ra & pm, hb = rb & pm;
-    const uint64_t *pa = R + (size_t)(ha ? ra - 1 : 0) * stride, *pb = R + (size_t)(hb ? rb - 1 : 0) * stride;
+    uint32_t *w = reinterpret_cast<uint32_t *>(p);
+    if ((uint32_t)v) atomicXor(w, (uint32_t)v);
+    if ((uint32_t)(v >> 32)) atomicXor(w + 1, (uint32_t)(v >> 32));
+}
+
+// Level list li's prefix sums are completed (x_scan_blocks): when the windows
+// that read it span more than kScanSpan blocks on average, and for long levels,
+// where a few windows of thousands of rows hold their teams up. Otherwise the
+// pass and its barrier (5 us) cost more than the extra reads: dense contacts,
+// k = 12, 264 us scanning every layer of 48 blocks, 230 us so; at-most-k, k = 10,
+// on n = 1e6, m = 1e7 5.23 ms by the average alone, 4.99 ms so.
+__device__ __forceinline__ bool x_scans(const XTmpl &t, uint32_t li)
+{
+    const XShape sh = x_shape_of(t.shape[li]);
+    if (!sh.scan || t.ll[li].level >= t.maxlev) return false;
+    if (t.cnt[li] >= kScanLong * sh.rows) return true;
+    uint64_t readers = 0;
+    for (uint32_t i = t.runs[t.ll[li].level + 1].first, e = i + t.runs[t.ll[li].level + 1].count; i < e; ++i) readers += t.cnt[i];
+    return t.span[li] > readers * sh.rows * kScanSpan;
+}
+
+// What a level reads of the level below: per needed row `stride` values, prefix
+// sums within blocks of `rows` rows.
+struct XBelow {
+    const uint64_t *R, *IP;    // the rows; scanned levels: the sums of all blocks up to each
+    const uint64_t *s1, *s2, *s3;
+    uint32_t stride, rows, scan;
+};
+__device__ __forceinline__ XBelow x_below(const XTmpl &t, uint32_t prev, bool U)
+{
+    const XLL &P = t.ll[prev];
+    const XShape sh = x_shape_of(t.shape[prev]);
+    const uint32_t cnt = t.cnt[prev], nb = (cnt + sh.rows - 1u) / sh.rows;
+    XBelow b;
+    b.stride = U ? P.uout : P.cout;
+    b.rows = sh.rows;
+    b.scan = x_scans(t, prev) ? 1u : 0u;
+    b.R = U ? P.U : P.R;
+    // (P.IP: the cout columns of ipcap blocks, then the uout ones)
+    b.IP = sh.rows == 1u ? b.R : P.IP + (U ? (size_t)P.ipcap * P.cout : 0);
+    b.s1 = P.sup + (U ? (size_t)x_sup_rows(nb) * P.cout : 0);
+    b.s2 = b.s1 + (size_t)(nb / kSup1 + 1u) * b.stride;
+    b.s3 = b.s2 + (size_t)(nb / kSup2 + 1u) * b.stride;
+    return b;
+}
+// A window's two ends in its block structure.
+struct XEnds {
+    uint32_t b0, b1;        // first and end block: whole blocks [b0, b1) lie between
+    const uint64_t *p0, *p1;  // the row before each end inside its block, or null
+};
+__device__ __forceinline__ XEnds x_ends(const XBelow &B, uint32_t ra, uint32_t rb)
+{
+    XEnds e;
+    e.b0 = ra / B.rows;
+    e.b1 = rb / B.rows;
+    e.p0 = ra - e.b0 * B.rows ? B.R + (size_t)(ra - 1u) * B.stride : nullptr;
+    e.p1 = rb - e.b1 * B.rows ? B.R + (size_t)(rb - 1u) * B.stride : nullptr;
+    if (B.scan && e.b0 == e.b1) e.b0 = e.b1 = 0;
+    return e;
+}
+// One value of a window of a scanned level: at most four reads.
+__device__ __forceinline__ uint64_t x_scanned(const XBelow &B, const XEnds &e, uint32_t s)
+{
+    uint64_t v = 0;
+    if (e.p0) v ^= e.p0[s];
+    if (e.p1) v ^= e.p1[s];
+    if (e.b0) v ^= B.IP[(size_t)(e.b0 - 1u) * B.stride + s];
+    if (e.b1) v ^= B.IP[(size_t)(e.b1 - 1u) * B.stride + s];
+    return v;
+}
+// The blocks [i, e) in as few pieces as the partial sums allow: the next one.
+__device__ __forceinline__ const uint64_t *x_piece(const XBelow &B, uint32_t &i, uint32_t e)
+{
+    const uint64_t *p;
+    if (!(i % kSup3) && i + kSup3 <= e) {
+        p = B.s3 + (size_t)(i / kSup3) * B.stride;
+        i += kSup3;
+    } else if (!(i % kSup2) && i + kSup2 <= e) {
+        p = B.s2 + (size_t)(i / kSup2) * B.stride;
+        i += kSup2;
+    } else if (!(i % kSup1) && i + kSup1 <= e) {
+        p = B.s1 + (size_t)(i / kSup1) * B.stride;
+        i += kSup1;
+    } else {
+        p = B.R + ((size_t)(i + 1u) * B.rows - 1u) * B.stride;
+        ++i;
+    }
+    return p;
+}
+// XOR of the rows [ra, rb)'s values first, first + step, .. into dst; one warp,
+// several loads in flight.
+__device__ __forceinline__ void window_sum(const XBelow &B, uint32_t ra, uint32_t rb, uint32_t count, uint32_t first,
+                                           uint32_t step, uint64_t *dst)
+{
+    const XEnds e = x_ends(B, ra, rb);
+    if (B.scan) {
 #pragma unroll 4
-    for (uint32_t s = lane; s < count; s += 32u) dst[s] = (ha ? pa[s] : 0ull) ^ (hb ? pb[s] : 0ull);
-    uint32_t i = ra >> ps;
-    const uint32_t e = rb >> ps;
-    while (i < e) {  // warp-uniform
-        const uint64_t *p;
-        if (!(i % kSup2) && i + kSup2 <= e) {
-            p = sup2 + (size_t)(i / kSup2) * stride;
-            i += kSup2;
-        } else if (!(i % kSup1) && i + kSup1 <= e) {
-            p = sup1 + (size_t)(i / kSup1) * stride;
-            i += kSup1;
-        } else {
-            p = R + ((size_t)(i << ps) + pm) * stride;
-            ++i;
+        for (uint32_t s = first; s < count; s += step) dst[s] = x_scanned(B, e, s);
+        return;
+    }
+#pragma unroll 4
+    for (uint32_t s = first; s < count; s += step) dst[s] = (e.p0 ? e.p0[s] : 0ull) ^ (e.p1 ? e.p1[s] : 0ull);
+    for (uint32_t i = e.b0; i < e.b1;) {  // warp-uniform
+        const uint64_t *const p = x_piece(B, i, e.b1);
+#pragma unroll 4
+        for (uint32_t s = first; s < count; s += step) dst[s] ^= p[s];
+    }
+}
+
+// Completes a level's prefix sums: IP[b] = the XOR of the blocks up to b (rows of
+// one: in place). A warp takes 16 blocks and 32 columns, the sums before them
+// from the partial sums. A window then takes four reads instead of one per
+// piece: of a layer of 136,000 rows of 126 values the windows were a quarter of
+// the time with up to 30 pieces one after another.
+__device__ __forceinline__ void x_scan_blocks(const XTmpl &t, uint32_t li, const View &v)
+{
+    const XLL &X = t.ll[li];
+    const uint32_t lane = threadIdx.x & 31u, gw = v.b * kWarps + (threadIdx.x >> 5), nw = v.n * kWarps;
+    const uint32_t cnt = t.cnt[li], rows = x_shape_of(t.shape[li]).rows, nb = (cnt + rows - 1u) / rows;
+    const uint32_t groups = (nb + kSup1 - 1u) / kSup1;
+    const uint32_t cr = X.R ? (X.cout + 31u) / 32u : 0u, cu = (X.uout + 31u) / 32u, cols = cr + cu;
+    for (uint32_t i = gw; i < groups * cols; i += nw) {
+        const uint32_t g = i / cols, c = i - g * cols;
+        const bool U = c >= cr;
+        const XBelow B = x_below(t, li, U);
+        const uint32_t s = (U ? c - cr : c) * 32u + lane;
+        if (s >= B.stride) continue;
+        uint64_t *const R = (U ? X.U : X.R) + s;
+        uint64_t *const IP = rows == 1u ? R : X.IP + (U ? (size_t)X.ipcap * X.cout : 0) + s;
+        uint64_t acc = 0;
+        const uint32_t first = g * kSup1;
+        for (uint32_t b = 0; b < first / kSup3; ++b) acc ^= B.s3[(size_t)b * B.stride + s];
+#pragma unroll 4
+        for (uint32_t b = first / kSup3 * (kSup3 / kSup2); b < first / kSup2; ++b) acc ^= B.s2[(size_t)b * B.stride + s];
+#pragma unroll 4
+        for (uint32_t b = first / kSup2 * (kSup2 / kSup1); b < g; ++b) acc ^= B.s1[(size_t)b * B.stride + s];
+        uint64_t tot[kSup1];
+#pragma unroll
+        for (uint32_t b = 0; b < kSup1; ++b)
+            tot[b] = first + b < nb ? R[(size_t)(min(cnt, (first + b + 1u) * rows) - 1u) * B.stride] : 0ull;
+#pragma unroll
+        for (uint32_t b = 0; b < kSup1; ++b) {
+            acc ^= tot[b];
+            if (first + b < nb) IP[(size_t)(first + b) * B.stride] = acc;
         }
-#pragma unroll 4
-        for (uint32_t s = lane; s < count; s += 32u) dst[s] ^= p[s];
     }
 }
 
@@ -636,7 +814,8 @@ __device__ __forceinline__ void window_sum(const uint64_t *R, const uint64_t *su
 // The store level below an out level keeps U = z'_v ^ (its value), v the row's
 // head, on the label sets the output needs: the window of an out row lies in one
 // vertex's rows, so the wedge with that vertex is taken once per stored row, not
-// per out row, and an out row needs y U only.
+// per out row, and an out row needs y sum_j z'_{w,j} U_j only, one product per
+// label and one per row.
 __device__ __noinline__ bool x_wedge(const XArgs &a, const XOne &o, View &v, uint32_t lbeg, uint32_t lend, bool last_sync)
 {
     extern __shared__ __align__(16) uint64_t sm_all[];
@@ -647,156 +826,185 @@ __device__ __noinline__ bool x_wedge(const XArgs &a, const XOne &o, View &v, uin
     for (uint32_t l = lbeg; l <= lend; ++l) {
         bool any = false;
         uint32_t base_item = 0;
-            for (uint32_t li = t_.runs[l].first; li < t_.runs[l].first + t_.runs[l].count; ++li) {
-                const uint32_t cnt = t_.cnt[li];
-                if (!cnt) continue;
-                any = true;
-                const XLL &X = t_.ll[li];
-                const uint32_t cin = X.cin, cout = X.cout, uout = X.uout, d = X.d;
-                const uint32_t K = X.out ? cout : Q.K;  // labels in use
-                const XShape sh = x_shape_of(t_.shape[li]);
-                const uint32_t qs = sh.rows, rows = 1u << qs;
-                const uint32_t nb = (cnt + rows - 1) >> qs;
-                // the thread's team, its number in the grid and its shared memory
-                const uint32_t tsize = 32u << sh.team, team = threadIdx.x / tsize, tid = threadIdx.x % tsize;
-                const uint32_t per_block = (1u << kTeamLog) >> sh.team;
-                const uint32_t nteam = v.n * per_block, gteam = team * v.n + v.b;
-                const uint32_t tsmem = a.smem >> (kTeamLog - sh.team);
-                uint64_t *const sm = sm_all + (size_t)team * (tsmem / 8);
-                uint32_t *const msp = reinterpret_cast<uint32_t *>(sm);  // rows x K split multipliers
-                uint64_t *const dr = sm + (size_t)rows * K * (kSplit / 2), *const G = dr + rows * cin, *const Us = G + rows * cout;
-                uint4 *const smeta = reinterpret_cast<uint4 *>(sm + (tsmem / 8 - rows * 4u));
-                uint32_t *const shead = reinterpret_cast<uint32_t *>(smeta + rows);
-                auto sync = [&] {
-                    if (sh.team == 0) __syncwarp();
-                    else if (sh.team == kTeamLog) __syncthreads();
-                    else asm volatile("bar.sync %0, %1;" ::"r"(team + 1u), "r"(tsize) : "memory");
-                };
-                // the level below: its prefix sums come in blocks of 1 << ps rows
-                const XLL &P = t_.ll[X.prev];
-                const uint32_t pcnt = l > 1 ? t_.cnt[X.prev] : 0u;
-                const uint32_t ps = l > 1 ? x_shape_of(t_.shape[X.prev]).rows : 0u;
-                const uint32_t pn1 = (((pcnt + (1u << ps) - 1) >> ps) / kSup1) + 1, pn2 = (((pcnt + (1u << ps) - 1) >> ps) / kSup2) + 1;
-                const uint32_t pst = X.out ? P.uout : P.cout;  // values per row read from below
-                const uint64_t *const pR = X.out ? P.U : P.R;
-                const uint64_t *const psup1 = P.sup + (X.out ? (size_t)(pn1 + pn2) * P.cout : 0), *const psup2 = psup1 + (size_t)pn1 * pst;
-                const uint32_t n1 = nb / kSup1 + 1, n2 = nb / kSup2 + 1;
-                uint64_t *const E = X.out ? Q.E : nullptr, *const S = Q.S + (size_t)X.row * a.n;
-                const bool per_row = E || X.Ec;  // out levels: every row's own sum is wanted
-                for (uint32_t it = View::first_item(base_item, gteam, nteam); it < nb; it += nteam) {
-                    const uint32_t row0 = it << qs, nr = min(rows, cnt - row0);
-                    sync();
-                    for (uint32_t t = tid; t < nr; t += tsize) {
-                        smeta[t] = X.meta[row0 + t];
-                        if (X.mhead) shead[t] = X.mhead[row0 + t];
+        for (uint32_t li = t_.runs[l].first; li < t_.runs[l].first + t_.runs[l].count; ++li) {
+            const uint32_t cnt = t_.cnt[li];
+            if (!cnt) continue;
+            any = true;
+            const XLL &X = t_.ll[li];
+            const uint32_t cin = X.cin, cout = X.cout, uout = X.uout, d = X.d;
+            const uint32_t K = X.out ? cout : Q.K;  // labels in use
+            const XShape sh = x_shape_of(t_.shape[li]);
+            const uint32_t rows = sh.rows, nb = (cnt + rows - 1) / rows;
+            // the thread's team, its number in the grid and its shared memory
+            const uint32_t tsize = team_threads(sh.team), team = threadIdx.x / tsize, tid = threadIdx.x % tsize;
+            const uint32_t nteam = v.n * team_count(sh.team), gteam = team * v.n + v.b, twarps = tsize / 32u;
+            const uint32_t tsmem = team_smem(a.smem, sh.team);
+            uint64_t *const sm = sm_all + (size_t)team * (tsmem / 8);
+            uint32_t *const msp = reinterpret_cast<uint32_t *>(sm);  // rows x K split multipliers
+            uint64_t *const dr = sm + (size_t)rows * K * (kSplit / 2), *const G = dr + rows * cin, *const Us = G + rows * cout;
+            uint4 *const smeta = reinterpret_cast<uint4 *>(sm + (tsmem / 8 - rows * 8u));
+            uint32_t *const shead = reinterpret_cast<uint32_t *>(smeta + rows), *const srun = shead + rows;
+            auto sync = [&] {
+                if (sh.team == 0) __syncwarp();
+                else if (sh.team + 1u == kTeams) __syncthreads();
+                else asm volatile("bar.sync %0, %1;" ::"r"(team + 1u), "r"(tsize) : "memory");
+            };
+            XBelow B{};
+            if (l > 1) B = x_below(t_, X.prev, X.out != 0);
+            uint64_t *const E = X.out ? Q.E : nullptr, *const S = Q.S + (size_t)X.row * a.n;
+            for (uint32_t it = View::first_item(base_item, gteam, nteam); it < nb; it += nteam) {
+                const uint32_t row0 = it * rows, nr = min(rows, cnt - row0);
+                sync();
+                // (at most 16 rows: the first half warp of the team)
+                if (tid < 32u) {
+                    uint32_t h = 0xffffffffu;
+                    if (tid < nr) {
+                        smeta[tid] = X.meta[row0 + tid];
+                        if (X.mhead) shead[tid] = h = X.mhead[row0 + tid];
                     }
-                    sync();
-                    if (l > 1)
-                        for (uint32_t q = tid >> 5; q < nr; q += 1u << sh.team)
-                            window_sum(pR, psup1, psup2, pst, ps, smeta[q].x, smeta[q].y, X.out ? cout : cin, lane,
-                                       (X.out ? G + q * cout : dr + q * cin));
-                    if (!X.out) {
-                        if (l == 1) {
-                            // y_{e,1} z_{s,p}; a set of sources: y_{e,1} z_{s,j}
-                            for (uint32_t t = tid; t < nr * cout; t += tsize) {
-                                const uint32_t q = t / cout;
-                                G[t] = gf64_mul(sm_draw(Q.key_y, (uint64_t)smeta[q].z * 32u),
-                                                Q.multi ? zprime(Q, t_.omega, a.color, smeta[q].w, t - q * cout) : Q.d0);
-                            }
-                        } else {
-                            for (uint32_t t = tid; t < nr * K; t += tsize) {
-                                const uint32_t q = t / K, j = t - q * K;
-                                const uint64_t y = sm_draw(Q.key_y, (uint64_t)smeta[q].z * 32u + (l - 1u));
-                                store_split(msp + (size_t)t * kSplit, gf64_mul(y, zprime(Q, t_.omega, a.color, smeta[q].w, j)));
-                            }
-                            sync();
-                            const uint32_t *const tb = a.tab + x_tab_off_dev(d);
-                            const uint32_t cm = x_binom_dev(kXMaxLabels, d);
-                            for (uint32_t t = tid; t < nr * cout; t += tsize) {
-                                const uint32_t q = t / cout, T = t - q * cout;
-                                G[t] = wedge_at(tb, cm, T, d, msp + (size_t)q * K * kSplit, dr + q * cin);
-                            }
+                    // the row's run of equal heads, by its first row
+                    const uint32_t up = __shfl_up_sync(0xffffffffu, h, 1);
+                    const uint32_t starts = __ballot_sync(0xffffffffu, tid == 0 || h != up);
+                    if (tid < nr) srun[tid] = 31u - __clz(starts & (0xffffffffu >> (31u - tid)));
+                }
+                sync();
+                if (!X.out) {
+                    if (l > 1) {
+                        // a warp takes whole rows, or with fewer rows than warps a share of
+                        // one row's columns
+                        const uint32_t w = tid >> 5, share = twarps / nr;
+                        if (share <= 1u) {
+                            for (uint32_t q = w; q < nr; q += twarps)
+                                window_sum(B, smeta[q].x, smeta[q].y, cin, lane, 32u, dr + q * cin);
+                        } else if (w < share * nr) {
+                            const uint32_t q = w / share;
+                            window_sum(B, smeta[q].x, smeta[q].y, cin, (w - q * share) * 32u + lane, 32u * share, dr + q * cin);
                         }
-                        sync();
-                        if (uout) {  // U on the d+1-subsets of the first d + 2 labels
-                            for (uint32_t t = tid; t < nr * uout; t += tsize) {
-                                const uint32_t q = t / uout, j = t - q * uout;
-                                store_split(msp + (size_t)t * kSplit, zprime(Q, t_.omega, a.color, shead[q], j));
-                            }
-                            sync();
-                            const uint32_t *const tb = a.tab + x_tab_off_dev(d + 1u);
-                            const uint32_t cm = x_binom_dev(kXMaxLabels, d + 1u);
-                            for (uint32_t t = tid; t < nr * uout; t += tsize) {
-                                const uint32_t q = t / uout, T = t - q * uout;
-                                Us[t] = wedge_at(tb, cm, T, d + 1u, msp + (size_t)q * uout * kSplit, G + q * cout);
-                            }
-                            sync();
-                        }
-                        const bool whole = nb >= kSup1 && nr == rows;
-                        for (uint32_t s = tid; s < cout + uout; s += tsize) {
-                            const bool isU = s >= cout;
-                            const uint32_t st = isU ? uout : cout, c = isU ? s - cout : s;
-                            const uint64_t *const g = (isU ? Us : G) + c;
-                            uint64_t *const o = (isU ? X.U : X.R) + c;
-                            uint64_t acc = 0;
-                            if (isU || X.R) {
-                                for (uint32_t q = 0; q < nr; ++q) {
-                                    acc ^= g[q * st];
-                                    o[(size_t)(row0 + q) * st] = acc;
-                                }
-                                if (whole) {
-                                    uint64_t *const s1 = X.sup + (isU ? (size_t)(n1 + n2) * cout : 0) + c;
-                                    atomicXor(reinterpret_cast<unsigned long long *>(s1 + (size_t)(it / kSup1) * st), (unsigned long long)acc);
-                                    if (nb >= kSup2)
-                                        atomicXor(reinterpret_cast<unsigned long long *>(s1 + (size_t)(n1 + it / kSup2) * st), (unsigned long long)acc);
-                                }
-                            }
+                    }
+                    if (l == 1) {
+                        // y_{e,1} z_{s,p}; a set of sources: y_{e,1} z_{s,j}
+                        for (uint32_t t = tid; t < nr * cout; t += tsize) {
+                            const uint32_t q = t / cout;
+                            G[t] = gf64_mul(sm_draw(Q.key_y, (uint64_t)smeta[q].z * 32u),
+                                            Q.multi ? zprime(Q, t_.omega, a.color, smeta[q].w, t - q * cout) : Q.d0);
                         }
                     } else {
-                        // y U per row (layer 1: the source's z row itself), then z'_w over runs of
-                        // equal heads -- or row by row when every row's own sum is wanted
-                        sync();
                         for (uint32_t t = tid; t < nr * K; t += tsize) {
-                            const uint32_t q = t / K;
+                            const uint32_t q = t / K, j = t - q * K;
                             const uint64_t y = sm_draw(Q.key_y, (uint64_t)smeta[q].z * 32u + (l - 1u));
-                            G[t] = gf64_mul(y, l > 1 ? G[t] : Q.multi ? zprime(Q, t_.omega, a.color, smeta[q].w, t - q * K) : Q.d0);
+                            store_split(msp + (size_t)t * kSplit, gf64_mul(y, zprime(Q, t_.omega, a.color, smeta[q].w, j)));
                         }
                         sync();
-                        for (uint32_t t = tid; t < nr * K; t += tsize) {
-                            const uint32_t q = t / K, T = t - q * K;
-                            if (!per_row && q && shead[q] == shead[q - 1]) continue;
-                            uint64_t x = G[t];
-                            if (!per_row)
-                                for (uint32_t o = q + 1; o < nr && shead[o] == shead[q]; ++o) x ^= G[o * K + T];
-                            sm[t] = gf64_mul(x, zprime(Q, t_.omega, a.color, shead[q], K - 1u - T));  // the label T misses
-                        }
-                        sync();
-                        for (uint32_t q = tid; q < nr; q += tsize) {
-                            if (!per_row && q && shead[q] == shead[q - 1]) continue;
-                            uint64_t x = 0;
-                            for (uint32_t s = 0; s < K; ++s) x ^= sm[q * K + s];
-                            if (E) E[smeta[q].z] = x;
-                            if (X.Ec) X.Ec[row0 + q] = x;
-                            if (x) atomicXor(reinterpret_cast<unsigned long long *>(S + shead[q]), (unsigned long long)x);
+                        const uint32_t *const tb = a.tab + x_tab_off_dev(d);
+                        const uint32_t cm = x_binom_dev(kXMaxLabels, d);
+                        for (uint32_t t = tid; t < nr * cout; t += tsize) {
+                            const uint32_t q = t / cout, T = t - q * cout;
+                            G[t] = wedge_at(tb, cm, T, d, msp + (size_t)q * K * kSplit, dr + q * cin);
                         }
                     }
+                    sync();
+                    if (uout) {  // U on the d+1-subsets of the first d + 2 labels; z' once per run of heads
+                        for (uint32_t t = tid; t < nr * uout; t += tsize) {
+                            const uint32_t q = t / uout, j = t - q * uout;
+                            if (srun[q] == q) store_split(msp + (size_t)t * kSplit, zprime(Q, t_.omega, a.color, shead[q], j));
+                        }
+                        sync();
+                        const uint32_t *const tb = a.tab + x_tab_off_dev(d + 1u);
+                        const uint32_t cm = x_binom_dev(kXMaxLabels, d + 1u);
+                        for (uint32_t t = tid; t < nr * uout; t += tsize) {
+                            const uint32_t q = t / uout, T = t - q * uout;
+                            Us[t] = wedge_at(tb, cm, T, d + 1u, msp + (size_t)srun[q] * uout * kSplit, G + q * cout);
+                        }
+                        sync();
+                    }
+                    const bool whole = nb >= kSup1 && nr == rows;
+                    for (uint32_t s = X.R ? tid : cout + tid; s < cout + uout; s += tsize) {
+                        const bool isU = s >= cout;
+                        const uint32_t st = isU ? uout : cout, c = isU ? s - cout : s;
+                        const uint64_t *const g = (isU ? Us : G) + c;
+                        uint64_t *const out = (isU ? X.U : X.R) + c;
+                        uint64_t acc = 0;
+                        for (uint32_t q = 0; q < nr; ++q) {
+                            acc ^= g[q * st];
+                            out[(size_t)(row0 + q) * st] = acc;
+                        }
+                        if (whole) {
+                            auto add = [&](uint64_t *p) { atomicXor(reinterpret_cast<unsigned long long *>(p), (unsigned long long)acc); };
+                            uint64_t *const s1 = X.sup + (isU ? (size_t)x_sup_rows(nb) * cout : 0) + c;
+                            uint64_t *const s2 = s1 + (size_t)(nb / kSup1 + 1u) * st, *const s3 = s2 + (size_t)(nb / kSup2 + 1u) * st;
+                            add(s1 + (size_t)(it / kSup1) * st);
+                            if (nb >= kSup2) add(s2 + (size_t)(it / kSup2) * st);
+                            if (nb >= kSup3) add(s3 + (size_t)(it / kSup3) * st);
+                        }
+                    }
+                } else {
+                    // z'_w of the runs' heads, and the sums of the rows
+                    uint64_t *const zw = sm, *const sum = sm + rows * K;
+                    for (uint32_t t = tid; t < nr * K; t += tsize) {
+                        const uint32_t q = t / K;
+                        if (srun[q] == q) zw[t] = zprime(Q, t_.omega, a.color, shead[q], t - q * K);
+                    }
+                    for (uint32_t q = tid; q < nr; q += tsize) sum[q] = 0;
+                    sync();
+                    for (uint32_t t = tid; t < nr * K; t += tsize) {
+                        const uint32_t q = t / K, T = t - q * K;
+                        uint64_t u;
+                        if (l == 1) {  // the source's z row itself
+                            u = Q.multi ? zprime(Q, t_.omega, a.color, smeta[q].w, T) : Q.d0;
+                        } else {
+                            const XEnds e = x_ends(B, smeta[q].x, smeta[q].y);
+                            if (B.scan) {
+                                u = x_scanned(B, e, T);
+                            } else {
+                                u = (e.p0 ? e.p0[T] : 0ull) ^ (e.p1 ? e.p1[T] : 0ull);
+                                for (uint32_t i = e.b0; i < e.b1;) u ^= x_piece(B, i, e.b1)[T];
+                            }
+                        }
+                        // T misses one label, whose z' it meets
+                        xor_shared(sum + q, gf64_mul(u, zw[srun[q] * K + (K - 1u - T)]));
+                    }
+                    sync();
+                    if (tid < 32u) {
+                        uint64_t x = 0;
+                        if (tid < nr) {
+                            const uint32_t e = smeta[tid].z;
+                            x = gf64_mul(sum[tid], sm_draw(Q.key_y, (uint64_t)e * 32u + (l - 1u)));
+                            if (E) E[e] = x;
+                            if (X.Ec) X.Ec[row0 + tid] = x;
+                        }
+                        // runs of equal heads: one atomic, by the run's last row
+                        const uint32_t first = tid < nr ? srun[tid] : tid;
+#pragma unroll
+                        for (int f = 1; f < 16; f <<= 1) {
+                            const uint64_t y = __shfl_up_sync(0xffffffffu, (unsigned long long)x, f);
+                            if (tid >= first + f) x ^= y;
+                        }
+                        if (tid < nr && x && (tid + 1u == nr || srun[tid + 1u] != first))
+                            atomicXor(reinterpret_cast<unsigned long long *>(S + shead[tid]), (unsigned long long)x);
+                    }
                 }
-                base_item += nb;
-                __syncthreads();  // the next level list may form other teams
             }
+            base_item += nb;
+            __syncthreads();  // the next level list may form other teams
+        }
         if (l < t_.maxlev)  // clear the next level's partial sums
             for (uint32_t li = t_.runs[l + 1].first; li < t_.runs[l + 1].first + t_.runs[l + 1].count; ++li) {
                 const uint32_t cnt = t_.cnt[li];
                 const XLL &X = t_.ll[li];
                 if (X.out || !cnt) continue;
-                const uint32_t qs = x_shape_of(t_.shape[li]).rows;
-                const uint32_t nb = (cnt + (1u << qs) - 1) >> qs;
+                const uint32_t rows = x_shape_of(t_.shape[li]).rows, nb = (cnt + rows - 1u) / rows;
                 if (nb < kSup1) continue;
-                const uint32_t w = (nb / kSup1 + 1 + nb / kSup2 + 1) * (X.cout + X.uout);
+                const uint32_t w = x_sup_rows(nb) * (X.cout + X.uout);
                 for (uint32_t i = gt; i < w; i += nt) X.sup[i] = 0;
             }
-        if (any && (l < lend || last_sync))
+        const uint32_t st = t_.runs[l].first;  // the store level list, if the level has one
+        const bool scan = l < t_.maxlev && t_.cnt[st] && x_scans(t_, st);
+        if (any && (l < lend || last_sync || scan))
             if (!v.sync()) return false;
+        if (scan) {
+            x_scan_blocks(t_, st, v);
+            if (!v.sync()) return false;
+        }
     }
     return true;
 }
@@ -822,16 +1030,15 @@ __device__ __noinline__ void x_outputs(const XArgs &a, const XOne &o, const View
         }
     }
     if (!Q.bitmap) return;
-    const uint32_t nbytes = (a.n + 7) / 8, rows = o.t.every ? Q.k - 1 : 1u;
-    for (uint32_t b = gt; b < nbytes; b += nt) {
-        uint32_t bits = 0;
-        for (uint32_t w = 0; w < rows; ++w)
-#pragma unroll
-            for (uint32_t i = 0; i < 8; ++i) {
-                const uint32_t x = b * 8 + i;
-                if (x < a.n && Q.S[(size_t)w * a.n + x] != 0) bits |= 1u << i;
-            }
-        Q.bitmap[b] = (uint8_t)bits;
+    // a warp takes 32 vertices: whole lines of the witness rows
+    const uint32_t rows = o.t.every ? Q.k - 1 : 1u, lane = threadIdx.x & 31u;
+    for (uint32_t w = gt >> 5; w < (a.n + 31u) / 32u; w += nt >> 5) {
+        const uint32_t x = w * 32u + lane;
+        uint64_t any = 0;
+        if (x < a.n)
+            for (uint32_t r = 0; r < rows; ++r) any |= Q.S[(size_t)r * a.n + x];
+        const uint32_t word = __ballot_sync(0xffffffffu, any != 0);
+        if (lane < 4u && w * 4u + lane < (a.n + 7u) / 8u) Q.bitmap[w * 4u + lane] = (uint8_t)(word >> (8u * lane));
     }
 }
 
@@ -874,13 +1081,6 @@ struct TinyMem {
     uint64_t acc[kTinyTotal];               // their sums
     uint64_t omega[(kXMaxLabels + 1) * (kXMaxLabels + 1)];
 };
-
-__device__ __forceinline__ void xor_shared(uint64_t *p, uint64_t v)
-{
-    uint32_t *w = reinterpret_cast<uint32_t *>(p);
-    if ((uint32_t)v) atomicXor(w, (uint32_t)v);
-    if ((uint32_t)(v >> 32)) atomicXor(w + 1, (uint32_t)(v >> 32));
-}
 
 // XOR of the level below's values s of the rows in `mk`, by their places among
 // its needed rows `nd`.
@@ -1219,7 +1419,7 @@ __device__ __forceinline__ void relocate(XTmpl &t, uint8_t *base)
         XLL &x = t.ll[i];
         fix(x.A);
         fix(x.N);
-        fix(x.pc);
+        fix(x.rank);
         fix(x.tsum);
         fix(x.meta);
         fix(x.mhead);
@@ -1227,6 +1427,7 @@ __device__ __forceinline__ void relocate(XTmpl &t, uint8_t *base)
         fix(x.R);
         fix(x.U);
         fix(x.sup);
+        fix(x.IP);
         fix(x.Ec);
     }
     if (threadIdx.x == 0) {
@@ -1234,6 +1435,7 @@ __device__ __forceinline__ void relocate(XTmpl &t, uint8_t *base)
         fix(t.live);
         fix(t.cnt);
         fix(t.shape);
+        fix(t.span);
         fix(t.omega);
     }
 }
@@ -1544,22 +1746,26 @@ static uint64_t x_template(const XList *lists, uint32_t k, bool every, bool mult
         for (uint32_t i = 0; i < t.nll; ++i)
             if (!t.ll[i].out) t.ll[i].N = b.take<uint32_t>(t.ll[i].words);
     t.clear4 = (uint32_t)(b.used / 16);
-    uint64_t ping[2] = {0, 0}, supw = 0;
+    uint64_t ping[2] = {0, 0}, ipw[2] = {0, 0}, supw = 0;
     for (uint32_t i = 0; i < t.nll; ++i) {
         const XLL &x = t.ll[i];
         if (x.out) continue;
         const uint64_t c = lists[x.list].count, w = x.cout + x.uout;
-        if (x.level >= 3) ping[x.level & 1u] = std::max<uint64_t>(ping[x.level & 1u], c * w);
-        supw = std::max<uint64_t>(supw, (c / kSup1 + c / kSup2 + 2) * w);
+        if (x.level >= 3) {
+            ping[x.level & 1u] = std::max<uint64_t>(ping[x.level & 1u], c * w);
+            ipw[x.level & 1u] = std::max<uint64_t>(ipw[x.level & 1u], (c / 4 + 1) * w);
+        }
+        supw = std::max<uint64_t>(supw, (uint64_t)x_sup_rows(c) * w);
     }
     uint64_t *pp[2] = {b.take<uint64_t>(ping[0]), b.take<uint64_t>(ping[1])};
+    uint64_t *ip[2] = {b.take<uint64_t>(ipw[0]), b.take<uint64_t>(ipw[1])};
     uint64_t *sup[3] = {b.take<uint64_t>(supw), b.take<uint64_t>(supw), b.take<uint64_t>(supw)};
     for (uint32_t i = 0; i < t.nll; ++i) {
         XLL &x = t.ll[i];
         const uint64_t c = lists[x.list].count;
         x.A = b.take<uint32_t>(x.words);
         if (x.out || every) x.N = x.A;
-        x.pc = b.take<uint32_t>(x.words);
+        x.rank = b.take<uint2>(x.words);
         x.tsum = b.take<uint32_t>(256);
         x.meta = b.take<uint4>(c);
         if (x.out || x.uout) x.mhead = b.take<uint32_t>(c);
@@ -1568,8 +1774,12 @@ static uint64_t x_template(const XList *lists, uint32_t k, bool every, bool mult
             x.Ec = b.take<uint64_t>(c);
         }
         if (!x.out) {
+            const bool up = x.level + 1 <= k - 2;  // a store level above reads R
             x.R = x.level >= 3 ? pp[x.level & 1u] : b.take<uint64_t>(c * (x.cout + x.uout));
             if (x.uout) x.U = x.R + c * x.cout;
+            if (!up) x.R = nullptr;
+            x.ipcap = (uint32_t)(c / 4 + 1);  // blocks IP holds (four rows or more a block)
+            x.IP = x.level >= 3 ? ip[x.level & 1u] : b.take<uint64_t>((uint64_t)x.ipcap * (x.cout + x.uout));
             x.sup = sup[x.level % 3];
         }
     }
@@ -1577,6 +1787,7 @@ static uint64_t x_template(const XList *lists, uint32_t k, bool every, bool mult
     t.live = b.take<uint32_t>(t.nll);
     t.cnt = b.take<uint32_t>(t.nll);
     t.shape = b.take<uint32_t>(t.nll);
+    t.span = b.take<unsigned long long>(t.nll);
     return b.used;
 }
 
@@ -1589,7 +1800,7 @@ static void x_args(const Graph &g, XArgs &a)
     a.ooff = g.o_off.as<uint32_t>();
     a.orec = g.o_rec.as<uint4>();
     a.olen = g.o_len.as<uint32_t>();
-    a.smem = g.x_smem_max / (16u << kTeamLog) * (16u << kTeamLog);  // 16-byte shares per warp
+    a.smem = g.x_smem_max / 16u * 16u;
 }
 
 // gf64 inverse by the extended Euclidean algorithm on binary polynomials.

@@ -50,13 +50,15 @@ struct XLL {
     uint32_t list, level, prev, out;  // prev: the store level below (itself at level 1)
     uint32_t d, cin, cout, uout;      // d: subset size of the values; cin / cout: values read / kept per row;
                                       // uout: store levels below an out level: values kept for it per row
-    uint32_t words, row;              // row: out levels' witness row
-    uint32_t *A, *N, *pc;             // active rows, needed rows (bitmaps), exclusive popcount per word of N
+    uint32_t words, row, ipcap, pad;  // row: out levels' witness row
+    uint32_t *A, *N;                  // active rows, needed rows (bitmaps)
+    uint2 *rank;                      // per word of N: the word and the needed rows before it
     uint32_t *tsum;                   // rows per scan tile (256)
     uint4 *meta;                      // per needed row: window [x, y) in needed rows of prev, edge, tail
     uint32_t *mhead, *mtime;          // heads; out levels with arrivals: times
     uint64_t *R, *U;                  // store levels: prefix sums of the cout values and of the uout ones
-    uint64_t *sup;                    // sums of 16 and of 256 blocks (R's, then U's)
+    uint64_t *sup;                    // sums of 16, 256 and 4,096 blocks (R's, then U's)
+    uint64_t *IP;                     // sums of all blocks up to each, of ipcap blocks at most (R's, then U's)
     uint64_t *Ec;                     // out levels with arrivals: per-row sums
 };
 
@@ -70,7 +72,8 @@ struct XTmpl {
     uint4 *clear;          // needed-row bitmaps to clear
     uint32_t *live;        // per level list: some row is active
     uint32_t *cnt;         // per level list: needed rows
-    uint32_t *shape;       // per level list: log2 warps per team | log2 rows per item << 8
+    uint32_t *shape;       // per level list: log2 warps per team | rows per item << 8 | scanned << 16
+    unsigned long long *span;  // per store level: rows of it in the windows of the level above, together
     uint64_t *omega;       // coloured: shade factors omega'_{d,j}, k x K
     XRun runs[kXMaxLevels + 1];
     XLL ll[kXMaxLL];
