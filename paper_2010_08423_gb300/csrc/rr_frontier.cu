@@ -84,6 +84,26 @@ __host__ __device__ constexpr uint32_t x_tab_off(uint32_t d)
 
 __device__ __forceinline__ uint32_t x_tab_off_dev(uint32_t d) { return c_tab_off[d]; }
 
+// For K <= kPackedLabels the tables of [K] once more, packed ([d][i][T], K 2^(K-1)
+// words), so that a block copies them in one go.
+constexpr uint32_t kPackedLabels = 11;
+constexpr uint32_t kPackedTab = x_tab_off(kXMaxLabels + 1);
+__host__ __device__ constexpr uint32_t x_packed_off(uint32_t K)  // sum of i 2^(i-1), i < K
+{
+    return (K - 2u) * (1u << (K - 1u)) + 1u;
+}
+
+__global__ void __launch_bounds__(128) k_packed_table(uint32_t *__restrict__ tab)
+{
+    const uint32_t K = blockIdx.y + 1;
+    uint32_t *o = tab + kPackedTab + x_packed_off(K);
+    for (uint32_t d = 1; d <= K; ++d) {
+        const uint32_t c = x_binom_dev(K, d), cm = x_binom_dev(kXMaxLabels, d), *src = tab + x_tab_off_dev(d);
+        for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < d * c; i += gridDim.x * blockDim.x) o[i] = src[i / c * cm + i % c];
+        o += d * c;
+    }
+}
+
 __global__ void __launch_bounds__(128) k_subset_table(uint32_t *__restrict__ tab)
 {
     constexpr uint32_t W = kXMaxLabels + 1;
@@ -130,6 +150,7 @@ __device__ __forceinline__ uint64_t now_ns()
 // on a counter in device memory), or one block with a query of its own. The
 // counter wait is bounded by time and by iterations; when it gives up it sets
 // the error flag, and the blocks return.
+constexpr uint32_t kLeftOne = 1u << 18;  // barrier counts stay below: 152 blocks, under 100 barriers a query
 struct View {
     uint32_t b, n;  // this block among n
     uint32_t *ctr, *err;
@@ -143,28 +164,36 @@ struct View {
     }
     // In two halves, for what may go on until the other blocks' part is needed:
     // arrive() publishes the block's writes, wait() returns once every block has
-    // arrived.
-    __device__ void arrive()
+    // arrived. The counter's upper bits count the queries that blocks left over.
+    __device__ void arrive(uint32_t left = 0)
     {
         target += n;
         __syncthreads();
         if (threadIdx.x == 0) {
             __threadfence();
-            atomicAdd(ctr, 1u);
+            atomicAdd(ctr, 1u + left * kLeftOne);
         }
     }
     __device__ bool wait()
     {
+        uint32_t left;
+        return wait(left);
+    }
+    __device__ bool wait(uint32_t &left)
+    {
         __shared__ int ok;
+        __shared__ uint32_t left_;
         __syncthreads();
         if (threadIdx.x == 0) {
             int good = 0;
+            uint32_t seen = 0;
             uint64_t t0 = 0;
             for (uint32_t it = 0; it < 200000000u; ++it) {
                 uint32_t v;
                 asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(ctr) : "memory");
-                if ((int32_t)(v - target) >= 0) {
+                if ((v & (kLeftOne - 1u)) >= target) {
                     good = 1;
+                    seen = v;
                     break;
                 }
                 if ((it & 1023u) != 1023u) continue;
@@ -174,8 +203,10 @@ struct View {
             if (!good) *(volatile uint32_t *)err = 1u;
             __threadfence();
             ok = good;
+            left_ = seen / kLeftOne;
         }
         __syncthreads();
+        left = left_;
         return ok != 0;
     }
     __device__ bool sync()
@@ -305,25 +336,34 @@ __device__ __forceinline__ uint64_t finish27(const uint32_t (&z)[27])
     return gf64_reduce(r[1] ^ (m >> 32), r[0] ^ (m << 32));
 }
 
+// One out-of-line multiply for the small queries' path: it runs each of its
+// products once or twice, and fetching 4 KB of instructions again for every
+// inlined copy took longer than the product (see x_tiny).
+__device__ __noinline__ uint64_t mul_call(uint64_t a, uint64_t b) { return gf64_mul(a, b); }
+
 // z'_{u,j}: the source's column eliminated (see the top of the file); a set of
 // sources keeps all k labels as they are.
+template <bool CALL = false>
 __device__ __forceinline__ uint64_t zprime(const XQuery &Q, const uint64_t *omega, const uint8_t *color, uint32_t u, uint32_t j)
 {
+    auto mul = [](uint64_t x, uint64_t y) { return CALL ? mul_call(x, y) : gf64_mul(x, y); };
     if (!Q.colored) {
         const uint64_t zj = sm_draw(Q.key_z, (uint64_t)u * 32u + (j < Q.pivot ? j : j + 1u));
-        return Q.multi ? zj : zj ^ gf64_mul(sm_draw(Q.key_z, (uint64_t)u * 32u + Q.pivot), Q.rho[j]);
+        return Q.multi ? zj : zj ^ mul(sm_draw(Q.key_z, (uint64_t)u * 32u + Q.pivot), Q.rho[j]);
     }
     const uint32_t c = color[u], d0 = Q.first[c], mu = Q.mu[c];
     uint64_t r = 0;
-    for (uint32_t d = d0; d < d0 + mu; ++d) r ^= gf64_mul(sm_draw(Q.key_g, (uint64_t)u * 32u + d), omega[d * Q.K + j]);
+    for (uint32_t d = d0; d < d0 + mu; ++d) r ^= mul(sm_draw(Q.key_g, (uint64_t)u * 32u + d), omega[d * Q.K + j]);
     return r;
 }
 // omega'_{d,j} at i = d K + j: the shade factor with the source's column eliminated
+template <bool CALL = false>
 __device__ __forceinline__ uint64_t shade_factor(const XQuery &Q, uint32_t i)
 {
+    auto mul = [](uint64_t x, uint64_t y) { return CALL ? mul_call(x, y) : gf64_mul(x, y); };
     const uint32_t d = i / Q.K, j = i - d * Q.K;
     const uint64_t oj = sm_draw(Q.key_o, (uint64_t)d * 32u + (j < Q.pivot ? j : j + 1u));
-    return Q.multi ? oj : oj ^ gf64_mul(sm_draw(Q.key_o, (uint64_t)d * 32u + Q.pivot), Q.rho[j]);
+    return Q.multi ? oj : oj ^ mul(sm_draw(Q.key_o, (uint64_t)d * 32u + Q.pivot), Q.rho[j]);
 }
 // A vertex walks may pass: it has a colour of M and is not deleted.
 __device__ __forceinline__ bool allowed(const XQuery &Q, const uint8_t *color, uint32_t v)
@@ -1056,14 +1096,19 @@ __device__ __noinline__ void x_outputs(const XArgs &a, const XOne &o, const View
 //  * a layer's products (row, subset, element) are spread over the threads and
 //    meet in shared memory, its window sums taken on the way: one block barrier
 //    a layer.
+//  * code that runs once is fetched once: one out-of-line multiply, no unrolled
+//    loops (inlined copies made the step with the multipliers 2.5 us, 1.1 so).
 // Uniform n = 1e5, m = 1e6, k = 8: 33.5 us with two loads, a window-sum step and
-// global tables a layer, 29.7 us so. Returns kTinyNoFit, with nothing written,
+// global tables a layer, 25.5 us so; 16 sources, k = 6, n = 20,011: 91 us over
+// the bitmaps (128 rows a level), 33 us here. A frontier that has kTinyGrow rows
+// and grows is given up with layers to go (it would not fit, and the bitmap
+// passes start that much later). Returns kTinyNoFit, with nothing written,
 // when the query does not fit. Witnesses are written only after every block has
 // cleared its part (clear: the barrier they arrived at).
 // ---------------------------------------------------------------------------
-constexpr uint32_t kTinyRows = 128, kTinyWords = kTinyRows / 32, kTinyTotal = 768, kTinyPairs = 1024, kTinyHash = 512;
+constexpr uint32_t kTinyRows = 256, kTinyWords = kTinyRows / 32, kTinyTotal = 1024, kTinyPairs = 1024, kTinyHash = 512;
+constexpr uint32_t kTinyGrow = 64;       // rows from which a growing frontier is given up early
 constexpr uint32_t kTinyRange = 1024;    // followers of one edge, at most
-constexpr uint32_t kTinyTable = 11264;   // subset-table words kept in shared memory (11 labels)
 enum { kTinyDone = 0, kTinyNoFit = 1, kTinyFailed = 2 };
 
 struct TinyMem {
@@ -1075,7 +1120,8 @@ struct TinyMem {
     uint32_t cn[kXMaxLevels + 2];           // needed rows before each level
     uint32_t hkey[2][kTinyHash], hval[kTinyHash];
     uint32_t pair[kTinyPairs];
-    uint32_t npair[2], count[2], over, need_g, need_d, toff[kXMaxLabels + 2];
+    uint32_t npair[2], count[2], over, need_g, need_d, toff[kXMaxLabels + 2], bin[kXMaxLabels + 2];
+    uint64_t warm;
     uint16_t list[kTinyTotal];              // needed rows
     uint8_t lev[kTinyTotal];                // and their levels
     uint64_t acc[kTinyTotal];               // their sums
@@ -1084,13 +1130,13 @@ struct TinyMem {
 
 // XOR of the level below's values s of the rows in `mk`, by their places among
 // its needed rows `nd`.
-__device__ __forceinline__ uint64_t tiny_window(const uint32_t *mk, const uint32_t *nd, const uint64_t *Gp, uint32_t cin,
-                                                uint32_t s)
+__device__ __forceinline__ uint64_t tiny_window(const uint32_t *mk, const uint32_t *nd, uint32_t words, const uint64_t *Gp,
+                                                uint32_t cin, uint32_t s)
 {
     uint64_t v = 0;
     uint32_t before = 0;
-#pragma unroll
-    for (uint32_t x = 0; x < kTinyWords; ++x) {
+#pragma unroll 1
+    for (uint32_t x = 0; x < words; ++x) {
         const uint32_t need = nd[x];
         for (uint32_t m = mk[x] & need; m; m &= m - 1)
             v ^= Gp[(before + __popc(need & ((m & (0u - m)) - 1u))) * cin + s];
@@ -1109,7 +1155,7 @@ __device__ __noinline__ int x_tiny(const XArgs &a, const XQuery &Q, bool every, 
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
     const uint32_t k = Q.k, K = Q.K, sh = Q.multi ? 1u : 0u, last = k - 1;
     // subset tables of the first K labels, where they are small
-    const bool tables = K * (1u << (K - 1u)) <= kTinyTable;
+    const bool tables = K <= kPackedLabels;
     uint32_t *const tab = reinterpret_cast<uint32_t *>(pool);
     if (tables) {
         const uint32_t w = K * (1u << (K - 1u));
@@ -1127,18 +1173,20 @@ __device__ __noinline__ int x_tiny(const XArgs &a, const XQuery &Q, bool every, 
     // subset tables and the shade factors
     if (warp >= kWarps / 2) {
         const uint32_t t = tid - kThreads / 2;
+        if (t == 0) M.warm = mul_call(Q.key_y, Q.d0);  // fetches the multiply's code
         if (tables) {
+            const uint32_t *const src = a.tab + kPackedTab + x_packed_off(K);
+#pragma unroll 4
+            for (uint32_t i = t; i < K << (K - 1u); i += kThreads / 2) tab[i] = __ldg(src + i);
+        }
+        if (t <= K) {  // C(K, t), and where the packed table of t-subsets starts
+            M.bin[t] = x_binom_dev(K, t);
             uint32_t off = 0;
-            for (uint32_t d = 1; d <= K; ++d) {
-                const uint32_t c = x_binom_dev(K, d), cm = x_binom_dev(kXMaxLabels, d), w = d * c;
-                const uint32_t *const src = a.tab + x_tab_off_dev(d);
-                if (t == 0) M.toff[d] = off;
-                for (uint32_t i = t; i < w; i += kThreads / 2) tab[off + i] = __ldg(src + i / c * cm + i % c);
-                off += w;
-            }
+            for (uint32_t d = 1; d < t; ++d) off += d * x_binom_dev(K, d);
+            M.toff[t] = off;
         }
         if (Q.colored)
-            for (uint32_t i = t; i < Q.k * K; i += kThreads / 2) M.omega[i] = shade_factor(Q, i);
+            for (uint32_t i = t; i < Q.k * K; i += kThreads / 2) M.omega[i] = shade_factor<true>(Q, i);
     } else if (!Q.dead) {
         const uint32_t ns = Q.multi ? Q.nslist : 1u;
         for (uint32_t i = warp; i < ns; i += kWarps / 2) {
@@ -1149,6 +1197,7 @@ __device__ __noinline__ int x_tiny(const XArgs &a, const XQuery &Q, bool every, 
                 if (lane == 0) M.over = 1;
                 continue;
             }
+#pragma unroll 1
             for (uint32_t o = o0 + lane; o < o1; o += 32u) {
                 const uint4 r = a.orec[o];  // head, time, edge, first follower
                 const uint32_t fl = a.olen[o];
@@ -1164,12 +1213,14 @@ __device__ __noinline__ int x_tiny(const XArgs &a, const XQuery &Q, bool every, 
     __syncthreads();
     uint32_t n = M.count[1], lmax = 1;
     const uint32_t n1 = n;
+    uint32_t prev = n;
     if (M.over || n > kTinyRows) return kTinyNoFit;
     if (tid == 0) M.base[2] = n;
     // forward; the hash table, counters and pairs of a level are cleared while
     // the one before it uses the other
     for (uint32_t l = 2; l <= last && n; ++l) {
         const uint32_t b1 = M.base[l - 1] + n, b0 = b1 - n, par = l & 1u;  // (base[l] is written by now or below)
+#pragma unroll 1
         for (uint32_t f = warp; f < n; f += kWarps) {
             const uint32_t v = M.row[b0 + f].y;
             const uint2 nx = M.next[b0 + f];
@@ -1177,6 +1228,7 @@ __device__ __noinline__ int x_tiny(const XArgs &a, const XQuery &Q, bool every, 
                 if (lane == 0) M.over = 1;
                 continue;
             }
+#pragma unroll 1
             for (uint32_t i = lane; i < nx.y; i += 32u) {
                 const uint32_t p = nx.x + i;
                 const uint4 r = a.orec[p];
@@ -1208,7 +1260,9 @@ __device__ __noinline__ int x_tiny(const XArgs &a, const XQuery &Q, bool every, 
         }
         __syncthreads();
         n = M.count[par];
-        if (M.over || n > kTinyRows || b1 + n > kTinyTotal) return kTinyNoFit;
+        if (M.over || n > kTinyRows || b1 + n > kTinyTotal || (n > kTinyGrow && n > prev + prev / 8u && l + 2u < last)) return kTinyNoFit;
+        prev = n;
+#pragma unroll 1
         for (uint32_t i = tid; i < M.npair[par]; i += kThreads) {
             const uint32_t f = M.pair[i] >> 16, e = M.hval[M.pair[i] & 0xffffu];
             atomicOr(&M.mask[b1 + e][f >> 5], 1u << (f & 31u));
@@ -1228,6 +1282,7 @@ __device__ __noinline__ int x_tiny(const XArgs &a, const XQuery &Q, bool every, 
 
     // backward, the row counts and the space the layers take: one warp
     if (warp == 0) {
+#pragma unroll 1
         for (uint32_t i = lane; i < (top + 1u) * kTinyWords; i += 32u) {
             const uint32_t l = i / kTinyWords;
             uint32_t all = 0;
@@ -1238,17 +1293,17 @@ __device__ __noinline__ int x_tiny(const XArgs &a, const XQuery &Q, bool every, 
             M.need[l][i % kTinyWords] = all;
         }
         __syncwarp();
+#pragma unroll 1
         for (uint32_t l = top; l >= 2 && !every; --l) {
-            const uint32_t b = M.base[l], c = M.base[l + 1] - b;
-            uint32_t m[kTinyWords] = {};
-            for (uint32_t e = lane; e < c; e += 32u)
-                if ((M.need[l][e >> 5] >> (e & 31u)) & 1u)
-#pragma unroll
-                    for (uint32_t x = 0; x < kTinyWords; ++x) m[x] |= M.mask[b + e][x];
-#pragma unroll
-            for (uint32_t x = 0; x < kTinyWords; ++x) {
-                const uint32_t o = __reduce_or_sync(0xffffffffu, m[x]);
-                if (lane == 0) M.need[l - 1][x] = o;
+            const uint32_t b = M.base[l], c = M.base[l + 1] - b, words = (b - M.base[l - 1] + 31u) / 32u;
+#pragma unroll 1
+            for (uint32_t x = 0; x < words; ++x) {
+                uint32_t m = 0;
+#pragma unroll 1
+                for (uint32_t e = lane; e < c; e += 32u)
+                    if ((M.need[l][e >> 5] >> (e & 31u)) & 1u) m |= M.mask[b + e][x];
+                m = __reduce_or_sync(0xffffffffu, m);
+                if (lane == 0) M.need[l - 1][x] = m;
             }
             __syncwarp();
         }
@@ -1265,8 +1320,8 @@ __device__ __noinline__ int x_tiny(const XArgs &a, const XQuery &Q, bool every, 
         if (lane >= 1 && lane <= top + 1u) M.cn[lane] = inc - c;
         const uint32_t d = lane - 1u + sh;
         const bool on = lane >= 1 && lane <= top;
-        const uint32_t g = __reduce_max_sync(0xffffffffu, on ? c * x_binom_dev(K, d) : 0u);
-        const uint32_t w = __reduce_max_sync(0xffffffffu, on && lane > 1 ? c * x_binom_dev(K, d - 1u) : 0u);
+        const uint32_t g = __reduce_max_sync(0xffffffffu, on ? c * M.bin[d] : 0u);
+        const uint32_t w = __reduce_max_sync(0xffffffffu, on && lane > 1 ? c * M.bin[d - 1u] : 0u);
         if (lane == 0) {
             M.need_g = g;
             M.need_d = w;
@@ -1280,10 +1335,12 @@ __device__ __noinline__ int x_tiny(const XArgs &a, const XQuery &Q, bool every, 
     // the needed rows by level
     for (uint32_t i = tid, rows = M.base[top + 1]; i < rows; i += kThreads) {
         uint32_t l = 1;
+#pragma unroll 1
         while (i >= M.base[l + 1]) ++l;
         const uint32_t e = i - M.base[l];
         if (!((M.need[l][e >> 5] >> (e & 31u)) & 1u)) continue;
         uint32_t at = M.cn[l] + __popc(M.need[l][e >> 5] & ((1u << (e & 31u)) - 1u));
+#pragma unroll 1
         for (uint32_t x = 0; x < (e >> 5); ++x) at += __popc(M.need[l][x]);
         M.list[at] = (uint16_t)i;
         M.lev[at] = (uint8_t)l;
@@ -1291,18 +1348,19 @@ __device__ __noinline__ int x_tiny(const XArgs &a, const XQuery &Q, bool every, 
     }
     for (uint32_t i = tid; i < need_g; i += kThreads) G[2][i] = 0;
     __syncthreads();
+#pragma unroll 1
     for (uint32_t i = tid; i < 2u * total * K; i += kThreads) {
         const bool second = i >= total * K;
         const uint32_t x = second ? i - total * K : i, at = x / K, j = x - at * K, l = M.lev[at];
         const uint4 r = M.row[M.list[at]];
         if (second) {
-            if (every || l == top) zw[x] = zprime(Q, M.omega, a.color, r.y, j);
+            if (every || l == top) zw[x] = zprime<true>(Q, M.omega, a.color, r.y, j);
         } else if (l > 1 || Q.multi) {
             const uint64_t y = sm_draw(Q.key_y, (uint64_t)r.w * 32u + (l - 1u));
-            mul[x] = gf64_mul(y, zprime(Q, M.omega, a.color, r.x, j));
+            mul[x] = mul_call(y, zprime<true>(Q, M.omega, a.color, r.x, j));
             if (l == 1) G[1][at * K + j] = mul[x];
         } else if (j == 0) {
-            G[1][at] = gf64_mul(sm_draw(Q.key_y, (uint64_t)r.w * 32u), Q.d0);
+            G[1][at] = mul_call(sm_draw(Q.key_y, (uint64_t)r.w * 32u), Q.d0);
         }
     }
     __syncthreads();
@@ -1310,45 +1368,50 @@ __device__ __noinline__ int x_tiny(const XArgs &a, const XQuery &Q, bool every, 
     for (uint32_t l = 2; l <= top + 1u; ++l) {
         uint64_t *const Gc = G[l % 3u], *const Gp = G[(l + 2u) % 3u], *const Gn = G[(l + 1u) % 3u];
         if (l <= top) {
-            const uint32_t c0 = M.cn[l], c = M.cn[l + 1] - c0, d = l - 1 + sh, cout = x_binom_dev(K, d), cin = x_binom_dev(K, d - 1);
+            const uint32_t c0 = M.cn[l], c = M.cn[l + 1] - c0, d = l - 1 + sh, cout = M.bin[d], cin = M.bin[d - 1];
             const uint64_t *const ml = mul + c0 * K;
             const uint32_t *const tb = tables ? tab + M.toff[d] : a.tab + x_tab_off_dev(d);
             const uint32_t cm = tables ? cout : x_binom_dev(kXMaxLabels, d);
             const uint32_t *const nd = M.need[l - 1];
+            const uint32_t words = (M.base[l] - M.base[l - 1] + 31u) / 32u;  // of the level below's masks
             if (c * cout * d <= 4u * kThreads) {
+#pragma unroll 1
                 for (uint32_t i = tid; i < c * cout * d; i += kThreads) {
                     const uint32_t q = i / (cout * d), r = i - q * cout * d, x = r / cout, T = r - x * cout;
                     const uint32_t e = tb[x * cm + T];
-                    const uint64_t w = tiny_window(M.mask[M.list[c0 + q]], nd, Gp, cin, e >> 8);
-                    xor_shared(&Gc[q * cout + T], gf64_mul(ml[q * K + (e & 255u)], w));
+                    const uint64_t w = tiny_window(M.mask[M.list[c0 + q]], nd, words, Gp, cin, e >> 8);
+                    xor_shared(&Gc[q * cout + T], mul_call(ml[q * K + (e & 255u)], w));
                 }
             } else {
+#pragma unroll 1
                 for (uint32_t i = tid; i < c * cin; i += kThreads) {
                     const uint32_t q = i / cin;
-                    dr[i] = tiny_window(M.mask[M.list[c0 + q]], nd, Gp, cin, i - q * cin);
+                    dr[i] = tiny_window(M.mask[M.list[c0 + q]], nd, words, Gp, cin, i - q * cin);
                 }
                 __syncthreads();
+#pragma unroll 1
                 for (uint32_t i = tid; i < c * cout; i += kThreads) {
                     const uint32_t q = i / cout, T = i - q * cout;
                     uint64_t v = 0;
                     for (uint32_t x = 0; x < d; ++x) {
                         const uint32_t e = tb[x * cm + T];
-                        v ^= gf64_mul(ml[q * K + (e & 255u)], dr[q * cin + (e >> 8)]);
+                        v ^= mul_call(ml[q * K + (e & 255u)], dr[q * cin + (e >> 8)]);
                     }
                     Gc[i] = v;
                 }
             }
             if (l < top) {  // the next level's products add up from zero (it was read two steps ago)
-                const uint32_t w = (M.cn[l + 2] - M.cn[l + 1]) * x_binom_dev(K, d + 1u);
+                const uint32_t w = (M.cn[l + 2] - M.cn[l + 1]) * M.bin[d + 1u];
                 for (uint32_t i = tid; i < w; i += kThreads) Gn[i] = 0;
             }
         }
         if (every ? !(Q.pivot > l - 1u && !Q.multi) : l == top + 1u) {
             // times z'_w over the first labels of k' = l
-            const uint32_t c0 = M.cn[l - 1], c = M.cn[l] - c0, K2 = l - 1u + sh, st = x_binom_dev(K, l - 2u + sh);
+            const uint32_t c0 = M.cn[l - 1], c = M.cn[l] - c0, K2 = l - 1u + sh, st = M.bin[l - 2u + sh];
+#pragma unroll 1
             for (uint32_t i = tid; i < c * K2; i += kThreads) {
                 const uint32_t q = i / K2, T = i - q * K2;
-                xor_shared(&M.acc[c0 + q], gf64_mul(Gp[q * st + T], zw[(c0 + q) * K + (K2 - 1u - T)]));
+                xor_shared(&M.acc[c0 + q], mul_call(Gp[q * st + T], zw[(c0 + q) * K + (K2 - 1u - T)]));
             }
         }
         __syncthreads();
@@ -1365,6 +1428,7 @@ __device__ __noinline__ int x_tiny(const XArgs &a, const XQuery &Q, bool every, 
         const size_t off = (size_t)(every ? l - 1u : 0u) * a.n + r.y;
         uint64_t sum = 0, same = 0;
         bool lead = true;
+#pragma unroll 1
         for (uint32_t x = c0; x < c1; ++x) {
             const uint4 o = M.row[M.list[x]];
             if (o.y != r.y) continue;
@@ -1445,6 +1509,21 @@ __device__ __forceinline__ void copy_words(void *dst, const void *src, uint32_t 
     for (uint32_t i = threadIdx.x; i < bytes / 4; i += blockDim.x)
         static_cast<uint32_t *>(dst)[i] = static_cast<const uint32_t *>(src)[i];
 }
+// From the parameter bank: it serves one address per warp at a time, so a warp
+// reads 32 words with the same index on all lanes and every lane keeps its own.
+__device__ __forceinline__ void copy_params(void *dst, const void *src, uint32_t bytes)
+{
+    const uint32_t lane = threadIdx.x & 31u;
+    for (uint32_t w = threadIdx.x & ~31u; w < bytes / 4; w += blockDim.x) {
+        uint32_t mine = 0;
+#pragma unroll
+        for (uint32_t i = 0; i < 32; ++i) {
+            const uint32_t x = w + i < bytes / 4 ? static_cast<const uint32_t *>(src)[w + i] : 0u;
+            if (lane == i) mine = x;
+        }
+        if (w + lane < bytes / 4) static_cast<uint32_t *>(dst)[w + lane] = mine;
+    }
+}
 
 // The description of one query, in shared memory (it is read all the time at
 // run-time indexes; indexed reads of the parameter bank took a microsecond a
@@ -1453,9 +1532,11 @@ template <bool BATCH>
 __device__ __forceinline__ void load_query(XOne &o, const XArgs &a, const XOne &one, uint32_t q, uint32_t lane)
 {
     __syncthreads();
-    copy_words(&o.q, BATCH ? a.xq + q : &one.q, sizeof(XQuery));
+    if (BATCH) copy_words(&o.q, a.xq + q, sizeof(XQuery));
+    else copy_params(&o.q, &one.q, sizeof(XQuery));
     __syncthreads();
-    copy_words(&o.t, BATCH ? a.xt + o.q.k : &one.t, sizeof(XTmpl));
+    if (BATCH) copy_words(&o.t, a.xt + o.q.k, sizeof(XTmpl));
+    else copy_params(&o.t, &one.t, sizeof(XTmpl));
     __syncthreads();
     relocate(o.t, a.scratch + lane * a.stride);
     __syncthreads();
@@ -1472,13 +1553,15 @@ k_frontier(const __grid_constant__ XArgs a_, const __grid_constant__ XOne one_, 
     __shared__ __align__(16) XArgs a;
     __shared__ __align__(16) XOne o;
     __shared__ uint32_t next;
-    copy_words(&a, &a_, sizeof(XArgs));
+    copy_params(&a, &a_, sizeof(XArgs));
     __syncthreads();
-    const uint32_t gt = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
     View grid{blockIdx.x, gridDim.x, a.ctl, a.err, 0u};
     bool ok = true;
-    if (plan) {
-        // cleared first: witnesses and bitmaps
+    // cleared first: witnesses and bitmaps (a single query's first block goes on
+    // with the query)
+    const uint32_t skip = !BATCH && a.tiny && gridDim.x > 1 ? 1u : 0u;
+    if (plan && blockIdx.x >= skip) {
+        const uint32_t gt = (blockIdx.x - skip) * blockDim.x + threadIdx.x, nt = (gridDim.x - skip) * blockDim.x;
         if ((reinterpret_cast<uint64_t>(a.szero) & 15u) == 0) {
             ulonglong2 *z = reinterpret_cast<ulonglong2 *>(a.szero);
             for (uint64_t i = gt; i < a.szero_n / 2; i += nt) z[i] = make_ulonglong2(0, 0);
@@ -1492,27 +1575,33 @@ k_frontier(const __grid_constant__ XArgs a_, const __grid_constant__ XOne one_, 
     if (plan && a.tiny) {
         grid.arrive();
         bool cleared = false;
-        for (;;) {
-            uint32_t q = blockIdx.x;  // one query: block 0's
-            if (BATCH) {
+        if (BATCH) {
+            while (ok) {
                 __syncthreads();
                 if (threadIdx.x == 0) next = atomicAdd(a.ctl + 2, 1u);
                 __syncthreads();
-                q = next;
+                const uint32_t q = next;
+                if (q >= a.nq) break;
+                copy_words(&o.q, a.xq + q, sizeof(XQuery));
+                __syncthreads();
+                const int r = x_tiny(a, o.q, false, grid, cleared);
+                ok = r != kTinyFailed;
+                if (r == kTinyNoFit && threadIdx.x == 0) a.left[atomicAdd(a.ctl + 3, 1u)] = q;
             }
-            if (q >= a.nq || !ok) break;
-            copy_words(&o.q, BATCH ? a.xq + q : &one_.q, sizeof(XQuery));
+            ok = ok && grid.sync();
+            if (ok) left = *(volatile uint32_t *)(a.ctl + 3);
+        } else if (blockIdx.x == 0) {
+            copy_params(&o.q, &one_.q, sizeof(XQuery));
             __syncthreads();
-            const int r = x_tiny(a, o.q, !BATCH && one_.t.every, grid, cleared);
-            if (r == kTinyFailed) ok = false;
-            if (r == kTinyNoFit && threadIdx.x == 0) {
-                const uint32_t at = atomicAdd(a.ctl + 3, 1u);
-                if (BATCH) a.left[at] = q;
-            }
-            if (!BATCH) break;
+            const int r = x_tiny(a, o.q, one_.t.every, grid, cleared);
+            ok = r != kTinyFailed;
+            left = r == kTinyNoFit ? 1u : 0u;
+            grid.arrive(left);  // done: the others leave, and so does this block
+            if (left) ok = grid.wait();
+        } else {
+            grid.arrive();
+            ok = grid.wait(left);
         }
-        ok = ok && grid.sync();
-        if (ok) left = *(volatile uint32_t *)(a.ctl + 3);
     }
     if (!BATCH && ok && left) load_query<BATCH>(o, a, one_, 0, 0);
     if (ok && left) {
@@ -1544,7 +1633,6 @@ k_frontier(const __grid_constant__ XArgs a_, const __grid_constant__ XOne one_, 
     // the last block to leave clears the counters for the next launch
     __syncthreads();
     if (threadIdx.x == 0) {
-        __threadfence();
         if (atomicAdd(a.ctl + 1, 1u) == gridDim.x - 1)
             for (int i = 0; i < 5; ++i) a.ctl[i] = 0;
     }
@@ -1632,7 +1720,7 @@ rr_status frontier_load(Graph &g, cudaStream_t st)
     g.x_smem_max = g.x_smem_max / 64 * 64;
     RR_CUDA(cudaFuncSetAttribute(k_frontier<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.x_smem_max));
     RR_CUDA(cudaFuncSetAttribute(k_frontier<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.x_smem_max));
-    RR_CUDA(g.x_tab.reserve((size_t)x_tab_off(kXMaxLabels + 1) * 4));
+    RR_CUDA(g.x_tab.reserve((size_t)(kPackedTab + x_packed_off(kPackedLabels + 1)) * 4));
     k_subset_table<<<dim3((x_binom(kXMaxLabels, kXMaxLabels / 2) + 127) / 128, kXMaxLabels), 128, 0, st>>>(g.x_tab.as<uint32_t>());
     RR_LAUNCHED();
     {
@@ -1646,6 +1734,8 @@ rr_status frontier_load(Graph &g, cudaStream_t st)
         RR_CUDA(cudaMemcpyToSymbolAsync(c_tab_off, off, sizeof off, 0, cudaMemcpyHostToDevice, st));
         RR_CUDA(cudaStreamSynchronize(st));
     }
+    k_packed_table<<<dim3(8, kPackedLabels), 128, 0, st>>>(g.x_tab.as<uint32_t>());
+    RR_LAUNCHED();
     struct {
         RowList *L, *prev;
         DevBuf *a, *b, *start;

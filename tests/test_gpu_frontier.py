@@ -1,6 +1,6 @@
 """GPU parity of the frontier engine at the edges of its two paths.
 
-A query whose walks are few runs in one block's shared memory (at most 128
+A query whose walks are few runs in one block's shared memory (at most 256
 rows a layer); any other goes through the bitmap passes, whose rows are kept as
 prefix sums in blocks with sums over 16 and 256 blocks. Both must equal the
 per-point engine (the dense-layout load flag) and the oracle bit for bit.
@@ -36,9 +36,10 @@ def _fan(width, tails=3, n_extra=5):
             "delta": np.full(n, 2, np.uint32), "color": (np.arange(n) % 2).astype(np.uint8)}
 
 
-@pytest.mark.parametrize("width,tails", [(1, 1), (31, 4), (42, 3), (43, 3), (127, 1), (128, 1), (129, 1), (64, 2), (65, 2)])
+@pytest.mark.parametrize("width,tails", [(1, 1), (31, 4), (42, 3), (43, 3), (127, 1), (128, 1), (129, 1), (64, 2), (65, 2),
+                                         (85, 3), (86, 3), (255, 1), (256, 1), (257, 1), (128, 2), (129, 2)])
 def test_rows_around_the_block_limit(width, tails):
-    # 127 / 128 / 129 rows at layer 1, 126 / 128 / 129 / 130 at layer 2
+    # 127 .. 257 rows at layer 1, 126 .. 258 at layer 2: word and limit edges
     g = _fan(width, tails)
     with capi.Graph(g) as G:
         for k in (2, 3, 4):
