@@ -51,11 +51,13 @@ constexpr uint32_t kMaxRows = 16;     // rows of one wedge item
 constexpr uint32_t kSplit = 36;       // words of a split multiplier: 9 pieces of 3 classes, each padded to 16 bytes
 constexpr uint32_t kSup1 = 16, kSup2 = 256, kSup3 = 4096;  // blocks per partial sum
 constexpr uint32_t kScanBlocks = 48, kScanSpan = 6, kScanLong = 1024;  // when a level's prefix sums are completed (x_scans)
-// Bitmap words per scan tile: one tile up to 8,192 words (a block scans them in
-// 8 steps), else at most 256 tiles of whole 1,024s.
+// Bitmap words per scan tile (a block takes four per thread at a time), and the
+// longest bitmap whose tiles count what lies before them themselves: 16 reads of
+// 16 bytes per thread at most, against a pass of its own and its barrier.
+constexpr uint32_t kTileWords = 2048, kDirectWords = 32768;
 __host__ __device__ constexpr uint32_t x_tile_words(uint32_t words)
 {
-    return words <= 8192u ? 8192u : ((words + 255u) / 256u + 1023u) / 1024u * 1024u;
+    return words <= kDirectWords ? kTileWords : ((words + 255u) / 256u + kTileWords - 1u) / kTileWords * kTileWords;
 }
 
 __host__ __device__ constexpr uint32_t x_binom(uint32_t n, uint32_t d)
@@ -154,7 +156,7 @@ constexpr uint32_t kLeftOne = 1u << 18;  // barrier counts stay below: 152 block
 struct View {
     uint32_t b, n;  // this block among n
     uint32_t *ctr, *err;
-    uint32_t target;
+    uint32_t target, told;  // told: the counter's upper bits at the last sync_or
     // worker w of n, the items before `base` dealt out: its first item from there on
     __device__ static uint32_t first_item(uint32_t base, uint32_t w, uint32_t n)
     {
@@ -217,6 +219,19 @@ struct View {
         }
         arrive();
         return wait();
+    }
+    // sync(), and whether any thread of any block came with `mine` (told by the
+    // counter itself: no flag to read after the barrier)
+    __device__ bool sync_or(bool mine, bool &any)
+    {
+        any = __syncthreads_or(mine);
+        if (n == 1) return true;
+        uint32_t left = 0;
+        arrive(any ? 1u : 0u);
+        const bool good = wait(left);
+        any = left != told;
+        told = left;
+        return good;
     }
 };
 
@@ -372,7 +387,11 @@ __device__ __forceinline__ bool allowed(const XQuery &Q, const uint8_t *color, u
     return !(Q.vmask && Q.vmask[v]);
 }
 
-// Forward and backward passes, ranks and row records of one query.
+// Forward and backward passes, ranks and row records of one query. Each pass is
+// short (10 MB of row windows and bitmaps on n = 1e6, m = 1e7), so the dependent
+// reads between two barriers bound it: a level's first windows are read before
+// the barrier they wait at, whether a level is alive comes with the barrier, the
+// warps take the steps of all level lists in one sequence.
 __device__ __noinline__ bool x_plan(const XArgs &a, const XOne &o, View &v)
 {
     const XQuery &Q = o.q;
@@ -382,11 +401,10 @@ __device__ __noinline__ bool x_plan(const XArgs &a, const XOne &o, View &v)
     const uint32_t gt = v.b * kThreads + threadIdx.x, nt = v.n * kThreads;
     constexpr uint32_t U = 2;  // bitmap words per warp and step
 
-    // cleared first: needed-row bitmaps, flags
+    // cleared first: needed-row bitmaps, counts
     for (uint32_t i = gt; i < t.clear4; i += nt) t.clear[i] = make_uint4(0, 0, 0, 0);
     if (v.b == 0)
         for (uint32_t i = threadIdx.x; i < t.nll; i += kThreads) {
-            t.live[i] = t.ll[i].level == 1 ? 1u : 0u;
             t.cnt[i] = 0;
             t.span[i] = 0;
         }
@@ -395,37 +413,50 @@ __device__ __noinline__ bool x_plan(const XArgs &a, const XOne &o, View &v)
         for (uint32_t i = threadIdx.x; i < Q.k * Q.K; i += kThreads) t.omega[i] = shade_factor(Q, i);
     const bool check = Q.colored || Q.vmask;
     uint32_t lmax = t.maxlev;
+    uint32_t nlo[U] = {}, nhi[U] = {};  // the next level's first windows
     for (uint32_t l = 1; l <= t.maxlev; ++l) {
+        bool live = false;
+        uint32_t base = 0;
         for (uint32_t li = t.runs[l].first; li < t.runs[l].first + t.runs[l].count; ++li) {
             const XLL &X = t.ll[li];
             const XList &L = a.lists[X.list];
-            const uint32_t steps = (L.words + U - 1) / U;
+            const uint32_t steps = (L.words + U - 1) / U, i0 = View::first_item(base, gw, nw);
             const uint32_t *const Ap = t.ll[X.prev].A;
-            if (l > 1 && !t.live[X.prev]) continue;
             const bool none = Q.dead || (X.out && Q.pivot > l && !Q.multi);  // z_s is zero over the labels of k' = l + 1
-            bool warp_live = false;
-            for (uint32_t i = gw; i < steps; i += nw) {
-                const uint32_t w0 = i * U;
-                bool act[U];
-                if (l == 1) {
-                    uint32_t u[U];
+            if (l == 1) {
+                // a stream of tails: eight words a step keep enough reads in flight
+                constexpr uint32_t U1 = 8;
+                const uint32_t steps1 = (L.words + U1 - 1) / U1;
+                for (uint32_t i = View::first_item(base, gw, nw); i < steps1; i += nw) {
+                    uint32_t u[U1];
 #pragma unroll
-                    for (uint32_t x = 0; x < U; ++x) {
-                        const uint32_t r = (w0 + x) * 32u + lane;
+                    for (uint32_t x = 0; x < U1; ++x) {
+                        const uint32_t r = (i * U1 + x) * 32u + lane;
                         u[x] = r < L.count ? L.src[r] : 0xffffffffu;
                     }
 #pragma unroll
-                    for (uint32_t x = 0; x < U; ++x) {
-                        act[x] = Q.multi ? u[x] != 0xffffffffu && Q.smask[u[x]] : u[x] == Q.source && u[x] != 0xffffffffu;
-                        if (act[x] && Q.vmask && Q.vmask[u[x]]) act[x] = false;
+                    for (uint32_t x = 0; x < U1; ++x) {
+                        bool on = u[x] != 0xffffffffu && !none && (Q.multi ? Q.smask[u[x]] != 0 : u[x] == Q.source);
+                        if (on && check) on = !(Q.vmask && Q.vmask[u[x]]) && allowed(Q, a.color, L.head[(i * U1 + x) * 32u + lane]);
+                        const uint32_t word = __ballot_sync(0xffffffffu, on);
+                        if (lane == x && i * U1 + x < L.words) X.A[i * U1 + x] = word;
+                        live |= word != 0;
                     }
-                } else {
+                }
+                base += steps1;
+                continue;
+            }
+            for (uint32_t i = i0; i < steps; i += nw) {
+                const uint32_t w0 = i * U;
+                bool act[U];
+                {
                     uint32_t lo[U], hi[U];
+                    const bool ready = base == 0 && i == gw;
 #pragma unroll
                     for (uint32_t x = 0; x < U; ++x) {
                         const uint32_t r = (w0 + x) * 32u + lane;
-                        lo[x] = r < L.count ? L.lo[r] : 0u;
-                        hi[x] = r < L.count ? L.hi[r] : 0u;
+                        lo[x] = ready ? nlo[x] : r < L.count ? L.lo[r] : 0u;
+                        hi[x] = ready ? nhi[x] : r < L.count ? L.hi[r] : 0u;
                     }
 #pragma unroll
                     for (uint32_t x = 0; x < U; ++x) act[x] = any_in(Ap, lo[x], hi[x]);
@@ -440,99 +471,109 @@ __device__ __noinline__ bool x_plan(const XArgs &a, const XOne &o, View &v)
                 for (uint32_t x = 0; x < U; ++x) {
                     const uint32_t word = __ballot_sync(0xffffffffu, act[x] && !none);
                     if (lane == x && w0 + x < L.words) X.A[w0 + x] = word;
-                    warp_live |= word != 0;
+                    live |= word != 0;
                 }
             }
-            // one write per block: one line written by every warp would queue in L2
-            const bool some = __syncthreads_or(warp_live);
-            if (some && threadIdx.x == 0 && l > 1) t.live[li] = 1u;
+            base += steps;
         }
-        if (!v.sync()) return false;
-        if (l == 1) continue;
-        bool some = false;
-        for (uint32_t li = t.runs[l].first; li < t.runs[l].first + t.runs[l].count; ++li) some |= t.live[li] != 0;
+        if (l < t.maxlev) {
+            const XList &L = a.lists[t.ll[t.runs[l + 1].first].list];
+#pragma unroll
+            for (uint32_t x = 0; x < U; ++x) {
+                const uint32_t r = (gw * U + x) * 32u + lane;
+                nlo[x] = r < L.count ? L.lo[r] : 0u;
+                nhi[x] = r < L.count ? L.hi[r] : 0u;
+            }
+        }
+        bool some;
+        if (!v.sync_or(live, some)) return false;
         if (!some) {
             lmax = l - 1;
             break;
         }
     }
+    // no walk as long as an output needs: every count stays zero
+    if (lmax == 0 || (!t.every && lmax < t.maxlev)) return v.sync();
 
     // backward: the rows of layer l - 1 in the window of a needed row of layer l
     // (at-most-k: every layer has outputs, every active row is needed)
     if (!t.every)
         for (uint32_t l = lmax; l >= 2; --l) {
-            for (uint32_t li = t.runs[l].first; li < t.runs[l].first + t.runs[l].count; ++li) {
-                const XLL &X = t.ll[li];
-                const XList &L = a.lists[X.list];
-                const uint32_t steps = (L.words + U - 1) / U;
-                if (!t.live[li]) continue;
-                const uint32_t *const Ap = t.ll[X.prev].A;
-                uint32_t *const Np = t.ll[X.prev].N;
-                for (uint32_t i = gw; i < steps; i += nw) {
-                    const uint32_t w0 = i * U;
-                    const uint32_t mine = lane < U && w0 + lane < L.words ? X.N[w0 + lane] : 0u;
-                    if (!__any_sync(0xffffffffu, mine != 0)) continue;
-                    uint32_t lo[U], hi[U];
+            const XLL &X = t.ll[t.runs[l].first];  // (one list a level)
+            const XList &L = a.lists[X.list];
+            const uint32_t steps = (L.words + U - 1) / U;
+            const uint32_t *const Ap = t.ll[X.prev].A;
+            uint32_t *const Np = t.ll[X.prev].N;
+            for (uint32_t i = gw; i < steps; i += nw) {
+                const uint32_t w0 = i * U;
+                const uint32_t mine = lane < U && w0 + lane < L.words ? X.N[w0 + lane] : 0u;
+                if (!__any_sync(0xffffffffu, mine != 0)) continue;
+                uint32_t lo[U], hi[U];
 #pragma unroll
-                    for (uint32_t x = 0; x < U; ++x) {
-                        const bool on = (__shfl_sync(0xffffffffu, mine, (int)x) >> lane) & 1u;
-                        const uint32_t r = (w0 + x) * 32u + lane;
-                        lo[x] = on ? L.lo[r] : 0u;
-                        hi[x] = on ? L.hi[r] : 0u;
+                for (uint32_t x = 0; x < U; ++x) {
+                    const bool on = (__shfl_sync(0xffffffffu, mine, (int)x) >> lane) & 1u;
+                    const uint32_t r = (w0 + x) * 32u + lane;
+                    lo[x] = on ? L.lo[r] : 0u;
+                    hi[x] = on ? L.hi[r] : 0u;
+                }
+                uint32_t m[U], have[U];  // the window's first words
+#pragma unroll
+                for (uint32_t x = 0; x < U; ++x) {
+                    m[x] = have[x] = 0;
+                    if (hi[x] > lo[x]) {
+                        m[x] = Ap[lo[x] >> 5] & (0xffffffffu << (lo[x] & 31u));
+                        have[x] = Np[lo[x] >> 5];
                     }
-                    uint32_t m[U], have[U];  // the window's first words
+                }
 #pragma unroll
-                    for (uint32_t x = 0; x < U; ++x) {
-                        m[x] = have[x] = 0;
-                        if (hi[x] > lo[x]) {
-                            m[x] = Ap[lo[x] >> 5] & (0xffffffffu << (lo[x] & 31u));
-                            have[x] = Np[lo[x] >> 5];
-                        }
-                    }
-#pragma unroll
-                    for (uint32_t x = 0; x < U; ++x) {
-                        if (hi[x] <= lo[x]) continue;
-                        const uint32_t b0 = lo[x] >> 5, b1 = (hi[x] - 1) >> 5;
-                        const uint32_t last = 0xffffffffu >> (31u - ((hi[x] - 1) & 31u));
-                        if (b1 == b0) m[x] &= last;
-                        if (m[x] & ~have[x]) atomicOr(Np + b0, m[x]);
-                        for (uint32_t w = b0 + 1; w <= b1; ++w) {
-                            const uint32_t mw = Ap[w] & (w == b1 ? last : 0xffffffffu);
-                            if (mw & ~Np[w]) atomicOr(Np + w, mw);
-                        }
+                for (uint32_t x = 0; x < U; ++x) {
+                    if (hi[x] <= lo[x]) continue;
+                    const uint32_t b0 = lo[x] >> 5, b1 = (hi[x] - 1) >> 5;
+                    const uint32_t last = 0xffffffffu >> (31u - ((hi[x] - 1) & 31u));
+                    if (b1 == b0) m[x] &= last;
+                    if (m[x] & ~have[x]) atomicOr(Np + b0, m[x]);
+                    for (uint32_t w = b0 + 1; w <= b1; ++w) {
+                        const uint32_t mw = Ap[w] & (w == b1 ? last : 0xffffffffu);
+                        if (mw & ~Np[w]) atomicOr(Np + w, mw);
                     }
                 }
             }
             if (!v.sync()) return false;
         }
 
-    // ranks: exclusive popcounts per bitmap word, and the levels' row counts.
-    // Long bitmaps are cut into tiles, whose sums come first.
+    // ranks: per bitmap word the rows before it, and the levels' row counts. A
+    // block takes a tile of kTileWords words; what lies before it, it counts
+    // itself in lists of at most kDirectWords words, else the tiles' sums come
+    // first.
     __shared__ uint32_t part[32];
     if (threadIdx.x < 32) part[threadIdx.x] = 0;
     __syncthreads();
-    bool tiled = false;
-    for (uint32_t l = 1; l <= lmax; ++l)
-        for (uint32_t li = t.runs[l].first; li < t.runs[l].first + t.runs[l].count; ++li)
-            tiled |= t.ll[li].words > x_tile_words(t.ll[li].words);
     const uint32_t nll = t.runs[lmax].first + t.runs[lmax].count;  // level lists up to lmax
+    bool tiled = false;
+    for (uint32_t li = 0; li < nll; ++li) tiled |= t.ll[li].words > kDirectWords;
     for (uint32_t pass = tiled ? 0u : 1u; pass < 2; ++pass) {
-        uint32_t base_item = 0;
+        uint32_t base = 0;
         for (uint32_t li = 0; li < nll; ++li) {
             const XLL &X = t.ll[li];
-            const uint32_t words = X.words;
-            const uint32_t tw = x_tile_words(words), tiles = (words + tw - 1) / tw;
-            if ((pass == 0 && tiles == 1) || !t.live[li]) continue;  // block-uniform
-            for (uint32_t i = View::first_item(base_item, v.b, v.n); i < tiles; i += v.n) {
+            const uint32_t words = X.words, tw = x_tile_words(words), tiles = (words + tw - 1) / tw;
+            const bool direct = words <= kDirectWords;
+            if (pass == 0 && direct) continue;
+            for (uint32_t i = View::first_item(base, v.b, v.n); i < tiles; i += v.n) {
                 const uint32_t end = min(words, (i + 1) * tw);
                 uint32_t sum = 0;
                 if (pass == 0) {
                     for (uint32_t w = i * tw + threadIdx.x; w < end; w += kThreads) sum += __popc(X.N[w]);
-                } else if (tiles > 1) {
-                    if (threadIdx.x < i) sum = X.tsum[threadIdx.x];  // rows before the tile
+                } else if (direct) {  // rows before the tile (tiles are whole 16-byte groups)
+                    const uint4 *const N4 = reinterpret_cast<const uint4 *>(X.N);
+                    for (uint32_t w = threadIdx.x; w < i * tw / 4u; w += kThreads) {
+                        const uint4 y = N4[w];
+                        sum += __popc(y.x) + __popc(y.y) + __popc(y.z) + __popc(y.w);
+                    }
+                } else if (threadIdx.x < i) {
+                    sum = X.tsum[threadIdx.x];
                 }
                 uint32_t run_base = 0;
-                if (tiles > 1) {
+                if (i || pass == 0) {
                     sum = __reduce_add_sync(0xffffffffu, sum);
                     __syncthreads();
                     if (lane == 0) part[warp] = sum;
@@ -579,26 +620,43 @@ __device__ __noinline__ bool x_plan(const XArgs &a, const XOne &o, View &v)
                     }
                 }
             }
-            base_item += tiles;
+            base += tiles;
         }
         if (!v.sync()) return false;
     }
 
     // the needed rows' windows, edges and tails, in list order, and how many rows
     // of the level below the windows hold together
+    uint32_t base = 0;
     for (uint32_t li = 0; li < nll; ++li) {
         const XLL &X = t.ll[li];
         const XList &L = a.lists[X.list];
-        const uint32_t steps = (L.words + U - 1) / U;
-        if (!t.live[li]) continue;
         const bool window = X.level > 1;
         const uint2 *const rank = X.rank, *const below = t.ll[X.prev].rank;
+        if (!window) {
+            // layer 1: few rows in long lists, a word per lane
+            const uint32_t steps1 = (L.words + 31u) / 32u;
+            for (uint32_t i = View::first_item(base, gw, nw); i < steps1; i += nw) {
+                const uint32_t w = i * 32u + lane;
+                const uint2 mine = w < L.words ? rank[w] : make_uint2(0, 0);
+                uint32_t at = mine.y;
+                for (uint32_t m = mine.x; m; m &= m - 1u, ++at) {
+                    const uint32_t r = w * 32u + (uint32_t)__ffs((int)m) - 1u;
+                    X.meta[at] = make_uint4(0, 0, L.eid[r], L.src[r]);
+                    if (X.mhead) X.mhead[at] = L.head[r];
+                    if (X.mtime) X.mtime[at] = L.time[r];
+                }
+            }
+            base += steps1;
+            continue;
+        }
+        const uint32_t steps = (L.words + U - 1) / U;
         uint64_t span = 0;
-        for (uint32_t i = gw; i < steps; i += nw) {
+        for (uint32_t i = View::first_item(base, gw, nw); i < steps; i += nw) {
             const uint32_t w0 = i * U;
             const uint2 mine = lane < U && w0 + lane < L.words ? rank[w0 + lane] : make_uint2(0, 0);
             if (!__any_sync(0xffffffffu, mine.x != 0)) continue;
-            uint32_t lo[U], hi[U], at[U];
+            uint32_t lo[U], hi[U], at[U], hd[U];
             uint4 m[U];
 #pragma unroll
             for (uint32_t x = 0; x < U; ++x) {
@@ -615,6 +673,7 @@ __device__ __noinline__ bool x_plan(const XArgs &a, const XOne &o, View &v)
                     }
                     m[x].z = L.eid[r];
                     m[x].w = L.src[r];
+                    if (X.mhead) hd[x] = L.head[r];
                 }
             }
 #pragma unroll
@@ -629,12 +688,12 @@ __device__ __noinline__ bool x_plan(const XArgs &a, const XOne &o, View &v)
 #pragma unroll
             for (uint32_t x = 0; x < U; ++x)
                 if (at[x] != 0xffffffffu) {
-                    const uint32_t r = (w0 + x) * 32u + lane;
                     X.meta[at[x]] = m[x];
-                    if (X.mhead) X.mhead[at[x]] = L.head[r];
-                    if (X.mtime) X.mtime[at[x]] = L.time[r];
+                    if (X.mhead) X.mhead[at[x]] = hd[x];
+                    if (X.mtime) X.mtime[at[x]] = L.time[(w0 + x) * 32u + lane];
                 }
         }
+        base += steps;
         if (window && __any_sync(0xffffffffu, span != 0)) {
 #pragma unroll
             for (int f = 16; f > 0; f >>= 1) span += __shfl_xor_sync(0xffffffffu, (unsigned long long)span, f);
@@ -1054,6 +1113,7 @@ __device__ __noinline__ void x_outputs(const XArgs &a, const XOne &o, const View
 {
     const XQuery &Q = o.q;
     const uint32_t gt = v.b * kThreads + threadIdx.x, nt = v.n * kThreads;
+    uint32_t base = 0;  // the threads take the rows of all levels in one sequence
     for (uint32_t li = 0; li < o.t.nll; ++li) {
         const XLL &X = o.t.ll[li];
         if (!X.Ec) continue;
@@ -1061,7 +1121,9 @@ __device__ __noinline__ void x_outputs(const XArgs &a, const XOne &o, const View
         // runs of equal head and time among the out rows (consecutive: the
         // rows keep the list's order)
         const uint32_t cnt = o.t.cnt[li];
-        for (uint32_t i = gt; i < cnt; i += nt) {
+        const uint32_t i0 = View::first_item(base, gt, nt);
+        base += cnt;
+        for (uint32_t i = i0; i < cnt; i += nt) {
             const uint32_t h = X.mhead[i], t = X.mtime[i];
             if (i && X.mhead[i - 1] == h && X.mtime[i - 1] == t) continue;
             uint64_t e = X.Ec[i];
@@ -1496,7 +1558,6 @@ __device__ __forceinline__ void relocate(XTmpl &t, uint8_t *base)
     }
     if (threadIdx.x == 0) {
         fix(t.clear);
-        fix(t.live);
         fix(t.cnt);
         fix(t.shape);
         fix(t.span);
@@ -1555,7 +1616,7 @@ k_frontier(const __grid_constant__ XArgs a_, const __grid_constant__ XOne one_, 
     __shared__ uint32_t next;
     copy_params(&a, &a_, sizeof(XArgs));
     __syncthreads();
-    View grid{blockIdx.x, gridDim.x, a.ctl, a.err, 0u};
+    View grid{blockIdx.x, gridDim.x, a.ctl, a.err, 0u, 0u};
     bool ok = true;
     // cleared first: witnesses and bitmaps (a single query's first block goes on
     // with the query)
@@ -1597,16 +1658,17 @@ k_frontier(const __grid_constant__ XArgs a_, const __grid_constant__ XOne one_, 
             ok = r != kTinyFailed;
             left = r == kTinyNoFit ? 1u : 0u;
             grid.arrive(left);  // done: the others leave, and so does this block
-            if (left) ok = grid.wait();
+            if (left) ok = grid.wait(grid.told);
         } else {
             grid.arrive();
             ok = grid.wait(left);
+            grid.told = left;
         }
     }
     if (!BATCH && ok && left) load_query<BATCH>(o, a, one_, 0, 0);
     if (ok && left) {
         if (BATCH && a.lanes > 1 && left >= gridDim.x / 4) {
-            View solo{0u, 1u, a.ctl, a.err, 0u};
+            View solo{0u, 1u, a.ctl, a.err, 0u, 0u};
             while (blockIdx.x < a.lanes) {
                 __syncthreads();
                 if (threadIdx.x == 0) next = atomicAdd(a.ctl + 4, 1u);
@@ -1874,7 +1936,6 @@ static uint64_t x_template(const XList *lists, uint32_t k, bool every, bool mult
         }
     }
     t.omega = b.take<uint64_t>((uint64_t)k * k);
-    t.live = b.take<uint32_t>(t.nll);
     t.cnt = b.take<uint32_t>(t.nll);
     t.shape = b.take<uint32_t>(t.nll);
     t.span = b.take<unsigned long long>(t.nll);

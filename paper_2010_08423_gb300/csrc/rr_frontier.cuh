@@ -70,7 +70,6 @@ struct XRun {
 struct XTmpl {
     uint32_t nll, maxlev, clear4, every;
     uint4 *clear;          // needed-row bitmaps to clear
-    uint32_t *live;        // per level list: some row is active
     uint32_t *cnt;         // per level list: needed rows
     uint32_t *shape;       // per level list: log2 warps per team | rows per item << 8 | scanned << 16
     unsigned long long *span;  // per store level: rows of it in the windows of the level above, together
