@@ -47,7 +47,7 @@ __host__ __device__ constexpr uint32_t team_threads(uint32_t t) { return t + 1 <
 __host__ __device__ constexpr uint32_t team_count(uint32_t t) { return (uint32_t)kThreads / team_threads(t); }
 // A team's share of the block's shared memory.
 __host__ __device__ constexpr uint32_t team_smem(uint32_t smem, uint32_t t) { return smem / team_count(t) / 16u * 16u; }
-constexpr uint32_t kMaxRows = 16;     // rows of one wedge item
+constexpr uint32_t kMaxRows = 16, kMaxOutRows = 32;  // rows of one item: store and out levels
 constexpr uint32_t kSplit = 36;       // words of a split multiplier: 9 pieces of 3 classes, each padded to 16 bytes
 constexpr uint32_t kSup1 = 16, kSup2 = 256, kSup3 = 4096;  // blocks per partial sum
 constexpr uint32_t kScanBlocks = 48, kScanSpan = 6, kScanLong = 1024;  // when a level's prefix sums are completed (x_scans)
@@ -287,14 +287,14 @@ struct XShape {
 __device__ __forceinline__ XShape x_shape_of(uint32_t s) { return XShape{s & 0xffu, (s >> 8) & 0xffu, s >> 16}; }
 __host__ __device__ __forceinline__ uint32_t x_item_bytes(uint32_t rows, uint32_t K, const XLL &X)
 {
-    return X.out ? rows * (K * 16u + 64u) : rows * (K * (4u * kSplit) + (X.cin + X.cout + X.uout) * 8u + 64u);
+    return X.out ? rows * (K * 8u + 8u + 64u) : rows * (K * (4u * kSplit) + (X.cin + X.cout + X.uout) * 8u + 64u);
 }
 // Quarter steps of one item.
 __device__ __forceinline__ uint32_t x_item_cost(uint32_t rows, uint32_t t, uint32_t K, const XLL &X)
 {
     const uint32_t T = team_threads(t), W = T / 32u;
     auto rounds = [&](uint32_t n) { return (n + T - 1u) / T; };
-    if (X.out) return 16u + 24u * rounds(rows * X.cout);
+    if (X.out) return 12u + 10u * rounds(rows * X.cout);
     const uint32_t per_warp = (rows + W - 1u) / W;
     uint32_t c = 16u + per_warp * (4u + X.cin / 64u) + rounds(rows * K) * 20u + rounds(rows * X.cout) * X.d * 4u +
                  rows * rounds(X.cout + X.uout);
@@ -306,8 +306,9 @@ __device__ __noinline__ uint32_t x_choose_shape(uint32_t smem, uint32_t blocks, 
 {
     const uint32_t lane = threadIdx.x & 31u;
     uint32_t best = 0xffffffffu, pick = 0;
-    for (uint32_t i = lane; i < kTeams * kMaxRows; i += 32u) {
-        const uint32_t t = i / kMaxRows, rows = i % kMaxRows + 1u;
+    const uint32_t most = X.out ? kMaxOutRows : kMaxRows;
+    for (uint32_t i = lane; i < kTeams * most; i += 32u) {
+        const uint32_t t = i / most, rows = i % most + 1u;
         if ((rows > 1u || t + 1u < kTeams) && x_item_bytes(rows, K, X) > team_smem(smem, t)) continue;
         const uint32_t items = (cnt + rows - 1u) / rows, teams = blocks * team_count(t);
         const uint32_t cost = (items + teams - 1u) / teams * x_item_cost(rows, t, K, X);
@@ -723,17 +724,51 @@ __device__ __forceinline__ void store_split(uint32_t *o, uint64_t v)
     }
 }
 
-// sum over the d elements j of subset T of m_j w_{T \ j} (m: split multipliers)
+// z += x y for one piece of the two operands: their three classes each
+struct Piece {
+    uint32_t c0, c1, c2;
+};
+__device__ __forceinline__ Piece piece_of(uint32_t v)
+{
+    return Piece{v & 0x9249u, v & 0x2492u, v & 0x4924u};
+}
+
+// sum over the d elements j of subset T of m_j w_{T \ j} (m: split multipliers).
+// Two products a round: their six class products and the accumulator meet in
+// three three-input XORs, 27 fewer a round than one product at a time (the ALU
+// pipe bounds the loop: 94 of its operations a product measured, 82 so; k = 12
+// from a hub of n = 2e5, m = 2e6 774 -> 733 us).
 __device__ __forceinline__ uint64_t wedge_at(const uint32_t *__restrict__ tb, uint32_t cm, uint32_t T, uint32_t d,
                                              const uint32_t *m, const uint64_t *w)
 {
     uint32_t z[27];
 #pragma unroll
     for (int i = 0; i < 27; ++i) z[i] = 0;
-    uint32_t e = __ldg(tb + T);
+    uint32_t e = __ldg(tb + T), i = 1;
 #pragma unroll 1
-    for (uint32_t i = 1; i <= d; ++i) {
-        const uint32_t next = i < d ? __ldg(tb + i * cm + T) : 0u;
+    for (; i < d; i += 2) {
+        const uint32_t f = __ldg(tb + i * cm + T), next = i + 1 < d ? __ldg(tb + (i + 1) * cm + T) : 0u;
+        const uint64_t v = w[e >> 8], u = w[f >> 8];
+        const uint4 *const mv = reinterpret_cast<const uint4 *>(m + (e & 255u) * kSplit);
+        const uint4 *const mu = reinterpret_cast<const uint4 *>(m + (f & 255u) * kSplit);
+#pragma unroll
+        for (int h = 0; h < 3; ++h) {
+            const uint32_t x = h == 0 ? (uint32_t)v : h == 1 ? (uint32_t)(v >> 32) : (uint32_t)v ^ (uint32_t)(v >> 32);
+            const uint32_t t = h == 0 ? (uint32_t)u : h == 1 ? (uint32_t)(u >> 32) : (uint32_t)u ^ (uint32_t)(u >> 32);
+            const uint32_t xh = x >> 16, th = t >> 16;
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                const Piece a = piece_of(j == 0 ? x : j == 1 ? xh : x ^ xh), b = piece_of(j == 0 ? t : j == 1 ? th : t ^ th);
+                const uint4 y = mv[3 * h + j], g = mu[3 * h + j];
+                uint32_t *const q = z + 9 * h + 3 * j;
+                q[0] = ((q[0] ^ (a.c0 * y.x) ^ (a.c1 * y.z)) ^ (a.c2 * y.y) ^ (b.c0 * g.x)) ^ (b.c1 * g.z) ^ (b.c2 * g.y);
+                q[1] = ((q[1] ^ (a.c0 * y.y) ^ (a.c1 * y.x)) ^ (a.c2 * y.z) ^ (b.c0 * g.y)) ^ (b.c1 * g.x) ^ (b.c2 * g.z);
+                q[2] = ((q[2] ^ (a.c0 * y.z) ^ (a.c1 * y.y)) ^ (a.c2 * y.x) ^ (b.c0 * g.z)) ^ (b.c1 * g.y) ^ (b.c2 * g.x);
+            }
+        }
+        e = next;
+    }
+    if (i == d) {  // the last of an odd number
         const uint64_t v = w[e >> 8];
         const uint4 *const mv = reinterpret_cast<const uint4 *>(m + (e & 255u) * kSplit);
 #pragma unroll
@@ -742,16 +777,14 @@ __device__ __forceinline__ uint64_t wedge_at(const uint32_t *__restrict__ tb, ui
             const uint32_t xh = x >> 16;
 #pragma unroll
             for (int j = 0; j < 3; ++j) {
-                const uint32_t piece = j == 0 ? x : j == 1 ? xh : x ^ xh;
-                const uint32_t x0 = piece & 0x9249u, x1 = piece & 0x2492u, x2 = piece & 0x4924u;
+                const Piece a = piece_of(j == 0 ? x : j == 1 ? xh : x ^ xh);
                 const uint4 y = mv[3 * h + j];
                 uint32_t *const q = z + 9 * h + 3 * j;
-                q[0] ^= (x0 * y.x) ^ (x1 * y.z) ^ (x2 * y.y);
-                q[1] ^= (x0 * y.y) ^ (x1 * y.x) ^ (x2 * y.z);
-                q[2] ^= (x0 * y.z) ^ (x1 * y.y) ^ (x2 * y.x);
+                q[0] ^= (a.c0 * y.x) ^ (a.c1 * y.z) ^ (a.c2 * y.y);
+                q[1] ^= (a.c0 * y.y) ^ (a.c1 * y.x) ^ (a.c2 * y.z);
+                q[2] ^= (a.c0 * y.z) ^ (a.c1 * y.y) ^ (a.c2 * y.x);
             }
         }
-        e = next;
     }
     return finish27(z);
 }
@@ -943,6 +976,7 @@ __device__ __noinline__ bool x_wedge(const XArgs &a, const XOne &o, View &v, uin
             uint64_t *const dr = sm + (size_t)rows * K * (kSplit / 2), *const G = dr + rows * cin, *const Us = G + rows * cout;
             uint4 *const smeta = reinterpret_cast<uint4 *>(sm + (tsmem / 8 - rows * 8u));
             uint32_t *const shead = reinterpret_cast<uint32_t *>(smeta + rows), *const srun = shead + rows;
+            uint32_t *const sfirst = srun + rows;  // (rows + 1)
             auto sync = [&] {
                 if (sh.team == 0) __syncwarp();
                 else if (sh.team + 1u == kTeams) __syncthreads();
@@ -954,17 +988,23 @@ __device__ __noinline__ bool x_wedge(const XArgs &a, const XOne &o, View &v, uin
             for (uint32_t it = View::first_item(base_item, gteam, nteam); it < nb; it += nteam) {
                 const uint32_t row0 = it * rows, nr = min(rows, cnt - row0);
                 sync();
-                // (at most 16 rows: the first half warp of the team)
+                // (at most 32 rows: the team's first warp)
                 if (tid < 32u) {
                     uint32_t h = 0xffffffffu;
                     if (tid < nr) {
-                        smeta[tid] = X.meta[row0 + tid];
+                        uint4 mt = X.meta[row0 + tid];
                         if (X.mhead) shead[tid] = h = X.mhead[row0 + tid];
+                        smeta[tid] = mt;
                     }
-                    // the row's run of equal heads, by its first row
+                    // runs of equal heads: their first rows, and each row's run
                     const uint32_t up = __shfl_up_sync(0xffffffffu, h, 1);
-                    const uint32_t starts = __ballot_sync(0xffffffffu, tid == 0 || h != up);
-                    if (tid < nr) srun[tid] = 31u - __clz(starts & (0xffffffffu >> (31u - tid)));
+                    const uint32_t starts = __ballot_sync(0xffffffffu, tid < nr && (tid == 0 || h != up));
+                    const uint32_t run = __popc(starts & (0xffffffffu >> (31u - tid))) - 1u;
+                    if (tid < nr) {
+                        srun[tid] = run;
+                        if ((starts >> tid) & 1u) sfirst[run] = tid;
+                        if (tid == 0) sfirst[nr] = __popc(starts);
+                    }
                 }
                 sync();
                 if (!X.out) {
@@ -1003,9 +1043,9 @@ __device__ __noinline__ bool x_wedge(const XArgs &a, const XOne &o, View &v, uin
                     }
                     sync();
                     if (uout) {  // U on the d+1-subsets of the first d + 2 labels; z' once per run of heads
-                        for (uint32_t t = tid; t < nr * uout; t += tsize) {
-                            const uint32_t q = t / uout, j = t - q * uout;
-                            if (srun[q] == q) store_split(msp + (size_t)t * kSplit, zprime(Q, t_.omega, a.color, shead[q], j));
+                        for (uint32_t t = tid, n = sfirst[nr] * uout; t < n; t += tsize) {
+                            const uint32_t r = t / uout, j = t - r * uout;
+                            store_split(msp + (size_t)t * kSplit, zprime(Q, t_.omega, a.color, shead[sfirst[r]], j));
                         }
                         sync();
                         const uint32_t *const tb = a.tab + x_tab_off_dev(d + 1u);
@@ -1039,28 +1079,30 @@ __device__ __noinline__ bool x_wedge(const XArgs &a, const XOne &o, View &v, uin
                 } else {
                     // z'_w of the runs' heads, and the sums of the rows
                     uint64_t *const zw = sm, *const sum = sm + rows * K;
-                    for (uint32_t t = tid; t < nr * K; t += tsize) {
-                        const uint32_t q = t / K;
-                        if (srun[q] == q) zw[t] = zprime(Q, t_.omega, a.color, shead[q], t - q * K);
+                    for (uint32_t t = tid, n = sfirst[nr] * K; t < n; t += tsize) {
+                        const uint32_t r = t / K;
+                        zw[t] = zprime(Q, t_.omega, a.color, shead[sfirst[r]], t - r * K);
                     }
                     for (uint32_t q = tid; q < nr; q += tsize) sum[q] = 0;
+                    auto value = [&](uint32_t t) -> uint64_t {  // U of (row, subset) t
+                        const uint32_t q = t / K, T = t - q * K;
+                        if (l == 1)  // the source's z row itself
+                            return Q.multi ? zprime(Q, t_.omega, a.color, smeta[q].w, T) : Q.d0;
+                        const XEnds e = x_ends(B, smeta[q].x, smeta[q].y);
+                        if (B.scan) return x_scanned(B, e, T);
+                        uint64_t u = (e.p0 ? e.p0[T] : 0ull) ^ (e.p1 ? e.p1[T] : 0ull);
+                        for (uint32_t i = e.b0; i < e.b1;) u ^= x_piece(B, i, e.b1)[T];
+                        return u;
+                    };
+                    // the next value is read while this one is multiplied
+                    uint64_t u = tid < nr * K ? value(tid) : 0ull;
                     sync();
                     for (uint32_t t = tid; t < nr * K; t += tsize) {
                         const uint32_t q = t / K, T = t - q * K;
-                        uint64_t u;
-                        if (l == 1) {  // the source's z row itself
-                            u = Q.multi ? zprime(Q, t_.omega, a.color, smeta[q].w, T) : Q.d0;
-                        } else {
-                            const XEnds e = x_ends(B, smeta[q].x, smeta[q].y);
-                            if (B.scan) {
-                                u = x_scanned(B, e, T);
-                            } else {
-                                u = (e.p0 ? e.p0[T] : 0ull) ^ (e.p1 ? e.p1[T] : 0ull);
-                                for (uint32_t i = e.b0; i < e.b1;) u ^= x_piece(B, i, e.b1)[T];
-                            }
-                        }
+                        const uint64_t next = t + tsize < nr * K ? value(t + tsize) : 0ull;
                         // T misses one label, whose z' it meets
                         xor_shared(sum + q, gf64_mul(u, zw[srun[q] * K + (K - 1u - T)]));
+                        u = next;
                     }
                     sync();
                     if (tid < 32u) {
@@ -1072,13 +1114,13 @@ __device__ __noinline__ bool x_wedge(const XArgs &a, const XOne &o, View &v, uin
                             if (X.Ec) X.Ec[row0 + tid] = x;
                         }
                         // runs of equal heads: one atomic, by the run's last row
-                        const uint32_t first = tid < nr ? srun[tid] : tid;
+                        const uint32_t first = tid < nr ? sfirst[srun[tid]] : tid;
 #pragma unroll
-                        for (int f = 1; f < 16; f <<= 1) {
+                        for (int f = 1; f < 32; f <<= 1) {
                             const uint64_t y = __shfl_up_sync(0xffffffffu, (unsigned long long)x, f);
                             if (tid >= first + f) x ^= y;
                         }
-                        if (tid < nr && x && (tid + 1u == nr || srun[tid + 1u] != first))
+                        if (tid < nr && x && (tid + 1u == nr || srun[tid + 1u] != srun[tid]))
                             atomicXor(reinterpret_cast<unsigned long long *>(S + shead[tid]), (unsigned long long)x);
                     }
                 }
