@@ -10,6 +10,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 
 import numpy as np
 
@@ -28,6 +29,9 @@ FLAG_ATMOST_LANES = 64
 FLAG_ATMOST_BRANCHES = 128
 FLAG_K4_PER_POINT = 256
 FLAG_K5_CLOSED = 512
+
+
+M64 = (1 << 64) - 1
 
 
 class RRError(RuntimeError):
@@ -246,14 +250,28 @@ def rr_reach_device_noalloc(g, source, k, seed, d_witness, d_bitmap=None, stream
     del keep
 
 
+_pack_query = struct.Struct("=IIQQ").pack  # rr_query: source, k, seed, motif
+
+
 def _query_array(queries):
-    arr = (rr_query * len(queries))()
-    keep = []
-    for i, qd in enumerate(queries):
-        q, m = make_query(qd["source"], qd["k"], qd["seed"], qd.get("motif"))
-        arr[i] = q
-        keep.append(m)
-    return arr, keep
+    """Returns (rr_query[len(queries)], keepalive) of a list of query dicts: the
+    motifs in one buffer, the structs packed in one pass."""
+    raws, size = [], 0
+    for qd in queries:
+        m = qd.get("motif")
+        if m is not None:
+            m = m.tobytes() if type(m) is np.ndarray and m.dtype == np.uint8 else np.asarray(m, dtype=np.uint8).tobytes()
+            size += len(m)
+        raws.append(m)
+    buf = ctypes.create_string_buffer(b"".join([m for m in raws if m is not None]), size + 1)
+    at = ctypes.addressof(buf)
+    out = []
+    for qd, m in zip(queries, raws):
+        out.append(_pack_query(int(qd["source"]) & 0xFFFFFFFF, int(qd["k"]) & 0xFFFFFFFF, int(qd["seed"]) & M64,
+                               0 if m is None else at))
+        if m is not None:
+            at += len(m)
+    return (rr_query * len(queries)).from_buffer_copy(b"".join(out)), buf
 
 
 def rr_reach_batch_device(g, queries, d_witness, d_bitmaps=None, d_status=None, stream=None):

@@ -47,27 +47,51 @@ __global__ void k_arrival_bitmap(uint32_t n, const uint32_t *__restrict__ R, uin
     }
 }
 
+// What an extraction has chosen so far (device): the vertex and time its next
+// step goes back from, the step's best candidate, and the path. fail: 1 the
+// target has no arrival, 2 a step found no candidate; later steps do nothing.
+struct ExtractState {
+    unsigned long long best;
+    uint32_t cur, tc, fail, done;
+    uint32_t vertices[32], edges[32], times[32];
+};
+
+// The target's minimum arrival time starts the path.
+__global__ void k_extract_begin(ExtractState *st, const uint32_t *__restrict__ R, uint32_t target, uint32_t k, uint8_t *vmask)
+{
+    st->best = ~0ull;
+    st->cur = target;
+    st->tc = R[target];
+    st->fail = st->tc == 0xFFFFFFFFu ? 1u : 0u;
+    st->done = 0;
+    st->vertices[k - 1] = target;
+    st->times[k - 2] = st->tc;
+    vmask[target] = 1;  // deleted from the next query on
+}
+
 // One extraction step (Sec. "Extracting an optimal solution using k queries").
-// Among the rows r of `cur`'s segment with time tc whose tail u is not
+// Among the rows r of cur's segment with time tc whose tail u is not
 // deleted, find the earliest time i inside r's restless window at which u's
 // (u, i) polynomial -- the XOR of E over u's rows at time i -- is non-zero;
 // best = min over such rows of (i << 32 | r). Rows of one (head, time) run are
-// in input-edge order, so the smallest r is the smallest edge index. With
-// `first` set, the candidates are instead the rows from `source` (the path's
-// first edge) and best = min r.
-__global__ void k_extract_step(uint32_t cur, uint32_t tc, const uint32_t *__restrict__ off,
+// in input-edge order, so the smallest r is the smallest edge index. At ell = 1
+// the candidates are instead the rows from `source` (the path's first edge) and
+// best = min r. The last block to finish records the choice, so that the next
+// query and step can be enqueued at once.
+__global__ void k_extract_step(ExtractState *st, uint32_t ell, const uint32_t *__restrict__ off,
                                const uint32_t *__restrict__ row_t, const uint32_t *__restrict__ row_src,
                                const uint32_t *__restrict__ row_lo, const uint32_t *__restrict__ row_hi,
                                const uint32_t *__restrict__ row_eid, const uint64_t *__restrict__ E,
-                               const uint8_t *__restrict__ vmask, uint32_t source, int first,
-                               unsigned long long *best)
+                               uint8_t *vmask, uint32_t source)
 {
+    if (st->fail) return;
+    const uint32_t cur = st->cur, tc = st->tc;
     const uint32_t r0 = off[cur], r1 = off[cur + 1];
     for (uint32_t r = r0 + blockIdx.x * blockDim.x + threadIdx.x; r < r1; r += gridDim.x * blockDim.x) {
         if (row_t[r] != tc) continue;
         const uint32_t u = row_src[r];
-        if (first) {
-            if (u == source) atomicMin(best, (unsigned long long)r);
+        if (ell == 1) {
+            if (u == source) atomicMin(&st->best, (unsigned long long)r);
             continue;
         }
         if (vmask[u]) continue;
@@ -78,11 +102,31 @@ __global__ void k_extract_step(uint32_t cur, uint32_t tc, const uint32_t *__rest
             uint64_t x = 0;
             for (; f < hi && row_t[f] == t; ++f) x ^= E[row_eid[f]];
             if (x) {
-                atomicMin(best, ((unsigned long long)t << 32) | r);
+                atomicMin(&st->best, ((unsigned long long)t << 32) | r);
                 break;
             }
         }
     }
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    __threadfence();
+    if (atomicAdd(&st->done, 1u) != gridDim.x - 1) return;
+    __threadfence();
+    const unsigned long long best = *(volatile unsigned long long *)&st->best;
+    st->done = 0;
+    st->best = ~0ull;
+    if (best == ~0ull) {
+        st->fail = 2;
+        return;
+    }
+    const uint32_t r = (uint32_t)best;
+    st->edges[ell - 1] = row_eid[r];
+    st->vertices[ell - 1] = ell == 1 ? source : row_src[r];
+    if (ell == 1) return;
+    st->times[ell - 2] = (uint32_t)(best >> 32);
+    st->cur = row_src[r];
+    st->tc = (uint32_t)(best >> 32);
+    vmask[row_src[r]] = 1;
 }
 
 unsigned grid_for(uint64_t count, unsigned block)
@@ -187,7 +231,11 @@ rr_status arrival_on(const Graph &g, Workspace &ws, const rr_query *q, uint64_t 
 // queries"): the fine-grained query for k vertices gives the target's minimum
 // arrival time; each further query, for one vertex fewer on the graph without
 // the chosen vertices (and, for motif queries, without their colours in M),
-// certifies the next vertex back. Synchronous on the graph's stream.
+// certifies the next vertex back. The choices stay on the device, so a plain
+// extraction is one sequence of launches with one wait at its end (k = 7 on
+// n = 20,011: 436 us with four waits a step, 240 us so); a motif query's next
+// motif needs the vertex on the host, one wait a step. Synchronous on the
+// graph's stream.
 rr_status extract_path(const Graph &g, const rr_query *q, uint32_t target, uint32_t *vertices,
                        uint32_t *edges, uint32_t *times)
 {
@@ -197,18 +245,15 @@ rr_status extract_path(const Graph &g, const rr_query *q, uint32_t target, uint3
     RR_CUDA(ws.S.reserve((size_t)g.n * 8));
     RR_CUDA(ws.arrival.reserve((size_t)g.n * 4));
     RR_CUDA(ws.vmask.reserve(g.n));
-    RR_CUDA(ws.pick.reserve(8));
+    RR_CUDA(ws.pick.reserve(sizeof(ExtractState)));
     RR_CUDA(ws.edges.reserve((size_t)std::max<uint64_t>(1, g.m) * 8));
     uint8_t *vm = ws.vmask.as<uint8_t>();
+    ExtractState *ds = ws.pick.as<ExtractState>(), hs;
     RR_CUDA(cudaMemsetAsync(vm, 0, g.n, st));
     std::vector<uint8_t> M;
     if (q->motif) M.assign(q->motif, q->motif + k);
     auto drop_colour = [&](uint32_t v) -> rr_status {
-        if (!q->motif) return RR_OK;
-        uint8_t c = 0;
-        RR_CUDA(cudaMemcpyAsync(&c, g.color.as<uint8_t>() + v, 1, cudaMemcpyDeviceToHost, st));
-        RR_CUDA(cudaStreamSynchronize(st));
-        auto it = std::find(M.begin(), M.end(), c);
+        auto it = std::find(M.begin(), M.end(), g.h_color[v]);
         if (it == M.end()) return fail(RR_ECUDA, "rr_extract_path: chosen vertex colour not in M");
         M.erase(it);
         return RR_OK;
@@ -218,60 +263,49 @@ rr_status extract_path(const Graph &g, const rr_query *q, uint32_t target, uint3
         return arrival_device(g, &qq, ws.S.as<uint64_t>(), ws.edges.as<uint64_t>(),
                               ws.arrival.as<uint32_t>(), nullptr, st, mask);
     };
-    auto pick = [&](uint32_t cur, uint32_t tc, int first, uint64_t *out) -> rr_status {
-        RR_CUDA(cudaMemsetAsync(ws.pick.p, 0xFF, 8, st));
-        k_extract_step<<<152, 256, 0, st>>>(cur, tc, g.off.as<uint32_t>(), g.row_t.as<uint32_t>(),
-                                            g.row_src.as<uint32_t>(), g.row_lo.as<uint32_t>(),
-                                            g.row_hi.as<uint32_t>(), g.row_eid.as<uint32_t>(),
-                                            ws.edges.as<uint64_t>(), vm, q->source, first,
-                                            ws.pick.as<unsigned long long>());
+    auto step = [&](uint32_t ell) -> rr_status {
+        k_extract_step<<<38, 256, 0, st>>>(ds, ell, g.off.as<uint32_t>(), g.row_t.as<uint32_t>(),
+                                           g.row_src.as<uint32_t>(), g.row_lo.as<uint32_t>(),
+                                           g.row_hi.as<uint32_t>(), g.row_eid.as<uint32_t>(),
+                                           ws.edges.as<uint64_t>(), vm, q->source);
         RR_LAUNCHED();
-        RR_CUDA(cudaMemcpyAsync(out, ws.pick.p, 8, cudaMemcpyDeviceToHost, st));
-        RR_CUDA(cudaStreamSynchronize(st));
         return RR_OK;
     };
-    auto row_field = [&](const DevBuf &b, uint32_t r, uint32_t *out) -> rr_status {
-        RR_CUDA(cudaMemcpyAsync(out, b.as<uint32_t>() + r, 4, cudaMemcpyDeviceToHost, st));
+    // the state so far, and what went wrong
+    auto look = [&]() -> rr_status {
+        RR_CUDA(cudaMemcpyAsync(&hs, ds, sizeof hs, cudaMemcpyDeviceToHost, st));
         RR_CUDA(cudaStreamSynchronize(st));
+        rr_status e = frontier_error(ws);
+        if (e != RR_OK) return e;
+        if (hs.fail == 1) return fail(RR_ENOPATH, "rr_extract_path: the target has no arrival");
+        if (hs.fail == 2)
+            return fail(RR_ENOPATH, "rr_extract_path: a step's polynomials vanished (probability <= (3k-1)/2^64)");
         return RR_OK;
     };
 
     // the target's minimum arrival time
     rr_status s = run(k, nullptr);
     if (s != RR_OK) return s;
-    uint32_t tc = 0;
-    RR_CUDA(cudaMemcpyAsync(&tc, ws.arrival.as<uint32_t>() + target, 4, cudaMemcpyDeviceToHost, st));
-    RR_CUDA(cudaStreamSynchronize(st));
-    if (tc == 0xFFFFFFFFu) return fail(RR_ENOPATH, "rr_extract_path: the target has no arrival");
+    k_extract_begin<<<1, 1, 0, st>>>(ds, ws.arrival.as<uint32_t>(), target, k, vm);
+    RR_LAUNCHED();
     uint32_t cur = target;
-    vertices[k - 1] = target;
-    times[k - 2] = tc;
     for (uint32_t ell = k - 1; ell >= 2; --ell) {
-        RR_CUDA(cudaMemsetAsync(vm + cur, 1, 1, st));  // delete the vertex chosen last
-        if ((s = drop_colour(cur)) != RR_OK) return s;
+        if (q->motif) {
+            if ((s = look()) != RR_OK) return s;
+            if (ell < k - 1) cur = hs.cur;
+            if ((s = drop_colour(cur)) != RR_OK) return s;
+        }
         if ((s = run(ell, vm)) != RR_OK) return s;
-        uint64_t best = 0;
-        if ((s = pick(cur, tc, 0, &best)) != RR_OK) return s;
-        if (best == ~0ull)
-            return fail(RR_ENOPATH, "rr_extract_path: a step's polynomials vanished (probability <= (3k-1)/2^64)");
-        const uint32_t r = (uint32_t)best, i = (uint32_t)(best >> 32);
-        uint32_t u = 0, e = 0;
-        if ((s = row_field(g.row_src, r, &u)) != RR_OK) return s;
-        if ((s = row_field(g.row_eid, r, &e)) != RR_OK) return s;
-        vertices[ell - 1] = u;
-        edges[ell - 1] = e;
-        times[ell - 2] = i;
-        cur = u;
-        tc = i;
+        if ((s = step(ell)) != RR_OK) return s;
     }
     // the first edge: from the source into vertices[1] at its chosen time
-    uint64_t best = 0;
-    if ((s = pick(cur, tc, 1, &best)) != RR_OK) return s;
-    if (best == ~0ull) return fail(RR_ECUDA, "rr_extract_path: no source edge at the chosen time");
-    uint32_t e0 = 0;
-    if ((s = row_field(g.row_eid, (uint32_t)best, &e0)) != RR_OK) return s;
-    vertices[0] = q->source;
-    edges[0] = e0;
+    if ((s = step(1)) != RR_OK) return s;
+    if ((s = look()) != RR_OK) return s;
+    for (uint32_t i = 0; i < k; ++i) vertices[i] = hs.vertices[i];
+    for (uint32_t i = 0; i + 1 < k; ++i) {
+        edges[i] = hs.edges[i];
+        times[i] = hs.times[i];
+    }
     return RR_OK;
 }
 

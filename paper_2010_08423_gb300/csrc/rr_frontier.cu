@@ -1576,6 +1576,65 @@ __device__ __noinline__ int x_tiny(const XArgs &a, const XQuery &Q, bool every, 
     return kTinyDone;
 }
 
+// Inverse (x != 0) by the extended Euclidean algorithm on binary polynomials.
+__host__ __device__ static uint64_t gf64_inverse(uint64_t x)
+{
+    unsigned __int128 u = x, v = ((unsigned __int128)1 << 64) | 0x1B, g1 = 1, g2 = 0;
+    auto deg = [](unsigned __int128 w) {
+        const uint64_t hi = (uint64_t)(w >> 64), lo = (uint64_t)w;
+#ifdef __CUDA_ARCH__
+        return hi ? 127 - __clzll((long long)hi) : (lo ? 63 - __clzll((long long)lo) : -1);
+#else
+        return hi ? 127 - __builtin_clzll(hi) : (lo ? 63 - __builtin_clzll(lo) : -1);
+#endif
+    };
+    while (u != 1) {
+        int j = deg(u) - deg(v);
+        if (j < 0) {
+            const unsigned __int128 tu = u, tg = g1;
+            u = v;
+            v = tu;
+            g1 = g2;
+            g2 = tg;
+            j = -j;
+        }
+        u ^= v << j;
+        g1 ^= g2 << j;
+    }
+    return (uint64_t)g1;
+}
+
+// A batch's queries come without what depends on the source's z row (x_query
+// forms it on the host for a single query: 0.7 us each, 180 us of a batch of 256
+// with the blocks waiting); a warp forms it beside the clearing.
+__device__ __noinline__ void x_constants(XQuery &Q, const uint8_t *color)
+{
+    const uint32_t lane = threadIdx.x & 31u, s = Q.source, k = Q.k;
+    uint64_t z = 0;
+    if (lane < k) {
+        if (!Q.colored) {
+            z = sm_draw(Q.key_z, (uint64_t)s * 32u + lane);
+        } else {
+            const uint32_t c = color[s];
+            for (uint32_t d = Q.first[c]; d < (uint32_t)Q.first[c] + Q.mu[c]; ++d)
+                z ^= gf64_mul(sm_draw(Q.key_g, (uint64_t)s * 32u + d), sm_draw(Q.key_o, (uint64_t)d * 32u + lane));
+        }
+    }
+    const uint32_t set = __ballot_sync(0xffffffffu, z != 0);
+    if (!set) {  // x_s is zero at every point
+        if (lane == 0) Q.dead = 1;
+        return;
+    }
+    const uint32_t p = (uint32_t)__ffs((int)set) - 1u;
+    const uint64_t d0 = __shfl_sync(0xffffffffu, (unsigned long long)z, (int)p);
+    const uint64_t rho = gf64_mul(z, gf64_inverse(d0));
+    if (lane < k && lane != p) Q.rho[lane - (lane > p ? 1u : 0u)] = rho;
+    if (lane == 0) {
+        Q.pivot = p;
+        Q.d0 = d0;
+    }
+}
+
 // The scratch pointers of a template, from offsets + 1 to addresses.
 __device__ __forceinline__ void relocate(XTmpl &t, uint8_t *base)
 {
@@ -1663,6 +1722,8 @@ k_frontier(const __grid_constant__ XArgs a_, const __grid_constant__ XOne one_, 
     // cleared first: witnesses and bitmaps (a single query's first block goes on
     // with the query)
     const uint32_t skip = !BATCH && a.tiny && gridDim.x > 1 ? 1u : 0u;
+    if (BATCH)
+        for (uint32_t q = blockIdx.x + (threadIdx.x >> 5) * gridDim.x; q < a.nq; q += kWarps * gridDim.x) x_constants(a.xq[q], a.color);
     if (plan && blockIdx.x >= skip) {
         const uint32_t gt = (blockIdx.x - skip) * blockDim.x + threadIdx.x, nt = (gridDim.x - skip) * blockDim.x;
         if ((reinterpret_cast<uint64_t>(a.szero) & 15u) == 0) {
@@ -1679,6 +1740,7 @@ k_frontier(const __grid_constant__ XArgs a_, const __grid_constant__ XOne one_, 
         grid.arrive();
         bool cleared = false;
         if (BATCH) {
+            ok = cleared = grid.wait();  // the queries' constants are any block's
             while (ok) {
                 __syncthreads();
                 if (threadIdx.x == 0) next = atomicAdd(a.ctl + 2, 1u);
@@ -1996,27 +2058,6 @@ static void x_args(const Graph &g, XArgs &a)
     a.smem = g.x_smem_max / 16u * 16u;
 }
 
-// gf64 inverse by the extended Euclidean algorithm on binary polynomials.
-static uint64_t gf64_inverse(uint64_t x)
-{
-    unsigned __int128 u = x, v = ((unsigned __int128)1 << 64) | 0x1B, g1 = 1, g2 = 0;
-    auto deg = [](unsigned __int128 w) {
-        const uint64_t hi = (uint64_t)(w >> 64), lo = (uint64_t)w;
-        return hi ? 127 - __builtin_clzll(hi) : (lo ? 63 - __builtin_clzll(lo) : -1);
-    };
-    while (u != 1) {
-        int j = deg(u) - deg(v);
-        if (j < 0) {
-            std::swap(u, v);
-            std::swap(g1, g2);
-            j = -j;
-        }
-        u ^= v << j;
-        g1 ^= g2 << j;
-    }
-    return (uint64_t)g1;
-}
-
 // Products with one factor: its 16 multiples by polynomials of degree < 4, and
 // the other factor four bits at a time.
 struct GfTimes {
@@ -2039,7 +2080,8 @@ struct GfTimes {
     }
 };
 
-static void x_query(const Graph &g, const rr_query &q, bool multi, XQuery &X)
+// constants: with what depends on the source's z row.
+static void x_query(const Graph &g, const rr_query &q, bool multi, bool constants, XQuery &X)
 {
     std::memset(&X, 0, sizeof X);
     const QueryKeys keys = make_keys(q.seed);
@@ -2053,6 +2095,7 @@ static void x_query(const Graph &g, const rr_query &q, bool multi, XQuery &X)
     X.key_g = keys.key_gamma;
     X.key_o = keys.key_omega;
     uint64_t zs[kXMaxLabels + 1];
+    constants = constants && !multi;
     if (multi) {
         X.multi = 1;
         X.K = X.pivot = k;
@@ -2064,7 +2107,7 @@ static void x_query(const Graph &g, const rr_query &q, bool multi, XQuery &X)
             X.first[c] = (uint8_t)sh.first[c];
             X.mu[c] = (uint8_t)sh.mu[c];
         }
-        if (multi) return;
+        if (!constants) return;
         const uint32_t c = g.h_color[s];
         for (uint32_t j = 0; j < k; ++j) {
             zs[j] = 0;
@@ -2072,7 +2115,7 @@ static void x_query(const Graph &g, const rr_query &q, bool multi, XQuery &X)
                 zs[j] ^= gf64_mul(sm_draw(X.key_g, (uint64_t)s * 32u + d), sm_draw(X.key_o, (uint64_t)d * 32u + j));
         }
     } else {
-        if (multi) return;
+        if (!constants) return;
         for (uint32_t j = 0; j < k; ++j) zs[j] = sm_draw(X.key_z, (uint64_t)s * 32u + j);
     }
     uint32_t p = 0;
@@ -2197,7 +2240,7 @@ rr_status frontier_query(const Graph &g, Workspace &ws, const rr_query *q, bool 
     if (s != RR_OK) return s;
     XOne one;
     x_template(a.lists, q->k, every, src != nullptr, d_R != nullptr, one.t);
-    x_query(g, *q, src != nullptr, one.q);
+    x_query(g, *q, src != nullptr, true, one.q);
     XQuery &Q = one.q;
     Q.S = d_witness;
     Q.E = d_E;
@@ -2261,7 +2304,7 @@ bool frontier_batch(const Graph &g, const rr_query *qs, uint32_t nq, const std::
         const size_t nb = (g.n + 7) / 8;
         for (uint32_t j = 0; j < count; ++j) {
             const uint32_t i = idx[j];
-            x_query(g, qs[i], false, hq[j]);
+            x_query(g, qs[i], false, false, hq[j]);
             hq[j].S = d_witness + (size_t)i * g.n;
             hq[j].bitmap = d_bitmaps ? d_bitmaps + (size_t)i * nb : nullptr;
         }
@@ -2269,7 +2312,7 @@ bool frontier_batch(const Graph &g, const rr_query *qs, uint32_t nq, const std::
         s = B.stage_done(st);
         if (s != RR_OK) return s;
         a.xt = B.xq.as<XTmpl>();
-        a.xq = reinterpret_cast<const XQuery *>(B.xq.as<uint8_t>() + tbytes);
+        a.xq = reinterpret_cast<XQuery *>(B.xq.as<uint8_t>() + tbytes);
         a.left = B.left.as<uint32_t>();
         a.nq = count;
         a.scratch = ws.state.as<uint8_t>();

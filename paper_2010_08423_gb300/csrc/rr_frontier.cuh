@@ -81,7 +81,7 @@ struct XTmpl {
 struct XArgs {
     XList lists[kXLists];
     uint32_t n, nq;
-    const XQuery *xq;      // batch form (device); null: the launch's own parameter block
+    XQuery *xq;            // batch form (device); null: the launch's own parameter block
     const XTmpl *xt;       // batch form: by k
     uint8_t *scratch;      // `lanes` regions of `stride` bytes
     uint64_t stride;

@@ -94,7 +94,7 @@ struct Workspace {
     DevBuf edges;   // m * 8: per-edge sums (fine-grained output) when the caller gives none
     DevBuf arrival; // n * 4: minimum arrival times (path extraction)
     DevBuf vmask;   // n: deleted vertices (path extraction)
-    DevBuf pick;    // 8: the extraction step's choice
+    DevBuf pick;    // the extraction's state
     DevBuf srcmask; // n: a set of sources (rr_reach_sources_device)
     DevBuf bS, bE, bR;  // at-most-k branches' witnesses (n), per-edge sums (m), arrivals (n)
     cudaStream_t capture = nullptr;           // stream used only to capture graphs
