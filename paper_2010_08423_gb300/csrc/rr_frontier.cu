@@ -48,7 +48,7 @@ __host__ __device__ constexpr uint32_t team_count(uint32_t t) { return (uint32_t
 // A team's share of the block's shared memory.
 __host__ __device__ constexpr uint32_t team_smem(uint32_t smem, uint32_t t) { return smem / team_count(t) / 16u * 16u; }
 constexpr uint32_t kMaxRows = 16, kMaxOutRows = 32;  // rows of one item: store and out levels
-constexpr uint32_t kSplit = 36;       // words of a split multiplier: 9 pieces of 3 classes, each padded to 16 bytes
+constexpr uint32_t kSplit = 28;       // words of a split multiplier: 9 pieces of 3 classes, padded to whole 16-byte loads
 constexpr uint32_t kSup1 = 16, kSup2 = 256, kSup3 = 4096;  // blocks per partial sum
 constexpr uint32_t kScanBlocks = 48, kScanSpan = 6, kScanLong = 1024;  // when a level's prefix sums are completed (x_scans)
 // Bitmap words per scan tile (a block takes four per thread at a time), and the
@@ -330,8 +330,9 @@ __device__ __noinline__ uint32_t x_choose_shape(uint32_t smem, uint32_t blocks, 
 // (two Karatsuba levels) of 3 bit classes; everything after the 81 integer
 // products of classes is linear, so a sum of products XORs them class by class
 // and is put together and reduced once. The multipliers of a row serve all its
-// subsets: their 27 words are formed once and read from shared memory, a piece
-// (three classes) at a time, so that a product holds few registers.
+// subsets: their 27 words are formed once and read from shared memory in seven
+// 16-byte loads (nine, a piece each, kept the shared-memory pipe as busy as the
+// ALU: at-most-k, k = 10, on n = 1e6, m = 1e7 4.82 -> 4.62 ms).
 // Per product this leaves 81 IMAD, about 41 three-input XORs and the 31
 // instructions that split the other operand, against 240 of gf64_mul.
 __device__ __forceinline__ uint64_t finish27(const uint32_t (&z)[27])
@@ -715,13 +716,21 @@ __device__ __noinline__ bool x_plan(const XArgs &a, const XOne &o, View &v)
 __device__ __forceinline__ void store_split(uint32_t *o, uint64_t v)
 {
     const uint32_t w[3] = {(uint32_t)v, (uint32_t)(v >> 32), (uint32_t)v ^ (uint32_t)(v >> 32)};
-    uint4 *q = reinterpret_cast<uint4 *>(o);
+    uint32_t p[28];
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
         const uint32_t x[3] = {w[i], w[i] >> 16, w[i] ^ (w[i] >> 16)};
 #pragma unroll
-        for (int j = 0; j < 3; ++j) q[3 * i + j] = make_uint4(x[j] & 0x9249u, x[j] & 0x2492u, x[j] & 0x4924u, 0u);
+        for (int j = 0; j < 3; ++j) {
+            p[9 * i + 3 * j] = x[j] & 0x9249u;
+            p[9 * i + 3 * j + 1] = x[j] & 0x2492u;
+            p[9 * i + 3 * j + 2] = x[j] & 0x4924u;
+        }
     }
+    p[27] = 0;
+    uint4 *q = reinterpret_cast<uint4 *>(o);
+#pragma unroll
+    for (int i = 0; i < 7; ++i) q[i] = make_uint4(p[4 * i], p[4 * i + 1], p[4 * i + 2], p[4 * i + 3]);
 }
 
 // z += x y for one piece of the two operands: their three classes each
@@ -731,6 +740,19 @@ struct Piece {
 __device__ __forceinline__ Piece piece_of(uint32_t v)
 {
     return Piece{v & 0x9249u, v & 0x2492u, v & 0x4924u};
+}
+
+__device__ __forceinline__ void load_split(const uint32_t *m, uint32_t (&y)[28])
+{
+    const uint4 *const q = reinterpret_cast<const uint4 *>(m);
+#pragma unroll
+    for (int i = 0; i < 7; ++i) {
+        const uint4 t = q[i];
+        y[4 * i] = t.x;
+        y[4 * i + 1] = t.y;
+        y[4 * i + 2] = t.z;
+        y[4 * i + 3] = t.w;
+    }
 }
 
 // sum over the d elements j of subset T of m_j w_{T \ j} (m: split multipliers).
@@ -749,8 +771,9 @@ __device__ __forceinline__ uint64_t wedge_at(const uint32_t *__restrict__ tb, ui
     for (; i < d; i += 2) {
         const uint32_t f = __ldg(tb + i * cm + T), next = i + 1 < d ? __ldg(tb + (i + 1) * cm + T) : 0u;
         const uint64_t v = w[e >> 8], u = w[f >> 8];
-        const uint4 *const mv = reinterpret_cast<const uint4 *>(m + (e & 255u) * kSplit);
-        const uint4 *const mu = reinterpret_cast<const uint4 *>(m + (f & 255u) * kSplit);
+        uint32_t y[28], g[28];
+        load_split(m + (e & 255u) * kSplit, y);
+        load_split(m + (f & 255u) * kSplit, g);
 #pragma unroll
         for (int h = 0; h < 3; ++h) {
             const uint32_t x = h == 0 ? (uint32_t)v : h == 1 ? (uint32_t)(v >> 32) : (uint32_t)v ^ (uint32_t)(v >> 32);
@@ -759,18 +782,20 @@ __device__ __forceinline__ uint64_t wedge_at(const uint32_t *__restrict__ tb, ui
 #pragma unroll
             for (int j = 0; j < 3; ++j) {
                 const Piece a = piece_of(j == 0 ? x : j == 1 ? xh : x ^ xh), b = piece_of(j == 0 ? t : j == 1 ? th : t ^ th);
-                const uint4 y = mv[3 * h + j], g = mu[3 * h + j];
+                const uint32_t y0 = y[9 * h + 3 * j], y1 = y[9 * h + 3 * j + 1], y2 = y[9 * h + 3 * j + 2];
+                const uint32_t g0 = g[9 * h + 3 * j], g1 = g[9 * h + 3 * j + 1], g2 = g[9 * h + 3 * j + 2];
                 uint32_t *const q = z + 9 * h + 3 * j;
-                q[0] = ((q[0] ^ (a.c0 * y.x) ^ (a.c1 * y.z)) ^ (a.c2 * y.y) ^ (b.c0 * g.x)) ^ (b.c1 * g.z) ^ (b.c2 * g.y);
-                q[1] = ((q[1] ^ (a.c0 * y.y) ^ (a.c1 * y.x)) ^ (a.c2 * y.z) ^ (b.c0 * g.y)) ^ (b.c1 * g.x) ^ (b.c2 * g.z);
-                q[2] = ((q[2] ^ (a.c0 * y.z) ^ (a.c1 * y.y)) ^ (a.c2 * y.x) ^ (b.c0 * g.z)) ^ (b.c1 * g.y) ^ (b.c2 * g.x);
+                q[0] = ((q[0] ^ (a.c0 * y0) ^ (a.c1 * y2)) ^ (a.c2 * y1) ^ (b.c0 * g0)) ^ (b.c1 * g2) ^ (b.c2 * g1);
+                q[1] = ((q[1] ^ (a.c0 * y1) ^ (a.c1 * y0)) ^ (a.c2 * y2) ^ (b.c0 * g1)) ^ (b.c1 * g0) ^ (b.c2 * g2);
+                q[2] = ((q[2] ^ (a.c0 * y2) ^ (a.c1 * y1)) ^ (a.c2 * y0) ^ (b.c0 * g2)) ^ (b.c1 * g1) ^ (b.c2 * g0);
             }
         }
         e = next;
     }
     if (i == d) {  // the last of an odd number
         const uint64_t v = w[e >> 8];
-        const uint4 *const mv = reinterpret_cast<const uint4 *>(m + (e & 255u) * kSplit);
+        uint32_t y[28];
+        load_split(m + (e & 255u) * kSplit, y);
 #pragma unroll
         for (int h = 0; h < 3; ++h) {
             const uint32_t x = h == 0 ? (uint32_t)v : h == 1 ? (uint32_t)(v >> 32) : (uint32_t)v ^ (uint32_t)(v >> 32);
@@ -778,11 +803,11 @@ __device__ __forceinline__ uint64_t wedge_at(const uint32_t *__restrict__ tb, ui
 #pragma unroll
             for (int j = 0; j < 3; ++j) {
                 const Piece a = piece_of(j == 0 ? x : j == 1 ? xh : x ^ xh);
-                const uint4 y = mv[3 * h + j];
+                const uint32_t y0 = y[9 * h + 3 * j], y1 = y[9 * h + 3 * j + 1], y2 = y[9 * h + 3 * j + 2];
                 uint32_t *const q = z + 9 * h + 3 * j;
-                q[0] ^= (a.c0 * y.x) ^ (a.c1 * y.z) ^ (a.c2 * y.y);
-                q[1] ^= (a.c0 * y.y) ^ (a.c1 * y.x) ^ (a.c2 * y.z);
-                q[2] ^= (a.c0 * y.z) ^ (a.c1 * y.y) ^ (a.c2 * y.x);
+                q[0] ^= (a.c0 * y0) ^ (a.c1 * y2) ^ (a.c2 * y1);
+                q[1] ^= (a.c0 * y1) ^ (a.c1 * y0) ^ (a.c2 * y2);
+                q[2] ^= (a.c0 * y2) ^ (a.c1 * y1) ^ (a.c2 * y0);
             }
         }
     }
