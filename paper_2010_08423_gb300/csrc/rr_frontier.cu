@@ -235,16 +235,10 @@ struct View {
     }
 };
 
-// Some active row at positions [lo, hi) of a bitmap.
-__device__ __forceinline__ bool any_in(const uint32_t *A, uint32_t lo, uint32_t hi)
+// Some bit in the words [w, w1) of a bitmap, four at a time (bitmaps start on
+// 256-byte boundaries).
+__device__ __forceinline__ bool any_words(const uint32_t *A, uint32_t w, uint32_t w1)
 {
-    if (hi <= lo) return false;
-    const uint32_t w0 = lo >> 5, w1 = (hi - 1) >> 5;
-    const uint32_t m0 = 0xffffffffu << (lo & 31u), m1 = 0xffffffffu >> (31u - ((hi - 1) & 31u));
-    if (w0 == w1) return (A[w0] & m0 & m1) != 0;
-    if ((A[w1] & m1) || (A[w0] & m0)) return true;
-    // the whole words between, four at a time (bitmaps start on 256-byte boundaries)
-    uint32_t w = w0 + 1;
     for (; w < w1 && (w & 3u); ++w)
         if (A[w]) return true;
     for (; w + 4u <= w1; w += 4u) {
@@ -448,26 +442,40 @@ __device__ __noinline__ bool x_plan(const XArgs &a, const XOne &o, View &v)
                 base += steps1;
                 continue;
             }
+            // first the rows' windows, then both end words of each, then what lies
+            // between
             for (uint32_t i = i0; i < steps; i += nw) {
+                const bool ready = base == 0 && i == gw;
                 const uint32_t w0 = i * U;
+                uint32_t lo[U], hi[U], fw[U], lw[U];
                 bool act[U];
-                {
-                    uint32_t lo[U], hi[U];
-                    const bool ready = base == 0 && i == gw;
 #pragma unroll
-                    for (uint32_t x = 0; x < U; ++x) {
-                        const uint32_t r = (w0 + x) * 32u + lane;
-                        lo[x] = ready ? nlo[x] : r < L.count ? L.lo[r] : 0u;
-                        hi[x] = ready ? nhi[x] : r < L.count ? L.hi[r] : 0u;
-                    }
+                for (uint32_t x = 0; x < U; ++x) {
+                    const uint32_t r = (w0 + x) * 32u + lane;
+                    lo[x] = ready ? nlo[x] : r < L.count ? L.lo[r] : 0u;
+                    hi[x] = ready ? nhi[x] : r < L.count ? L.hi[r] : 0u;
+                }
 #pragma unroll
-                    for (uint32_t x = 0; x < U; ++x) act[x] = any_in(Ap, lo[x], hi[x]);
+                for (uint32_t x = 0; x < U; ++x) {
+                    fw[x] = hi[x] > lo[x] ? Ap[lo[x] >> 5] : 0u;
+                    lw[x] = hi[x] > lo[x] ? Ap[(hi[x] - 1u) >> 5] : 0u;
+                }
+#pragma unroll
+                for (uint32_t x = 0; x < U; ++x) {
+                    const uint32_t m0 = 0xffffffffu << (lo[x] & 31u), m1 = 0xffffffffu >> (31u - ((hi[x] - 1u) & 31u));
+                    const uint32_t first = lo[x] >> 5, last = (hi[x] - 1u) >> 5;
+                    if (hi[x] <= lo[x]) act[x] = false;
+                    else if (first == last) act[x] = (fw[x] & m0 & m1) != 0;
+                    else act[x] = (fw[x] & m0) || (lw[x] & m1) || any_words(Ap, first + 1u, last);
                 }
                 if (check) {
+                    uint32_t h[U];
+#pragma unroll
+                    for (uint32_t x = 0; x < U; ++x) h[x] = act[x] ? L.head[(w0 + x) * 32u + lane] : 0u;
 #pragma unroll
                     for (uint32_t x = 0; x < U; ++x)
                         // walks through vertices without a colour of M, or deleted ones, are zero
-                        if (act[x] && !allowed(Q, a.color, L.head[(w0 + x) * 32u + lane])) act[x] = false;
+                        if (act[x] && !allowed(Q, a.color, h[x])) act[x] = false;
                 }
 #pragma unroll
                 for (uint32_t x = 0; x < U; ++x) {
