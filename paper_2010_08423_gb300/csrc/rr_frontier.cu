@@ -152,11 +152,24 @@ __device__ __forceinline__ uint64_t now_ns()
 // on a counter in device memory), or one block with a query of its own. The
 // counter wait is bounded by time and by iterations; when it gives up it sets
 // the error flag, and the blocks return.
-constexpr uint32_t kLeftOne = 1u << 18;  // barrier counts stay below: 152 blocks, under 100 barriers a query
+//
+// Two counters take turns, so that a block that is late to look at one barrier
+// does not see what others said at the next (nobody reaches the one after that
+// without it). A counter holds the arrivals there, plus 2^20 for each block that
+// came with something to tell, modulo 2^32: once all have arrived, what is above
+// the arrivals known to be there is what was told, also after the thousands of
+// barriers of a batch whose queries run one after another.
+constexpr uint32_t kTellOne = 1u << 20;  // above the blocks of a launch
+struct Meetings {
+    uint32_t count;    // so far
+    uint32_t told[2];  // at each counter
+    uint32_t result;   // of the last: 1 all came, 2 some told
+};
 struct View {
     uint32_t b, n;  // this block among n
-    uint32_t *ctr, *err;
-    uint32_t target, told;  // told: the counter's upper bits at the last sync_or
+    uint32_t *ctr, *err;  // ctr: two, 128 bytes apart
+    Meetings *meet;       // shared memory, kept by thread 0
+    bool some = false;    // some block came to the last barrier with something to tell
     // worker w of n, the items before `base` dealt out: its first item from there on
     __device__ static uint32_t first_item(uint32_t base, uint32_t w, uint32_t n)
     {
@@ -166,36 +179,29 @@ struct View {
     }
     // In two halves, for what may go on until the other blocks' part is needed:
     // arrive() publishes the block's writes, wait() returns once every block has
-    // arrived. The counter's upper bits count the queries that blocks left over.
-    __device__ void arrive(uint32_t left = 0)
+    // arrived.
+    __device__ void arrive(bool tell = false)
     {
-        target += n;
         __syncthreads();
         if (threadIdx.x == 0) {
+            const uint32_t turn = meet->count++ & 1u;
             __threadfence();
-            atomicAdd(ctr, 1u + left * kLeftOne);
+            atomicAdd(ctr + turn * 32u, tell ? kTellOne + 1u : 1u);
         }
     }
     __device__ bool wait()
     {
-        uint32_t left;
-        return wait(left);
-    }
-    __device__ bool wait(uint32_t &left)
-    {
-        __shared__ int ok;
-        __shared__ uint32_t left_;
         __syncthreads();
         if (threadIdx.x == 0) {
-            int good = 0;
-            uint32_t seen = 0;
+            const uint32_t s = meet->count - 1u, turn = s & 1u;
+            const uint32_t target = (s / 2u + 1u) * n;
+            uint32_t v = 0, good = 0;
             uint64_t t0 = 0;
             for (uint32_t it = 0; it < 200000000u; ++it) {
-                uint32_t v;
-                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(ctr) : "memory");
-                if ((v & (kLeftOne - 1u)) >= target) {
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(ctr + turn * 32u) : "memory");
+                v -= target;
+                if (!(v & (kTellOne - 1u))) {
                     good = 1;
-                    seen = v;
                     break;
                 }
                 if ((it & 1023u) != 1023u) continue;
@@ -204,12 +210,14 @@ struct View {
             }
             if (!good) *(volatile uint32_t *)err = 1u;
             __threadfence();
-            ok = good;
-            left_ = seen / kLeftOne;
+            v /= kTellOne;
+            meet->result = good | (v != meet->told[turn] ? 2u : 0u);
+            meet->told[turn] = v;
         }
         __syncthreads();
-        left = left_;
-        return ok != 0;
+        const uint32_t r = meet->result;
+        some = (r & 2u) != 0;
+        return (r & 1u) != 0;
     }
     __device__ bool sync()
     {
@@ -226,11 +234,9 @@ struct View {
     {
         any = __syncthreads_or(mine);
         if (n == 1) return true;
-        uint32_t left = 0;
-        arrive(any ? 1u : 0u);
-        const bool good = wait(left);
-        any = left != told;
-        told = left;
+        arrive(any);
+        const bool good = wait();
+        any = some;
         return good;
     }
 };
@@ -1748,9 +1754,11 @@ k_frontier(const __grid_constant__ XArgs a_, const __grid_constant__ XOne one_, 
     __shared__ __align__(16) XArgs a;
     __shared__ __align__(16) XOne o;
     __shared__ uint32_t next;
+    __shared__ Meetings meet;
     copy_params(&a, &a_, sizeof(XArgs));
     __syncthreads();
-    View grid{blockIdx.x, gridDim.x, a.ctl, a.err, 0u, 0u};
+    if (threadIdx.x == 0) meet = Meetings{};
+    View grid{blockIdx.x, gridDim.x, a.ctl, a.err, &meet};
     bool ok = true;
     // cleared first: witnesses and bitmaps (a single query's first block goes on
     // with the query)
@@ -1794,18 +1802,18 @@ k_frontier(const __grid_constant__ XArgs a_, const __grid_constant__ XOne one_, 
             const int r = x_tiny(a, o.q, one_.t.every, grid, cleared);
             ok = r != kTinyFailed;
             left = r == kTinyNoFit ? 1u : 0u;
-            grid.arrive(left);  // done: the others leave, and so does this block
-            if (left) ok = grid.wait(grid.told);
+            grid.arrive(left != 0);  // done: the others leave, and so does this block
+            if (left) ok = grid.wait();
         } else {
             grid.arrive();
-            ok = grid.wait(left);
-            grid.told = left;
+            ok = grid.wait();
+            left = grid.some ? 1u : 0u;
         }
     }
     if (!BATCH && ok && left) load_query<BATCH>(o, a, one_, 0, 0);
     if (ok && left) {
         if (BATCH && a.lanes > 1 && left >= gridDim.x / 4) {
-            View solo{0u, 1u, a.ctl, a.err, 0u, 0u};
+            View solo{0u, 1u, a.ctl, a.err, &meet};
             while (blockIdx.x < a.lanes) {
                 __syncthreads();
                 if (threadIdx.x == 0) next = atomicAdd(a.ctl + 4, 1u);
@@ -1832,8 +1840,10 @@ k_frontier(const __grid_constant__ XArgs a_, const __grid_constant__ XOne one_, 
     // the last block to leave clears the counters for the next launch
     __syncthreads();
     if (threadIdx.x == 0) {
-        if (atomicAdd(a.ctl + 1, 1u) == gridDim.x - 1)
+        if (atomicAdd(a.ctl + 1, 1u) == gridDim.x - 1) {
             for (int i = 0; i < 5; ++i) a.ctl[i] = 0;
+            a.ctl[32] = 0;
+        }
     }
 }
 

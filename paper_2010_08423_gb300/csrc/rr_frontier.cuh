@@ -90,7 +90,7 @@ struct XArgs {
     uint64_t szero_n;
     uint8_t *bzero;
     uint64_t bzero_n;
-    uint32_t *ctl;         // [0] barrier, [1] blocks done, [2] next query, [3] queries left, [4] next of them
+    uint32_t *ctl;         // [0], [32] barriers, [1] blocks done, [2] next query, [3] queries left, [4] next of them
     uint32_t *left;        // batch form: the queries left to the bitmap passes
     int32_t *status;       // batch form: per query, RR_ETIMEDOUT when a wait gave up
     uint32_t *err;         // set when a bounded wait gave up

@@ -126,3 +126,25 @@ def test_batches_whose_queries_fill_the_rows(nq):
             assert np.array_equal(w[i], w1) and np.array_equal(bm[i], b1), i
             if q["k"] <= 6:
                 assert np.array_equal(w1, oracle.sieve(g, q["source"], q["k"], q["seed"], motif=q["motif"])), i
+
+
+def test_long_queries_one_after_another():
+    # 37 queries of 14 to 16 vertices that no block's memory holds: a launch whose
+    # blocks meet some 2,000 times, 300,000 arrivals
+    import torch
+    g = W.uniform(300, 5_001, 40, 0, 8, 17, ncolors=2)
+    n = g["n"]
+    nq = 37
+    qs = [{"source": (7 * i) % n, "k": 14 + i % 3, "seed": 100 + i, "motif": None} for i in range(nq)]
+    with capi.Graph(g) as G:
+        d_w = torch.full((nq, n), -1, dtype=torch.int64, device="cuda")
+        d_b = torch.full((nq, (n + 7) // 8), 255, dtype=torch.uint8, device="cuda")
+        d_s = torch.full((nq,), -1, dtype=torch.int32, device="cuda")
+        capi.rr_reach_batch_device(G.handle, qs, d_w, d_b, d_s)
+        torch.cuda.synchronize()
+        assert not d_s.cpu().numpy().any()
+        w = d_w.cpu().numpy().view(np.uint64)
+        for i in range(0, nq, 6):
+            _, w1 = G.reach(qs[i]["source"], qs[i]["k"], qs[i]["seed"])
+            assert np.array_equal(w[i], w1), i
+        assert w.any()
