@@ -183,15 +183,17 @@ struct View {
     __device__ void arrive(bool tell = false)
     {
         __syncthreads();
+        arrived(tell);
+    }
+    __device__ void arrived(bool tell)
+    {
         if (threadIdx.x == 0) {
             const uint32_t turn = meet->count++ & 1u;
-            __threadfence();
-            atomicAdd(ctr + turn * 32u, tell ? kTellOne + 1u : 1u);
+            asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(ctr + turn * 32u), "r"(tell ? kTellOne + 1u : 1u) : "memory");
         }
     }
     __device__ bool wait()
     {
-        __syncthreads();
         if (threadIdx.x == 0) {
             const uint32_t s = meet->count - 1u, turn = s & 1u;
             const uint32_t target = (s / 2u + 1u) * n;
@@ -209,7 +211,6 @@ struct View {
                 if (*(volatile uint32_t *)err || now_ns() - t0 > 10000000000ull) break;
             }
             if (!good) *(volatile uint32_t *)err = 1u;
-            __threadfence();
             v /= kTellOne;
             meet->result = good | (v != meet->told[turn] ? 2u : 0u);
             meet->told[turn] = v;
@@ -234,7 +235,7 @@ struct View {
     {
         any = __syncthreads_or(mine);
         if (n == 1) return true;
-        arrive(any);
+        arrived(any);
         const bool good = wait();
         any = some;
         return good;
