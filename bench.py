@@ -1,8 +1,8 @@
 #!/usr/bin/env python3
 """Benchmark: restless-reachability sieve queries on a resident temporal graph.
 
-Headline workload (one step = one complete query: z-table, every layer over
-all 2^k sieve points, fused per-vertex reduce, reach bitmap):
+Headline workload (one step = one complete query: the rows walks pass, every
+layer of their values, fused per-vertex reduce, reach bitmap):
   Chung-Lu power-law temporal multigraph (degree exponent 2.5), n = 1,000,000,
   m = 10,000,000, timestamps in [1, 10000] drawn as Poisson(50) bursts of width
   20, delta(v) ~ U{5..50}, 8 vertex colours; k-RestlessMotifReach with k = 10
@@ -13,13 +13,14 @@ all 2^k sieve points, fused per-vertex reduce, reach bitmap):
 Metric: GF(2^64) edge-updates/s counted as the nominal 2^k * k * m per query.
 `value` is device-timed (CUDA events on the launching stream, L2 flushed
 between steps, graph resident in HBM); `work` states what one query performs
-(GF(2^64) multiplications and stored state values, from the per-kernel counts)
+(GF(2^64) multiplications, counted here from the rows that its walks pass)
 beside the nominal count, and `value_performed` the performed multiplications
 per second; `e2e` is the same metric through the host-buffer C-ABI call
 rr_reach_sync (descriptor uploaded and results copied back into pinned host
 buffers every step). `roofline` reports the dominant kernel against the
 measured copy bandwidth or the measured GF(2^64) multiply rate, whichever
-binds. Extra lines: the uniform k = 8 query, the dense per-point engine on the
+binds (one rank: the query's one kernel; sharded, --dense and --shape runs: the
+per-point engine's kernels). Extra lines: the uniform k = 8 query, the dense per-point engine on the
 headline query, the small n = 1,000 graph with the full oracle, batched,
 served (with the same query list one at a time), at-most-k / bounded and
 fine-grained queries, and serving on an n = 1e7 graph.
@@ -110,7 +111,8 @@ def cpu_model() -> str:
 
 # the sources whose change invalidates a recorded ncu capture of the query
 # kernels (their code, the device arithmetic and the row lists they read)
-KERNEL_SOURCES = ("rr_device.cuh", "rr_v2_device.cuh", "rr_sieve2.cu", "rr_graph.cu", "rr_internal.h")
+KERNEL_SOURCES = ("rr_device.cuh", "rr_v2_device.cuh", "rr_sieve2.cu", "rr_frontier.cu", "rr_frontier.cuh", "rr_graph.cu",
+                  "rr_internal.h")
 
 
 def code_tokens(text: str) -> str:
@@ -281,6 +283,116 @@ def kernel_rooflines_dense(info, k, chunk, ppl, m, n, kt, queries, hbm_peak, mul
     return out
 
 
+def frontier_rows(g, s, k, motif=None):
+    """The edges that k-vertex walks from s use as their l-th edge, l = 1..k-1:
+    edge indices per layer, in (head, time) order. An edge (u, v, t) may follow
+    an edge into u no more than delta(u) before t."""
+    src, dst, t = (np.asarray(g[x], dtype=np.int64) for x in ("src", "dst", "t"))
+    delta = np.asarray(g["delta"], dtype=np.int64)
+    ok = src != dst
+    if motif is not None:
+        has = np.zeros(256, dtype=bool)
+        has[np.asarray(motif, dtype=np.int64)] = True
+        color = has[np.asarray(g["color"], dtype=np.int64)]
+        ok &= color[src] & color[dst]
+    span = int(t.max()) + 1
+    order = np.argsort(dst * span + t, kind="stable")
+    order = order[ok[order]]
+    src, dst, t = src[order], dst[order], t[order]
+    key = dst * span + t
+    lo = np.searchsorted(key, src * span + np.maximum(t - delta[src], 0), "left")
+    hi = np.searchsorted(key, src * span + t, "right")
+    act = [src == s]
+    for _ in range(2, k):
+        c = np.concatenate(([0], np.cumsum(act[-1])))
+        act.append(c[hi] > c[lo])
+    need = act[-1]
+    rows = [order[need]]
+    for l in range(k - 2, 0, -1):
+        w = np.flatnonzero(need)
+        w = w[hi[w] > lo[w]]
+        d = np.bincount(lo[w], minlength=len(t) + 1) - np.bincount(hi[w], minlength=len(t) + 1)
+        need = act[l - 1] & (np.cumsum(d[:-1]) > 0)
+        rows.insert(0, order[need])
+    return rows
+
+
+def frontier_work(g, s, k, motif=None):
+    """What the frontier engine cannot do without for the query: rows per layer,
+    GF(2^64) products and bytes. With K = k-1 labels left, a layer l <= k-2 keeps
+    C(K, l-1) values a row, each a sum of l-1 products, from K multipliers
+    y z'_{tail}; layer k-2 extends them by the head (K values of K-1 products);
+    layer k-1 takes one product per label, and y. z' costs one product, in a
+    motif query one per occurrence of the vertex's colour. Bytes: every row's
+    record, the values it keeps (written) and its window's two ends (read), and
+    the witness. The fewest a query of this form takes: a row's z' is counted
+    once per layer, a head's once per layer."""
+    from math import comb
+    rows = frontier_rows(g, s, k, motif)
+    dst, src = np.asarray(g["dst"]), np.asarray(g["src"])
+    K = k - 1
+    zc = np.ones(g["n"], dtype=np.int64)
+    if motif is not None:
+        mu = np.bincount(np.asarray(motif, dtype=np.int64), minlength=256)
+        zc = mu[np.asarray(g["color"], dtype=np.int64)]
+    mults, nbytes = 0, 8 * g["n"]
+    for l, e in enumerate(rows, 1):
+        cnt = len(e)
+        heads = int(zc[np.unique(dst[e])].sum())
+        nbytes += cnt * 16
+        if l == k - 1:
+            mults += K * heads + cnt * (K + 1)
+            nbytes += cnt * 2 * 8 * (K if l > 1 else 0)
+            continue
+        mults += cnt if l == 1 else K * (int(zc[src[e]].sum()) + cnt) + cnt * comb(K, l - 1) * (l - 1)
+        nbytes += cnt * 8 * comb(K, l - 1) + (cnt * 2 * 8 * comb(K, l - 2) if l > 1 else 0)
+        if l == k - 2:
+            mults += K * heads + cnt * K * (K - 1)
+            nbytes += cnt * 8 * K
+    return {"rows_per_layer": [len(e) for e in rows], "gf_mults": int(mults), "bytes": int(nbytes)}
+
+
+def frontier_accounting(fw, k, m, info, ms_per_query):
+    """What one query performs against the nominal count, and what the dense
+    per-point engine multiplies for the same query."""
+    mults = fw["gf_mults"]
+    nominal = units_per_query(k, m)
+    # the per-point engine multiplies once per point for every row with a
+    # non-empty window at layers 2..k-1 (layer 1: the source's out-edges)
+    dense = float(2 ** k) * (k - 2) * info["window_rows"]
+    return {
+        "nominal_units_per_query": nominal,
+        "method_edge_point_layer_values_per_query": float(2 ** k) * (k - 1) * m,
+        "rows_per_layer": fw["rows_per_layer"],
+        "performed_gf_mults_per_query": mults,
+        "dense_engine_gf_mults_per_query": dense,
+        "dense_over_performed_mults": dense / max(1.0, mults),
+        "nominal_over_performed": nominal / max(1.0, mults),
+        "value_performed": {"value": mults / (ms_per_query / 1e3), "unit": "GF(2^64) multiplications/s"},
+        "note": "performed = products of the rows that a k-vertex walk from the source passes, over label "
+                "subsets instead of 2^k points (counted on the host); nominal = 2^k*k*m",
+    }
+
+
+def frontier_roofline(fw, ms_per_query, mul_peak, hbm_peak, peak_kind):
+    """The whole query is one kernel: its products and bytes over the query's
+    device time. A query with few rows is bound by neither: its one launch and
+    the reads that wait for each other."""
+    sec = ms_per_query / 1e3
+    gms, gbs = fw["gf_mults"] / sec / 1e9, fw["bytes"] / sec / 1e9
+    fa, fh = gms / (mul_peak / 1e9), gbs / hbm_peak
+    common = {"traffic": None, "kernel": "k_frontier", "avg_launch_us": round(ms_per_query * 1e3, 2),
+              "alg_bytes_per_launch": fw["bytes"], "alg_gf_mults_per_launch": fw["gf_mults"],
+              "hbm_frac": round(fh, 4), "alu_frac": round(fa, 4)}
+    if fa >= fh:
+        return {"bound": "alu", "achieved": round(gms, 2), "peak": round(mul_peak / 1e9, 2),
+                "unit": "GF(2^64) Gmul/s", "frac": round(fa, 4),
+                "peak_kind": "measured live: rr_bench_gf_mul, register-only multiply chains on all "
+                             "SMs, each operand value in one product (ALU-pipe bound)", **common}
+    return {"bound": "hbm", "achieved": round(gbs, 1), "peak": hbm_peak, "unit": "GB/s", "frac": round(fh, 4),
+            "peak_kind": peak_kind + " (MEASURED_PEAKS.json hbm_gbs)", **common}
+
+
 def work_accounting(by_kernel, k, m, info, ms_per_query):
     """What one query performs against the nominal count: GF(2^64)
     multiplications and stored state values summed over the kernels' per-launch
@@ -363,12 +475,11 @@ def motif_ztable_mults(g, motif, k):
 
 def uniform_metrics(capi, torch, g, mul_peak, hbm_peak, peak_kind, steps=20):
     """The uniform n=1e5 / m=1e6 graph, plain k=8 from vertex 0 (no restless
-    path of 3 or more vertices leaves it, so the witness is zero; the full
-    sieve still runs), autotuned shape."""
+    path of 3 or more vertices leaves it, so the witness is zero and the query
+    ends where its walks do)."""
     n, m = g["n"], len(g["src"])
     with capi.Graph(g) as G:
         info = G.info()
-        ppl, chunk = capi.rr_autotune(G.handle, K_UNIFORM)
         st = torch.cuda.Stream()
         d_w = torch.empty(n, dtype=torch.int64, device="cuda")
         d_bm = torch.empty((n + 7) // 8, dtype=torch.uint8, device="cuda")
@@ -379,16 +490,12 @@ def uniform_metrics(capi, torch, g, mul_peak, hbm_peak, peak_kind, steps=20):
                                  st.cuda_stream)
         timed_queries(torch, st, run, 3, flush)
         ms = timed_queries(torch, st, lambda i: run(100 + i), steps, flush)
-        kt = kernel_times(capi, torch, st, lambda i: run(200 + i), 5)
-    by_kernel = kernel_rooflines(info, K_UNIFORM, chunk, ppl, n, kt, 5, hbm_peak, mul_peak)
+    fw = frontier_work(g, 0, K_UNIFORM)
     per_q = sum(ms) / steps
-    roof = dominant_roofline(by_kernel, kt, mul_peak, hbm_peak, peak_kind,
-                             lambda kern: recorded_traffic("uniform", kern, ppl, chunk))
     return {"workload": UNIFORM_WORKLOAD, "value": units_per_query(K_UNIFORM, m) / (per_q / 1e3),
             "unit": UNIT, "ms_per_query": per_q, "steps": steps,
-            "shape": {"points_per_lane": ppl, "points_per_chunk": chunk},
-            "work": work_accounting(by_kernel, K_UNIFORM, m, info, per_q),
-            "roofline": roof, "roofline_by_kernel": by_kernel,
+            "work": frontier_accounting(fw, K_UNIFORM, m, info, per_q),
+            "roofline": frontier_roofline(fw, per_q, mul_peak, hbm_peak, peak_kind),
             "rows": {"state": info["producer_window_rows"] + 1, "deep": info["state_compute_rows"],
                      "deep_compute": info["deep_compute_rows"], "last_layer": info["deep_tail_rows"]},
             "l2": "flushed between queries",
@@ -503,55 +610,15 @@ def cpu_baseline(g, s, motif):
                       "shift-and-add GF(2^64) multiply (gcc -O2 -fopenmp)"}
 
 
-def batch_kernel_alg(info, qs, max_chunk, n):
-    """Algorithmic bytes and GF(2^64) multiplications of the persistent batch
-    kernel for the queries qs: per unit (one query's chunk of points) the same
-    per-layer counts as the one-query kernels, with layer 3 per point (the
-    batch has no pair-label form); k <= 3 and the label-space layer 2 run in
-    the prologue kernels and are not counted here."""
-    S = info["producer_window_rows"]
-    D = info["state_compute_rows"]
-    DC = info["deep_compute_rows"]
-    T3 = info["deep_tail_rows"]
-    T2 = info["tail_rows"]
-    R3 = info["deep_head_runs"]
-    tot_b = tot_m = 0.0
-    for q in qs:
-        k = q["k"]
-        if k <= 3:
-            continue
-        npts = 2 ** k
-        ppl = 4 if npts >= 128 else 2
-        c = max(32 * ppl, min(npts, max_chunk))
-        lg = 7 if ppl == 4 else 6
-        rs = c // (32 * ppl) * (lg + 1)
-        nch = (npts + c - 1) // c
-        if k == 4:
-            layers = [(S * rs * 8 + S * 20 + 2 * S * 8, S * (1 + k + c)),
-                      (2 * T2 * rs * 8 + T2 * 16 + n * 8, T2 * rs)]
-        else:
-            l3 = (D * (rs if k == 5 else c) * 8 + 2 * D * k * 8 + D * 20, D * (k + 2 * c) + R3 * c)
-            mid = (D * c * 8 + 2 * DC * c * 8 + D * 20, DC * (c + k))
-            tail = (D * rs * 8 + 2 * DC * c * 8 + D * 20, DC * (c + k))
-            last = (2 * T3 * rs * 8 + T3 * 16 + n * 8, T3 * rs)
-            layers = [l3] + ([mid] * (k - 6) + [tail] if k >= 6 else []) + [last]
-        tot_b += nch * sum(x[0] for x in layers)
-        tot_m += nch * sum(x[1] for x in layers)
-    return tot_b, tot_m
-
-
-def batched_metrics(capi, torch, gc, mul_peak, hbm_peak, nq=256, seed=UNIFORM_SEED):
+def batched_metrics(capi, torch, gc, nq=256, seed=UNIFORM_SEED):
     """The same graph with 8 colours; nq queries, s ~ U, k ~ U{4..12}, odd q
-    with a motif (source colour + k-1 uniform colours): one persistent batched
-    launch in the automatic shape and in the shape rr_autotune_batch picks on
-    this query list, against one launch sequence per query; results compared
-    bit for bit."""
+    with a motif (source colour + k-1 uniform colours): one batched launch
+    against one launch per query; results compared bit for bit."""
     qs = W.query_set(gc, nq, 4, 12, seed)
     n = gc["n"]
     m = len(gc["src"])
     units = sum(units_per_query(q["k"], m) for q in qs)
     with capi.Graph(gc) as G:
-        info = G.info()
         stream = torch.cuda.Stream()
         d_b = torch.zeros((nq, n), dtype=torch.int64, device="cuda")
         d_s = torch.zeros((nq, n), dtype=torch.int64, device="cuda")
@@ -569,20 +636,7 @@ def batched_metrics(capi, torch, gc, mul_peak, hbm_peak, nq=256, seed=UNIFORM_SE
                 stream.synchronize()
                 best = min(best, e0.elapsed_time(e1))
             return best / 1e3
-        t_auto = batch_ms()
-        t0 = time.perf_counter()
-        tuned = capi.rr_autotune_batch(G.handle, qs)
-        tune_s = time.perf_counter() - t0
         t_batch = batch_ms()
-        # the batch kernel alone, from the library's per-launch events
-        capi.rr_timing_enable(True)
-        capi.rr_timing_read(reset=True)
-        try:
-            capi.rr_reach_batch_device(G.handle, qs, d_b, None, d_st, stream.cuda_stream)
-            stream.synchronize()
-            kt = capi.rr_timing_read(reset=True)
-        finally:
-            capi.rr_timing_enable(False)
         for q in qs[:8]:
             capi.rr_reach_device(G.handle, q["source"], q["k"], q["seed"], d_s[0], None,
                                  stream.cuda_stream, motif=q["motif"])
@@ -597,28 +651,15 @@ def batched_metrics(capi, torch, gc, mul_peak, hbm_peak, nq=256, seed=UNIFORM_SE
             stream.synchronize()
             t_single = e0.elapsed_time(e1) / 1e3
         same = bool(torch.equal(d_b, d_s)) and int(d_st.abs().sum().item()) == 0
-    kms, kn = kt.get("batch", (0.0, 0))
-    roof = None
-    if kn:
-        ab, am = batch_kernel_alg(info, qs, tuned["max_chunk"], n)
-        ks = kms / kn / 1e3
-        fa, fh = am / ks / mul_peak, ab / ks / 1e9 / hbm_peak
-        roof = {"kernel": "k_batch", "avg_launch_us": round(ks * 1e6, 1),
-                "alg_gf_mults_per_launch": int(am), "alg_bytes_per_launch": int(ab),
-                "achieved_gmul_s": round(am / ks / 1e9, 2), "alu_frac": round(fa, 4),
-                "achieved_gbs": round(ab / ks / 1e9, 1), "hbm_frac": round(fh, 4),
-                "bound": "alu" if fa >= fh else "hbm",
-                "peak": "the multiply rate measured live (rr_bench_gf_mul) and the measured copy bandwidth"}
     return {"workload": f"{nq} queries on the n=100000 m=1000000 graph with 8 colours, "
                         "k~U{4..12}, odd queries coloured (motif = source colour + k-1 uniform)",
             "queries_per_s": nq / t_batch, "value": units / t_batch, "unit": UNIT,
-            "autotuned_shape": tuned, "autotune_s": round(tune_s, 2),
-            "automatic_shape_queries_per_s": nq / t_auto,
             "one_query_per_launch_queries_per_s": nq / t_single,
             "one_query_per_launch_value": units / t_single,
             "speedup": t_single / t_batch, "bit_exact_vs_single": same,
-            "roofline": roof,
-            "launches": "1 persistent kernel (+ z-table, first-layer and bitmap prologue/epilogue)"}
+            "roofline": None,
+            "bound": "latency: each query is one block's chain of dependent reads in its shared memory",
+            "launches": "1 kernel (+ bitmap epilogue)"}
 
 
 def served_metrics(capi, g, nq=160, seed=UNIFORM_SEED ^ 0x5E,
@@ -848,7 +889,7 @@ def kernel_rooflines(info, k, chunk, ppl, n, kt, queries, hbm_peak, mul_peak, zt
 
 
 def atmost_metrics(capi, torch, g, k=10, reps=5, source=0):
-    """at-most-k (the exact-k' queries for k' = 2..k, run concurrently) against
+    """at-most-k (the exact-k' queries for k' = 2..k, one launch) against
     the exact-k query on the benchmark graph. The paper's experiments report the
     ratio of the two runtimes (column 4 of its scalability tables; below 2 on
     most graphs), which the nominal work sum_{k'} k' 2^k' / (k 2^k) predicts."""
@@ -1007,10 +1048,14 @@ def main():
     G = capi.Graph(g, capi.FLAG_DENSE_STATE if args.dense else 0)
     load_s = time.perf_counter() - t0
     info = G.info()
+    # whole queries of a compact graph take the frontier engine; a range of
+    # points, the dense layout and a fixed shape the per-point engine
+    frontier = world == 1 and not args.shape and not args.dense
+    ppl = chunk = None
     if args.shape:
         ppl, chunk = (int(x) for x in args.shape.lower().split("x"))
         capi.rr_set_tuning(G.handle, K, ppl, chunk)
-    else:
+    elif not frontier:
         ppl, chunk = capi.rr_autotune(G.handle, K)
     first, count = shard.point_range(K, rank, world)
 
@@ -1057,8 +1102,10 @@ def main():
         clocks = sampler.stop()
     reach = int((d_w != 0).sum().item())
     # profiling pass (not timed above): per-kernel CUDA-event durations recorded
-    # by the library on the launching stream, this rank's share of the points
+    # by the library on the launching stream (frontier engine: one launch a
+    # layer); sharded: this rank's share of the points
     kt = kernel_times(capi, torch, stream,
+                      (lambda i: step(10_000 + i)) if frontier else
                       lambda i: capi.rr_reach_range_device(G.handle, s, K, step_seed(10_000 + i), first,
                                                            count, d_w, stream.cuda_stream, motif),
                       2)
@@ -1105,14 +1152,22 @@ def main():
 
     peaks, peak_kind = measured_peaks()
     mul_peak = gf_mul_peak(capi, torch)
-    by_kernel = {} if args.dense else kernel_rooflines(
-        info, K, chunk, ppl, n, kt, 2, peaks["hbm_gbs"], mul_peak,
-        ztable_mults=motif_ztable_mults(g, motif, K))
-    roofline = dominant_roofline(by_kernel, kt, mul_peak, peaks["hbm_gbs"], peak_kind,
-                                 lambda kern: recorded_traffic("motif", kern, ppl, chunk))
+    ms_per_step = tot_ms / args.steps
+    by_kernel, work = {}, None
+    if frontier:
+        fw = frontier_work(g, s, K, motif)
+        work = frontier_accounting(fw, K, m, info, ms_per_step)
+        roofline = frontier_roofline(fw, ms_per_step, mul_peak, peaks["hbm_gbs"], peak_kind)
+    else:
+        if not args.dense:
+            by_kernel = kernel_rooflines(info, K, chunk, ppl, n, kt, 2, peaks["hbm_gbs"], mul_peak,
+                                         ztable_mults=motif_ztable_mults(g, motif, K))
+        roofline = dominant_roofline(by_kernel, kt, mul_peak, peaks["hbm_gbs"], peak_kind,
+                                     lambda kern: recorded_traffic("motif", kern, ppl, chunk))
+        if by_kernel and world == 1:  # (per-rank kernel counts cover one share of the points)
+            work = work_accounting(by_kernel, K, m, info, ms_per_step)
     tot_k = max(1e-9, sum(v[0] for v in kt.values()))
     kernel_share = {k_: round(v[0] / tot_k, 4) for k_, v in kt.items() if v[1]}
-    ms_per_step = tot_ms / args.steps
 
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world,
             "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms_per_step,
@@ -1121,6 +1176,7 @@ def main():
             "config": {"workload": WORKLOAD, "graph_seed": GRAPH_SEED, "source": s, "k": K,
                        "motif": [int(c) for c in motif], "l2": "flushed between steps",
                        "state_layout": "dense" if args.dense else "compact",
+                       "engine": "frontier" if frontier else "per-point",
                        "points_per_lane": ppl, "points_per_chunk": chunk,
                        "parallelism": "single GPU" if world == 1 else
                        f"sieve points split over {world} ranks, partial witnesses all-gathered "
@@ -1134,7 +1190,7 @@ def main():
                        "max_in_degree": info["max_in_degree"],
                        "pair_layer3": info["pair_layer3_min_k"] <= K, "head_table": info["head_table"],
                        "graph_load_s": round(load_s, 3), "reachable_vertices": reach},
-            "work": work_accounting(by_kernel, K, m, info, ms_per_step) if by_kernel else None,
+            "work": work,
             "roofline": roofline,
             "roofline_by_kernel": by_kernel,
             "kernel_time_share": kernel_share,
@@ -1145,9 +1201,8 @@ def main():
                            if world == 1 else "shard.reach_sharded + witness copied to pinned host memory"},
             "gpu_launches": int(launches), "clocks": clocks,
             "parity": "tests/test_gpu_scale_parity.py: sieve points 640..703 of this query on this "
-                      "graph, autotuned shape, bit-exact vs the oracle"}
-    if world > 1:
-        line["work"] = None  # per-rank kernel counts cover one share of the points
+                      "graph bit-exact vs the oracle; tests/test_gpu_frontier.py: whole witnesses "
+                      "bit-exact vs the oracle and the per-point engine"}
     G.close()
     if rank == 0 and not args.no_extra:
         line["uniform_k8"] = uniform_metrics(capi, torch, W.scale_uniform(), mul_peak,
@@ -1161,8 +1216,7 @@ def main():
         line["atmost_k_powerlaw"]["workload"] = ("plain k-RestlessReach from the headline source on the "
                                                  "Chung-Lu n=1e6 m=1e7 graph")
         gu = W.scale_uniform()
-        line["batched"] = batched_metrics(capi, torch, W.scale_uniform(ncolors=8), mul_peak,
-                                          peaks["hbm_gbs"])
+        line["batched"] = batched_metrics(capi, torch, W.scale_uniform(ncolors=8))
         line["served"] = served_metrics(capi, gu)
         line["atmost_k"] = atmost_metrics(capi, torch, gu)
         line["fine_grained"] = fine_metrics(capi, torch, gu)
