@@ -369,14 +369,20 @@ rr_status rr_server_stats(rr_server *s, uint64_t *single, uint64_t *batched, uin
 rr_status rr_server_set_batching(rr_server *s, uint32_t min_batch, uint32_t max_batch);
 
 /* ---- tuning ----------------------------------------------------------------
- * Kernel shape used for a (graph, k): points per lane (2 or 4) and points per
- * chunk. rr_autotune times the candidates on the resident graph for the given
- * k and stores the winner in the graph; rr_set_tuning forces one. */
+ * Kernel shape of the per-point engine for a (graph, k): points per lane (2 or
+ * 4) and points per chunk. rr_autotune times the candidates on the resident
+ * graph for the given k and stores the winner in the graph; rr_set_tuning forces
+ * one. Whole queries of k <= 16 on a graph loaded without a load flag that picks
+ * a form of the per-point engine do without sieve points and have no shape;
+ * rr_set_tuning with a shape keeps the queries of that k on the per-point engine
+ * (0, 0 gives the choice back). */
 rr_status rr_autotune(rr_graph *g, uint32_t k, uint32_t *best_ppl, uint32_t *best_chunk);
 rr_status rr_set_tuning(rr_graph *g, uint32_t k, uint32_t ppl, uint32_t chunk);
 
-/* Shape of the persistent batch (rr_reach_batch_device and the server's batch
- * lanes), kept per graph; 0 in a field = the automatic rule.
+/* Shape of the persistent per-point batch (rr_reach_batch_device and the
+ * server's batch lanes), kept per graph; 0 in a field = the automatic rule.
+ * Without rr_set_batch_tuning it takes the queries that need the per-point
+ * engine (see above); a shape set there keeps whole batches on it.
  *   blocks_per_sm  kernel variant by the blocks per SM its register budget is
  *                  set for: 2 (168 registers), 4 (128), 5 (96, a few spills) or 6
  *                  (80, more spills);
@@ -452,7 +458,10 @@ rr_status rr_debug_draw(uint64_t key, uint64_t first, uint64_t count, uint64_t *
  * 6 = the last per-point layer, writing the transformed state (layer k-2, or
  * k-3 with the pair tail), 7 = layer 3 in pair-label space, 8 = the pair
  * tail's layer k-2 in label space. While timing is enabled the
- * launches are issued one by one instead of as a captured CUDA graph. */
+ * launches are issued one by one instead of as a captured CUDA graph. A whole
+ * query without sieve points is one launch otherwise and one per layer here:
+ * 0 = its passes over the row lists and layer 1, 5, 7, 1 = layers 2, 3 and the
+ * following, 2 = the last; a batch of them is one launch, 4. */
 typedef struct {
     double ms[9];
     uint64_t launches[9];

@@ -32,6 +32,7 @@
 // k = 8 (a handful of rows): 0.053 -> 0.033 ms; n = 1,000, k = 5: 26 -> 25 us.
 #include <algorithm>
 #include <cstring>
+#include <iterator>
 #include <type_traits>
 
 #include "rr_frontier.cuh"
@@ -69,9 +70,16 @@ __host__ __device__ constexpr uint32_t x_binom(uint32_t n, uint32_t d)
 }
 
 // the same at run time (n, d <= kXMaxLabels + 1)
-__constant__ uint16_t c_binom[kXMaxLabels + 2][kXMaxLabels + 2];
-__constant__ uint32_t c_tab_off[kXMaxLabels + 2];
-__device__ __forceinline__ uint32_t x_binom_dev(uint32_t n, uint32_t d) { return c_binom[n][d]; }
+struct XBinomials {
+    uint16_t v[kXMaxLabels + 2][kXMaxLabels + 2];
+    constexpr XBinomials() : v()
+    {
+        for (uint32_t i = 0; i < kXMaxLabels + 2; ++i)
+            for (uint32_t d = 0; d < kXMaxLabels + 2; ++d) v[i][d] = (uint16_t)x_binom(i, d);
+    }
+};
+__constant__ XBinomials c_binom;
+__device__ __forceinline__ uint32_t x_binom_dev(uint32_t n, uint32_t d) { return c_binom.v[n][d]; }
 
 // Subset tables: for every subset size d and d-subset T of [kXMaxLabels] in
 // colexicographic order, element i of T and the rank of T without it, packed
@@ -84,21 +92,28 @@ __host__ __device__ constexpr uint32_t x_tab_off(uint32_t d)
     return o;
 }
 
-__device__ __forceinline__ uint32_t x_tab_off_dev(uint32_t d) { return c_tab_off[d]; }
+struct XTabOffsets {
+    uint32_t v[kXMaxLabels + 2];
+    constexpr XTabOffsets() : v()
+    {
+        for (uint32_t d = 1; d < kXMaxLabels + 2; ++d) v[d] = x_tab_off(d);
+    }
+};
+__constant__ XTabOffsets c_tab_off;
+__device__ __forceinline__ uint32_t x_tab_off_dev(uint32_t d) { return c_tab_off.v[d]; }
 
 // For K <= kPackedLabels the tables of [K] once more, packed ([d][i][T], K 2^(K-1)
 // words), so that a block copies them in one go.
 constexpr uint32_t kPackedLabels = 11;
-constexpr uint32_t kPackedTab = x_tab_off(kXMaxLabels + 1);
 __host__ __device__ constexpr uint32_t x_packed_off(uint32_t K)  // sum of i 2^(i-1), i < K
 {
     return (K - 2u) * (1u << (K - 1u)) + 1u;
 }
 
-__global__ void __launch_bounds__(128) k_packed_table(uint32_t *__restrict__ tab)
+__global__ void __launch_bounds__(128) k_packed_table(const uint32_t *__restrict__ tab, uint32_t *__restrict__ packed)
 {
     const uint32_t K = blockIdx.y + 1;
-    uint32_t *o = tab + kPackedTab + x_packed_off(K);
+    uint32_t *o = packed + x_packed_off(K);
     for (uint32_t d = 1; d <= K; ++d) {
         const uint32_t c = x_binom_dev(K, d), cm = x_binom_dev(kXMaxLabels, d), *src = tab + x_tab_off_dev(d);
         for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < d * c; i += gridDim.x * blockDim.x) o[i] = src[i / c * cm + i % c];
@@ -1369,7 +1384,7 @@ __device__ __noinline__ int x_tiny(const XArgs &a, const XQuery &Q, bool every, 
         const uint32_t t = tid - kThreads / 2;
         if (t == 0) M.warm = mul_call(Q.key_y, Q.d0);  // fetches the multiply's code
         if (tables) {
-            const uint32_t *const src = a.tab + kPackedTab + x_packed_off(K);
+            const uint32_t *const src = a.packed + x_packed_off(K);
 #pragma unroll 4
             for (uint32_t i = t; i < K << (K - 1u); i += kThreads / 2) tab[i] = __ldg(src + i);
         }
@@ -1926,40 +1941,57 @@ __global__ void k_out_records(uint32_t m, const uint32_t *__restrict__ off, cons
     }
 }
 
-// start[i] = first position of entry i's window in the list `prev` (0-based):
+// start[i] = first position of entry i's window in the list before (0-based):
 // its index b when set, else the first row of the tail's segment there (the
-// rows with smaller heads come before it).
-__global__ void k_window_start(uint32_t count, const uint32_t *__restrict__ a, const uint32_t *__restrict__ b,
-                               const uint32_t *__restrict__ src, const uint32_t *__restrict__ prev_head,
-                               uint32_t prev_count, uint32_t *__restrict__ start)
+// rows with smaller heads come before it). A row of blocks per list.
+struct WindowList {
+    uint32_t count, prev_count;
+    const uint32_t *a, *b, *src, *prev_head;
+    uint32_t *start;
+};
+struct WindowLists {
+    WindowList l[6];
+};
+__global__ void k_window_start(const __grid_constant__ WindowLists lists)
 {
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) {
-        uint32_t s = b[i];
-        if (!s && a[i]) {
-            const uint32_t u = src[i];
-            uint32_t lo = 0, hi = prev_count;
+    const WindowList &L = lists.l[blockIdx.y];
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < L.count; i += gridDim.x * blockDim.x) {
+        uint32_t s = L.b[i];
+        if (!s && L.a[i]) {
+            const uint32_t u = L.src[i];
+            uint32_t lo = 0, hi = L.prev_count;
             while (lo < hi) {
                 const uint32_t mid = lo + (hi - lo) / 2;
-                if (prev_head[mid] < u) lo = mid + 1;
+                if (L.prev_head[mid] < u) lo = mid + 1;
                 else hi = mid;
             }
             s = lo;
         }
-        start[i] = s;
+        L.start[i] = s;
     }
 }
 
 }  // namespace
 
+rr_status frontier_out_reserve(Graph &g)
+{
+    // (with the packed subset tables behind them; both buffers of a small graph
+    // stay below 1 MiB, where an allocation needs no mapping of its own: 120 us)
+    const uint64_t m = std::max<uint64_t>(1, g.m);
+    RR_CUDA(g.o_buf.reserve(m * (sizeof(uint4) + 4) + ((uint64_t)g.n + 1 + x_packed_off(kPackedLabels + 1)) * 4));
+    RR_CUDA(g.x_tab.reserve((size_t)x_tab_off(kXMaxLabels + 1) * 4));
+    g.o_rec = g.o_buf.as<uint4>();
+    g.o_len = reinterpret_cast<uint32_t *>(g.o_rec + m);
+    g.o_off = g.o_len + m;
+    g.x_packed = g.o_off + g.n + 1;
+    return RR_OK;
+}
+
 rr_status frontier_out_records(Graph &g, const uint32_t *d_time, const uint32_t *d_dst, const uint32_t *d_eid,
                                const uint32_t *d_delta, cudaStream_t st)
 {
-    RR_CUDA(g.o_rec.reserve(std::max<uint64_t>(1, g.m) * sizeof(uint4)));
-    RR_CUDA(g.o_len.reserve(std::max<uint64_t>(1, g.m) * 4));
-    if (!g.m) return RR_OK;
     const unsigned grid = (unsigned)std::min<uint64_t>(152ull * 64, (g.m + 255) / 256);
-    k_out_records<<<grid, 256, 0, st>>>((uint32_t)g.m, g.o_off.as<uint32_t>(), d_time, d_dst, d_eid, d_delta,
-                                        g.o_rec.as<uint4>(), g.o_len.as<uint32_t>());
+    k_out_records<<<grid, 256, 0, st>>>((uint32_t)g.m, g.o_off, d_time, d_dst, d_eid, d_delta, g.o_rec, g.o_len);
     RR_LAUNCHED();
     return RR_OK;
 }
@@ -1980,47 +2012,45 @@ rr_status frontier_load(Graph &g, cudaStream_t st)
     g.x_smem_max = g.x_smem_max / 64 * 64;
     RR_CUDA(cudaFuncSetAttribute(k_frontier<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.x_smem_max));
     RR_CUDA(cudaFuncSetAttribute(k_frontier<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.x_smem_max));
-    RR_CUDA(g.x_tab.reserve((size_t)(kPackedTab + x_packed_off(kPackedLabels + 1)) * 4));
     k_subset_table<<<dim3((x_binom(kXMaxLabels, kXMaxLabels / 2) + 127) / 128, kXMaxLabels), 128, 0, st>>>(g.x_tab.as<uint32_t>());
     RR_LAUNCHED();
-    {
-        uint16_t bin[kXMaxLabels + 2][kXMaxLabels + 2];
-        uint32_t off[kXMaxLabels + 2];
-        for (uint32_t i = 0; i < kXMaxLabels + 2; ++i) {
-            for (uint32_t d = 0; d < kXMaxLabels + 2; ++d) bin[i][d] = (uint16_t)x_binom(i, d);
-            off[i] = i ? x_tab_off(i) : 0u;
-        }
-        RR_CUDA(cudaMemcpyToSymbolAsync(c_binom, bin, sizeof bin, 0, cudaMemcpyHostToDevice, st));
-        RR_CUDA(cudaMemcpyToSymbolAsync(c_tab_off, off, sizeof off, 0, cudaMemcpyHostToDevice, st));
-        RR_CUDA(cudaStreamSynchronize(st));
-    }
-    k_packed_table<<<dim3(8, kPackedLabels), 128, 0, st>>>(g.x_tab.as<uint32_t>());
+    k_packed_table<<<dim3(8, kPackedLabels), 128, 0, st>>>(g.x_tab.as<uint32_t>(), g.x_packed);
     RR_LAUNCHED();
     struct {
         RowList *L, *prev;
-        DevBuf *a, *b, *start;
+        DevBuf *a, *b;
+        uint32_t **start;
     } w[] = {{&g.state_list, &g.prod_list, &g.state_list.a0, &g.state_list.b0, &g.state_list.w0},
              {&g.win_list, &g.prod_list, &g.win_list.a0, &g.win_list.b0, &g.win_list.w0},
              {&g.deep_list, &g.state_list, &g.deep_list.a1, &g.deep_list.b1, &g.deep_list.w1},
              {&g.tail_list, &g.state_list, &g.tail_list.a1, &g.tail_list.b1, &g.tail_list.w1},
              {&g.deep_list, &g.deep_list, &g.deep_list.a3, &g.deep_list.b3, &g.deep_list.w3},
              {&g.tail3_list, &g.deep_list, &g.tail3_list.a3, &g.tail3_list.b3, &g.tail3_list.w3}};
+    uint64_t total = 0, most = 0;
     for (auto &x : w) {
-        if (!x.L->count) continue;
-        RR_CUDA(x.start->reserve(x.L->count * 4));
-        const unsigned grid = (unsigned)std::min<uint64_t>(152ull * 32, (x.L->count + 255) / 256);
-        k_window_start<<<grid, 256, 0, st>>>((uint32_t)x.L->count, x.a->as<uint32_t>(), x.b->as<uint32_t>(),
-                                             x.L->src.as<uint32_t>(), x.prev->head.as<uint32_t>(),
-                                             (uint32_t)x.prev->count, x.start->as<uint32_t>());
-        RR_LAUNCHED();
+        total += (x.L->count + 63u) / 64u * 64u;  // each on a 256-byte boundary
+        most = std::max<uint64_t>(most, x.L->count);
     }
+    if (!most) return RR_OK;
+    RR_CUDA(g.x_win.reserve(total * 4));
+    uint32_t *at = g.x_win.as<uint32_t>();
+    WindowLists lists{};
+    for (size_t i = 0; i < std::size(w); ++i) {
+        auto &x = w[i];
+        *x.start = at;
+        at += (x.L->count + 63u) / 64u * 64u;
+        lists.l[i] = WindowList{(uint32_t)x.L->count, (uint32_t)x.prev->count, x.a->as<uint32_t>(), x.b->as<uint32_t>(),
+                                x.L->src.as<uint32_t>(), x.prev->head.as<uint32_t>(), *x.start};
+    }
+    k_window_start<<<dim3((unsigned)std::min<uint64_t>(152ull * 32, (most + 255) / 256), (unsigned)std::size(w)), 256, 0, st>>>(lists);
+    RR_LAUNCHED();
     return RR_OK;
 }
 
 static void x_lists(const Graph &g, XList *out)
 {
-    auto set = [&](uint32_t id, const RowList &L, const DevBuf &lo, const DevBuf &hi) {
-        out[id] = XList{L.head.as<uint32_t>(), L.eid.as<uint32_t>(), L.src.as<uint32_t>(), lo.as<uint32_t>(),
+    auto set = [&](uint32_t id, const RowList &L, const uint32_t *lo, const DevBuf &hi) {
+        out[id] = XList{L.head.as<uint32_t>(), L.eid.as<uint32_t>(), L.src.as<uint32_t>(), lo,
                         hi.as<uint32_t>(), L.time.as<uint32_t>(), (uint32_t)L.count, (uint32_t)(L.count / 32 + 1)};
     };
     set(kXProd, g.prod_list, g.prod_list.w0, g.prod_list.a0);
@@ -2146,9 +2176,10 @@ static void x_args(const Graph &g, XArgs &a)
     a.n = g.n;
     a.color = g.color.as<uint8_t>();
     a.tab = g.x_tab.as<uint32_t>();
-    a.ooff = g.o_off.as<uint32_t>();
-    a.orec = g.o_rec.as<uint4>();
-    a.olen = g.o_len.as<uint32_t>();
+    a.packed = g.x_packed;
+    a.ooff = g.o_off;
+    a.orec = g.o_rec;
+    a.olen = g.o_len;
     a.smem = g.x_smem_max / 16u * 16u;
 }
 

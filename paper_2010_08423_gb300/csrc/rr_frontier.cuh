@@ -95,7 +95,7 @@ struct XArgs {
     int32_t *status;       // batch form: per query, RR_ETIMEDOUT when a wait gave up
     uint32_t *err;         // set when a bounded wait gave up
     const uint8_t *color;
-    const uint32_t *tab;   // subset tables
+    const uint32_t *tab, *packed;  // subset tables
     const uint32_t *ooff;  // edges by (tail, time): offsets (n + 1),
     const uint4 *orec;     // head, time, input index, first edge that may follow
     const uint32_t *olen;  // and how many

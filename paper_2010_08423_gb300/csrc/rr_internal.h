@@ -191,10 +191,11 @@ struct RowList {
     // frontier engine: the windows' first positions in the list of the layer
     // before (w0 producers, w1 state rows, w3 deep rows; the ends are a0/a1/a3),
     // and of the lists a last layer reads the edges' times
-    DevBuf w0, w1, w3, time;
+    DevBuf time;
+    uint32_t *w0 = nullptr, *w1 = nullptr, *w3 = nullptr;  // (parts of Graph::x_win)
     size_t bytes() const
     {
-        return w0.bytes + w1.bytes + w3.bytes + time.bytes + head.bytes + eid.bytes + src.bytes + a0.bytes + b0.bytes + a1.bytes + b1.bytes +
+        return time.bytes + head.bytes + eid.bytes + src.bytes + a0.bytes + b0.bytes + a1.bytes + b1.bytes +
                a3.bytes + b3.bytes + items.bytes + items_coarse.bytes + chains.bytes + fix2.bytes +
                heads.bytes + trank.bytes + row_carry.bytes + chain_slot0.bytes;
     }
@@ -352,7 +353,9 @@ struct Graph {
     // offsets (n + 1), records (head, time, input index, first edge that may
     // follow), numbers of followers --, subset tables, launch limits, and the
     // colours on the host (the source's z row is formed there)
-    DevBuf o_off, o_rec, o_len;
+    DevBuf o_buf, x_win;  // (x_win: the row lists' window starts)
+    uint4 *o_rec = nullptr;
+    uint32_t *o_len = nullptr, *o_off = nullptr, *x_packed = nullptr;
     DevBuf x_tab;
     int x_sms = 0;
     uint32_t x_smem_max = 0;
@@ -388,7 +391,7 @@ struct Graph {
 
     size_t device_bytes() const
     {
-        return x_tab.bytes + o_off.bytes + o_rec.bytes + o_len.bytes + off.bytes + row_a.bytes + row_b.bytes + row_s.bytes + row_eid.bytes +
+        return x_tab.bytes + o_buf.bytes + x_win.bytes + off.bytes + row_a.bytes + row_b.bytes + row_s.bytes + row_eid.bytes +
                row_src.bytes + row_lo.bytes + row_hi.bytes + row_t.bytes + row_head.bytes +
                color.bytes + color_order.bytes + items.bytes +
                prod_list.bytes() + state_list.bytes() + win_list.bytes() + tail_list.bytes() +
@@ -540,6 +543,7 @@ rr_status frontier_reserve(Workspace &ws, cudaStream_t st);
 // RR_ETIMEDOUT, once, when a bounded wait of a finished query on ws gave up.
 rr_status frontier_error(Workspace &ws);
 rr_status frontier_load(Graph &g, cudaStream_t st);
+rr_status frontier_out_reserve(Graph &g);
 rr_status frontier_out_records(Graph &g, const uint32_t *d_time, const uint32_t *d_dst, const uint32_t *d_eid,
                                const uint32_t *d_delta, cudaStream_t st);
 rr_status frontier_query(const Graph &g, Workspace &ws, const rr_query *q, bool every, uint8_t *d_bitmap,
