@@ -5,9 +5,9 @@
 // source ends with e, and it reaches an output only when a walk goes on from e
 // to the query's last layer. Both sets are found first, per layer, as bitmaps
 // over the row lists: forward, a row is active at layer l when its window holds
-// a row active at l - 1 (k_plan); backward, an active row is needed when a
+// a row active at l - 1 (x_plan); backward, an active row is needed when a
 // needed row of the next layer has it in its window. The layers then run over
-// the needed rows alone, stored densely in list order (k_wedge).
+// the needed rows alone, stored densely in list order (x_wedge).
 //
 // Wedge form. Summed over all sieve points L, a walk contributes the permanent
 // of its vertices' z rows, which in characteristic 2 is their determinant.
@@ -26,10 +26,16 @@
 // Why. On a Chung-Lu graph with n = 1e6, m = 1e7 the sieve-point engine
 // multiplies 1,024 points for each of 330,000 rows at each layer of a k = 10
 // query; walks from the source that reach the last layer pass 1,400 to 62,000
-// of them per layer, with at most 126 values each. Measured there 21 to 25 ms ->
-// 0.9 to 1.0 ms a query; n = 2e5, m = 2e6, k = 12: 23 -> 0.9 ms; a dense contact
-// graph (n = 2,000, m = 30,011, k = 12): 4.6 -> 0.26 ms; uniform n = 1e5, m = 1e6,
-// k = 8 (a handful of rows): 0.053 -> 0.033 ms; n = 1,000, k = 5: 26 -> 25 us.
+// of them per layer, with at most 126 values each. Measured against that engine:
+//   motif, k = 10, n = 1e6, m = 1e7                 23.1 -> 0.71 ms a query
+//   from a hub, k = 12, n = 2e5, m = 2e6            27.3 -> 0.73 ms
+//   dense contacts, k = 12, n = 2,000, m = 30,011   4.59 -> 0.19 ms
+//   uniform, k = 8, n = 1e5, m = 1e6                52 -> 24 us (a handful of rows)
+//   n = 1,000, m = 10,000, k = 5                    26 -> 18 us
+// What bounds it now: with many rows the products (issue slots of the integer
+// multiplies and XORs: 257 cycles per warp product and scheduler, the loop alone),
+// with few the chain of layers, some 50 grid barriers of 1.6 us at k = 12, and in
+// one block's shared memory about 2 us a layer.
 #include <algorithm>
 #include <cstring>
 #include <iterator>
@@ -51,7 +57,7 @@ __host__ __device__ constexpr uint32_t team_smem(uint32_t smem, uint32_t t) { re
 constexpr uint32_t kMaxRows = 16, kMaxOutRows = 32;  // rows of one item: store and out levels
 constexpr uint32_t kSplit = 28;       // words of a split multiplier: 9 pieces of 3 classes, padded to whole 16-byte loads
 constexpr uint32_t kSup1 = 16, kSup2 = 256, kSup3 = 4096;  // blocks per partial sum
-constexpr uint32_t kScanBlocks = 48, kScanSpan = 6, kScanLong = 1024;  // when a level's prefix sums are completed (x_scans)
+constexpr uint32_t kScanBlocks = 48, kScanSpan = 6, kScanLong = 4096;  // when a level's prefix sums are completed (x_scans)
 // Bitmap words per scan tile (a block takes four per thread at a time), and the
 // longest bitmap whose tiles count what lies before them themselves: 16 reads of
 // 16 bytes per thread at most, against a pass of its own and its barrier.
@@ -350,7 +356,10 @@ __device__ __noinline__ uint32_t x_choose_shape(uint32_t smem, uint32_t blocks, 
 // 16-byte loads (nine, a piece each, kept the shared-memory pipe as busy as the
 // ALU: at-most-k, k = 10, on n = 1e6, m = 1e7 4.82 -> 4.62 ms).
 // Per product this leaves 81 IMAD, about 41 three-input XORs and the 31
-// instructions that split the other operand, against 240 of gf64_mul.
+// instructions that split the other operand, against 240 of gf64_mul. An IMAD
+// takes two issue cycles of its scheduler and the others one each, together 257
+// cycles a product and warp with the loads and the end of a sum. Forms with fewer
+// IMADs cost more: 48 64-bit multiplies of 32-bit pieces in four classes 350.
 __device__ __forceinline__ uint64_t finish27(const uint32_t (&z)[27])
 {
     uint64_t r[3];
@@ -854,9 +863,10 @@ __device__ __forceinline__ void xor_shared(uint64_t *p, uint64_t v)
 // Level list li's prefix sums are completed (x_scan_blocks): when the windows
 // that read it span more than kScanSpan blocks on average, and for long levels,
 // where a few windows of thousands of rows hold their teams up. Otherwise the
-// pass and its barrier (5 us) cost more than the extra reads: dense contacts,
-// k = 12, 264 us scanning every layer of 48 blocks, 230 us so; at-most-k, k = 10,
-// on n = 1e6, m = 1e7 5.23 ms by the average alone, 4.99 ms so.
+// pass and its barrier (4 us) cost more than the extra reads: levels from 256,
+// 1,024, 4,096, 16,384 blocks on: arrival, k = 8, 269, 258, 248, 248 us; bounded,
+// k = 8, 368, 368, 353, 353 us; at-most-k, k = 10, on n = 1e6, m = 1e7 4.15, 4.15,
+// 4.14, 4.15 ms, and 4.45 ms by the average alone.
 __device__ __forceinline__ bool x_scans(const XTmpl &t, uint32_t li)
 {
     const XShape sh = x_shape_of(t.shape[li]);
