@@ -319,6 +319,10 @@ void Server::run()
                     t.state = Ticket::Failed;
                     t.status = RR_ECUDA;
                     t.error = std::string("query failed on device: ") + cudaGetErrorString(q);
+                } else if (const rr_status fs = frontier_error(sl.ws); fs != RR_OK) {
+                    t.state = Ticket::Failed;
+                    t.status = fs;
+                    t.error = rr_last_error();
                 } else if (t.cancel_requested) {
                     t.state = Ticket::Canceled;
                     t.status = RR_ECANCELED;
