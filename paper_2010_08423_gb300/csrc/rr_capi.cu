@@ -170,11 +170,8 @@ rr_status rr_reach_sync(const rr_graph *g, const rr_query *q, uint8_t *bitmap, u
     rr_status s = reach_on_stream(*g, g->ws, q, g->ws.bitmap.as<uint8_t>(),
                                   g->ws.S.as<uint64_t>(), 0, g->stream);
     if (s != RR_OK) return s;
-    if (witness)
-        RR_CUDA(cudaMemcpyAsync(witness, g->ws.S.p, (size_t)g->n * 8, cudaMemcpyDeviceToHost,
-                                g->stream));
-    if (bitmap)
-        RR_CUDA(cudaMemcpyAsync(bitmap, g->ws.bitmap.p, nb, cudaMemcpyDeviceToHost, g->stream));
+    s = copy_out(g->ws.S.as<uint64_t>(), witness, g->n, g->ws.bitmap.as<uint8_t>(), bitmap, nb, g->stream);
+    if (s != RR_OK) return s;
     RR_CUDA(cudaStreamSynchronize(g->stream));
     return frontier_error(g->ws);
 }

@@ -388,11 +388,7 @@ void Server::run()
                                      share, sl.stream);
             if (st == RR_OK) {
                 const ResultBuf &rb = results[sl.result];
-                if (cudaMemcpyAsync(rb.w, sl.ws.S.p, (size_t)g->n * 8, cudaMemcpyDeviceToHost,
-                                    sl.stream) != cudaSuccess ||
-                    cudaMemcpyAsync(rb.bm, sl.ws.bitmap.p, nb, cudaMemcpyDeviceToHost, sl.stream) !=
-                        cudaSuccess)
-                    st = RR_ECUDA;
+                st = copy_out(sl.ws.S.as<uint64_t>(), rb.w, g->n, sl.ws.bitmap.as<uint8_t>(), rb.bm, nb, sl.stream);
             }
             if (st == RR_OK && cudaEventRecord(sl.done, sl.stream) != cudaSuccess) st = RR_ECUDA;
             if (st == RR_OK && cudaLaunchHostFunc(sl.stream, on_query_copied, this) != cudaSuccess)

@@ -148,3 +148,21 @@ def test_long_queries_one_after_another():
             _, w1 = G.reach(qs[i]["source"], qs[i]["k"], qs[i]["seed"])
             assert np.array_equal(w[i], w1), i
         assert w.any()
+
+
+@pytest.mark.parametrize("n,ow,ob", [(33, 0, 0), (37, 1, 1), (2000, 0, 3), (2001, 1, 16), (4097, 2, 0)])
+def test_results_into_pinned_buffers(n, ow, ob):
+    # one kernel writes both; every alignment, words and bytes left over, and
+    # nothing beyond them
+    import torch
+    g = W.uniform(n, 15 * n, 40, 0, 6, 5)
+    nb = (n + 7) // 8
+    w = torch.full((n + ow + 2,), -7, dtype=torch.int64, pin_memory=True).numpy().view(np.uint64)
+    b = torch.full((nb + ob + 2,), 99, dtype=torch.uint8, pin_memory=True).numpy()
+    with capi.Graph(g) as G:
+        b1, w1 = G.reach(1, 5, 3)
+        G.reach(1, 5, 3, out=(b[ob:ob + nb], w[ow:ow + n]))
+    assert np.array_equal(w[ow:ow + n], w1) and np.array_equal(b[ob:ob + nb], b1)
+    assert w1.any()
+    assert (w[:ow].view(np.int64) == -7).all() and (w[ow + n:].view(np.int64) == -7).all()
+    assert (b[:ob] == 99).all() and (b[ob + nb:] == 99).all()
