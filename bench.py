@@ -151,10 +151,7 @@ def kernel_sources_sha1() -> str:
     return h.hexdigest()
 
 
-TRAFFIC_RECORDS = {
-    "motif": "ncu_traffic_k10_motif_powerlaw_n1e6_m1e7.json",
-    "uniform": "ncu_traffic_k8_uniform_n1e5_m1e6.json",
-}
+TRAFFIC_RECORDS = {"motif": "ncu_traffic_k10_motif_powerlaw_n1e6_m1e7.json"}
 
 
 def recorded_traffic(workload: str, kernel: str, ppl: int, chunk: int):
