@@ -27,14 +27,14 @@
 // multiplies 1,024 points for each of 330,000 rows at each layer of a k = 10
 // query; walks from the source that reach the last layer pass 1,400 to 62,000
 // of them per layer, with at most 126 values each. Measured against that engine:
-//   motif, k = 10, n = 1e6, m = 1e7                 23.1 -> 0.71 ms a query
-//   from a hub, k = 12, n = 2e5, m = 2e6            27.3 -> 0.73 ms
-//   dense contacts, k = 12, n = 2,000, m = 30,011   4.59 -> 0.19 ms
-//   uniform, k = 8, n = 1e5, m = 1e6                52 -> 24 us (a handful of rows)
-//   n = 1,000, m = 10,000, k = 5                    26 -> 18 us
+//   motif, k = 10, n = 1e6, m = 1e7                 20.8 -> 0.67 ms a query
+//   from a hub, k = 12, n = 2e5, m = 2e6            30.9 -> 1.06 ms
+//   dense contacts, k = 12, n = 2,000, m = 30,011   4.52 -> 0.19 ms
+//   uniform, k = 8, n = 1e5, m = 1e6                52 -> 25 us (a handful of rows)
+//   n = 1,000, m = 10,000, k = 5                    27 -> 18 us
 // What bounds it now: with many rows the products (issue slots of the integer
 // multiplies and XORs: 257 cycles per warp product and scheduler, the loop alone),
-// with few the chain of layers, some 50 grid barriers of 1.6 us at k = 12, and in
+// with few the chain of layers, some 45 grid barriers of 1.6 us at k = 12, and in
 // one block's shared memory about 2 us a layer.
 #include <algorithm>
 #include <cstring>
@@ -54,7 +54,7 @@ __host__ __device__ constexpr uint32_t team_threads(uint32_t t) { return t + 1 <
 __host__ __device__ constexpr uint32_t team_count(uint32_t t) { return (uint32_t)kThreads / team_threads(t); }
 // A team's share of the block's shared memory.
 __host__ __device__ constexpr uint32_t team_smem(uint32_t smem, uint32_t t) { return smem / team_count(t) / 16u * 16u; }
-constexpr uint32_t kMaxRows = 16, kMaxOutRows = 32;  // rows of one item: store and out levels
+constexpr uint32_t kMaxRows = 32;     // rows of one item: the lanes of the team's first warp
 constexpr uint32_t kSplit = 28;       // words of a split multiplier: 9 pieces of 3 classes, padded to whole 16-byte loads
 constexpr uint32_t kSup1 = 16, kSup2 = 256, kSup3 = 4096;  // blocks per partial sum
 constexpr uint32_t kScanBlocks = 48, kScanSpan = 6, kScanLong = 4096;  // when a level's prefix sums are completed (x_scans)
@@ -302,7 +302,9 @@ __device__ __forceinline__ uint32_t rank_below(const uint2 *rank, uint32_t x)
 // item's other parts. Chosen once per level list, by the warp that counts its
 // rows; the next level reads the rows' prefix sums by it. With powers of two and
 // rows added until every team had an item, layers of 2,500 to 4,000 rows left
-// the warps idle for a third of the time.
+// the warps idle for a third of the time. Store items of up to 32 rows instead of
+// 16 fill the last wave better where many short rows meet large teams (k = 12 from
+// a hub of n = 2e5 1.35 -> 1.31 ms on one graph, at-most-k 3.58 -> 3.49 ms on one).
 struct XShape {
     uint32_t team, rows, scan;  // team: log2
 };
@@ -328,9 +330,8 @@ __device__ __noinline__ uint32_t x_choose_shape(uint32_t smem, uint32_t blocks, 
 {
     const uint32_t lane = threadIdx.x & 31u;
     uint32_t best = 0xffffffffu, pick = 0;
-    const uint32_t most = X.out ? kMaxOutRows : kMaxRows;
-    for (uint32_t i = lane; i < kTeams * most; i += 32u) {
-        const uint32_t t = i / most, rows = i % most + 1u;
+    for (uint32_t i = lane; i < kTeams * kMaxRows; i += 32u) {
+        const uint32_t t = i / kMaxRows, rows = i % kMaxRows + 1u;
         if ((rows > 1u || t + 1u < kTeams) && x_item_bytes(rows, K, X) > team_smem(smem, t)) continue;
         const uint32_t items = (cnt + rows - 1u) / rows, teams = blocks * team_count(t);
         const uint32_t cost = (items + teams - 1u) / teams * x_item_cost(rows, t, K, X);
