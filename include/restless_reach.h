@@ -165,7 +165,9 @@ rr_status rr_reach_sync(const rr_graph *g, const rr_query *q, uint8_t *bitmap,
  * one graph that use it (this one, rr_reach_sync, the batched, at-most-k,
  * fine-grained, set-of-sources and extraction calls, rr_autotune) may be
  * issued on different streams -- each call's stream first waits, on the
- * device, for the previous such call's work. */
+ * device, for the previous such call's work. A query whose kernel gave up a
+ * bounded wait is reported as RR_ETIMEDOUT by rr_reach_sync itself, for the
+ * calls that only enqueue by the next call on the graph. */
 rr_status rr_reach_device(const rr_graph *g, const rr_query *q, uint8_t *d_bitmap,
                           uint64_t *d_witness, void *stream);
 

@@ -27,9 +27,9 @@
 // multiplies 1,024 points for each of 330,000 rows at each layer of a k = 10
 // query; walks from the source that reach the last layer pass 1,400 to 62,000
 // of them per layer, with at most 126 values each. Measured against that engine:
-//   motif, k = 10, n = 1e6, m = 1e7                 20.8 -> 0.67 ms a query
-//   from a hub, k = 12, n = 2e5, m = 2e6            30.9 -> 1.06 ms
-//   dense contacts, k = 12, n = 2,000, m = 30,011   4.52 -> 0.19 ms
+//   motif, k = 10, n = 1e6, m = 1e7                 20.8 -> 0.68 ms a query
+//   from a hub, k = 12, n = 2e5, m = 2e6            30.9 -> 1.02 ms
+//   dense contacts, k = 12, n = 2,000, m = 30,011   4.53 -> 0.19 ms
 //   uniform, k = 8, n = 1e5, m = 1e6                52 -> 25 us (a handful of rows)
 //   n = 1,000, m = 10,000, k = 5                    27 -> 18 us
 // What bounds it now: with many rows the products (issue slots of the integer
