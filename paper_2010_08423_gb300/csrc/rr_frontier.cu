@@ -2023,6 +2023,16 @@ rr_status frontier_load(Graph &g, cudaStream_t st)
     g.x_smem_max = g.x_smem_max / 64 * 64;
     RR_CUDA(cudaFuncSetAttribute(k_frontier<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.x_smem_max));
     RR_CUDA(cudaFuncSetAttribute(k_frontier<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.x_smem_max));
+    // blocks that wait on one another need a cooperative launch with a block on
+    // every SM; where that is not to be had, queries run over sieve points
+    int coop = 0;
+    RR_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, g.dev));
+    for (const void *f : {(const void *)k_frontier<false>, (const void *)k_frontier<true>}) {
+        int per = 0;
+        RR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, f, kThreads, g.x_smem_max));
+        if (!coop || per < 1) g.x_sms = 0;
+    }
+    if (!g.x_sms) return RR_OK;
     k_subset_table<<<dim3((x_binom(kXMaxLabels, kXMaxLabels / 2) + 127) / 128, kXMaxLabels), 128, 0, st>>>(g.x_tab.as<uint32_t>());
     RR_LAUNCHED();
     k_packed_table<<<dim3(8, kPackedLabels), 128, 0, st>>>(g.x_tab.as<uint32_t>(), g.x_packed);
@@ -2269,7 +2279,7 @@ static void x_query(const Graph &g, const rr_query &q, bool multi, bool constant
 
 bool uses_frontier(const Graph &g, uint32_t k)
 {
-    return g.compact && !g.point_flags && k >= 2 && k - 1 <= kXMaxLabels && !g.tune_forced[k];
+    return g.x_sms && g.compact && !g.point_flags && k >= 2 && k - 1 <= kXMaxLabels && !g.tune_forced[k];
 }
 
 uint64_t frontier_bytes(const Graph &g, uint32_t k, bool every, bool multi, bool arrivals)
