@@ -1391,6 +1391,7 @@ __device__ __noinline__ int x_tiny(const XArgs &a, const XQuery &Q, bool every, 
     __syncthreads();
     // layer 1: the edges leaving the source(s); beside it (the upper warps) the
     // subset tables and the shade factors
+    bool wide = false;  // a source with more edges than kTinyRange
     if (warp >= kWarps / 2) {
         const uint32_t t = tid - kThreads / 2;
         if (t == 0) M.warm = mul_call(Q.key_y, Q.d0);  // fetches the multiply's code
@@ -1414,7 +1415,7 @@ __device__ __noinline__ int x_tiny(const XArgs &a, const XQuery &Q, bool every, 
             if (Q.vmask && Q.vmask[s]) continue;
             const uint32_t o0 = a.ooff[s], o1 = a.ooff[s + 1];
             if (o1 - o0 > kTinyRange) {
-                if (lane == 0) M.over = 1;
+                wide = true;
                 continue;
             }
 #pragma unroll 1
@@ -1430,11 +1431,13 @@ __device__ __noinline__ int x_tiny(const XArgs &a, const XQuery &Q, bool every, 
             }
         }
     }
-    __syncthreads();
+    // (the barrier's own answer, not M.over: the first warps past it may set that
+    // for layer 2 before the last ones have looked)
+    const bool over1 = __syncthreads_or(wide);
     uint32_t n = M.count[1], lmax = 1;
     const uint32_t n1 = n;
     uint32_t prev = n;
-    if (M.over || n > kTinyRows) return kTinyNoFit;
+    if (over1 || n > kTinyRows) return kTinyNoFit;
     if (tid == 0) M.base[2] = n;
     // forward; the hash table, counters and pairs of a level are cleared while
     // the one before it uses the other
@@ -1502,6 +1505,7 @@ __device__ __noinline__ int x_tiny(const XArgs &a, const XQuery &Q, bool every, 
 
     // backward, the row counts and the space the layers take: one warp
     if (warp == 0) {
+        __syncwarp();  // base[2] is lane 0's (k = 2: no layer's barriers came between)
 #pragma unroll 1
         for (uint32_t i = lane; i < (top + 1u) * kTinyWords; i += 32u) {
             const uint32_t l = i / kTinyWords;
