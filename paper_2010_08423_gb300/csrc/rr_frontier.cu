@@ -278,6 +278,99 @@ __device__ __forceinline__ bool any_words(const uint32_t *A, uint32_t w, uint32_
     return false;
 }
 
+// Long windows. A pass that reads every word of every window takes (rows that
+// leave a vertex) x (rows that enter it) / 32 words a layer: k = 5 through two
+// vertices with 20,000, 100,000 and 400,000 edges each way and waits as long as the
+// time range took 0.44, 4.0 and 48.9 ms (0.24, 0.34 and 1.25 ms with summaries), and
+// larger ones would outlast a barrier's wait. So a bitmap that windows of more than
+// kLongWords words read has three summaries, each a bit per word of the level below
+// it (at most 2^26 words, 2,048 in the last): S, the words of A that hold a row, and
+// F, the words of N that some window covers whole. A window then takes at most
+// 2 kLongWords words of each level, and the passes are linear in the rows, with a
+// barrier more a layer. Graphs without such windows have no summaries, and passes of
+// their own that read what lies between a window's end words directly (x_plan<false>;
+// with the tests for summaries in one form for both, k = 12 on n = 2,000, m = 30,011
+// took 1.4 % longer). The summaries' functions are inlined: x_plan makes no call
+// where the lanes of a warp have parted.
+constexpr uint32_t kLongWords = 128;
+// Words of the first summary of `words` words, and of all three.
+__host__ __device__ __forceinline__ uint32_t x_sum_level(uint32_t words) { return ((words + 31u) / 32u + 3u) / 4u * 4u; }
+__host__ __device__ __forceinline__ uint32_t x_sum_words(uint32_t words)
+{
+    const uint32_t a = x_sum_level(words), b = x_sum_level(a);
+    return a + b + x_sum_level(b);
+}
+// The summaries of a level's A (the upper two were cleared): a warp a word of the first.
+__device__ __forceinline__ void sum_level(const XLL &X, uint32_t gw, uint32_t nw)
+{
+    const uint32_t lane = threadIdx.x & 31u, n1 = (X.words + 31u) / 32u, l1 = x_sum_level(X.words);
+    uint32_t *const S2 = X.S + l1, *const S3 = S2 + x_sum_level(l1);
+    for (uint32_t i = gw; i < n1; i += nw) {
+        const uint32_t w = i * 32u + lane;
+        const uint32_t on = __ballot_sync(0xffffffffu, w < X.words && X.A[w] != 0);
+        if (lane == 0) {
+            X.S[i] = on;
+            if (on) {
+                const uint32_t b2 = 1u << (i & 31u), b3 = 1u << ((i >> 5) & 31u);
+                if (!(__ldcg(S2 + (i >> 5)) & b2)) atomicOr(S2 + (i >> 5), b2);
+                if (!(__ldcg(S3 + (i >> 10)) & b3)) atomicOr(S3 + (i >> 10), b3);
+            }
+        }
+    }
+}
+// any_words over [a, b), by the summaries.
+__device__ __forceinline__ bool any_long(const uint32_t *A, const uint32_t *S, uint32_t words, uint32_t a, uint32_t b)
+{
+    for (int level = 0;; ++level) {
+        if (level == 3 || b - a <= kLongWords) return any_words(A, a, b);
+        const uint32_t a1 = (a + 31u) & ~31u, b1 = b & ~31u;
+        if (any_words(A, a, a1) || any_words(A, b1, b)) return true;
+        a = a1 >> 5;
+        b = b1 >> 5;
+        A = level ? A + words : S;
+        words = x_sum_level(words);
+    }
+}
+// The words [a, b) are needed whole.
+__device__ __forceinline__ void mark_long(uint32_t *F, uint32_t words, uint32_t a, uint32_t b)
+{
+    auto set = [&](uint32_t w, uint32_t mask) {
+        if (mask & ~__ldcg(F + w)) atomicOr(F + w, mask);
+    };
+    for (int level = 0;; ++level) {  // the bits [a, b) of this summary
+        const uint32_t w0 = a >> 5, w1 = (b - 1u) >> 5;
+        const uint32_t first = 0xffffffffu << (a & 31u), last = 0xffffffffu >> (31u - ((b - 1u) & 31u));
+        if (w0 == w1) {
+            set(w0, first & last);
+            return;
+        }
+        if (level == 2 || w1 - w0 <= 8u) {
+            set(w0, first);
+            for (uint32_t w = w0 + 1u; w < w1; ++w) set(w, 0xffffffffu);
+            set(w1, last);
+            return;
+        }
+        set(w0, first);
+        set(w1, last);
+        a = w0 + 1u;  // the words between, whole: bits of the next summary
+        b = w1;
+        words = x_sum_level(words);
+        F += words;
+    }
+}
+// Whether word w is marked.
+__device__ __forceinline__ bool covered(const uint32_t *F, uint32_t words, uint32_t w)
+{
+    bool on = false;
+    for (int level = 0; level < 3; ++level) {
+        on |= (F[w >> 5] >> (w & 31u)) & 1u;
+        w >>= 5;
+        words = x_sum_level(words);
+        F += words;
+    }
+    return on;
+}
+
 // Rows of partial sums over nb blocks: of 16, 256 and 4,096 blocks.
 __host__ __device__ __forceinline__ uint32_t x_sup_rows(uint64_t nb)
 {
@@ -419,7 +512,8 @@ __device__ __forceinline__ bool allowed(const XQuery &Q, const uint8_t *color, u
 // short (10 MB of row windows and bitmaps on n = 1e6, m = 1e7), so the dependent
 // reads between two barriers bound it: a level's first windows are read before
 // the barrier they wait at, whether a level is alive comes with the barrier, the
-// warps take the steps of all level lists in one sequence.
+// warps take the steps of all level lists in one sequence. WIDE: with summaries.
+template <bool WIDE>
 __device__ __noinline__ bool x_plan(const XArgs &a, const XOne &o, View &v)
 {
     const XQuery &Q = o.q;
@@ -429,7 +523,7 @@ __device__ __noinline__ bool x_plan(const XArgs &a, const XOne &o, View &v)
     const uint32_t gt = v.b * kThreads + threadIdx.x, nt = v.n * kThreads;
     constexpr uint32_t U = 2;  // bitmap words per warp and step
 
-    // cleared first: needed-row bitmaps, counts
+    // cleared first: needed-row bitmaps, summaries, counts
     for (uint32_t i = gt; i < t.clear4; i += nt) t.clear[i] = make_uint4(0, 0, 0, 0);
     if (v.b == 0)
         for (uint32_t i = threadIdx.x; i < t.nll; i += kThreads) {
@@ -449,7 +543,8 @@ __device__ __noinline__ bool x_plan(const XArgs &a, const XOne &o, View &v)
             const XLL &X = t.ll[li];
             const XList &L = a.lists[X.list];
             const uint32_t steps = (L.words + U - 1) / U, i0 = View::first_item(base, gw, nw);
-            const uint32_t *const Ap = t.ll[X.prev].A;
+            const XLL &P = t.ll[X.prev];
+            const uint32_t *const Ap = P.A;
             const bool none = Q.dead || (X.out && Q.pivot > l && !Q.multi);  // z_s is zero over the labels of k' = l + 1
             if (l == 1) {
                 // a stream of tails: eight words a step keep enough reads in flight
@@ -498,7 +593,9 @@ __device__ __noinline__ bool x_plan(const XArgs &a, const XOne &o, View &v)
                     const uint32_t first = lo[x] >> 5, last = (hi[x] - 1u) >> 5;
                     if (hi[x] <= lo[x]) act[x] = false;
                     else if (first == last) act[x] = (fw[x] & m0 & m1) != 0;
-                    else act[x] = (fw[x] & m0) || (lw[x] & m1) || any_words(Ap, first + 1u, last);
+                    else if ((fw[x] & m0) || (lw[x] & m1)) act[x] = true;
+                    else if (WIDE && last - first > kLongWords) act[x] = any_long(Ap, P.S, P.words, first + 1u, last);
+                    else act[x] = any_words(Ap, first + 1u, last);
                 }
                 if (check) {
                     uint32_t h[U];
@@ -533,22 +630,33 @@ __device__ __noinline__ bool x_plan(const XArgs &a, const XOne &o, View &v)
             lmax = l - 1;
             break;
         }
+        if (const XLL &X = t.ll[t.runs[l].first]; WIDE && l < t.maxlev && X.S) {  // (the store level comes first)
+            sum_level(X, gw, nw);
+            if (!v.sync()) return false;
+        }
     }
     // no walk as long as an output needs: every count stays zero
     if (lmax == 0 || (!t.every && lmax < t.maxlev)) return v.sync();
 
     // backward: the rows of layer l - 1 in the window of a needed row of layer l
     // (at-most-k: every layer has outputs, every active row is needed)
+    // Word w of level X's N, with what the long windows need whole.
+    auto needed = [](const XLL &X, uint32_t w) {
+        uint32_t m = X.N[w];
+        if (WIDE && X.F && covered(X.F, X.words, w)) X.N[w] = m = X.A[w];
+        return m;
+    };
     if (!t.every)
         for (uint32_t l = lmax; l >= 2; --l) {
             const XLL &X = t.ll[t.runs[l].first];  // (one list a level)
             const XList &L = a.lists[X.list];
             const uint32_t steps = (L.words + U - 1) / U;
-            const uint32_t *const Ap = t.ll[X.prev].A;
-            uint32_t *const Np = t.ll[X.prev].N;
+            const XLL &P = t.ll[X.prev];
+            const uint32_t *const Ap = P.A;
+            uint32_t *const Np = P.N;
             for (uint32_t i = gw; i < steps; i += nw) {
                 const uint32_t w0 = i * U;
-                const uint32_t mine = lane < U && w0 + lane < L.words ? X.N[w0 + lane] : 0u;
+                const uint32_t mine = lane < U && w0 + lane < L.words ? needed(X, w0 + lane) : 0u;
                 if (!__any_sync(0xffffffffu, mine != 0)) continue;
                 uint32_t lo[U], hi[U];
 #pragma unroll
@@ -574,7 +682,12 @@ __device__ __noinline__ bool x_plan(const XArgs &a, const XOne &o, View &v)
                     const uint32_t last = 0xffffffffu >> (31u - ((hi[x] - 1) & 31u));
                     if (b1 == b0) m[x] &= last;
                     if (m[x] & ~have[x]) atomicOr(Np + b0, m[x]);
-                    for (uint32_t w = b0 + 1; w <= b1; ++w) {
+                    uint32_t w = b0 + 1;
+                    if (WIDE && b1 - b0 > kLongWords) {
+                        mark_long(P.F, P.words, w, b1);
+                        w = b1;
+                    }
+                    for (; w <= b1; ++w) {
                         const uint32_t mw = Ap[w] & (w == b1 ? last : 0xffffffffu);
                         if (mw & ~Np[w]) atomicOr(Np + w, mw);
                     }
@@ -582,6 +695,10 @@ __device__ __noinline__ bool x_plan(const XArgs &a, const XOne &o, View &v)
             }
             if (!v.sync()) return false;
         }
+    if (const XLL &X = t.ll[t.runs[1].first]; WIDE && X.F) {  // (the other levels' words were completed on the way)
+        for (uint32_t w = gt; w < X.words; w += nt) needed(X, w);
+        if (!v.sync()) return false;
+    }
 
     // ranks: per bitmap word the rows before it, and the levels' row counts. A
     // block takes a tile of kTileWords words; what lies before it, it counts
@@ -1766,6 +1883,8 @@ __device__ __forceinline__ void relocate(XTmpl &t, uint8_t *base)
         XLL &x = t.ll[i];
         fix(x.A);
         fix(x.N);
+        fix(x.S);
+        fix(x.F);
         fix(x.rank);
         fix(x.tsum);
         fix(x.meta);
@@ -1901,14 +2020,15 @@ k_frontier(const __grid_constant__ XArgs a_, const __grid_constant__ XOne one_, 
                 __syncthreads();
                 if (next >= left) break;
                 load_query<BATCH>(o, a, one_, a.left[next], blockIdx.x);
-                x_plan(a, o, solo);
+                if (o.t.wide) x_plan<true>(a, o, solo);
+                else x_plan<false>(a, o, solo);
                 x_wedge(a, o, solo, 1u, o.t.maxlev, true);
                 x_outputs(a, o, solo);
             }
         } else {
             for (uint32_t i = 0; i < left && ok; ++i) {
                 if (BATCH) load_query<BATCH>(o, a, one_, a.left[i], 0);
-                if (plan) ok = x_plan(a, o, grid);
+                if (plan) ok = o.t.wide ? x_plan<true>(a, o, grid) : x_plan<false>(a, o, grid);
                 const uint32_t l1 = BATCH ? o.t.maxlev : lend;
                 if (ok && l1) ok = x_wedge(a, o, grid, BATCH ? 1u : lbeg, l1, fin != 0);
                 if (ok && fin) x_outputs(a, o, grid);
@@ -1958,7 +2078,8 @@ __global__ void k_out_records(uint32_t m, const uint32_t *__restrict__ off, cons
 
 // start[i] = first position of entry i's window in the list before (0-based):
 // its index b when set, else the first row of the tail's segment there (the
-// rows with smaller heads come before it). A row of blocks per list.
+// rows with smaller heads come before it); and the longest window. A row of
+// blocks per list.
 struct WindowList {
     uint32_t count, prev_count;
     const uint32_t *a, *b, *src, *prev_head;
@@ -1966,10 +2087,12 @@ struct WindowList {
 };
 struct WindowLists {
     WindowList l[6];
+    uint32_t *longest;  // per list
 };
 __global__ void k_window_start(const __grid_constant__ WindowLists lists)
 {
     const WindowList &L = lists.l[blockIdx.y];
+    uint32_t most = 0;
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < L.count; i += gridDim.x * blockDim.x) {
         uint32_t s = L.b[i];
         if (!s && L.a[i]) {
@@ -1983,7 +2106,10 @@ __global__ void k_window_start(const __grid_constant__ WindowLists lists)
             s = lo;
         }
         L.start[i] = s;
+        if (L.a[i] > s) most = max(most, L.a[i] - s);
     }
+    most = __reduce_max_sync(0xffffffffu, most);
+    if ((threadIdx.x & 31u) == 0 && most) atomicMax(lists.longest + blockIdx.y, most);
 }
 
 }  // namespace
@@ -2057,9 +2183,11 @@ rr_status frontier_load(Graph &g, cudaStream_t st)
         most = std::max<uint64_t>(most, x.L->count);
     }
     if (!most) return RR_OK;
-    RR_CUDA(g.x_win.reserve(total * 4));
+    RR_CUDA(g.x_win.reserve((total + std::size(w)) * 4));
     uint32_t *at = g.x_win.as<uint32_t>();
     WindowLists lists{};
+    lists.longest = at + total;
+    RR_CUDA(cudaMemsetAsync(lists.longest, 0, sizeof g.x_longest, st));
     for (size_t i = 0; i < std::size(w); ++i) {
         auto &x = w[i];
         *x.start = at;
@@ -2069,24 +2197,27 @@ rr_status frontier_load(Graph &g, cudaStream_t st)
     }
     k_window_start<<<dim3((unsigned)std::min<uint64_t>(152ull * 32, (most + 255) / 256), (unsigned)std::size(w)), 256, 0, st>>>(lists);
     RR_LAUNCHED();
+    // (the load waits for the stream at its end)
+    RR_CUDA(cudaMemcpyAsync(g.x_longest, lists.longest, sizeof g.x_longest, cudaMemcpyDeviceToHost, st));
     return RR_OK;
 }
 
 static void x_lists(const Graph &g, XList *out)
 {
-    auto set = [&](uint32_t id, const RowList &L, const uint32_t *lo, const DevBuf &hi) {
+    auto set = [&](uint32_t id, const RowList &L, const uint32_t *lo, const DevBuf &hi, uint32_t longest) {
         out[id] = XList{L.head.as<uint32_t>(), L.eid.as<uint32_t>(), L.src.as<uint32_t>(), lo,
-                        hi.as<uint32_t>(), L.time.as<uint32_t>(), (uint32_t)L.count, (uint32_t)(L.count / 32 + 1)};
+                        hi.as<uint32_t>(), L.time.as<uint32_t>(), (uint32_t)L.count, (uint32_t)(L.count / 32 + 1), longest};
     };
-    set(kXProd, g.prod_list, g.prod_list.w0, g.prod_list.a0);
-    set(kXState, g.state_list, g.state_list.w0, g.state_list.a0);
-    set(kXDeep1, g.deep_list, g.deep_list.w1, g.deep_list.a1);
-    set(kXDeep3, g.deep_list, g.deep_list.w3, g.deep_list.a3);
-    set(kXWin, g.win_list, g.win_list.w0, g.win_list.a0);
-    set(kXTail, g.tail_list, g.tail_list.w1, g.tail_list.a1);
-    set(kXTail3, g.tail3_list, g.tail3_list.w3, g.tail3_list.a3);
+    // (in the order of frontier_load's windows)
+    set(kXProd, g.prod_list, g.prod_list.w0, g.prod_list.a0, 0);
+    set(kXState, g.state_list, g.state_list.w0, g.state_list.a0, g.x_longest[0]);
+    set(kXDeep1, g.deep_list, g.deep_list.w1, g.deep_list.a1, g.x_longest[2]);
+    set(kXDeep3, g.deep_list, g.deep_list.w3, g.deep_list.a3, g.x_longest[4]);
+    set(kXWin, g.win_list, g.win_list.w0, g.win_list.a0, g.x_longest[1]);
+    set(kXTail, g.tail_list, g.tail_list.w1, g.tail_list.a1, g.x_longest[3]);
+    set(kXTail3, g.tail3_list, g.tail3_list.w3, g.tail3_list.a3, g.x_longest[5]);
     out[kXAll] = XList{g.row_head.as<uint32_t>(), g.row_eid.as<uint32_t>(), g.row_src.as<uint32_t>(), nullptr, nullptr,
-                       g.row_t.as<uint32_t>(), (uint32_t)g.m, (uint32_t)(g.m / 32 + 1)};
+                       g.row_t.as<uint32_t>(), (uint32_t)g.m, (uint32_t)(g.m / 32 + 1), 0};
 }
 
 // Bump allocation of the scratch: offsets + 1 in place of addresses.
@@ -2150,6 +2281,14 @@ static uint64_t x_template(const XList *lists, uint32_t k, bool every, bool mult
     if (!every)
         for (uint32_t i = 0; i < t.nll; ++i)
             if (!t.ll[i].out) t.ll[i].N = b.take<uint32_t>(t.ll[i].words);
+    for (uint32_t i = 0; i < t.nll; ++i) {  // levels read by long windows
+        const XLL &x = t.ll[i];
+        if (x.level < 2 || lists[x.list].longest <= kLongWords * 32u || t.ll[x.prev].S) continue;
+        XLL &p = t.ll[x.prev];
+        t.wide = 1;
+        p.S = b.take<uint32_t>(x_sum_words(p.words));
+        if (!every) p.F = b.take<uint32_t>(x_sum_words(p.words));
+    }
     t.clear4 = (uint32_t)(b.used / 16);
     uint64_t ping[2] = {0, 0}, ipw[2] = {0, 0}, supw = 0;
     for (uint32_t i = 0; i < t.nll; ++i) {

@@ -359,6 +359,7 @@ struct Graph {
     DevBuf x_tab;
     int x_sms = 0;
     uint32_t x_smem_max = 0;
+    uint32_t x_longest[6] = {0};  // rows of the longest window of each such list (as frontier_load orders them)
     std::vector<uint8_t> h_color;
     // load flags that choose a form of the sieve-point engine keep every query on it
     bool point_flags = false;

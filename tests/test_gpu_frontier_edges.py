@@ -66,3 +66,52 @@ def test_a_source_edge_into_a_hub(followers, edges):
         for i, q in enumerate(qs):
             b1, w1 = G.reach(0, q["k"], q["seed"])
             assert np.array_equal(w[i], w1) and np.array_equal(bm[i], b1), i
+
+
+def exchange(d, wait, ncolors=0, seed=0):
+    """A hub 0 and d leaves, an edge from and to every leaf; leaf 1 is the source."""
+    rng = np.random.default_rng([seed, d])
+    leaf = 1 + np.arange(d)
+    tau = 1000
+    t = np.concatenate([rng.integers(1, tau, d), rng.integers(1, tau, d)])
+    t[0] = tau // 8  # the source's only edge: rows before it have windows without a walk
+    delta = np.concatenate([[wait], rng.integers(0, tau, d)])
+    src, dst = np.concatenate([leaf, np.zeros(d, int)]), np.concatenate([np.zeros(d, int), leaf])
+    return graph_of(src, dst, t, delta, ncolors)
+
+
+@pytest.mark.parametrize("d,wait", [(4_000, 1000), (4_500, 1000), (6_000, 700), (150_001, 900), (4_600_000, 1000)])
+def test_windows_longer_than_the_direct_reads(d, wait):
+    # one dominant vertex and long waits: windows of d rows, by each level of
+    # their summaries (from 4,097, 131,000 and 4,194,000 rows on). A second hub
+    # continues the paths: leaf, hub, leaf, hub, leaf, and no longer ones (walks
+    # of six vertices exist, and cancel)
+    import torch
+    g = exchange(d, wait, ncolors=2)
+    h2 = g["n"]
+    rng = np.random.default_rng(d)
+    leaf = 1 + np.arange(d)
+    g = graph_of(np.concatenate([g["src"], leaf, np.full(d, h2)]), np.concatenate([g["dst"], np.full(d, h2), leaf]),
+                 np.concatenate([g["t"], rng.integers(1, 1000, 2 * d)]), np.concatenate([g["delta"], [wait]]), 2)
+    n = g["n"]
+    ks = (3, 4, 5, 6) if d < 1_000_000 else (5,)
+    with capi.Graph(g) as G, capi.Graph(g, capi.FLAG_DENSE_STATE) as H:
+        for k in ks:
+            for m in (None, [0, 1] * (k // 2) + [1] * (k % 2)):
+                b, w = G.reach(1, k, 3 + k, motif=m)
+                b1, w1 = H.reach(1, k, 3 + k, motif=m)
+                assert np.array_equal(w, w1) and np.array_equal(b, b1), (k, m)
+                assert m is not None or w.any() == (k <= 5), k
+        if d < 1_000_000:
+            d_w = torch.full((4, n), -1, dtype=torch.int64, device="cuda")
+            capi.rr_reach_atmost_device(G.handle, 1, 5, 9, d_w)
+            torch.cuda.synchronize()
+            for k in (2, 3, 4, 5):
+                assert np.array_equal(d_w[k - 2].cpu().numpy().view(np.uint64), H.reach(1, k, 9)[1]), k
+            for a, b in zip(G.arrival(1, 5, 9), H.arrival(1, 5, 9)):
+                assert np.array_equal(a, b)
+            qs = [{"source": 1 + i % 3, "k": 4 + i % 3, "seed": i, "motif": None} for i in range(45)]
+            w, _, st = batch(G, n, qs)
+            assert not st.any()
+            for i in range(0, 45, 4):
+                assert np.array_equal(w[i], H.reach(qs[i]["source"], qs[i]["k"], i)[1]), i
