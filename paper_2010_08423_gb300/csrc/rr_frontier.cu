@@ -2612,8 +2612,8 @@ rr_status frontier_query(const Graph &g, Workspace &ws, const rr_query *q, bool 
 
 // A batch in one launch: the queries' descriptions go to the device with one
 // copy, blocks take queries from a counter (x_tiny), and the queries that do not
-// fit follow, one per block when there are many (each block with its own region
-// of scratch) or one at a time by the whole grid. idx: the queries of qs to run
+// fit follow, one per block when there are many and their regions of scratch are
+// small, or one at a time by the whole grid. idx: the queries of qs to run
 // (the witnesses of all nq are cleared); false when one query's scratch does not
 // fit `budget`.
 bool frontier_batch(const Graph &g, const rr_query *qs, uint32_t nq, const std::vector<uint32_t> &idx, uint64_t budget,
@@ -2635,10 +2635,17 @@ bool frontier_batch(const Graph &g, const rr_query *qs, uint32_t nq, const std::
             if (used[k]) stride = std::max(stride, x_template(a.lists, k, false, false, false, tm[k]));
         stride = (stride + 255) / 256 * 256;
         if (stride > budget) return RR_EAGAIN;
-        // a region per block while they stay within kBatchScratch
+        // Queries one per block only where kBatchScratch holds a region for every
+        // block of the grid. Larger regions belong to graphs whose queries are long
+        // on one SM, and fewer of them leave SMs idle: 64 queries on n = 1e6, m = 1e7,
+        // k = 6..12, took 1,322 ms from hubs on six blocks, 64 ms one after another
+        // over the grid (k = 5..8, 53 blocks: 59 and 21 ms; 256 of k = 6..12 from any
+        // vertex: 576 and 48 ms). On n = 2e5, m = 2e6 regions of 87 MB, k = 5..8, take
+        // 5.4 ms one per block and 7.7 ms over the grid, of 226 MB 9.5 and 9.6 ms, of
+        // 726 MB (35 blocks) 26.7 and 11.8 ms.
         constexpr uint64_t kBatchScratch = 24ull << 30;
-        const uint64_t room = std::max<uint64_t>(stride, std::min<uint64_t>(budget, kBatchScratch));
-        a.lanes = (uint32_t)std::min<uint64_t>({(uint64_t)g.x_sms, (uint64_t)count, room / stride});
+        const uint64_t room = std::min<uint64_t>(budget, kBatchScratch);
+        a.lanes = room / stride >= (uint64_t)g.x_sms ? std::min<uint32_t>((uint32_t)g.x_sms, count) : 1u;
         RR_CUDA(ws.state.reserve(a.lanes * stride));
         rr_status s = x_control(ws, st, a);
         if (s != RR_OK) return s;

@@ -115,3 +115,36 @@ def test_windows_longer_than_the_direct_reads(d, wait):
             assert not st.any()
             for i in range(0, 45, 4):
                 assert np.array_equal(w[i], H.reach(qs[i]["source"], qs[i]["k"], i)[1]), i
+
+
+def test_a_batch_of_long_queries_uses_the_whole_grid():
+    # scratch for a few queries at a time (4 GB each): over the grid one after
+    # another, in about the time of single queries, not on as many blocks as fit
+    # (20 times that); the margin of three is for the clock
+    import torch
+    g = W.motif_powerlaw()
+    n = g["n"]
+    qs = [{"source": i, "k": 12 if i % 8 == 0 else 9, "seed": 60 + i, "motif": None} for i in range(40)]
+    with capi.Graph(g) as G:
+        d_w = torch.zeros((len(qs), n), dtype=torch.int64, device="cuda")
+        d_1 = torch.zeros((len(qs), n), dtype=torch.int64, device="cuda")
+        st = torch.cuda.current_stream().cuda_stream
+
+        def singles():
+            for i, q in enumerate(qs):
+                capi.rr_reach_device(G.handle, q["source"], q["k"], q["seed"], d_1[i], None, st)
+
+        def timed(f):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            f()
+            torch.cuda.synchronize()
+            a.record()
+            f()
+            b.record()
+            torch.cuda.synchronize()
+            return a.elapsed_time(b)
+
+        one = timed(singles)
+        many = timed(lambda: capi.rr_reach_batch_device(G.handle, qs, d_w, None, None, st))
+        assert torch.equal(d_w, d_1) and bool(d_w.any())
+        assert many < 3 * one, (many, one)
