@@ -283,15 +283,17 @@ __device__ __forceinline__ bool any_words(const uint32_t *A, uint32_t w, uint32_
 // vertices with 20,000, 100,000 and 400,000 edges each way and waits as long as the
 // time range took 0.44, 4.0 and 48.9 ms (0.24, 0.34 and 1.25 ms with summaries), and
 // larger ones would outlast a barrier's wait. So a bitmap that windows of more than
-// kLongWords words read has three summaries, each a bit per word of the level below
+// kWideWords words read has three summaries, each a bit per word of the level below
 // it (at most 2^26 words, 2,048 in the last): S, the words of A that hold a row, and
-// F, the words of N that some window covers whole. A window then takes at most
-// 2 kLongWords words of each level, and the passes are linear in the rows, with a
-// barrier more a layer. Graphs without such windows have no summaries, and passes of
-// their own that read what lies between a window's end words directly (x_plan<false>;
-// with the tests for summaries in one form for both, k = 12 on n = 2,000, m = 30,011
-// took 1.4 % longer). The summaries' functions are inlined: x_plan makes no call
-// where the lanes of a warp have parted.
+// F, the words of N that some window covers whole. A window of more than kLongWords
+// words then takes at most 2 kLongWords words of each level: the passes are linear in
+// the rows, with a barrier more a layer. That barrier is why shorter windows are read
+// directly. Graphs without such windows have kernels without the tests for summaries
+// (x_plan<false>; one form for both: k = 12 on n = 2,000, m = 30,011 +1.4 %, both
+// forms in one kernel: k = 8 arrival and bounded queries on n = 2e5, m = 2e6 +1 %). The
+// summaries' functions are inlined: x_plan makes no call where the lanes of a warp
+// have parted.
+constexpr uint32_t kWideWords = 512;
 constexpr uint32_t kLongWords = 128;
 // Words of the first summary of `words` words, and of all three.
 __host__ __device__ __forceinline__ uint32_t x_sum_level(uint32_t words) { return ((words + 31u) / 32u + 3u) / 4u * 4u; }
@@ -594,7 +596,7 @@ __device__ __noinline__ bool x_plan(const XArgs &a, const XOne &o, View &v)
                     if (hi[x] <= lo[x]) act[x] = false;
                     else if (first == last) act[x] = (fw[x] & m0 & m1) != 0;
                     else if ((fw[x] & m0) || (lw[x] & m1)) act[x] = true;
-                    else if (WIDE && last - first > kLongWords) act[x] = any_long(Ap, P.S, P.words, first + 1u, last);
+                    else if (WIDE && P.S && last - first > kLongWords) act[x] = any_long(Ap, P.S, P.words, first + 1u, last);
                     else act[x] = any_words(Ap, first + 1u, last);
                 }
                 if (check) {
@@ -683,7 +685,7 @@ __device__ __noinline__ bool x_plan(const XArgs &a, const XOne &o, View &v)
                     if (b1 == b0) m[x] &= last;
                     if (m[x] & ~have[x]) atomicOr(Np + b0, m[x]);
                     uint32_t w = b0 + 1;
-                    if (WIDE && b1 - b0 > kLongWords) {
+                    if (WIDE && P.F && b1 - b0 > kLongWords) {
                         mark_long(P.F, P.words, w, b1);
                         w = b1;
                     }
@@ -1946,7 +1948,8 @@ __device__ __forceinline__ void load_query(XOne &o, const XArgs &a, const XOne &
 // First: every query in one block's shared memory (x_tiny). Those that do not
 // fit are left to the bitmap passes: one query at a time by the whole grid, or,
 // when there are many, one per block.
-template <bool BATCH>
+// WIDE: the passes with summaries (x_plan).
+template <bool BATCH, bool WIDE>
 __global__ void __launch_bounds__(kThreads, 1)
 k_frontier(const __grid_constant__ XArgs a_, const __grid_constant__ XOne one_, uint32_t plan, uint32_t lbeg, uint32_t lend,
            uint32_t fin)
@@ -2020,15 +2023,14 @@ k_frontier(const __grid_constant__ XArgs a_, const __grid_constant__ XOne one_, 
                 __syncthreads();
                 if (next >= left) break;
                 load_query<BATCH>(o, a, one_, a.left[next], blockIdx.x);
-                if (o.t.wide) x_plan<true>(a, o, solo);
-                else x_plan<false>(a, o, solo);
+                x_plan<WIDE>(a, o, solo);
                 x_wedge(a, o, solo, 1u, o.t.maxlev, true);
                 x_outputs(a, o, solo);
             }
         } else {
             for (uint32_t i = 0; i < left && ok; ++i) {
                 if (BATCH) load_query<BATCH>(o, a, one_, a.left[i], 0);
-                if (plan) ok = o.t.wide ? x_plan<true>(a, o, grid) : x_plan<false>(a, o, grid);
+                if (plan) ok = x_plan<WIDE>(a, o, grid);
                 const uint32_t l1 = BATCH ? o.t.maxlev : lend;
                 if (ok && l1) ok = x_wedge(a, o, grid, BATCH ? 1u : lbeg, l1, fin != 0);
                 if (ok && fin) x_outputs(a, o, grid);
@@ -2145,19 +2147,20 @@ rr_status frontier_load(Graph &g, cudaStream_t st)
     int smem = 0;
     RR_CUDA(cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, g.dev));
     g.x_smem_max = (uint32_t)smem;
-    for (const void *f : {(const void *)k_frontier<false>, (const void *)k_frontier<true>}) {
+    const void *const kernels[] = {(const void *)k_frontier<false, false>, (const void *)k_frontier<true, false>,
+                                   (const void *)k_frontier<false, true>, (const void *)k_frontier<true, true>};
+    for (const void *f : kernels) {
         cudaFuncAttributes at{};
         RR_CUDA(cudaFuncGetAttributes(&at, f));
         g.x_smem_max = std::min<uint32_t>(g.x_smem_max, (uint32_t)(smem - (int)at.sharedSizeBytes));
     }
     g.x_smem_max = g.x_smem_max / 64 * 64;
-    RR_CUDA(cudaFuncSetAttribute(k_frontier<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.x_smem_max));
-    RR_CUDA(cudaFuncSetAttribute(k_frontier<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.x_smem_max));
+    for (const void *f : kernels) RR_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.x_smem_max));
     // blocks that wait on one another need a cooperative launch with a block on
     // every SM; where that is not to be had, queries run over sieve points
     int coop = 0;
     RR_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, g.dev));
-    for (const void *f : {(const void *)k_frontier<false>, (const void *)k_frontier<true>}) {
+    for (const void *f : kernels) {
         int per = 0;
         RR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, f, kThreads, g.x_smem_max));
         if (!coop || per < 1) g.x_sms = 0;
@@ -2283,7 +2286,7 @@ static uint64_t x_template(const XList *lists, uint32_t k, bool every, bool mult
             if (!t.ll[i].out) t.ll[i].N = b.take<uint32_t>(t.ll[i].words);
     for (uint32_t i = 0; i < t.nll; ++i) {  // levels read by long windows
         const XLL &x = t.ll[i];
-        if (x.level < 2 || lists[x.list].longest <= kLongWords * 32u || t.ll[x.prev].S) continue;
+        if (x.level < 2 || lists[x.list].longest <= kWideWords * 32u || t.ll[x.prev].S) continue;
         XLL &p = t.ll[x.prev];
         t.wide = 1;
         p.S = b.take<uint32_t>(x_sum_words(p.words));
@@ -2453,7 +2456,7 @@ bool frontier_fits(const Graph &g, Workspace &ws, uint32_t k, uint64_t budget, b
     return true;
 }
 
-template <bool BATCH>
+template <bool BATCH, bool WIDE>
 static rr_status x_launch(const Graph &g, const XArgs &a, const XOne &one, cudaStream_t st)
 {
     cudaLaunchAttribute at[1];
@@ -2468,7 +2471,7 @@ static rr_status x_launch(const Graph &g, const XArgs &a, const XOne &one, cudaS
     cfg.numAttrs = 1;
     if (BATCH || a.tiny) {
         const int ts = timing_begin(st);
-        RR_CUDA(cudaLaunchKernelEx(&cfg, k_frontier<BATCH>, a, one, 1u, 1u, one.t.maxlev, 1u));
+        RR_CUDA(cudaLaunchKernelEx(&cfg, k_frontier<BATCH, WIDE>, a, one, 1u, 1u, one.t.maxlev, 1u));
         timing_end(ts, kTimeBatch, st);
         RR_LAUNCHED();
         return RR_OK;
@@ -2477,7 +2480,7 @@ static rr_status x_launch(const Graph &g, const XArgs &a, const XOne &one, cudaS
     // layer, each timed
     for (uint32_t l = 0; l <= one.t.maxlev; ++l) {
         const int ts = timing_begin(st);
-        RR_CUDA(cudaLaunchKernelEx(&cfg, k_frontier<BATCH>, a, one, l ? 0u : 1u, l, l, l == one.t.maxlev ? 1u : 0u));
+        RR_CUDA(cudaLaunchKernelEx(&cfg, k_frontier<BATCH, WIDE>, a, one, l ? 0u : 1u, l, l, l == one.t.maxlev ? 1u : 0u));
         timing_end(ts, l == one.t.maxlev ? kTimeLast : l <= 1 ? kTimeFirst : l == 2 ? kTimeSecond : l == 3 ? kTimeThird : kTimeMid, st);
         RR_LAUNCHED();
     }
@@ -2607,7 +2610,7 @@ rr_status frontier_query(const Graph &g, Workspace &ws, const rr_query *q, bool 
     a.bzero = d_bitmap;
     a.bzero_n = d_bitmap ? (g.n + 7) / 8 : 0;
     a.tiny = g_timing.load(std::memory_order_relaxed) ? 0u : 1u;
-    return x_launch<false>(g, a, one, st);
+    return one.t.wide ? x_launch<false, true>(g, a, one, st) : x_launch<false, false>(g, a, one, st);
 }
 
 // A batch in one launch: the queries' descriptions go to the device with one
@@ -2630,9 +2633,13 @@ bool frontier_batch(const Graph &g, const rr_query *qs, uint32_t nq, const std::
     const size_t tbytes = sizeof(XTmpl) * (kXMaxLabels + 2), qbytes = sizeof(XQuery) * (size_t)count;
     auto run = [&]() -> rr_status {
         uint64_t stride = 0;
+        bool wide = false;
         std::vector<XTmpl> tm(kXMaxLabels + 2);
         for (uint32_t k = 2; k <= kXMaxLabels + 1; ++k)
-            if (used[k]) stride = std::max(stride, x_template(a.lists, k, false, false, false, tm[k]));
+            if (used[k]) {
+                stride = std::max(stride, x_template(a.lists, k, false, false, false, tm[k]));
+                wide |= tm[k].wide != 0;
+            }
         stride = (stride + 255) / 256 * 256;
         if (stride > budget) return RR_EAGAIN;
         // Queries one per block only where kBatchScratch holds a region for every
@@ -2678,7 +2685,7 @@ bool frontier_batch(const Graph &g, const rr_query *qs, uint32_t nq, const std::
         a.status = d_status && count == nq ? d_status : nullptr;
         a.tiny = 1;
         static const XOne none{};
-        return x_launch<true>(g, a, none, st);
+        return wide ? x_launch<true, true>(g, a, none, st) : x_launch<true, false>(g, a, none, st);
     };
     *ret = run();
     if (*ret != RR_EAGAIN) return true;

@@ -80,10 +80,11 @@ def exchange(d, wait, ncolors=0, seed=0):
     return graph_of(src, dst, t, delta, ncolors)
 
 
-@pytest.mark.parametrize("d,wait", [(4_000, 1000), (4_500, 1000), (6_000, 700), (150_001, 900), (4_600_000, 1000)])
+@pytest.mark.parametrize("d,wait", [(4_000, 1000), (16_000, 1000), (17_000, 1000), (23_000, 800),
+                                    (150_001, 900), (4_600_000, 1000)])
 def test_windows_longer_than_the_direct_reads(d, wait):
     # one dominant vertex and long waits: windows of d rows, by each level of
-    # their summaries (from 4,097, 131,000 and 4,194,000 rows on). A second hub
+    # their summaries (from 16,385, 131,000 and 4,194,000 rows on). A second hub
     # continues the paths: leaf, hub, leaf, hub, leaf, and no longer ones (walks
     # of six vertices exist, and cancel)
     import torch
