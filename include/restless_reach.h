@@ -166,8 +166,9 @@ rr_status rr_reach_sync(const rr_graph *g, const rr_query *q, uint8_t *bitmap,
  * fine-grained, set-of-sources and extraction calls, rr_autotune) may be
  * issued on different streams -- each call's stream first waits, on the
  * device, for the previous such call's work. A query whose kernel gave up a
- * bounded wait is reported as RR_ETIMEDOUT by rr_reach_sync itself, for the
- * calls that only enqueue by the next call on the graph. */
+ * bounded wait is reported as RR_ETIMEDOUT by rr_reach_sync itself, in a batch
+ * by the query's d_status, for other calls that only enqueue (a batch without
+ * d_status too) once by a later call on the graph, which then enqueues nothing. */
 rr_status rr_reach_device(const rr_graph *g, const rr_query *q, uint8_t *d_bitmap,
                           uint64_t *d_witness, void *stream);
 
@@ -447,6 +448,14 @@ rr_status rr_bench_gf_mul(uint32_t blocks, uint32_t threads, uint32_t iters, uin
  * above 10 s. Not part of the paper's method. */
 rr_status rr_debug_wait_probe(uint64_t timeout_ns, int32_t abort_preset, int32_t *status,
                               uint64_t *elapsed_ns);
+/* rr_debug_frontier: how whole queries on `g` meet inside their kernel, so that
+ * the failure path of its bounded waits can be tested without a fault. wait_ns:
+ * the longest a block waits for the others (0: the 10 s it is otherwise). absent:
+ * the kernel's last block leaves before this meeting, and the others wait in vain:
+ * 1 the first, 2 (batches) the one after the queries that fit a block, 0 none.
+ * Call it while no query on the graph is queued or running. RR_EINVAL for a NULL
+ * graph, a limit above 10 s, absent > 2. Not part of the paper's method. */
+rr_status rr_debug_frontier(rr_graph *g, uint64_t wait_ns, uint32_t absent);
 /* rr_debug_draw: out[i] = draw(key, first + i) on the device, HOST out. */
 rr_status rr_debug_draw(uint64_t key, uint64_t first, uint64_t count, uint64_t *out);
 

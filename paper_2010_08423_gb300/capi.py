@@ -82,7 +82,7 @@ EXPORTED = [
     "rr_timing_enable", "rr_timing_read", "rr_reach_device_noalloc", "rr_reach_atmost_device",
     "rr_reach_arrival_device", "rr_extract_path", "rr_reach_sources_device", "rr_bench_gf_mul",
     "rr_debug_wait_probe", "rr_reach_bounded_device", "rr_reach_range_device",
-    "rr_autotune_batch", "rr_set_batch_tuning", "rr_get_batch_tuning",
+    "rr_autotune_batch", "rr_set_batch_tuning", "rr_get_batch_tuning", "rr_debug_frontier",
 ]
 
 _lib = None
@@ -119,6 +119,7 @@ def load(build_if_missing: bool = True):
         "rr_reach_arrival_device": [vp, pq, vp, vp, vp, vp, vp],
         "rr_extract_path": [vp, pq, u32, vp, vp, vp],
         "rr_bench_gf_mul": [u32, u32, u32, vp, ctypes.POINTER(u64), vp],
+        "rr_debug_frontier": [vp, u64, u32],
         "rr_debug_wait_probe": [u64, i32, ctypes.POINTER(i32), ctypes.POINTER(u64)],
         "rr_reach_sources_device": [vp, vp, u32, u32, u64, vp, vp, vp, vp, vp],
         "rr_server_create": [vp, u64, u32, ctypes.POINTER(vp)],
@@ -314,6 +315,11 @@ def rr_debug_wait_probe(timeout_ns: int, abort_preset: bool = False):
     _check(load().rr_debug_wait_probe(int(timeout_ns), 1 if abort_preset else 0, ctypes.byref(st),
                                       ctypes.byref(ns)))
     return st.value, ns.value
+
+
+def rr_debug_frontier(g, wait_ns: int = 0, absent: int = 0):
+    """Limit of the waits inside a whole query's kernel, and the meeting its last block misses."""
+    _check(load().rr_debug_frontier(g, int(wait_ns), int(absent)))
 
 
 def rr_bench_gf_mul(blocks, threads, iters, d_sink, stream=None) -> int:

@@ -427,6 +427,18 @@ rr_status rr_debug_wait_probe(uint64_t timeout_ns, int32_t abort_preset, int32_t
     return debug_wait_probe(timeout_ns, abort_preset, status, elapsed_ns);
 }
 
+rr_status rr_debug_frontier(rr_graph *g, uint64_t wait_ns, uint32_t absent)
+{
+    clear_error();
+    if (!g) return fail(RR_EINVAL, "rr_debug_frontier: NULL graph");
+    if (wait_ns > 10000000000ull) return fail(RR_EINVAL, "rr_debug_frontier: limit above 10 s");
+    if (absent > 2) return fail(RR_EINVAL, "rr_debug_frontier: absent must be 0, 1 or 2");
+    std::lock_guard<std::mutex> lk(g->mu);
+    g->x_wait_ns = wait_ns ? wait_ns : 10000000000ull;
+    g->x_absent = absent;
+    return RR_OK;
+}
+
 rr_status rr_bench_gf_mul(uint32_t blocks, uint32_t threads, uint32_t iters, uint64_t *d_sink,
                           uint64_t *mults, void *stream)
 {

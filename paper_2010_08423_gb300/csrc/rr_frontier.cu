@@ -190,6 +190,7 @@ struct View {
     uint32_t b, n;  // this block among n
     uint32_t *ctr, *err;  // ctr: two, 128 bytes apart
     Meetings *meet;       // shared memory, kept by thread 0
+    uint64_t limit;       // of a wait (ns)
     bool some = false;    // some block came to the last barrier with something to tell
     // worker w of n, the items before `base` dealt out: its first item from there on
     __device__ static uint32_t first_item(uint32_t base, uint32_t w, uint32_t n)
@@ -229,7 +230,7 @@ struct View {
                 }
                 if ((it & 1023u) != 1023u) continue;
                 if (!t0) t0 = now_ns();
-                if (*(volatile uint32_t *)err || now_ns() - t0 > 10000000000ull) break;
+                if (*(volatile uint32_t *)err || now_ns() - t0 > limit) break;
             }
             if (!good) *(volatile uint32_t *)err = 1u;
             v /= kTellOne;
@@ -281,7 +282,7 @@ __device__ __forceinline__ bool any_words(const uint32_t *A, uint32_t w, uint32_
 // Long windows. A pass that reads every word of every window takes (rows that
 // leave a vertex) x (rows that enter it) / 32 words a layer: k = 5 through two
 // vertices with 20,000, 100,000 and 400,000 edges each way and waits as long as the
-// time range took 0.44, 4.0 and 48.9 ms (0.24, 0.34 and 1.25 ms with summaries), and
+// time range took 0.44, 4.0 and 48.9 ms (0.36, 0.34 and 1.26 ms with summaries), and
 // larger ones would outlast a barrier's wait. So a bitmap that windows of more than
 // kWideWords words read has three summaries, each a bit per word of the level below
 // it (at most 2^26 words, 2,048 in the last): S, the words of A that hold a row, and
@@ -1961,8 +1962,9 @@ k_frontier(const __grid_constant__ XArgs a_, const __grid_constant__ XOne one_, 
     copy_params(&a, &a_, sizeof(XArgs));
     __syncthreads();
     if (threadIdx.x == 0) meet = Meetings{};
-    View grid{blockIdx.x, gridDim.x, a.ctl, a.err, &meet};
-    bool ok = true;
+    View grid{blockIdx.x, gridDim.x, a.ctl, a.err, &meet, a.limit};
+    auto absent = [&](uint32_t at) { return a.absent == at && blockIdx.x == gridDim.x - 1u; };
+    bool ok = !absent(1);
     // cleared first: witnesses and bitmaps (a single query's first block goes on
     // with the query)
     const uint32_t skip = !BATCH && a.tiny && gridDim.x > 1 ? 1u : 0u;
@@ -1980,7 +1982,7 @@ k_frontier(const __grid_constant__ XArgs a_, const __grid_constant__ XOne one_, 
         for (uint64_t i = gt; i < a.bzero_n; i += nt) a.bzero[i] = 0;
     }
     uint32_t left = BATCH ? 0u : 1u;
-    if (plan && a.tiny) {
+    if (plan && a.tiny && ok) {
         grid.arrive();
         bool cleared = false;
         if (BATCH) {
@@ -1995,9 +1997,12 @@ k_frontier(const __grid_constant__ XArgs a_, const __grid_constant__ XOne one_, 
                 __syncthreads();
                 const int r = x_tiny(a, o.q, false, grid, cleared);
                 ok = r != kTinyFailed;
-                if (r == kTinyNoFit && threadIdx.x == 0) a.left[atomicAdd(a.ctl + 3, 1u)] = q;
+                if (threadIdx.x == 0) {
+                    if (r == kTinyNoFit) a.left[atomicAdd(a.ctl + 3, 1u)] = q;
+                    else if (r == kTinyDone) a.xq[q].done = 1;
+                }
             }
-            ok = ok && grid.sync();
+            ok = ok && !absent(2) && grid.sync();
             if (ok) left = *(volatile uint32_t *)(a.ctl + 3);
         } else if (blockIdx.x == 0) {
             copy_params(&o.q, &one_.q, sizeof(XQuery));
@@ -2016,7 +2021,7 @@ k_frontier(const __grid_constant__ XArgs a_, const __grid_constant__ XOne one_, 
     if (!BATCH && ok && left) load_query<BATCH>(o, a, one_, 0, 0);
     if (ok && left) {
         if (BATCH && a.lanes > 1 && left >= gridDim.x / 4) {
-            View solo{0u, 1u, a.ctl, a.err, &meet};
+            View solo{0u, 1u, a.ctl, a.err, &meet, a.limit};
             while (blockIdx.x < a.lanes) {
                 __syncthreads();
                 if (threadIdx.x == 0) next = atomicAdd(a.ctl + 4, 1u);
@@ -2026,6 +2031,7 @@ k_frontier(const __grid_constant__ XArgs a_, const __grid_constant__ XOne one_, 
                 x_plan<WIDE>(a, o, solo);
                 x_wedge(a, o, solo, 1u, o.t.maxlev, true);
                 x_outputs(a, o, solo);
+                if (threadIdx.x == 0) a.xq[a.left[next]].done = 1;
             }
         } else {
             for (uint32_t i = 0; i < left && ok; ++i) {
@@ -2035,15 +2041,24 @@ k_frontier(const __grid_constant__ XArgs a_, const __grid_constant__ XOne one_, 
                 if (ok && l1) ok = x_wedge(a, o, grid, BATCH ? 1u : lbeg, l1, fin != 0);
                 if (ok && fin) x_outputs(a, o, grid);
                 if (BATCH && ok) ok = grid.sync();  // the scratch is the next query's
+                if (BATCH && ok && blockIdx.x == 0 && threadIdx.x == 0) a.xq[a.left[i]].done = 1;
             }
         }
     }
-    if (BATCH && !ok && a.status)
-        for (uint32_t i = threadIdx.x; i < a.nq; i += blockDim.x) a.status[i] = (int32_t)RR_ETIMEDOUT;
-    // the last block to leave clears the counters for the next launch
+    // the last block to leave marks a failed batch's unfinished queries, and clears
+    // the counters for the next launch
     __syncthreads();
     if (threadIdx.x == 0) {
+        if (!ok) __threadfence();  // (wait() has set err)
         if (atomicAdd(a.ctl + 1, 1u) == gridDim.x - 1) {
+            if (BATCH && a.status) {
+                if (*(volatile uint32_t *)a.err) {
+                    __threadfence();
+                    for (uint32_t q = 0; q < a.nq; ++q)
+                        if (!*(volatile uint32_t *)&a.xq[q].done) a.status[a.xq[q].index] = (int32_t)RR_ETIMEDOUT;
+                }
+                a.ctl[5] = 0;
+            }
             for (int i = 0; i < 5; ++i) a.ctl[i] = 0;
             a.ctl[32] = 0;
         }
@@ -2507,8 +2522,10 @@ rr_status frontier_error(Workspace &ws)
     return fail(RR_ETIMEDOUT, "a bounded wait of the query's kernel expired");
 }
 
-static rr_status x_control(Workspace &ws, cudaStream_t st, XArgs &a)
+static rr_status x_control(const Graph &g, Workspace &ws, cudaStream_t st, XArgs &a)
 {
+    a.limit = g.x_wait_ns;
+    a.absent = g.x_absent;
     rr_status s = frontier_reserve(ws, st);
     if (s == RR_OK) s = frontier_error(ws);
     if (s != RR_OK) return s;
@@ -2586,7 +2603,7 @@ rr_status frontier_query(const Graph &g, Workspace &ws, const rr_query *q, bool 
 {
     XArgs a{};
     x_args(g, a);
-    rr_status s = x_control(ws, st, a);
+    rr_status s = x_control(g, ws, st, a);
     if (s != RR_OK) return s;
     XOne one;
     x_template(a.lists, q->k, every, src != nullptr, d_R != nullptr, one.t);
@@ -2654,7 +2671,7 @@ bool frontier_batch(const Graph &g, const rr_query *qs, uint32_t nq, const std::
         const uint64_t room = std::min<uint64_t>(budget, kBatchScratch);
         a.lanes = room / stride >= (uint64_t)g.x_sms ? std::min<uint32_t>((uint32_t)g.x_sms, count) : 1u;
         RR_CUDA(ws.state.reserve(a.lanes * stride));
-        rr_status s = x_control(ws, st, a);
+        rr_status s = x_control(g, ws, st, a);
         if (s != RR_OK) return s;
         RR_CUDA(B.xq.reserve(tbytes + qbytes));
         RR_CUDA(B.left.reserve((size_t)count * 4));
@@ -2666,6 +2683,7 @@ bool frontier_batch(const Graph &g, const rr_query *qs, uint32_t nq, const std::
         for (uint32_t j = 0; j < count; ++j) {
             const uint32_t i = idx[j];
             x_query(g, qs[i], false, false, hq[j]);
+            hq[j].index = i;
             hq[j].S = d_witness + (size_t)i * g.n;
             hq[j].bitmap = d_bitmaps ? d_bitmaps + (size_t)i * nb : nullptr;
         }
@@ -2682,7 +2700,8 @@ bool frontier_batch(const Graph &g, const rr_query *qs, uint32_t nq, const std::
         a.szero_n = (uint64_t)g.n * nq;
         a.bzero = d_bitmaps;
         a.bzero_n = d_bitmaps ? (uint64_t)nb * nq : 0;
-        a.status = d_status && count == nq ? d_status : nullptr;
+        a.status = d_status;
+        if (d_status) a.err = a.ctl + 5;  // the caller looks at the statuses: nothing left for the next call to report
         a.tiny = 1;
         static const XOne none{};
         return wide ? x_launch<true, true>(g, a, none, st) : x_launch<true, false>(g, a, none, st);

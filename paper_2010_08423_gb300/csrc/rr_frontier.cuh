@@ -41,6 +41,7 @@ struct XQuery {
     const uint8_t *vmask;                 // deleted vertices or null
     const uint32_t *slist;
     const uint8_t *smask;
+    uint32_t index, done;                 // batch form: place in the call's list; its results are written
     uint8_t first[256], mu[256];          // coloured: first shade and multiplicity per colour
 };
 
@@ -93,10 +94,13 @@ struct XArgs {
     uint64_t szero_n;
     uint8_t *bzero;
     uint64_t bzero_n;
-    uint32_t *ctl;         // [0], [32] barriers, [1] blocks done, [2] next query, [3] queries left, [4] next of them
+    uint32_t *ctl;         // [0], [32] barriers, [1] blocks done, [2] next query, [3] queries left, [4] next of them,
+                           // [5] batch form with status: its err
     uint32_t *left;        // batch form: the queries left to the bitmap passes
-    int32_t *status;       // batch form: per query, RR_ETIMEDOUT when a wait gave up
-    uint32_t *err;         // set when a bounded wait gave up
+    int32_t *status;       // batch form: by index, RR_ETIMEDOUT for queries unfinished when a wait gave up, or null
+    uint32_t *err;         // set when a bounded wait gave up: the host's flag, with status ctl[5]
+    uint64_t limit;        // of such a wait (ns)
+    uint32_t absent;       // (tests) the last block leaves before this meeting: 1 the first, 2 a batch's second
     const uint8_t *color;
     const uint32_t *tab, *packed;  // subset tables
     const uint32_t *ooff;  // edges by (tail, time): offsets (n + 1),

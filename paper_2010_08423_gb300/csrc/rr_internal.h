@@ -359,6 +359,8 @@ struct Graph {
     DevBuf x_tab;
     int x_sms = 0;
     uint32_t x_smem_max = 0;
+    uint64_t x_wait_ns = 10000000000ull;  // limit of a wait at its kernel's barriers
+    uint32_t x_absent = 0;                // rr_debug_frontier
     uint32_t x_longest[6] = {0};  // rows of the longest window of each such list (as frontier_load orders them)
     std::vector<uint8_t> h_color;
     // load flags that choose a form of the sieve-point engine keep every query on it
