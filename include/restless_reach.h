@@ -453,9 +453,11 @@ rr_status rr_debug_wait_probe(uint64_t timeout_ns, int32_t abort_preset, int32_t
  * the longest a block waits for the others (0: the 10 s it is otherwise). absent:
  * the kernel's last block leaves before this meeting, and the others wait in vain:
  * 1 the first, 2 (batches) the one after the queries that fit a block, 0 none.
+ * scratch: device bytes above which a query goes to the engines over sieve points
+ * as if they could not be had (0: what the device has).
  * Call it while no query on the graph is queued or running. RR_EINVAL for a NULL
  * graph, a limit above 10 s, absent > 2. Not part of the paper's method. */
-rr_status rr_debug_frontier(rr_graph *g, uint64_t wait_ns, uint32_t absent);
+rr_status rr_debug_frontier(rr_graph *g, uint64_t wait_ns, uint32_t absent, uint64_t scratch);
 /* rr_debug_draw: out[i] = draw(key, first + i) on the device, HOST out. */
 rr_status rr_debug_draw(uint64_t key, uint64_t first, uint64_t count, uint64_t *out);
 

@@ -119,7 +119,7 @@ def load(build_if_missing: bool = True):
         "rr_reach_arrival_device": [vp, pq, vp, vp, vp, vp, vp],
         "rr_extract_path": [vp, pq, u32, vp, vp, vp],
         "rr_bench_gf_mul": [u32, u32, u32, vp, ctypes.POINTER(u64), vp],
-        "rr_debug_frontier": [vp, u64, u32],
+        "rr_debug_frontier": [vp, u64, u32, u64],
         "rr_debug_wait_probe": [u64, i32, ctypes.POINTER(i32), ctypes.POINTER(u64)],
         "rr_reach_sources_device": [vp, vp, u32, u32, u64, vp, vp, vp, vp, vp],
         "rr_server_create": [vp, u64, u32, ctypes.POINTER(vp)],
@@ -317,9 +317,10 @@ def rr_debug_wait_probe(timeout_ns: int, abort_preset: bool = False):
     return st.value, ns.value
 
 
-def rr_debug_frontier(g, wait_ns: int = 0, absent: int = 0):
-    """Limit of the waits inside a whole query's kernel, and the meeting its last block misses."""
-    _check(load().rr_debug_frontier(g, int(wait_ns), int(absent)))
+def rr_debug_frontier(g, wait_ns: int = 0, absent: int = 0, scratch: int = 0):
+    """Limit of the waits inside a whole query's kernel, the meeting its last block misses, the
+    largest scratch of a query it takes."""
+    _check(load().rr_debug_frontier(g, int(wait_ns), int(absent), int(scratch)))
 
 
 def rr_bench_gf_mul(blocks, threads, iters, d_sink, stream=None) -> int:

@@ -427,7 +427,7 @@ rr_status rr_debug_wait_probe(uint64_t timeout_ns, int32_t abort_preset, int32_t
     return debug_wait_probe(timeout_ns, abort_preset, status, elapsed_ns);
 }
 
-rr_status rr_debug_frontier(rr_graph *g, uint64_t wait_ns, uint32_t absent)
+rr_status rr_debug_frontier(rr_graph *g, uint64_t wait_ns, uint32_t absent, uint64_t scratch)
 {
     clear_error();
     if (!g) return fail(RR_EINVAL, "rr_debug_frontier: NULL graph");
@@ -436,6 +436,7 @@ rr_status rr_debug_frontier(rr_graph *g, uint64_t wait_ns, uint32_t absent)
     std::lock_guard<std::mutex> lk(g->mu);
     g->x_wait_ns = wait_ns ? wait_ns : 10000000000ull;
     g->x_absent = absent;
+    g->x_scratch_max = scratch ? scratch : UINT64_MAX;
     return RR_OK;
 }
 

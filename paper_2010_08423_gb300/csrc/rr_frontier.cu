@@ -2460,6 +2460,7 @@ bool frontier_fits(const Graph &g, Workspace &ws, uint32_t k, uint64_t budget, b
     for (uint32_t kk = 2; every && kk < k; ++kk)
         if (!uses_frontier(g, kk)) return false;
     const uint64_t need = frontier_bytes(g, k, every, multi, arrivals);
+    if (need > g.x_scratch_max) return false;
     if (need > ws.state.bytes && budget == 0) {
         size_t free_b = 0, total_b = 0;
         if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return false;
@@ -2467,6 +2468,10 @@ bool frontier_fits(const Graph &g, Workspace &ws, uint32_t k, uint64_t budget, b
     }
     if (need > ws.state.bytes && need > budget) return false;
     const cudaError_t e = ws.state.reserve(need);
+    if (e == cudaErrorMemoryAllocation) {  // (not in one piece, or taken meanwhile: the sieve points need less)
+        (void)cudaGetLastError();
+        return false;
+    }
     if (e != cudaSuccess) *st = cuda_fail(e, "cudaMalloc (query scratch)", __FILE__, __LINE__);
     return true;
 }
@@ -2634,9 +2639,9 @@ rr_status frontier_query(const Graph &g, Workspace &ws, const rr_query *q, bool 
 // copy, blocks take queries from a counter (x_tiny), and the queries that do not
 // fit follow, one per block when there are many and their regions of scratch are
 // small, or one at a time by the whole grid. idx: the queries of qs to run
-// (the witnesses of all nq are cleared); false when one query's scratch does not
-// fit `budget`.
-bool frontier_batch(const Graph &g, const rr_query *qs, uint32_t nq, const std::vector<uint32_t> &idx, uint64_t budget,
+// (the witnesses of all nq are cleared), those whose scratch does not fit `budget`
+// taken out; false when none is left.
+bool frontier_batch(const Graph &g, const rr_query *qs, uint32_t nq, std::vector<uint32_t> &idx, uint64_t budget,
                     uint8_t *d_bitmaps, uint64_t *d_witness, int32_t *d_status, cudaStream_t st, rr_status *ret)
 {
     *ret = RR_OK;
@@ -2644,21 +2649,27 @@ bool frontier_batch(const Graph &g, const rr_query *qs, uint32_t nq, const std::
     BatchBuffers &B = g.batch;
     XArgs a{};
     x_args(g, a);
-    const uint32_t count = (uint32_t)idx.size();
     bool used[kXMaxLabels + 2] = {false};
     for (uint32_t i : idx) used[qs[i].k] = true;
-    const size_t tbytes = sizeof(XTmpl) * (kXMaxLabels + 2), qbytes = sizeof(XQuery) * (size_t)count;
+    budget = std::min(budget, g.x_scratch_max);
     auto run = [&]() -> rr_status {
         uint64_t stride = 0;
-        bool wide = false;
+        bool wide = false, fits = true;
         std::vector<XTmpl> tm(kXMaxLabels + 2);
         for (uint32_t k = 2; k <= kXMaxLabels + 1; ++k)
             if (used[k]) {
-                stride = std::max(stride, x_template(a.lists, k, false, false, false, tm[k]));
+                const uint64_t need = x_template(a.lists, k, false, false, false, tm[k]);  // (whole 256-byte groups)
+                if (need > budget) {
+                    used[k] = fits = false;
+                    continue;
+                }
+                stride = std::max(stride, need);
                 wide |= tm[k].wide != 0;
             }
-        stride = (stride + 255) / 256 * 256;
-        if (stride > budget) return RR_EAGAIN;
+        if (!fits) idx.erase(std::remove_if(idx.begin(), idx.end(), [&](uint32_t i) { return !used[qs[i].k]; }), idx.end());
+        if (idx.empty()) return RR_EAGAIN;
+        const uint32_t count = (uint32_t)idx.size();
+        const size_t tbytes = sizeof(XTmpl) * (kXMaxLabels + 2), qbytes = sizeof(XQuery) * (size_t)count;
         // Queries one per block only where kBatchScratch holds a region for every
         // block of the grid. Larger regions belong to graphs whose queries are long
         // on one SM, and fewer of them leave SMs idle: 64 queries on n = 1e6, m = 1e7,
@@ -2670,7 +2681,17 @@ bool frontier_batch(const Graph &g, const rr_query *qs, uint32_t nq, const std::
         constexpr uint64_t kBatchScratch = 24ull << 30;
         const uint64_t room = std::min<uint64_t>(budget, kBatchScratch);
         a.lanes = room / stride >= (uint64_t)g.x_sms ? std::min<uint32_t>((uint32_t)g.x_sms, count) : 1u;
-        RR_CUDA(ws.state.reserve(a.lanes * stride));
+        cudaError_t e = ws.state.reserve(a.lanes * stride);
+        if (e == cudaErrorMemoryAllocation && a.lanes > 1) {
+            (void)cudaGetLastError();
+            a.lanes = 1;
+            e = ws.state.reserve(stride);
+        }
+        if (e == cudaErrorMemoryAllocation) {
+            (void)cudaGetLastError();
+            return RR_EAGAIN;
+        }
+        RR_CUDA(e);
         rr_status s = x_control(g, ws, st, a);
         if (s != RR_OK) return s;
         RR_CUDA(B.xq.reserve(tbytes + qbytes));

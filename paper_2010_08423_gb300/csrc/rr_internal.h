@@ -361,6 +361,7 @@ struct Graph {
     uint32_t x_smem_max = 0;
     uint64_t x_wait_ns = 10000000000ull;  // limit of a wait at its kernel's barriers
     uint32_t x_absent = 0;                // rr_debug_frontier
+    uint64_t x_scratch_max = UINT64_MAX;  // largest scratch of a query (rr_debug_frontier)
     uint32_t x_longest[6] = {0};  // rows of the longest window of each such list (as frontier_load orders them)
     std::vector<uint8_t> h_color;
     // load flags that choose a form of the sieve-point engine keep every query on it
@@ -535,7 +536,7 @@ struct SourceSet {
     uint32_t count;
 };
 uint64_t frontier_bytes(const Graph &g, uint32_t k, bool every = false, bool multi = false, bool arrivals = false);
-bool frontier_batch(const Graph &g, const rr_query *qs, uint32_t nq, const std::vector<uint32_t> &idx, uint64_t budget,
+bool frontier_batch(const Graph &g, const rr_query *qs, uint32_t nq, std::vector<uint32_t> &idx, uint64_t budget,
                     uint8_t *d_bitmaps, uint64_t *d_witness, int32_t *d_status, cudaStream_t st, rr_status *ret);
 // Reserves ws.state for such a query when it fits `budget` (0: 60% of free device
 // memory, the workspace's own counted in); false: it does not.

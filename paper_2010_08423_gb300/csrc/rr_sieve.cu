@@ -487,7 +487,7 @@ uint64_t query_scratch_bytes(const Graph &g, uint32_t k, uint64_t budget)
     const uint64_t z = (uint64_t)g.n * k * 8ull + 2048;
     if (uses_frontier(g, k)) {
         const uint64_t need = frontier_bytes(g, k);
-        if (need <= budget) return need + z;
+        if (need <= std::min(budget, g.x_scratch_max)) return need + z;
     }
     if (uses_v2(g, k)) {
         if (!choose_shape_v2(g, k, budget, &ppl, &chunk)) return UINT64_MAX;

@@ -149,3 +149,55 @@ def test_a_batch_of_long_queries_uses_the_whole_grid():
         many = timed(lambda: capi.rr_reach_batch_device(G.handle, qs, d_w, None, None, st))
         assert torch.equal(d_w, d_1) and bool(d_w.any())
         assert many < 3 * one, (many, one)
+
+
+@pytest.mark.parametrize("k,scratch", [(4, 1), (7, 1), (9, 1), (9, 3_000_000), (10, 1)])
+def test_calls_whose_scratch_cannot_be_had(k, scratch):
+    # the engines over sieve points in their automatic shapes take what the
+    # frontier engine declines (all of it, or the long queries only), with the
+    # same results
+    import torch
+    g = W.uniform(700, 9_001, 60, 0, 12, 31 + k, ncolors=2)
+    n, s = g["n"], W.first_source(g)
+    motif = [int(g["color"][s])] + [i % 2 for i in range(k - 1)]
+    rng = np.random.default_rng(k)
+    srcs = [int(x) for x in rng.choice(n, 5, replace=False)]
+    qs = [{"source": int(rng.integers(0, n)), "k": 3 + i % (k - 2), "seed": i, "motif": None} for i in range(24)]
+    qs[5]["k"], qs[7]["k"] = k, 2
+
+    def every_call(G):
+        def dev(*shape, dtype=torch.int64):
+            return torch.full(shape, -1, dtype=dtype, device="cuda")
+        out = list(G.reach(s, k, 5)) + list(G.reach(s, k, 6, motif=motif)) + list(G.arrival(s, k, 7)) + list(G.arrival(s, k, 8, motif=motif))
+        w = [dev(n), dev(k - 1, n), dev(n)]
+        r, l = dev(n, dtype=torch.int32), dev(n, dtype=torch.uint8)
+        capi.rr_reach_sources_device(G.handle, srcs, k, 9, w[0])
+        capi.rr_reach_atmost_device(G.handle, s, k, 10, w[1])
+        capi.rr_reach_bounded_device(G.handle, s, k, 11, r, l)
+        capi.rr_reach_device(G.handle, s, k, 12, w[2])
+        torch.cuda.synchronize()
+        out += [x.cpu().numpy() for x in w] + [r.cpu().numpy(), l.cpu().numpy()]
+        bw, bb, bs = batch(G, n, qs)
+        reach = np.nonzero(out[2 * 2 + 2] != capi.NO_ARRIVAL)[0]
+        target = int(reach[0]) if len(reach) else (s + 1) % n
+        path = G.extract_path(s, k, 7, target)
+        return out + [bw, bb, bs], path
+
+    with capi.Graph(g) as G:
+        want, path = every_call(G)
+        assert want[1].any() and path is not None
+        capi.rr_debug_frontier(G.handle, 0, 0, scratch)
+        before = capi.rr_kernel_launches()
+        G.reach(s, k, 5)
+        assert capi.rr_kernel_launches() - before > 2  # (a frontier query: one kernel and the results')
+        got, path2 = every_call(G)
+        assert path2 == path
+        for i, (a, b) in enumerate(zip(want, got)):
+            assert np.array_equal(a, b), i
+        srv = capi.rr_server_create(G.handle, 0, 2)
+        try:
+            ts = [capi.rr_query_submit(srv, q["source"], q["k"], q["seed"]) for q in qs]
+            for i, t in enumerate(ts):
+                assert np.array_equal(capi.rr_query_poll(srv, t, n)[2], want[-3][i]), i
+        finally:
+            capi.rr_server_destroy(srv)
