@@ -1076,6 +1076,8 @@ rr_status atmost_device(const Graph &g, uint32_t source, uint32_t k, uint64_t se
         rr_status fs = RR_OK;
         if (frontier_fits(g, g.ws, k, 0, true, false, false, &fs))
             return fs != RR_OK ? fs : frontier_query(g, g.ws, &q, true, d_bitmap, d_witness, st);
+        fs = frontier_error(g);
+        if (fs != RR_OK) return fs;
     }
     const uint32_t lanes = k - 1;
     size_t free_b = 0, total_b = 0;

@@ -375,6 +375,8 @@ rr_status atmost_arrival_device(const Graph &g, uint32_t source, uint32_t k, uin
             }
             return RR_OK;
         }
+        fs = frontier_error(g);
+        if (fs != RR_OK) return fs;
     }
     const uint32_t lanes = k - 1;
     const size_t mb = (size_t)std::max<uint64_t>(1, g.m) * 8;

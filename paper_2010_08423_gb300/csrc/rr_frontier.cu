@@ -2527,12 +2527,20 @@ rr_status frontier_error(Workspace &ws)
     return fail(RR_ETIMEDOUT, "a bounded wait of the query's kernel expired");
 }
 
+rr_status frontier_error(const Graph &g)
+{
+    rr_status s = frontier_error(g.ws);
+    for (const auto &w : g.fan.ws)  // (every flag, so that a call is reported once)
+        if (const rr_status f = frontier_error(*w); f != RR_OK) s = f;
+    return s;
+}
+
 static rr_status x_control(const Graph &g, Workspace &ws, cudaStream_t st, XArgs &a)
 {
     a.limit = g.x_wait_ns;
     a.absent = g.x_absent;
     rr_status s = frontier_reserve(ws, st);
-    if (s == RR_OK) s = frontier_error(ws);
+    if (s == RR_OK) s = &ws == &g.ws ? frontier_error(g) : frontier_error(ws);
     if (s != RR_OK) return s;
     a.ctl = ws.x_bar.as<uint32_t>();
     uint32_t *d = nullptr;

@@ -546,6 +546,8 @@ bool frontier_fits(const Graph &g, Workspace &ws, uint32_t k, uint64_t budget, b
 rr_status frontier_reserve(Workspace &ws, cudaStream_t st);
 // RR_ETIMEDOUT, once, when a bounded wait of a finished query on ws gave up.
 rr_status frontier_error(Workspace &ws);
+// The same for the graph's own workspace and its lanes'.
+rr_status frontier_error(const Graph &g);
 // Copies a query's results to host buffers (either may be null).
 rr_status copy_out(const uint64_t *d_w, uint64_t *h_w, uint64_t n, const uint8_t *d_b, uint8_t *h_b, uint64_t nb, cudaStream_t st);
 rr_status frontier_load(Graph &g, cudaStream_t st);

@@ -136,3 +136,42 @@ def test_argument_errors(graph):
         with pytest.raises(capi.RRError) as ei:
             capi.rr_debug_frontier(G.handle, *args)
         assert ei.value.status == capi.RR_EINVAL
+
+
+def test_queries_on_lanes_are_reported_once(graph):
+    # at-most-k whose own scratch cannot be had runs its queries on lanes, which
+    # take the frontier engine where a single query's scratch can be had
+    import torch
+    g, G = graph
+    k, n = 7, g["n"]
+    d_w = torch.zeros((k - 1, n), dtype=torch.int64, device="cuda")
+
+    def atmost():
+        before = capi.rr_kernel_launches()
+        capi.rr_reach_atmost_device(G.handle, 3, k, 11, d_w)
+        torch.cuda.synchronize()
+        return capi.rr_kernel_launches() - before
+
+    def launches(scratch):
+        capi.rr_debug_frontier(G.handle, 0, 0, scratch)
+        return atmost()
+
+    want = launches(0) and d_w.cpu().numpy()
+    lo, hi = 1, 1 << 34  # the least scratch for which at-most-k is one launch
+    while lo < hi:
+        mid = (lo + hi) // 2
+        lo, hi = (lo, mid) if launches(mid) == 1 else (mid + 1, hi)
+    assert launches(lo) == 1 and launches(lo - 1) == k - 1  # one frontier query a lane
+    assert np.array_equal(d_w.cpu().numpy(), want)
+    d_r = torch.zeros(n, dtype=torch.int32, device="cuda")
+    for call in (atmost, lambda: capi.rr_reach_bounded_device(G.handle, 3, k, 11, d_r)):
+        for again in (atmost, lambda: usable(g, G)):
+            capi.rr_debug_frontier(G.handle, LIMIT, 1, lo - 1)
+            call()
+            torch.cuda.synchronize()
+            capi.rr_debug_frontier(G.handle, 0, 0, lo - 1)
+            with pytest.raises(capi.RRError) as ei:
+                again()
+            assert ei.value.status == capi.RR_ETIMEDOUT
+            usable(g, G)
+            assert atmost() == k - 1 and np.array_equal(d_w.cpu().numpy(), want)
