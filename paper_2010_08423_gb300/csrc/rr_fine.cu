@@ -47,6 +47,16 @@ __global__ void k_arrival_bitmap(uint32_t n, const uint32_t *__restrict__ R, uin
     }
 }
 
+// Per-edge sums and arrival times cleared for a query that is still wanted.
+__global__ void __launch_bounds__(256) k_clear_unless(const uint32_t *skip, uint64_t *__restrict__ E, uint64_t m,
+                                                      uint32_t *__restrict__ R, uint32_t n)
+{
+    if (*skip) return;
+    const uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x, step = (uint64_t)gridDim.x * blockDim.x;
+    for (uint64_t i = t; i < m; i += step) E[i] = 0;
+    for (uint64_t i = t; i < n; i += step) R[i] = 0xFFFFFFFFu;
+}
+
 // What an extraction has chosen so far (device): the vertex and time its next
 // step goes back from, the step's best candidate, and the path. fail: 1 the
 // target has no arrival, 2 a step found no candidate; later steps do nothing.
@@ -168,23 +178,29 @@ __global__ void k_merge_rows(uint32_t n, uint32_t k, const uint32_t *__restrict_
 }
 
 rr_status arrival_device(const Graph &g, const rr_query *q, uint64_t *d_witness, uint64_t *d_E,
-                         uint32_t *d_R, uint8_t *d_bitmap, cudaStream_t st, const uint8_t *d_vmask)
+                         uint32_t *d_R, uint8_t *d_bitmap, cudaStream_t st, const uint8_t *d_vmask,
+                         const uint32_t *d_skip)
 {
-    return arrival_on(g, g.ws, q, d_witness, d_E, d_R, d_bitmap, st, d_vmask, 0);
+    return arrival_on(g, g.ws, q, d_witness, d_E, d_R, d_bitmap, st, d_vmask, 0, 0, d_skip);
 }
 
 rr_status arrival_on(const Graph &g, Workspace &ws, const rr_query *q, uint64_t *d_witness,
                      uint64_t *d_E, uint32_t *d_R, uint8_t *d_bitmap, cudaStream_t st,
-                     const uint8_t *d_vmask, uint64_t budget, uint32_t bfirst)
+                     const uint8_t *d_vmask, uint64_t budget, uint32_t bfirst, const uint32_t *d_skip)
 {
     rr_status xs = RR_OK;
     if (!bfirst && frontier_fits(g, ws, q->k, budget, false, false, true, &xs)) {
         // frontier engine: the arrival times from the out rows alone; the
         // per-edge sums only when the caller wants them
         if (xs != RR_OK) return xs;
-        if (d_E && g.m) RR_CUDA(cudaMemsetAsync(d_E, 0, (size_t)g.m * 8, st));
-        RR_CUDA(cudaMemsetAsync(d_R, 0xFF, (size_t)g.n * 4, st));
-        xs = frontier_query(g, ws, q, false, nullptr, d_witness, st, d_E, d_vmask, d_R);
+        if (d_skip) {
+            k_clear_unless<<<grid_for(std::max<uint64_t>(g.m, g.n), 256), 256, 0, st>>>(d_skip, d_E, d_E ? g.m : 0, d_R, g.n);
+            RR_LAUNCHED();
+        } else {
+            if (d_E && g.m) RR_CUDA(cudaMemsetAsync(d_E, 0, (size_t)g.m * 8, st));
+            RR_CUDA(cudaMemsetAsync(d_R, 0xFF, (size_t)g.n * 4, st));
+        }
+        xs = frontier_query(g, ws, q, false, nullptr, d_witness, st, d_E, d_vmask, d_R, nullptr, d_skip);
         if (xs != RR_OK) return xs;
         if (d_bitmap) {
             k_arrival_bitmap<<<grid_for((g.n + 7) / 8, 256), 256, 0, st>>>(g.n, d_R, d_bitmap);
@@ -232,10 +248,13 @@ rr_status arrival_on(const Graph &g, Workspace &ws, const rr_query *q, uint64_t 
 // arrival time; each further query, for one vertex fewer on the graph without
 // the chosen vertices (and, for motif queries, without their colours in M),
 // certifies the next vertex back. The choices stay on the device, so a plain
-// extraction is one sequence of launches with one wait at its end (k = 7 on
-// n = 20,011: 436 us with four waits a step, 240 us so); a motif query's next
-// motif needs the vertex on the host, one wait a step. Synchronous on the
-// graph's stream.
+// extraction on the frontier engine is one sequence of launches with one wait at
+// its end (k = 7 on n = 20,011: 436 us with four waits a step, 216 us so), and its
+// queries are called off once there is nothing to extract (k = 8 from a hub of
+// n = 2e5, m = 2e6: 1,011 us to a reachable vertex, 315 us -- the first query and
+// the launches -- to an unreachable one). A motif query's next motif needs the
+// vertex on the host, one wait a step; so do the engines over sieve points, whose
+// queries cannot be called off. Synchronous on the graph's stream.
 rr_status extract_path(const Graph &g, const rr_query *q, uint32_t target, uint32_t *vertices,
                        uint32_t *edges, uint32_t *times)
 {
@@ -258,10 +277,15 @@ rr_status extract_path(const Graph &g, const rr_query *q, uint32_t target, uint3
         M.erase(it);
         return RR_OK;
     };
+    bool ahead = !q->motif;  // whether steps are enqueued before the one before them is known
+    for (uint32_t kk = 2; ahead && kk <= k; ++kk) ahead = uses_frontier(g, kk);
+    rr_status xs = RR_OK;
+    ahead = ahead && frontier_fits(g, ws, k, 0, false, false, true, &xs);
+    if (xs != RR_OK) return xs;
     auto run = [&](uint32_t kk, const uint8_t *mask) -> rr_status {
         rr_query qq{q->source, kk, q->seed, q->motif ? M.data() : nullptr};
         return arrival_device(g, &qq, ws.S.as<uint64_t>(), ws.edges.as<uint64_t>(),
-                              ws.arrival.as<uint32_t>(), nullptr, st, mask);
+                              ws.arrival.as<uint32_t>(), nullptr, st, mask, ahead && kk < k ? &ds->fail : nullptr);
     };
     auto step = [&](uint32_t ell) -> rr_status {
         k_extract_step<<<38, 256, 0, st>>>(ds, ell, g.off.as<uint32_t>(), g.row_t.as<uint32_t>(),
@@ -288,13 +312,9 @@ rr_status extract_path(const Graph &g, const rr_query *q, uint32_t target, uint3
     if (s != RR_OK) return s;
     k_extract_begin<<<1, 1, 0, st>>>(ds, ws.arrival.as<uint32_t>(), target, k, vm);
     RR_LAUNCHED();
-    uint32_t cur = target;
     for (uint32_t ell = k - 1; ell >= 2; --ell) {
-        if (q->motif) {
-            if ((s = look()) != RR_OK) return s;
-            if (ell < k - 1) cur = hs.cur;
-            if ((s = drop_colour(cur)) != RR_OK) return s;
-        }
+        if (!ahead && (s = look()) != RR_OK) return s;
+        if (q->motif && (s = drop_colour(hs.cur)) != RR_OK) return s;
         if ((s = run(ell, vm)) != RR_OK) return s;
         if ((s = step(ell)) != RR_OK) return s;
     }

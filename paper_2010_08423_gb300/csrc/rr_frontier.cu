@@ -1959,6 +1959,7 @@ k_frontier(const __grid_constant__ XArgs a_, const __grid_constant__ XOne one_, 
     __shared__ __align__(16) XOne o;
     __shared__ uint32_t next;
     __shared__ Meetings meet;
+    if (!BATCH && a_.skip && *a_.skip) return;  // (an earlier kernel's: the same for every block)
     copy_params(&a, &a_, sizeof(XArgs));
     __syncthreads();
     if (threadIdx.x == 0) meet = Meetings{};
@@ -2609,10 +2610,10 @@ rr_status copy_out(const uint64_t *d_w, uint64_t *h_w, uint64_t n, const uint8_t
 
 // One query on st. every: witness rows of k' = 2..k (plain queries); d_R: the
 // minimum arrival times (n per witness row, set to UINT32_MAX by the caller).
-// src: a set of sources.
+// src: a set of sources. d_skip: a device word that calls the query off when set.
 rr_status frontier_query(const Graph &g, Workspace &ws, const rr_query *q, bool every, uint8_t *d_bitmap,
                          uint64_t *d_witness, cudaStream_t st, uint64_t *d_E, const uint8_t *d_vmask, uint32_t *d_R,
-                         const SourceSet *src)
+                         const SourceSet *src, const uint32_t *d_skip)
 {
     XArgs a{};
     x_args(g, a);
@@ -2633,6 +2634,7 @@ rr_status frontier_query(const Graph &g, Workspace &ws, const rr_query *q, bool 
         Q.nslist = src->count;
     }
     a.nq = 1;
+    a.skip = d_skip;
     a.scratch = ws.state.as<uint8_t>();
     a.lanes = 1;
     a.szero = d_witness;

@@ -106,6 +106,7 @@ struct XArgs {
     const uint32_t *ooff;  // edges by (tail, time): offsets (n + 1),
     const uint4 *orec;     // head, time, input index, first edge that may follow
     const uint32_t *olen;  // and how many
+    const uint32_t *skip;  // set: the query is not wanted any more (or null)
     uint32_t smem;         // dynamic shared memory of a block
     uint32_t tiny;         // try every query in one block's shared memory first
 };

@@ -557,7 +557,7 @@ rr_status frontier_out_records(Graph &g, const uint32_t *d_time, const uint32_t 
 rr_status frontier_query(const Graph &g, Workspace &ws, const rr_query *q, bool every, uint8_t *d_bitmap,
                          uint64_t *d_witness, cudaStream_t st, uint64_t *d_E = nullptr,
                          const uint8_t *d_vmask = nullptr, uint32_t *d_R = nullptr,
-                         const SourceSet *src = nullptr);
+                         const SourceSet *src = nullptr, const uint32_t *d_skip = nullptr);
 
 // Held (under the graph's lock) by every call that uses the graph's scratch:
 // the call's stream first waits for the previous such call's work, and the
@@ -584,14 +584,16 @@ struct ScratchOrder {
 // D as a bitmap (or null); d_vmask deletes vertices.
 rr_status arrival_device(const Graph &g, const rr_query *q, uint64_t *d_witness, uint64_t *d_E,
                          uint32_t *d_R, uint8_t *d_bitmap, cudaStream_t st,
-                         const uint8_t *d_vmask = nullptr);
+                         const uint8_t *d_vmask = nullptr, const uint32_t *d_skip = nullptr);
 // The fine-grained query on workspace `ws` (budget as reach_on_stream).
 // bfirst > 0: also the at-most-k branches k' = bfirst..k-1 (reach_v2), their
 // witnesses, per-edge sums and minimum arrivals in ws.bS / ws.bE / ws.bR at
-// row k' - bfirst.
+// row k' - bfirst. d_skip (the frontier engine only): a device word that calls the
+// query off when it is set.
 rr_status arrival_on(const Graph &g, Workspace &ws, const rr_query *q, uint64_t *d_witness,
                      uint64_t *d_E, uint32_t *d_R, uint8_t *d_bitmap, cudaStream_t st,
-                     const uint8_t *d_vmask, uint64_t budget, uint32_t bfirst = 0);
+                     const uint8_t *d_vmask, uint64_t budget, uint32_t bfirst = 0,
+                     const uint32_t *d_skip = nullptr);
 // Bounded RestlessReach: minimum arrival over k' = 2..k, shortest length, D.
 rr_status atmost_arrival_device(const Graph &g, uint32_t source, uint32_t k, uint64_t seed,
                                 uint32_t *d_R, uint8_t *d_L, uint8_t *d_bitmap, cudaStream_t st);
