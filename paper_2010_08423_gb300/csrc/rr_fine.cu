@@ -59,7 +59,8 @@ __global__ void __launch_bounds__(256) k_clear_unless(const uint32_t *skip, uint
 
 // What an extraction has chosen so far (device): the vertex and time its next
 // step goes back from, the step's best candidate, and the path. fail: 1 the
-// target has no arrival, 2 a step found no candidate; later steps do nothing.
+// target has no arrival, 2 a step found no candidate, 3 the last step no edge from
+// the source (no sums that hold lead there); later steps do nothing.
 struct ExtractState {
     unsigned long long best;
     uint32_t cur, tc, fail, done;
@@ -126,7 +127,7 @@ __global__ void k_extract_step(ExtractState *st, uint32_t ell, const uint32_t *_
     st->done = 0;
     st->best = ~0ull;
     if (best == ~0ull) {
-        st->fail = 2;
+        st->fail = ell == 1 ? 3u : 2u;
         return;
     }
     const uint32_t r = (uint32_t)best;
@@ -304,6 +305,7 @@ rr_status extract_path(const Graph &g, const rr_query *q, uint32_t target, uint3
         if (hs.fail == 1) return fail(RR_ENOPATH, "rr_extract_path: the target has no arrival");
         if (hs.fail == 2)
             return fail(RR_ENOPATH, "rr_extract_path: a step's polynomials vanished (probability <= (3k-1)/2^64)");
+        if (hs.fail == 3) return fail(RR_ECUDA, "rr_extract_path: no source edge at the chosen time");
         return RR_OK;
     };
 
