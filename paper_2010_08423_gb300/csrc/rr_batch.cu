@@ -1149,11 +1149,12 @@ rr_status autotune_batch(Graph &g, const rr_query *qs, uint32_t nq, uint32_t *mi
     RR_CUDA(cudaEventCreate(&e1));
     const uint32_t save[3] = {g.batch_minb, g.batch_ranges, g.batch_max_chunk};
     // the candidates are shapes of the persistent kernel: keep the batch on it
-    // while they are timed (afterwards the frontier engine takes what it can)
+    // while they are timed (afterwards, unless rr_set_batch_tuning chose a shape,
+    // the frontier engine takes what it can)
     struct Forced {
-        bool &f;
-        explicit Forced(bool &x) : f(x) { f = true; }
-        ~Forced() { f = false; }
+        bool &f, saved;
+        explicit Forced(bool &x) : f(x), saved(x) { f = true; }
+        ~Forced() { f = saved; }
     } forced(g.batch_forced);
     uint32_t best[3] = {0, 0, 0};
     float best_ms = 1e30f;
