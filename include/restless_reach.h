@@ -142,6 +142,9 @@ typedef struct {
  * words) are part of a query's scratch and, unlike the per-point state, do not
  * shrink with the point chunk: a server whose per-slot budget cannot hold them
  * for its largest k refuses to start (RR_ENOMEM); bit 2 avoids that.
+ * The arrays of whole queries without sieve points take up to 56 bytes an edge;
+ * a graph that fits the device only without them is loaded without, and its
+ * queries run over sieve points.
  * Errors: RR_EINVAL for n == 0, m >= 2^31, an endpoint >= n or a self-loop;
  * RR_ENOMEM / RR_ECUDA on device failure (nothing is leaked). */
 rr_status rr_graph_load(uint32_t n, uint64_t m, const uint32_t *src, const uint32_t *dst,

@@ -246,7 +246,8 @@ __global__ void k_v2_scatter3(const uint32_t *__restrict__ row_dst, const uint32
         if (c4[r]) {
             const uint32_t i = rank4[r] - 1;
             T.head[i] = row_dst[r]; T.eid[i] = row_eid[r]; T.src[i] = row_src[r];
-            T.a3[i] = a3[r]; T.b3[i] = b3[r]; T.time[i] = row_t[r];
+            T.a3[i] = a3[r]; T.b3[i] = b3[r];
+            if (T.time) T.time[i] = row_t[r];
         }
     }
 }
@@ -276,12 +277,12 @@ __global__ void k_v2_scatter(const uint32_t *__restrict__ row_dst, const uint32_
         if (c0[r]) {
             const uint32_t i = rank0[r] - 1;
             W.head[i] = h; W.eid[i] = e; W.src[i] = u; W.a0[i] = a0[r]; W.b0[i] = b0[r];
-            W.time[i] = row_t[r];
+            if (W.time) W.time[i] = row_t[r];
         }
         if (c2[r]) {
             const uint32_t i = rank2[r] - 1;
             T.head[i] = h; T.eid[i] = e; T.src[i] = u; T.a1[i] = a1[r]; T.b1[i] = b1[r];
-            T.time[i] = row_t[r];
+            if (T.time) T.time[i] = row_t[r];
         }
     }
 }
@@ -397,8 +398,8 @@ static cudaError_t reserve_parts(DevBuf &all, std::initializer_list<std::pair<Pa
 
 // Builds the reduced-state engine's row lists (rr_internal.h, RowList) from
 // the windows [row_lo, row_hi), the head of every row and the true producer
-// flags (rows inside some window).
-rr_status build_lists_v2(Graph &g, const uint32_t *row_dst, const uint32_t *tprod, cudaStream_t st)
+// flags (rows inside some window). frontier: with the times its engine reads.
+rr_status build_lists_v2(Graph &g, const uint32_t *row_dst, const uint32_t *tprod, bool frontier, cudaStream_t st)
 {
     const uint64_t m = g.m;
     Part c0, c1, c2, rank_p, rank0, rank1, rank2, a0, b0, a1, b1;
@@ -442,7 +443,7 @@ rr_status build_lists_v2(Graph &g, const uint32_t *row_dst, const uint32_t *tpro
             RR_CUDA(R.a1.reserve(bytes));
             RR_CUDA(R.b1.reserve(bytes));
         }
-        if (i >= 2) RR_CUDA(R.time.reserve(bytes));
+        if (frontier && i >= 2) RR_CUDA(R.time.reserve(bytes));
         out[i] = ListOut{R.head.as<uint32_t>(), R.eid.as<uint32_t>(), R.src.as<uint32_t>(),
                          R.a0.as<uint32_t>(), R.b0.as<uint32_t>(), R.a1.as<uint32_t>(),
                          R.b1.as<uint32_t>(), nullptr, nullptr, R.time.as<uint32_t>()};
@@ -479,7 +480,8 @@ rr_status build_lists_v2(Graph &g, const uint32_t *row_dst, const uint32_t *tpro
         const size_t db = (size_t)std::max<uint32_t>(1, c3[0]) * 4;
         const size_t tb = (size_t)std::max<uint32_t>(1, c3[1]) * 4;
         for (DevBuf *b : {&D.head, &D.eid, &D.src, &D.a1, &D.b1, &D.a3, &D.b3}) RR_CUDA(b->reserve(db));
-        for (DevBuf *b : {&T.head, &T.eid, &T.src, &T.a3, &T.b3, &T.time}) RR_CUDA(b->reserve(tb));
+        for (DevBuf *b : {&T.head, &T.eid, &T.src, &T.a3, &T.b3}) RR_CUDA(b->reserve(tb));
+        if (frontier) RR_CUDA(T.time.reserve(tb));
         ListOut od{D.head.as<uint32_t>(), D.eid.as<uint32_t>(), D.src.as<uint32_t>(), nullptr, nullptr,
                    D.a1.as<uint32_t>(), D.b1.as<uint32_t>(), D.a3.as<uint32_t>(), D.b3.as<uint32_t>(), nullptr};
         ListOut ot{T.head.as<uint32_t>(), T.eid.as<uint32_t>(), T.src.as<uint32_t>(), nullptr, nullptr,
@@ -610,40 +612,35 @@ rr_status build_lists_v2(Graph &g, const uint32_t *row_dst, const uint32_t *tpro
     return RR_OK;
 }
 
-rr_status graph_load(uint32_t n, uint64_t m, const uint32_t *src, const uint32_t *dst,
-                     const uint32_t *t, const uint32_t *delta, const uint8_t *color,
-                     uint32_t flags, rr_graph **out)
-{
-    if (!out) return fail(RR_EINVAL, "rr_graph_load: out is NULL");
-    *out = nullptr;
-    if (n == 0) return fail(RR_EINVAL, "rr_graph_load: n must be >= 1");
-    if (m >= (1ull << 31)) return fail(RR_EINVAL, "rr_graph_load: m must be < 2^31");
-    if (m && (!src || !dst || !t)) return fail(RR_EINVAL, "rr_graph_load: NULL edge array");
-    if (!delta) return fail(RR_EINVAL, "rr_graph_load: NULL delta");
-    uint32_t times = 0;
-    for (uint64_t e = 0; e < m; ++e) {
-        times |= t[e];
-        if (src[e] >= n || dst[e] >= n)
-            return fail(RR_EINVAL, "rr_graph_load: endpoint >= n at edge " + std::to_string(e));
-        if (src[e] == dst[e])
-            return fail(RR_EINVAL, "rr_graph_load: self-loop at edge " + std::to_string(e));
+// A graph that was not loaded to its end.
+struct DropGraph {
+    void operator()(rr_graph *g) const
+    {
+        if (g->stream) {
+            cudaStreamSynchronize(g->stream);
+            cudaStreamDestroy(g->stream);
+        }
+        delete g;
     }
+};
 
+// times: all times or-ed together; frontier: with the frontier engine's arrays.
+static rr_status load_graph(uint32_t n, uint64_t m, const uint32_t *src, const uint32_t *dst, const uint32_t *t,
+                            const uint32_t *delta, const uint8_t *color, uint32_t flags, uint32_t times, bool frontier,
+                            rr_graph **out)
+{
     rr_graph *g = new rr_graph();
-    std::unique_ptr<rr_graph> guard(g);
+    std::unique_ptr<rr_graph, DropGraph> guard(g);
     RR_CUDA(cudaGetDevice(&g->dev));
     g->n = n;
     g->m = m;
     g->has_colors = color != nullptr;
     g->compact = !(flags & 1u);
-    if ((flags & 6u) == 6u) return fail(RR_EINVAL, "rr_graph_load: flags turn the pair-label layer 3 both on and off");
     g->pair_force = (flags & 2u) ? 2u : ((flags & 4u) ? 1u : 0u);
-    if ((flags & 24u) == 24u) return fail(RR_EINVAL, "rr_graph_load: flags turn the head-factor table both on and off");
     g->head_table_force = (flags & 8u) ? 2u : ((flags & 16u) ? 1u : 0u);
     g->pair_tail_off = (flags & 32u) != 0;
     g->k4_per_point = (flags & 256u) != 0;
     g->k5_closed = (flags & 512u) != 0;
-    if ((flags & 192u) == 192u) return fail(RR_EINVAL, "rr_graph_load: flags turn the at-most-k branches both on and off");
     g->atmost_branches = (flags & 128u) ? 2u : ((flags & 64u) ? 1u : 0u);
     RR_CUDA(cudaStreamCreateWithFlags(&g->stream, cudaStreamNonBlocking));
     cudaStream_t st = g->stream;
@@ -670,9 +667,6 @@ rr_status graph_load(uint32_t n, uint64_t m, const uint32_t *src, const uint32_t
     DevBuf d_delta;
     RR_CUDA(d_delta.reserve((size_t)n * 4));
     RR_CUDA(cudaMemcpyAsync(d_delta.p, delta, (size_t)n * 4, cudaMemcpyHostToDevice, st));
-    // (load flags that keep every query on the per-point engine: nothing of the
-    // frontier engine's)
-    const bool frontier = g->compact && !g->point_flags;
     if (frontier) {
         rr_status os = frontier_out_reserve(*g);
         if (os != RR_OK) return os;
@@ -786,7 +780,7 @@ rr_status graph_load(uint32_t n, uint64_t m, const uint32_t *src, const uint32_t
         g->state_rows = 1ull + last_rank;
         g->window_rows = nonempty;
         g->producer_window_rows = prod_window;
-        rr_status ls = build_lists_v2(*g, g->row_head.as<uint32_t>(), tprod.as<uint32_t>(), st);
+        rr_status ls = build_lists_v2(*g, g->row_head.as<uint32_t>(), tprod.as<uint32_t>(), frontier, st);
         if (ls != RR_OK) return ls;
     }
 
@@ -818,6 +812,40 @@ rr_status graph_load(uint32_t n, uint64_t m, const uint32_t *src, const uint32_t
     RR_CUDA(cudaStreamSynchronize(st));
     *out = guard.release();
     return RR_OK;
+}
+
+rr_status graph_load(uint32_t n, uint64_t m, const uint32_t *src, const uint32_t *dst,
+                     const uint32_t *t, const uint32_t *delta, const uint8_t *color,
+                     uint32_t flags, rr_graph **out)
+{
+    if (!out) return fail(RR_EINVAL, "rr_graph_load: out is NULL");
+    *out = nullptr;
+    if (n == 0) return fail(RR_EINVAL, "rr_graph_load: n must be >= 1");
+    if (m >= (1ull << 31)) return fail(RR_EINVAL, "rr_graph_load: m must be < 2^31");
+    if (m && (!src || !dst || !t)) return fail(RR_EINVAL, "rr_graph_load: NULL edge array");
+    if (!delta) return fail(RR_EINVAL, "rr_graph_load: NULL delta");
+    uint32_t times = 0;
+    for (uint64_t e = 0; e < m; ++e) {
+        times |= t[e];
+        if (src[e] >= n || dst[e] >= n)
+            return fail(RR_EINVAL, "rr_graph_load: endpoint >= n at edge " + std::to_string(e));
+        if (src[e] == dst[e])
+            return fail(RR_EINVAL, "rr_graph_load: self-loop at edge " + std::to_string(e));
+    }
+
+    if ((flags & 6u) == 6u) return fail(RR_EINVAL, "rr_graph_load: flags turn the pair-label layer 3 both on and off");
+    if ((flags & 24u) == 24u) return fail(RR_EINVAL, "rr_graph_load: flags turn the head-factor table both on and off");
+    if ((flags & 192u) == 192u) return fail(RR_EINVAL, "rr_graph_load: flags turn the at-most-k branches both on and off");
+    // load flags that keep every query on the engines over sieve points: nothing of
+    // the frontier engine's; nor where the device cannot hold that as well (up to
+    // 56 bytes an edge)
+    const bool frontier = !flags;
+    rr_status s = load_graph(n, m, src, dst, t, delta, color, flags, times, frontier, out);
+    if (s == RR_ENOMEM && frontier) {
+        clear_error();
+        s = load_graph(n, m, src, dst, t, delta, color, flags, times, false, out);
+    }
+    return s;
 }
 
 }  // namespace rr
