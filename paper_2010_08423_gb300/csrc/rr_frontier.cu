@@ -2581,22 +2581,33 @@ __global__ void __launch_bounds__(256) k_copy_out(const uint64_t *__restrict__ w
     }
 }
 
-// The device address of pinned host memory, or null.
+// The device address of `count` values in pinned host memory, or null: also where
+// their last byte is not pinned with the first (a registered range that ends inside
+// the caller's buffer) or they are not aligned as the kernel stores them. Those are
+// for the copy engine, whose checks are the runtime's.
 template <class T>
-static T *pinned(T *p)
+static T *pinned(T *p, uint64_t count)
 {
-    cudaPointerAttributes at{};
-    if (!p || cudaPointerGetAttributes(&at, p) != cudaSuccess) {
-        cudaGetLastError();
-        return nullptr;
+    if (!p || !count || reinterpret_cast<uintptr_t>(p) % sizeof(T)) return nullptr;
+    const void *const ends[2] = {p, reinterpret_cast<const uint8_t *>(p + count) - 1};
+    void *dev[2] = {nullptr, nullptr};
+    for (int i = 0; i < 2; ++i) {
+        cudaPointerAttributes at{};
+        if (cudaPointerGetAttributes(&at, ends[i]) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        if (at.type != cudaMemoryTypeHost || !at.devicePointer) return nullptr;
+        dev[i] = at.devicePointer;
     }
-    return at.type == cudaMemoryTypeHost ? static_cast<T *>(at.devicePointer) : nullptr;
+    if (static_cast<uint8_t *>(dev[1]) - static_cast<uint8_t *>(dev[0]) != (ptrdiff_t)(count * sizeof(T) - 1)) return nullptr;
+    return static_cast<T *>(dev[0]);
 }
 
 rr_status copy_out(const uint64_t *d_w, uint64_t *h_w, uint64_t n, const uint8_t *d_b, uint8_t *h_b, uint64_t nb, cudaStream_t st)
 {
-    uint64_t *const pw = pinned(h_w);
-    uint8_t *const pb = pinned(h_b);
+    uint64_t *const pw = pinned(h_w, n);
+    uint8_t *const pb = pinned(h_b, nb);
     if ((h_w && !pw) || (h_b && !pb) || n * 8 > kCopyOutMax) {
         if (h_w) RR_CUDA(cudaMemcpyAsync(h_w, d_w, n * 8, cudaMemcpyDeviceToHost, st));
         if (h_b) RR_CUDA(cudaMemcpyAsync(h_b, d_b, nb, cudaMemcpyDeviceToHost, st));

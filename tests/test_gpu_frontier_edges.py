@@ -201,3 +201,18 @@ def test_calls_whose_scratch_cannot_be_had(k, scratch):
                 assert np.array_equal(capi.rr_query_poll(srv, t, n)[2], want[-3][i]), i
         finally:
             capi.rr_server_destroy(srv)
+
+
+@pytest.mark.parametrize("ow", [1, 4, 7])
+def test_results_into_unaligned_pinned_buffers(ow):
+    # witness words that do not begin on a word's boundary: the copy engine's
+    import torch
+    g = W.uniform(2001, 30_000, 40, 0, 6, 5)
+    n, nb = g["n"], 251
+    raw = torch.full((8 * n + 16,), 99, dtype=torch.uint8, pin_memory=True).numpy()
+    b = torch.full((nb,), 99, dtype=torch.uint8, pin_memory=True).numpy()
+    with capi.Graph(g) as G:
+        b1, w1 = G.reach(1, 5, 3)
+        G.reach(1, 5, 3, out=(b, raw[ow:ow + 8 * n].view(np.uint64)))
+    assert np.array_equal(raw[ow:ow + 8 * n].copy().view(np.uint64), w1) and np.array_equal(b, b1) and w1.any()
+    assert (raw[:ow] == 99).all() and (raw[ow + 8 * n:] == 99).all()
