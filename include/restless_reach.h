@@ -461,6 +461,13 @@ rr_status rr_debug_wait_probe(uint64_t timeout_ns, int32_t abort_preset, int32_t
  * Call it while no query on the graph is queued or running. RR_EINVAL for a NULL
  * graph, a limit above 10 s, absent > 2. Not part of the paper's method. */
 rr_status rr_debug_frontier(rr_graph *g, uint64_t wait_ns, uint32_t absent, uint64_t scratch);
+/* rr_debug_levels: how the last whole query (atmost: at-most-k) of k vertices on
+ * `g` that did not fit one block was laid out, if no other call on the graph came
+ * after it: *count lists of rows (at most 32), five numbers each in out (HOST):
+ * level, whether its rows end walks, rows, rows per block of prefix sums, whether
+ * the sums of all blocks were completed. Synchronous. RR_EINVAL for a NULL argument
+ * or a k that has no such query. Not part of the paper's method. */
+rr_status rr_debug_levels(const rr_graph *g, uint32_t k, int32_t atmost, uint32_t *out, uint32_t *count);
 /* rr_debug_draw: out[i] = draw(key, first + i) on the device, HOST out. */
 rr_status rr_debug_draw(uint64_t key, uint64_t first, uint64_t count, uint64_t *out);
 

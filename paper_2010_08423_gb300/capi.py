@@ -83,6 +83,7 @@ EXPORTED = [
     "rr_reach_arrival_device", "rr_extract_path", "rr_reach_sources_device", "rr_bench_gf_mul",
     "rr_debug_wait_probe", "rr_reach_bounded_device", "rr_reach_range_device",
     "rr_autotune_batch", "rr_set_batch_tuning", "rr_get_batch_tuning", "rr_debug_frontier",
+    "rr_debug_levels",
 ]
 
 _lib = None
@@ -120,6 +121,7 @@ def load(build_if_missing: bool = True):
         "rr_extract_path": [vp, pq, u32, vp, vp, vp],
         "rr_bench_gf_mul": [u32, u32, u32, vp, ctypes.POINTER(u64), vp],
         "rr_debug_frontier": [vp, u64, u32, u64],
+        "rr_debug_levels": [vp, u32, i32, vp, ctypes.POINTER(u32)],
         "rr_debug_wait_probe": [u64, i32, ctypes.POINTER(i32), ctypes.POINTER(u64)],
         "rr_reach_sources_device": [vp, vp, u32, u32, u64, vp, vp, vp, vp, vp],
         "rr_server_create": [vp, u64, u32, ctypes.POINTER(vp)],
@@ -321,6 +323,13 @@ def rr_debug_frontier(g, wait_ns: int = 0, absent: int = 0, scratch: int = 0):
     """Limit of the waits inside a whole query's kernel, the meeting its last block misses, the
     largest scratch of a query it takes."""
     _check(load().rr_debug_frontier(g, int(wait_ns), int(absent), int(scratch)))
+
+
+def rr_debug_levels(g, k, atmost=False):
+    """[(level, ends walks, rows, rows per block, sums completed)] of the last whole query of k vertices."""
+    out, count = np.zeros((32, 5), dtype=np.uint32), ctypes.c_uint32()
+    _check(load().rr_debug_levels(g, int(k), 1 if atmost else 0, _hp(out), ctypes.byref(count)))
+    return [tuple(int(x) for x in r) for r in out[:count.value]]
 
 
 def rr_bench_gf_mul(blocks, threads, iters, d_sink, stream=None) -> int:

@@ -440,6 +440,15 @@ rr_status rr_debug_frontier(rr_graph *g, uint64_t wait_ns, uint32_t absent, uint
     return RR_OK;
 }
 
+rr_status rr_debug_levels(const rr_graph *g, uint32_t k, int32_t atmost, uint32_t *out, uint32_t *count)
+{
+    clear_error();
+    if (!g || !out || !count) return fail(RR_EINVAL, "rr_debug_levels: NULL argument");
+    std::lock_guard<std::mutex> lk(g->mu);
+    if (!uses_frontier(*g, k)) return fail(RR_EINVAL, "rr_debug_levels: no such query");
+    return frontier_levels(*g, k, atmost != 0, out, count);
+}
+
 rr_status rr_bench_gf_mul(uint32_t blocks, uint32_t threads, uint32_t iters, uint64_t *d_sink,
                           uint64_t *mults, void *stream)
 {

@@ -404,7 +404,7 @@ __device__ __forceinline__ uint32_t rank_below(const uint2 *rank, uint32_t x)
 struct XShape {
     uint32_t team, rows, scan;  // team: log2
 };
-__device__ __forceinline__ XShape x_shape_of(uint32_t s) { return XShape{s & 0xffu, (s >> 8) & 0xffu, s >> 16}; }
+__host__ __device__ __forceinline__ XShape x_shape_of(uint32_t s) { return XShape{s & 0xffu, (s >> 8) & 0xffu, s >> 16}; }
 __host__ __device__ __forceinline__ uint32_t x_item_bytes(uint32_t rows, uint32_t K, const XLL &X)
 {
     return X.out ? rows * (K * 8u + 8u + 64u) : rows * (K * (4u * kSplit) + (X.cin + X.cout + X.uout) * 8u + 64u);
@@ -988,7 +988,7 @@ __device__ __forceinline__ void xor_shared(uint64_t *p, uint64_t v)
 // 1,024, 4,096, 16,384 blocks on: arrival, k = 8, 269, 258, 248, 248 us; bounded,
 // k = 8, 368, 368, 353, 353 us; at-most-k, k = 10, on n = 1e6, m = 1e7 4.15, 4.15,
 // 4.14, 4.15 ms, and 4.45 ms by the average alone.
-__device__ __forceinline__ bool x_scans(const XTmpl &t, uint32_t li)
+__host__ __device__ __forceinline__ bool x_scans(const XTmpl &t, uint32_t li)
 {
     const XShape sh = x_shape_of(t.shape[li]);
     if (!sh.scan || t.ll[li].level >= t.maxlev) return false;
@@ -2654,6 +2654,37 @@ rr_status frontier_query(const Graph &g, Workspace &ws, const rr_query *q, bool 
     a.bzero_n = d_bitmap ? (g.n + 7) / 8 : 0;
     a.tiny = g_timing.load(std::memory_order_relaxed) ? 0u : 1u;
     return one.t.wide ? x_launch<false, true>(g, a, one, st) : x_launch<false, false>(g, a, one, st);
+}
+
+// The level lists of the last single query of k vertices that took the passes on
+// the graph's workspace: level, whether an out level, needed rows, rows per block,
+// whether its prefix sums were completed. Synchronous.
+rr_status frontier_levels(const Graph &g, uint32_t k, bool every, uint32_t *out, uint32_t *count)
+{
+    XList lists[kXLists];
+    x_lists(g, lists);
+    XTmpl t;
+    if (x_template(lists, k, every, false, false, t) > g.ws.state.bytes) return fail(RR_EINVAL, "rr_debug_levels: no such query");
+    RR_CUDA(cudaDeviceSynchronize());
+    uint32_t cnt[kXMaxLL], shape[kXMaxLL];
+    unsigned long long span[kXMaxLL];
+    auto host = [&](auto &p, auto *h) {
+        const cudaError_t e = cudaMemcpy(h, g.ws.state.as<uint8_t>() + (reinterpret_cast<uint64_t>(p) - 1u), t.nll * sizeof *h, cudaMemcpyDeviceToHost);
+        p = h;
+        return e;
+    };
+    RR_CUDA(host(t.cnt, cnt));
+    RR_CUDA(host(t.shape, shape));
+    RR_CUDA(host(t.span, span));
+    for (uint32_t li = 0; li < t.nll; ++li, out += 5) {
+        out[0] = t.ll[li].level;
+        out[1] = t.ll[li].out;
+        out[2] = cnt[li];
+        out[3] = cnt[li] ? x_shape_of(shape[li]).rows : 0u;
+        out[4] = cnt[li] && !t.ll[li].out && x_scans(t, li) ? 1u : 0u;
+    }
+    *count = t.nll;
+    return RR_OK;
 }
 
 // A batch in one launch: the queries' descriptions go to the device with one

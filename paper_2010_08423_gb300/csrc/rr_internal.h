@@ -551,6 +551,7 @@ rr_status frontier_error(const Graph &g);
 // Copies a query's results to host buffers (either may be null).
 rr_status copy_out(const uint64_t *d_w, uint64_t *h_w, uint64_t n, const uint8_t *d_b, uint8_t *h_b, uint64_t nb, cudaStream_t st);
 rr_status frontier_load(Graph &g, cudaStream_t st);
+rr_status frontier_levels(const Graph &g, uint32_t k, bool every, uint32_t *out, uint32_t *count);
 rr_status frontier_out_reserve(Graph &g);
 rr_status frontier_out_records(Graph &g, const uint32_t *d_time, const uint32_t *d_dst, const uint32_t *d_eid,
                                const uint32_t *d_delta, cudaStream_t st);

@@ -216,3 +216,66 @@ def test_results_into_unaligned_pinned_buffers(ow):
         G.reach(1, 5, 3, out=(b, raw[ow:ow + 8 * n].view(np.uint64)))
     assert np.array_equal(raw[ow:ow + 8 * n].copy().view(np.uint64), w1) and np.array_equal(b, b1) and w1.any()
     assert (raw[:ow] == 99).all() and (raw[ow + 8 * n:] == 99).all()
+
+
+def hub_reads(k, p, sparse, dense, wide):
+    """Edges p + 1 of the walks from vertex 0 are sparse + dense ones into a hub; each sparse one is read
+    by a window of its own, and `wide` windows read all the dense ones. 300 edges of 0 lead nowhere (too
+    many for one block)."""
+    rows, readers = sparse + dense, sparse + wide
+    chain, mid, hub = np.arange(p), p + np.arange(rows), p + rows
+    out = hub + 1 + np.arange(readers)
+    tail = out[-1] + 1 + np.arange(k)
+    dead = tail[-1] + 1 + np.arange(300)
+    t0, left = 200 + 20 * sparse, k - 3 - p  # the dense times; edges after the readers
+    td = np.sort(np.random.default_rng([k, p, sparse, dense]).integers(t0, t0 + 10, dense))
+    parts = [(chain[:-1], chain[1:], np.zeros(p - 1)), (np.full(rows, chain[-1]), mid, np.zeros(rows)),
+             (mid, np.full(rows, hub), np.concatenate([100 + 20 * np.arange(sparse), td])),
+             (np.full(readers, hub), out, np.concatenate([105 + 20 * np.arange(sparse), np.full(wide, t0 + 9)])),
+             (np.zeros(300), dead, np.zeros(300))]
+    if left >= 1:
+        parts += [(out, np.full(readers, tail[0]), np.full(readers, t0 + 20)),
+                  (tail[:left - 1], tail[1:left], t0 + 21 + np.arange(left - 1))]
+    delta = np.full(int(dead[-1]) + 1, t0 + 1000)
+    delta[hub] = 10
+    return graph_of(*(np.concatenate([x[i] for x in parts]) for i in range(3)), delta)
+
+
+@pytest.mark.parametrize("k,p,sparse,dense,wide,blocks,completed", [
+    (4, 1, 10, 20, 2, (16, 47), 0), (5, 1, 10, 37, 2, (16, 47), 0),        # sums over 16 blocks
+    (4, 1, 60, 60, 1, (48, 255), 0), (5, 1, 60, 60, 1, (48, 255), 0),
+    (4, 1, 800, 1000, 3, (256, 4095), 0), (5, 1, 800, 1000, 3, (256, 4095), 0),  # over 256
+    (12, 3, 6000, 6000, 3, (256, 4095), 0),
+    (4, 1, 60, 1000, 60, (256, 4095), 1), (5, 1, 60, 1000, 60, (256, 4095), 1),  # completed: wide on average
+    (4, 1, 100_000, 100_000, 3, (4096, 1 << 31), 1), (5, 1, 100_000, 100_000, 3, (4096, 1 << 31), 1),  # or long
+    (12, 4, 14_000, 500, 3, (4096, 1 << 31), 1)])
+def test_sums_over_blocks_and_completed_ones(k, p, sparse, dense, wide, blocks, completed):
+    # (from 4,096 blocks on, sums are completed wherever a level's rows are not
+    # nearly all of its list's)
+    g = hub_reads(k, p, sparse, dense, wide)
+    with capi.Graph(g) as G, capi.Graph(g, capi.FLAG_DENSE_STATE) as H:
+        b, w = G.reach(0, k, 3)
+        level, ends, rows, per, done = capi.rr_debug_levels(G.handle, k)[p]  # (one list a level)
+        assert (level, ends, rows) == (p + 1, 0, sparse + dense)
+        assert blocks[0] <= -(-rows // per) <= blocks[1] and done == completed
+        b1, w1 = H.reach(0, k, 3)
+        assert np.array_equal(w, w1) and np.array_equal(b, b1) and w.any()
+
+
+@pytest.mark.parametrize("k", [2, 3, 4, 5, 6, 9, 12, 14, 16])
+@pytest.mark.parametrize("dmax", [6, 25])
+def test_every_size_finds_a_planted_path(k, dmax):
+    # ragged sizes, a path of k vertices laid into the graph (its colours the
+    # motif): a non-zero witness in every combination
+    g = W.uniform(301, 3_007 if k < 14 else 1_201, 60, 0, dmax, 900 + k, ncolors=3)
+    rng = np.random.default_rng([k, dmax])
+    path = rng.choice(301, size=k, replace=False)
+    rows = rng.choice(len(g["src"]), size=k - 1, replace=False)
+    g["src"][rows], g["dst"][rows], g["t"][rows] = path[:-1], path[1:], 20 + np.arange(k - 1)
+    g["delta"][path] = np.maximum(g["delta"][path], 1)
+    s, end = int(path[0]), int(path[-1])
+    with capi.Graph(g) as G, capi.Graph(g, capi.FLAG_DENSE_STATE) as H:
+        for m in (None, g["color"][path]):
+            b, w = G.reach(s, k, 77 + k, motif=m)
+            b1, w1 = H.reach(s, k, 77 + k, motif=m)
+            assert np.array_equal(w, w1) and np.array_equal(b, b1) and w[end]
