@@ -793,9 +793,8 @@ __device__ __noinline__ bool x_plan(const XArgs &a, const XOne &o, View &v)
     for (uint32_t li = 0; li < nll; ++li) {
         const XLL &X = t.ll[li];
         const XList &L = a.lists[X.list];
-        const bool window = X.level > 1;
         const uint2 *const rank = X.rank, *const below = t.ll[X.prev].rank;
-        if (!window) {
+        if (X.level == 1) {
             // layer 1: few rows in long lists, a word per lane
             const uint32_t steps1 = (L.words + 31u) / 32u;
             for (uint32_t i = View::first_item(base, gw, nw); i < steps1; i += nw) {
@@ -829,10 +828,8 @@ __device__ __noinline__ bool x_plan(const XArgs &a, const XOne &o, View &v)
                 if (!((word >> lane) & 1u)) {
                     at[x] = 0xffffffffu;
                 } else {
-                    if (window) {
-                        lo[x] = L.lo[r];
-                        hi[x] = L.hi[r];
-                    }
+                    lo[x] = L.lo[r];
+                    hi[x] = L.hi[r];
                     m[x].z = L.eid[r];
                     m[x].w = L.src[r];
                     if (X.mhead) hd[x] = L.head[r];
@@ -841,7 +838,7 @@ __device__ __noinline__ bool x_plan(const XArgs &a, const XOne &o, View &v)
 #pragma unroll
             for (uint32_t x = 0; x < U; ++x) {
                 m[x].x = m[x].y = 0;
-                if (window && at[x] != 0xffffffffu) {
+                if (at[x] != 0xffffffffu) {
                     m[x].x = rank_below(below, lo[x]);
                     m[x].y = rank_below(below, hi[x]);
                     span += m[x].y - m[x].x;
@@ -856,7 +853,7 @@ __device__ __noinline__ bool x_plan(const XArgs &a, const XOne &o, View &v)
                 }
         }
         base += steps;
-        if (window && __any_sync(0xffffffffu, span != 0)) {
+        if (__any_sync(0xffffffffu, span != 0)) {
 #pragma unroll
             for (int f = 16; f > 0; f >>= 1) span += __shfl_xor_sync(0xffffffffu, (unsigned long long)span, f);
             if (lane == 0) atomicAdd(t.span + X.prev, (unsigned long long)span);
