@@ -1071,7 +1071,8 @@ rr_status atmost_device(const Graph &g, uint32_t source, uint32_t k, uint64_t se
 {
     {
         // frontier engine: the k query's rows, values on the first k' - 1 labels
-        // and one out level per k' (k = 10 from a hub of n = 1e6, m = 1e7: 24.5 -> 3.3 ms)
+        // and one out level per k' (k = 10 from a hub of n = 1e6, m = 1e7, three graphs:
+        // 26.9-31.1 -> 3.5-4.3 ms)
         const rr_query q{source, k, seed, nullptr};
         rr_status fs = RR_OK;
         if (frontier_fits(g, g.ws, k, 0, true, false, false, &fs))

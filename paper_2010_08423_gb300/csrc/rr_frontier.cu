@@ -26,12 +26,13 @@
 // Why. On a Chung-Lu graph with n = 1e6, m = 1e7 the sieve-point engine
 // multiplies 1,024 points for each of 330,000 rows at each layer of a k = 10
 // query; walks from the source that reach the last layer pass 1,400 to 62,000
-// of them per layer, with at most 126 values each. Measured against that engine:
-//   motif, k = 10, n = 1e6, m = 1e7                 20.8 -> 0.68 ms a query
-//   from a hub, k = 12, n = 2e5, m = 2e6            30.9 -> 1.02 ms
-//   dense contacts, k = 12, n = 2,000, m = 30,011   4.53 -> 0.19 ms
-//   uniform, k = 8, n = 1e5, m = 1e6                52 -> 25 us (a handful of rows)
-//   n = 1,000, m = 10,000, k = 5                    27 -> 18 us
+// of them per layer, with at most 126 values each. Measured against that engine
+// on three graphs of each kind (how many rows matter differs several times over):
+//   motif, k = 10, n = 1e6, m = 1e7                 23.1-26.8 -> 0.36-1.07 ms a query
+//   from a hub, k = 12, n = 2e5, m = 2e6            24.7-41.4 -> 0.61-1.31 ms
+//   contacts, k = 12, n = 2,000, m = 30,011         4.4-4.7 -> 0.19 ms
+//   uniform, k = 8, n = 1e5, m = 1e6                52-60 -> 25 us (a handful of rows)
+//   n = 1,000, m = 10,000, k = 5                    26-27 -> 19 us
 // What bounds it now: with many rows the products (issue slots of the integer
 // multiplies and XORs: 257 cycles per warp product and scheduler, the loop alone),
 // with few the chain of layers, some 45 grid barriers of 1.6 us at k = 12, and in
