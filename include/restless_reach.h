@@ -171,7 +171,8 @@ rr_status rr_reach_sync(const rr_graph *g, const rr_query *q, uint8_t *bitmap,
  * device, for the previous such call's work. A query whose kernel gave up a
  * bounded wait is reported as RR_ETIMEDOUT by rr_reach_sync itself, in a batch
  * by the query's d_status, for other calls that only enqueue (a batch without
- * d_status too) once by a later call on the graph, which then enqueues nothing. */
+ * d_status too) once by a later call on the graph, which then enqueues nothing (a
+ * batch with d_status goes ahead and leaves the report to another call). */
 rr_status rr_reach_device(const rr_graph *g, const rr_query *q, uint8_t *d_bitmap,
                           uint64_t *d_witness, void *stream);
 

@@ -2534,12 +2534,13 @@ rr_status frontier_error(const Graph &g)
     return s;
 }
 
-static rr_status x_control(const Graph &g, Workspace &ws, cudaStream_t st, XArgs &a)
+// report: an earlier call's expired wait is this call's to report.
+static rr_status x_control(const Graph &g, Workspace &ws, cudaStream_t st, bool report, XArgs &a)
 {
     a.limit = g.x_wait_ns;
     a.absent = g.x_absent;
     rr_status s = frontier_reserve(ws, st);
-    if (s == RR_OK) s = &ws == &g.ws ? frontier_error(g) : frontier_error(ws);
+    if (s == RR_OK && report) s = &ws == &g.ws ? frontier_error(g) : frontier_error(ws);
     if (s != RR_OK) return s;
     a.ctl = ws.x_bar.as<uint32_t>();
     uint32_t *d = nullptr;
@@ -2626,7 +2627,7 @@ rr_status frontier_query(const Graph &g, Workspace &ws, const rr_query *q, bool 
 {
     XArgs a{};
     x_args(g, a);
-    rr_status s = x_control(g, ws, st, a);
+    rr_status s = x_control(g, ws, st, true, a);
     if (s != RR_OK) return s;
     XOne one;
     x_template(a.lists, q->k, every, src != nullptr, d_R != nullptr, one.t);
@@ -2742,7 +2743,9 @@ bool frontier_batch(const Graph &g, const rr_query *qs, uint32_t nq, std::vector
             return RR_EAGAIN;
         }
         RR_CUDA(e);
-        rr_status s = x_control(g, ws, st, a);
+        // (with statuses a batch tells of itself alone: a server's tickets do not fail
+        // for another call's wait)
+        rr_status s = x_control(g, ws, st, !d_status, a);
         if (s != RR_OK) return s;
         RR_CUDA(B.xq.reserve(tbytes + qbytes));
         RR_CUDA(B.left.reserve((size_t)count * 4));

@@ -61,6 +61,12 @@ def test_an_enqueued_query_is_reported_once(graph):
         call()
         torch.cuda.synchronize()
         capi.rr_debug_frontier(G.handle)
+        # a batch with statuses is not refused for it, and leaves it to the next call
+        b_w = torch.zeros((1, g["n"]), dtype=torch.int64, device="cuda")
+        b_s = torch.full((1,), -1, dtype=torch.int32, device="cuda")
+        capi.rr_reach_batch_device(G.handle, [{"source": 3, "k": 5, "seed": 11, "motif": None}], b_w, None, b_s)
+        torch.cuda.synchronize()
+        assert int(b_s) == 0 and np.array_equal(b_w[0].cpu().numpy().view(np.uint64), oracle.sieve(g, 3, 5, 11))
         with pytest.raises(capi.RRError) as ei:
             capi.rr_reach_device(G.handle, 3, 5, 11, d_w)
         assert ei.value.status == capi.RR_ETIMEDOUT
