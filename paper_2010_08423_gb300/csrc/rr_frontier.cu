@@ -1957,7 +1957,6 @@ k_frontier(const __grid_constant__ XArgs a_, const __grid_constant__ XOne one_, 
     __shared__ __align__(16) XOne o;
     __shared__ uint32_t next;
     __shared__ Meetings meet;
-    if (!BATCH && a_.skip && *a_.skip) return;  // (an earlier kernel's: the same for every block)
     copy_params(&a, &a_, sizeof(XArgs));
     __syncthreads();
     if (threadIdx.x == 0) meet = Meetings{};
@@ -2006,6 +2005,10 @@ k_frontier(const __grid_constant__ XArgs a_, const __grid_constant__ XOne one_, 
         } else if (blockIdx.x == 0) {
             copy_params(&o.q, &one_.q, sizeof(XQuery));
             __syncthreads();
+            if (a.skip) {  // called off: no walks (an exit at the kernel's start cost every query 0.5 %)
+                if (threadIdx.x == 0 && *a.skip) o.q.dead = 1;
+                __syncthreads();
+            }
             const int r = x_tiny(a, o.q, one_.t.every, grid, cleared);
             ok = r != kTinyFailed;
             left = r == kTinyNoFit ? 1u : 0u;
