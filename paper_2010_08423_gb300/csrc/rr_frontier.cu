@@ -304,16 +304,25 @@ __host__ __device__ __forceinline__ uint32_t x_sum_words(uint32_t words)
     const uint32_t a = x_sum_level(words), b = x_sum_level(a);
     return a + b + x_sum_level(b);
 }
+// Where a level's summaries lie (X.sums: in 256-byte groups, from 1): S, then F.
+struct XSums {
+    uint32_t *S, *F;
+};
+__device__ __forceinline__ XSums x_sums(const XTmpl &t, const XLL &X)
+{
+    uint32_t *const S = reinterpret_cast<uint32_t *>(t.clear) + (size_t)(X.sums - 1u) * 64u;
+    return XSums{S, S + x_sum_words(X.words)};
+}
 // The summaries of a level's A (the upper two were cleared): a warp a word of the first.
-__device__ __forceinline__ void sum_level(const XLL &X, uint32_t gw, uint32_t nw)
+__device__ __forceinline__ void sum_level(const XLL &X, uint32_t *S, uint32_t gw, uint32_t nw)
 {
     const uint32_t lane = threadIdx.x & 31u, n1 = (X.words + 31u) / 32u, l1 = x_sum_level(X.words);
-    uint32_t *const S2 = X.S + l1, *const S3 = S2 + x_sum_level(l1);
+    uint32_t *const S2 = S + l1, *const S3 = S2 + x_sum_level(l1);
     for (uint32_t i = gw; i < n1; i += nw) {
         const uint32_t w = i * 32u + lane;
         const uint32_t on = __ballot_sync(0xffffffffu, w < X.words && X.A[w] != 0);
         if (lane == 0) {
-            X.S[i] = on;
+            S[i] = on;
             if (on) {
                 const uint32_t b2 = 1u << (i & 31u), b3 = 1u << ((i >> 5) & 31u);
                 if (!(__ldcg(S2 + (i >> 5)) & b2)) atomicOr(S2 + (i >> 5), b2);
@@ -598,7 +607,7 @@ __device__ __noinline__ bool x_plan(const XArgs &a, const XOne &o, View &v)
                     if (hi[x] <= lo[x]) act[x] = false;
                     else if (first == last) act[x] = (fw[x] & m0 & m1) != 0;
                     else if ((fw[x] & m0) || (lw[x] & m1)) act[x] = true;
-                    else if (WIDE && P.S && last - first > kLongWords) act[x] = any_long(Ap, P.S, P.words, first + 1u, last);
+                    else if (WIDE && P.sums && last - first > kLongWords) act[x] = any_long(Ap, x_sums(t, P).S, P.words, first + 1u, last);
                     else act[x] = any_words(Ap, first + 1u, last);
                 }
                 if (check) {
@@ -634,8 +643,8 @@ __device__ __noinline__ bool x_plan(const XArgs &a, const XOne &o, View &v)
             lmax = l - 1;
             break;
         }
-        if (const XLL &X = t.ll[t.runs[l].first]; WIDE && l < t.maxlev && X.S) {  // (the store level comes first)
-            sum_level(X, gw, nw);
+        if (const XLL &X = t.ll[t.runs[l].first]; WIDE && l < t.maxlev && X.sums) {  // (the store level comes first)
+            sum_level(X, x_sums(t, X).S, gw, nw);
             if (!v.sync()) return false;
         }
     }
@@ -645,9 +654,9 @@ __device__ __noinline__ bool x_plan(const XArgs &a, const XOne &o, View &v)
     // backward: the rows of layer l - 1 in the window of a needed row of layer l
     // (at-most-k: every layer has outputs, every active row is needed)
     // Word w of level X's N, with what the long windows need whole.
-    auto needed = [](const XLL &X, uint32_t w) {
+    auto needed = [&t](const XLL &X, uint32_t w) {
         uint32_t m = X.N[w];
-        if (WIDE && X.F && covered(X.F, X.words, w)) X.N[w] = m = X.A[w];
+        if (WIDE && X.sums && covered(x_sums(t, X).F, X.words, w)) X.N[w] = m = X.A[w];
         return m;
     };
     if (!t.every)
@@ -687,8 +696,8 @@ __device__ __noinline__ bool x_plan(const XArgs &a, const XOne &o, View &v)
                     if (b1 == b0) m[x] &= last;
                     if (m[x] & ~have[x]) atomicOr(Np + b0, m[x]);
                     uint32_t w = b0 + 1;
-                    if (WIDE && P.F && b1 - b0 > kLongWords) {
-                        mark_long(P.F, P.words, w, b1);
+                    if (WIDE && P.sums && b1 - b0 > kLongWords) {
+                        mark_long(x_sums(t, P).F, P.words, w, b1);
                         w = b1;
                     }
                     for (; w <= b1; ++w) {
@@ -699,7 +708,7 @@ __device__ __noinline__ bool x_plan(const XArgs &a, const XOne &o, View &v)
             }
             if (!v.sync()) return false;
         }
-    if (const XLL &X = t.ll[t.runs[1].first]; WIDE && X.F) {  // (the other levels' words were completed on the way)
+    if (const XLL &X = t.ll[t.runs[1].first]; WIDE && !t.every && X.sums) {  // (the other levels' words were completed on the way)
         for (uint32_t w = gt; w < X.words; w += nt) needed(X, w);
         if (!v.sync()) return false;
     }
@@ -1884,8 +1893,6 @@ __device__ __forceinline__ void relocate(XTmpl &t, uint8_t *base)
         XLL &x = t.ll[i];
         fix(x.A);
         fix(x.N);
-        fix(x.S);
-        fix(x.F);
         fix(x.rank);
         fix(x.tsum);
         fix(x.meta);
@@ -2224,20 +2231,19 @@ rr_status frontier_load(Graph &g, cudaStream_t st)
 
 static void x_lists(const Graph &g, XList *out)
 {
-    auto set = [&](uint32_t id, const RowList &L, const uint32_t *lo, const DevBuf &hi, uint32_t longest) {
+    auto set = [&](uint32_t id, const RowList &L, const uint32_t *lo, const DevBuf &hi) {
         out[id] = XList{L.head.as<uint32_t>(), L.eid.as<uint32_t>(), L.src.as<uint32_t>(), lo,
-                        hi.as<uint32_t>(), L.time.as<uint32_t>(), (uint32_t)L.count, (uint32_t)(L.count / 32 + 1), longest};
+                        hi.as<uint32_t>(), L.time.as<uint32_t>(), (uint32_t)L.count, (uint32_t)(L.count / 32 + 1)};
     };
-    // (in the order of frontier_load's windows)
-    set(kXProd, g.prod_list, g.prod_list.w0, g.prod_list.a0, 0);
-    set(kXState, g.state_list, g.state_list.w0, g.state_list.a0, g.x_longest[0]);
-    set(kXDeep1, g.deep_list, g.deep_list.w1, g.deep_list.a1, g.x_longest[2]);
-    set(kXDeep3, g.deep_list, g.deep_list.w3, g.deep_list.a3, g.x_longest[4]);
-    set(kXWin, g.win_list, g.win_list.w0, g.win_list.a0, g.x_longest[1]);
-    set(kXTail, g.tail_list, g.tail_list.w1, g.tail_list.a1, g.x_longest[3]);
-    set(kXTail3, g.tail3_list, g.tail3_list.w3, g.tail3_list.a3, g.x_longest[5]);
+    set(kXProd, g.prod_list, g.prod_list.w0, g.prod_list.a0);
+    set(kXState, g.state_list, g.state_list.w0, g.state_list.a0);
+    set(kXDeep1, g.deep_list, g.deep_list.w1, g.deep_list.a1);
+    set(kXDeep3, g.deep_list, g.deep_list.w3, g.deep_list.a3);
+    set(kXWin, g.win_list, g.win_list.w0, g.win_list.a0);
+    set(kXTail, g.tail_list, g.tail_list.w1, g.tail_list.a1);
+    set(kXTail3, g.tail3_list, g.tail3_list.w3, g.tail3_list.a3);
     out[kXAll] = XList{g.row_head.as<uint32_t>(), g.row_eid.as<uint32_t>(), g.row_src.as<uint32_t>(), nullptr, nullptr,
-                       g.row_t.as<uint32_t>(), (uint32_t)g.m, (uint32_t)(g.m / 32 + 1), 0};
+                       g.row_t.as<uint32_t>(), (uint32_t)g.m, (uint32_t)(g.m / 32 + 1)};
 }
 
 // Bump allocation of the scratch: offsets + 1 in place of addresses.
@@ -2265,9 +2271,11 @@ static uint32_t x_out_list(uint32_t l)
 // out level k-1 (every = false) or out levels 1..k-1 (every = true: at-most-k),
 // and their scratch. multi: a set of sources, all k labels, subsets larger by
 // one. Returns the scratch's bytes.
-static uint64_t x_template(const XList *lists, uint32_t k, bool every, bool multi, bool arrivals, XTmpl &t)
+static uint64_t x_template(const Graph &g, const XList *lists, uint32_t k, bool every, bool multi, bool arrivals, XTmpl &t)
 {
     std::memset(&t, 0, sizeof t);
+    // (by list: x_longest is in the order of frontier_load's windows)
+    const uint32_t *const w = g.x_longest, longest[kXLists] = {0, w[0], w[2], w[4], w[1], w[3], w[5], 0};
     const uint32_t sh = multi ? 1u : 0u, K = k - 1 + sh;
     t.maxlev = k - 1;
     t.every = every ? 1u : 0u;
@@ -2303,11 +2311,10 @@ static uint64_t x_template(const XList *lists, uint32_t k, bool every, bool mult
             if (!t.ll[i].out) t.ll[i].N = b.take<uint32_t>(t.ll[i].words);
     for (uint32_t i = 0; i < t.nll; ++i) {  // levels read by long windows
         const XLL &x = t.ll[i];
-        if (x.level < 2 || lists[x.list].longest <= kWideWords * 32u || t.ll[x.prev].S) continue;
         XLL &p = t.ll[x.prev];
-        t.wide = 1;
-        p.S = b.take<uint32_t>(x_sum_words(p.words));
-        if (!every) p.F = b.take<uint32_t>(x_sum_words(p.words));
+        if (x.level < 2 || longest[x.list] <= kWideWords * 32u || p.sums) continue;
+        p.sums = (uint32_t)(b.used / 256 + 1);
+        b.take<uint32_t>((uint64_t)x_sum_words(p.words) * (every ? 1 : 2));
     }
     t.clear4 = (uint32_t)(b.used / 16);
     uint64_t ping[2] = {0, 0}, ipw[2] = {0, 0}, supw = 0;
@@ -2352,6 +2359,12 @@ static uint64_t x_template(const XList *lists, uint32_t k, bool every, bool mult
     t.shape = b.take<uint32_t>(t.nll);
     t.span = b.take<unsigned long long>(t.nll);
     return b.used;
+}
+
+// Whether some level has summaries.
+static bool x_wide(const XTmpl &t)
+{
+    return std::any_of(t.ll, t.ll + t.nll, [](const XLL &x) { return x.sums != 0; });
 }
 
 static void x_args(const Graph &g, XArgs &a)
@@ -2450,7 +2463,7 @@ uint64_t frontier_bytes(const Graph &g, uint32_t k, bool every, bool multi, bool
     XList lists[kXLists];
     x_lists(g, lists);
     XTmpl t;
-    return x_template(lists, k, every, multi, arrivals, t);
+    return x_template(g, lists, k, every, multi, arrivals, t);
 }
 
 bool frontier_fits(const Graph &g, Workspace &ws, uint32_t k, uint64_t budget, bool every, bool multi, bool arrivals,
@@ -2633,7 +2646,7 @@ rr_status frontier_query(const Graph &g, Workspace &ws, const rr_query *q, bool 
     rr_status s = x_control(g, ws, st, true, a);
     if (s != RR_OK) return s;
     XOne one;
-    x_template(a.lists, q->k, every, src != nullptr, d_R != nullptr, one.t);
+    x_template(g, a.lists, q->k, every, src != nullptr, d_R != nullptr, one.t);
     x_query(g, *q, src != nullptr, true, one.q);
     XQuery &Q = one.q;
     Q.S = d_witness;
@@ -2655,7 +2668,7 @@ rr_status frontier_query(const Graph &g, Workspace &ws, const rr_query *q, bool 
     a.bzero = d_bitmap;
     a.bzero_n = d_bitmap ? (g.n + 7) / 8 : 0;
     a.tiny = g_timing.load(std::memory_order_relaxed) ? 0u : 1u;
-    return one.t.wide ? x_launch<false, true>(g, a, one, st) : x_launch<false, false>(g, a, one, st);
+    return x_wide(one.t) ? x_launch<false, true>(g, a, one, st) : x_launch<false, false>(g, a, one, st);
 }
 
 // The level lists of the last single query of k vertices that took the passes on
@@ -2666,7 +2679,7 @@ rr_status frontier_levels(const Graph &g, uint32_t k, bool every, uint32_t *out,
     XList lists[kXLists];
     x_lists(g, lists);
     XTmpl t;
-    if (x_template(lists, k, every, false, false, t) > g.ws.state.bytes) return fail(RR_EINVAL, "rr_debug_levels: no such query");
+    if (x_template(g, lists, k, every, false, false, t) > g.ws.state.bytes) return fail(RR_EINVAL, "rr_debug_levels: no such query");
     RR_CUDA(cudaDeviceSynchronize());
     uint32_t cnt[kXMaxLL], shape[kXMaxLL];
     unsigned long long span[kXMaxLL];
@@ -2712,13 +2725,13 @@ bool frontier_batch(const Graph &g, const rr_query *qs, uint32_t nq, std::vector
         std::vector<XTmpl> tm(kXMaxLabels + 2);
         for (uint32_t k = 2; k <= kXMaxLabels + 1; ++k)
             if (used[k]) {
-                const uint64_t need = x_template(a.lists, k, false, false, false, tm[k]);  // (whole 256-byte groups)
+                const uint64_t need = x_template(g, a.lists, k, false, false, false, tm[k]);  // (whole 256-byte groups)
                 if (need > budget) {
                     used[k] = fits = false;
                     continue;
                 }
                 stride = std::max(stride, need);
-                wide |= tm[k].wide != 0;
+                wide |= x_wide(tm[k]);
             }
         if (!fits) idx.erase(std::remove_if(idx.begin(), idx.end(), [&](uint32_t i) { return !used[qs[i].k]; }), idx.end());
         if (idx.empty()) return RR_EAGAIN;

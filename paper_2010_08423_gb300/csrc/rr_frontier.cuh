@@ -21,7 +21,6 @@ struct XList {
     const uint32_t *head, *eid, *src, *lo, *hi, *time;
     uint32_t count;
     uint32_t words;  // bitmap words: count / 32 + 1
-    uint32_t longest;  // rows of the longest window
 };
 enum XListId : uint32_t {
     kXProd = 0, kXState = 1, kXDeep1 = 2, kXDeep3 = 3, kXWin = 4, kXTail = 5, kXTail3 = 6, kXAll = 7, kXLists = 8
@@ -52,9 +51,8 @@ struct XLL {
     uint32_t list, level, prev, out;  // prev: the store level below (itself at level 1)
     uint32_t d, cin, cout, uout;      // d: subset size of the values; cin / cout: values read / kept per row;
                                       // uout: store levels below an out level: values kept for it per row
-    uint32_t words, row, ipcap, pad;  // row: out levels' witness row
+    uint32_t words, row, ipcap, sums; // row: out levels' witness row; sums: summaries, in the template's `clear` (x_sums)
     uint32_t *A, *N;                  // active rows, needed rows (bitmaps)
-    uint32_t *S, *F;                  // levels read by long windows: A's words with a row, words needed whole (x_sum_words)
     uint2 *rank;                      // per word of N: the word and the needed rows before it
     uint32_t *tsum;                   // rows per scan tile (256)
     uint4 *meta;                      // per needed row: window [x, y) in needed rows of prev, edge, tail
@@ -72,7 +70,6 @@ struct XRun {
 // The levels of a k-vertex query and their scratch.
 struct XTmpl {
     uint32_t nll, maxlev, clear4, every;
-    uint32_t wide, pad;    // wide: some level has summaries (S)
     uint4 *clear;          // needed-row bitmaps and summaries to clear
     uint32_t *cnt;         // per level list: needed rows
     uint32_t *shape;       // per level list: log2 warps per team | rows per item << 8 | scanned << 16
